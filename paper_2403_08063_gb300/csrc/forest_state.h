@@ -145,8 +145,8 @@ struct mg_forest {
     double omega = 0.8;                       // damping of the Jacobi smoother
     int *kerr = nullptr;                      // set by a device wait that gave up (staged smoother)
     double *AinvT = nullptr;                  // transpose of the coarsest inverses (adjoint cycles)
-    int32_t *gj_piv = nullptr, *gj_src = nullptr;  // device Gauss-Jordan: pivot rows, column permutation
-    double *gj_pinv = nullptr;                 // and the current pivot's reciprocal, per problem
+    double *gj_panel = nullptr;                // device Gauss-Jordan: the eliminated panel, its row exchanges
+    int32_t *gj_src = nullptr, *gj_org = nullptr;  // and the composed row origins (two buffers)
     cudaGraphExec_t coarse_graph = nullptr;    // recorded coarsest-level probe + inversion (assemble_coarse)
     int coarse_runs = 0;                       // calls of assemble_coarse so far
     bool coarse_nograph = false;               // its recording failed: launched directly
@@ -250,6 +250,10 @@ octmg::TailArgs tail_args(mg_forest *F);  // tail.cu: the forest's recorded tail
 // groups' tail arguments (device), with a grid of at most `need` CTAs
 mg_status launch_batch_tail32(mg_forest *const *groups, const octmg::TailArgs *args, const octmg::BatchEntry *entries,
                               int ne, unsigned *bar, int64_t need);
+// gauss_jordan.cu: inverses of the coarsest operators (input buffer, panel width, launches)
+double *gj_input(mg_forest *F, int maxN);
+int gj_width(int maxN);
+void enqueue_gauss_jordan(mg_forest *F, int maxN);
 int64_t tail_ctas(mg_forest *F);  // tail.cu: CTAs the largest phase of F's tail can use
 // solver.cu: one FP32 V-cycle in two parts around a joint tail: part 1 the steps down to the tail level's entry,
 // part 2 the steps after the tail (0: the whole cycle, its tail launched as usual)

@@ -1,0 +1,276 @@
+// Inversion of the coarsest-level operators (this library's direct coarsest solver), every problem's dense block at once:
+// in-place Gauss-Jordan elimination with partial pivoting, W columns (a panel) per step.
+//
+// One step on panel columns J = [c0, c0 + W): eliminating them one after another inside the panel alone leaves in it the
+// columns J of the product M of the W elementary transformations (in-place elimination stores exactly those; the other
+// columns of M are the identity's).  So the panel is eliminated first, by one thread-block cluster per problem that holds
+// it in distributed shared memory (k_gj_panel), and the W transformations then reach the rest of the matrix as one
+// product of rank W over the whole GPU (k_gj_update):
+//     Y[r, j] = (r in J ? 0 : X[src r, j]) + sum_w M[r, J_w] X[src J_w, j]   (j not in J),   Y[:, J] = M[:, J],
+// with src the row exchanges of the panel.  After all panels the matrix holds (P A)^-1 = A^-1 P^T for the exchanges P,
+// and org[r] the row of A that ended in row r, so A^-1[:, org r] is column r.
+//
+// What bounds it: the chain of N pivot searches (2.2 us each with 512 unknowns, 3.3 us with 1728: one cluster barrier, one
+// block barrier, a division, and the panel's update on the 2 FP64 FMA per clock of each of the cluster's SMs), then the
+// FP64 rate in the update (N^3 FMA in all: with 1728 unknowns 83.5 us per panel, 0.57 T FMA/s of the 0.63 measured).
+// Elimination of one column per step with two launches per column (every element rewritten each time) took 4.85 ms for
+// 512 unknowns and 58 ms for 1728 (three root blocks per axis); this takes 1.5 ms and 14.8 ms.
+#include <cooperative_groups.h>
+
+#include "forest_state.h"
+
+namespace octmg {
+namespace {
+namespace cg = cooperative_groups;
+
+constexpr int kGjCluster = 8;  // CTAs that share a panel's rows (the portable cluster size)
+constexpr int kGjThreads = 256;
+constexpr int kGjTile = 32;    // the update's output tile edge
+
+// One candidate pivot row of a panel column, as each CTA of the cluster receives it.
+template <int W>
+struct GjCand {
+    uint64_t key;   // magnitude bits + 1 (0: none): non-negative binary64 values order as their bits
+    double rcp;     // 1 / pivot
+    double row[W];  // the row's panel entries
+    int32_t r, id;  // its row and the row of the matrix it came from
+};
+template <int W>
+struct GjRow {
+    double row[W];
+    int32_t id;
+};
+
+// Rows of a problem held by one CTA, and its dynamic shared memory: rows x W doubles (rounded up to whole passes of the
+// CTA) and the rows' origins.
+__host__ __device__ constexpr int gj_rows(int N) { return (N + kGjCluster - 1) / kGjCluster; }
+__host__ __device__ constexpr int64_t gj_panel_elems(int N, int W) {
+    return (static_cast<int64_t>(gj_rows(N)) * W + kGjThreads - 1) / kGjThreads * kGjThreads;
+}
+constexpr int64_t gj_smem(int N, int W) { return gj_panel_elems(N, W) * 8 + static_cast<int64_t>(gj_rows(N)) * 4; }
+
+// Eliminates panel columns c0 .. c0 + W - 1 of every problem with more than c0 unknowns, one cluster per problem, rows
+// dealt out in contiguous chunks.  Per column one cluster barrier: before it each CTA sends the others its best pivot
+// candidate with the whole panel row and the reciprocal, and the owner of the diagonal row sends that one; after it every
+// CTA picks the same winner (largest magnitude, lowest row on ties) and updates its rows.  Messages alternate between two
+// buffers: a CTA that writes a buffer again has passed a barrier that every reader of it reached afterwards.  A thread
+// keeps one column of the panel (W divides the CTA); the W threads of a row share a warp, so the multiplier comes by
+// shuffle.  A zero or non-finite pivot sets *bad and the elimination goes on with the diagonal row.
+template <int W>
+__global__ void __cluster_dims__(kGjCluster, 1, 1) __launch_bounds__(kGjThreads)
+    k_gj_panel(const double *__restrict__ A, const int64_t *__restrict__ moff, const int64_t *__restrict__ ustart, int c0,
+               double *__restrict__ panel, int32_t *__restrict__ src, int *__restrict__ bad) {
+    extern __shared__ __align__(16) unsigned char gj_raw[];
+    __shared__ GjCand<W> cand[2][kGjCluster];
+    __shared__ GjRow<W> diag[2];
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int p = blockIdx.x / kGjCluster, rank = static_cast<int>(cluster.block_rank());
+    const int N = static_cast<int>(ustart[p + 1] - ustart[p]);
+    if (c0 >= N) return;  // uniform over the cluster, before any barrier
+    const int wn = min(W, N - c0), per = gj_rows(N), r0 = rank * per, nr = max(0, min(N - r0, per));
+    double *a = reinterpret_cast<double *>(gj_raw);
+    int32_t *id = reinterpret_cast<int32_t *>(a + gj_panel_elems(N, W));
+    const int tid = threadIdx.x, lane = tid & 31, col = tid & (W - 1);
+    const double *Ap = A + moff[p];
+    for (int e = tid; e < gj_panel_elems(N, W); e += kGjThreads) {
+        const int row = e / W;
+        a[e] = row < nr && col < wn ? Ap[static_cast<int64_t>(r0 + row) * N + c0 + col] : 0.0;
+    }
+    for (int i = tid; i < nr; i += kGjThreads) id[i] = r0 + i;
+    cluster.sync();
+    for (int cc = 0; cc < wn; ++cc) {
+        const int c = c0 + cc, buf = cc & 1;
+        if (tid < 32) {
+            uint64_t best = 0;
+            int at = -1;
+            for (int i = max(0, c - r0) + lane; i < nr; i += 32) {
+                const uint64_t bits = static_cast<uint64_t>(__double_as_longlong(a[i * W + cc])) & ~(1ull << 63);
+                if (bits <= 0x7ff0000000000000ull && bits + 1 > best) {
+                    best = bits + 1;
+                    at = i;
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const uint64_t ob = __shfl_xor_sync(0xffffffffu, best, o);
+                const int oa = __shfl_xor_sync(0xffffffffu, at, o);
+                if (ob > best || (ob == best && oa >= 0 && oa < at)) {
+                    best = ob;
+                    at = oa;
+                }
+            }
+            const double rcp = best ? 1.0 / a[at * W + cc] : 0.0;
+            for (int to = 0; to < kGjCluster; ++to) {
+                GjCand<W> *m = cluster.map_shared_rank(&cand[buf][rank], to);
+                if (best && lane < W) m->row[lane] = a[at * W + lane];
+                if (lane == 0) {
+                    m->key = best;
+                    m->rcp = rcp;
+                    m->r = r0 + at;
+                    m->id = best ? id[at] : -1;
+                }
+            }
+        } else if (tid < 64 && c >= r0 && c < r0 + nr) {
+            for (int to = 0; to < kGjCluster; ++to) {
+                GjRow<W> *m = cluster.map_shared_rank(&diag[buf], to);
+                if (lane < W) m->row[lane] = a[(c - r0) * W + lane];
+                if (lane == 0) m->id = id[c - r0];
+            }
+        }
+        cluster.sync();
+        int win = 0;
+#pragma unroll
+        for (int i = 1; i < kGjCluster; ++i)
+            if (cand[buf][i].key > cand[buf][win].key) win = i;  // ranks hold ascending rows: the lowest row on ties
+        const GjCand<W> &w = cand[buf][win];
+        // usable: found, not zero (key 1) and not infinite
+        const bool ok = w.key > 1 && w.key < 0x7ff0000000000001ull;
+        if (!ok && rank == 0 && tid == 0) atomicOr(bad, 1);
+        const int q = ok ? w.r : c;
+        const double *prow = ok ? w.row : diag[buf].row;
+        const double v = ok ? w.rcp : 1.0 / diag[buf].row[cc];
+        const double pv = col == cc ? v : prow[col] * v;  // row c of the eliminated panel
+        const double dc = diag[buf].row[col];
+        for (int base = 0; base < nr * W; base += kGjThreads) {
+            const int e = base + tid, r = r0 + e / W;
+            const double x = r == q ? dc : a[e];  // row q now holds the former row c
+            const double fr = W == 1 ? x : __shfl_sync(0xffffffffu, x, (lane & ~(W - 1)) | cc);
+            const double out = fma(-fr, pv, col == cc ? 0.0 : x);
+            if (e < nr * W) a[e] = r == c ? pv : out;
+        }
+        if (tid == 0) {  // q == c: the second store keeps the row's own origin
+            if (q >= r0 && q < r0 + nr) id[q - r0] = diag[buf].id;
+            if (c >= r0 && c < r0 + nr) id[c - r0] = ok ? w.id : diag[buf].id;
+        }
+        __syncthreads();
+    }
+    for (int e = tid; e < nr * W; e += kGjThreads) panel[(ustart[p] + r0) * W + e] = a[e];
+    for (int i = tid; i < nr; i += kGjThreads) src[ustart[p] + r0 + i] = id[i];
+    cluster.sync();  // no CTA leaves while another may still write to its shared memory
+}
+
+// The panel's transformations on the whole matrix, X -> Y (see the top), and the composed row origins org_in -> org_out
+// (c0 = 0: from the identity).  One CTA per 32 x 32 output tile, its 32 x W and W x 32 factors in shared memory.
+// Problems with c0 unknowns or fewer are copied through.
+template <int W>
+__global__ void __launch_bounds__(kGjThreads)
+    k_gj_update(const double *__restrict__ X, double *__restrict__ Y, const int64_t *__restrict__ moff,
+                const int64_t *__restrict__ ustart, int c0, const double *__restrict__ panel,
+                const int32_t *__restrict__ src, const int32_t *__restrict__ org_in, int32_t *__restrict__ org_out) {
+    constexpr int T = kGjTile, ROWS = kGjThreads / T;  // rows of the tile per pass
+    __shared__ double M[T][W], B[W][T];
+    __shared__ int32_t from[T];
+    const int p = blockIdx.z;
+    const int64_t u0 = ustart[p];
+    const int N = static_cast<int>(ustart[p + 1] - u0);
+    const int j0 = blockIdx.x * T, i0 = blockIdx.y * T;
+    if (j0 >= N || i0 >= N) return;
+    const double *x = X + moff[p];
+    double *y = Y + moff[p];
+    const int tx = threadIdx.x % T, ty = threadIdx.x / T, j = j0 + tx;
+    const bool done = c0 >= N;
+    if (threadIdx.x < T) {
+        const int r = i0 + threadIdx.x;
+        const int s = r < N && !done ? src[u0 + r] : r;
+        from[threadIdx.x] = s;
+        if (blockIdx.x == 0 && r < N) org_out[u0 + r] = c0 == 0 ? s : org_in[u0 + s];
+    }
+    if (!done) {
+        for (int e = threadIdx.x; e < T * W; e += kGjThreads) {
+            const int r = i0 + e / W;
+            M[e / W][e % W] = r < N ? panel[(u0 + r) * W + e % W] : 0.0;
+        }
+        for (int e = threadIdx.x; e < T * W; e += kGjThreads) {
+            const int w = e / T, jj = j0 + e % T;
+            B[w][e % T] = c0 + w < N && jj < N ? x[static_cast<int64_t>(src[u0 + c0 + w]) * N + jj] : 0.0;
+        }
+    }
+    __syncthreads();
+    if (j >= N) return;
+#pragma unroll
+    for (int k = 0; k < T / ROWS; ++k) {
+        const int i = ty + k * ROWS, r = i0 + i;
+        if (r >= N) continue;
+        const bool in_j = !done && r >= c0 && r < c0 + W;
+        double s = in_j ? 0.0 : x[static_cast<int64_t>(from[i]) * N + j];
+        if (!done) {
+            if (j >= c0 && j < c0 + W) {
+                s = M[i][j - c0];
+            } else {
+#pragma unroll
+                for (int w = 0; w < W; ++w) s = fma(M[i][w], B[w][tx], s);
+            }
+        }
+        y[static_cast<int64_t>(r) * N + j] = s;
+    }
+}
+
+// A^-1 from the eliminated matrix R, its columns put back: X[:, org r] = R[:, r].
+__global__ void k_gj_unpermute(const double *__restrict__ R, double *__restrict__ X, const int64_t *__restrict__ moff,
+                               const int64_t *__restrict__ ustart, const int32_t *__restrict__ org) {
+    const int p = blockIdx.y;
+    const int N = static_cast<int>(ustart[p + 1] - ustart[p]);
+    const int64_t NN = static_cast<int64_t>(N) * N;
+    for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < NN;
+         e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        const int r = static_cast<int>(e / N), k = static_cast<int>(e - static_cast<int64_t>(r) * N);
+        X[moff[p] + static_cast<int64_t>(r) * N + org[ustart[p] + k]] = R[moff[p] + e];
+    }
+}
+__global__ void k_gj_transpose(const double *__restrict__ X, double *__restrict__ T, const int64_t *__restrict__ moff,
+                               const int64_t *__restrict__ ustart) {
+    const int p = blockIdx.y;
+    const int N = static_cast<int>(ustart[p + 1] - ustart[p]);
+    const int64_t NN = static_cast<int64_t>(N) * N;
+    for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < NN;
+         e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        const int r = static_cast<int>(e / N), k = static_cast<int>(e - static_cast<int64_t>(r) * N);
+        T[moff[p] + static_cast<int64_t>(k) * N + r] = X[moff[p] + e];
+    }
+}
+
+constexpr int64_t kGjMaxSmem = 200 * 1024;
+
+template <int W>
+void invert(mg_forest *F, int maxN) {
+    cudaFuncSetAttribute(k_gj_panel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGjMaxSmem);
+    const unsigned tiles = static_cast<unsigned>((maxN + kGjTile - 1) / kGjTile);
+    const int steps = (maxN + W - 1) / W;
+    double *X = steps % 2 ? F->Ainv : F->AinvT, *Y = steps % 2 ? F->AinvT : F->Ainv;
+    int32_t *in = F->gj_org, *out = F->gj_org + F->Nc;
+    for (int c0 = 0; c0 < maxN; c0 += W) {
+        k_gj_panel<W><<<F->np * kGjCluster, kGjThreads, gj_smem(maxN, W), F->st>>>(X, F->moff, F->ustart, c0, F->gj_panel,
+                                                                                  F->gj_src, F->flag);
+        k_gj_update<W><<<dim3(tiles, tiles, F->np), kGjThreads, 0, F->st>>>(X, Y, F->moff, F->ustart, c0, F->gj_panel,
+                                                                            F->gj_src, in, out);
+        std::swap(X, Y);
+        std::swap(in, out);
+    }
+    const dim3 grid(static_cast<unsigned>(std::min<int64_t>(1024, (static_cast<int64_t>(maxN) * maxN + 255) / 256)),
+                    static_cast<unsigned>(F->np));
+    k_gj_unpermute<<<grid, 256, 0, F->st>>>(F->AinvT, F->Ainv, F->moff, F->ustart, in);
+    k_gj_transpose<<<grid, 256, 0, F->st>>>(F->Ainv, F->AinvT, F->moff, F->ustart);
+}
+
+}  // namespace
+
+// Panel width: 16 columns while a panel's rows fit the cluster's shared memory (12,800 unknowns in 8 x 200 KB), narrower
+// panels above.  Wider ones would make the panel's own FP64 work, which only the cluster's 8 SMs share, the longer part.
+int gj_width(int maxN) { return gj_smem(maxN, 16) <= kGjMaxSmem ? 16 : (gj_smem(maxN, 4) <= kGjMaxSmem ? 4 : 1); }
+
+// The buffer the caller fills with the operators before enqueue_gauss_jordan (the eliminated matrix ends in AinvT).
+double *gj_input(mg_forest *F, int maxN) {
+    const int w = gj_width(maxN);
+    return (maxN + w - 1) / w % 2 ? F->Ainv : F->AinvT;
+}
+
+// Ainv and AinvT (the transposes) from the operators in gj_input; a singular one sets *F->flag (cleared by the caller).
+void enqueue_gauss_jordan(mg_forest *F, int maxN) {
+    switch (gj_width(maxN)) {
+        case 16: invert<16>(F, maxN); break;
+        case 4: invert<4>(F, maxN); break;
+        default: invert<1>(F, maxN); break;
+    }
+}
+
+}  // namespace octmg

@@ -733,11 +733,10 @@ void apply64(mg_forest *F, DevLevel &d, const double *u, double *out) {
 }
 
 // The device part of assemble_coarse: the columns A e_m of every problem's coarsest operator (FP64 kernels on unit
-// vectors, all problems probed at once), then Gauss-Jordan on the device into Ainv and AinvT (transposes).
+// vectors, all problems probed at once), then Gauss-Jordan on the device into Ainv and AinvT (transposes; gauss_jordan.cu).
 void enqueue_coarse_inverse(mg_forest *F, DevLevel &d, int N, int maxN) {
     double *r = F->coarse_r;
-    // the columns go to the buffer that makes the eliminated matrix end up in AinvT after maxN steps
-    double *Adev = maxN % 2 == 0 ? F->AinvT : F->Ainv;
+    double *Adev = gj_input(F, maxN);
     cudaMemsetAsync(d.u64, 0, d.pool_elems() * sizeof(double), F->st);
     if (F->pcol) {  // no refinement interface: 27 colour probes
         cudaMemsetAsync(Adev, 0, F->moff_h[F->np] * sizeof(double), F->st);
@@ -758,18 +757,7 @@ void enqueue_coarse_inverse(mg_forest *F, DevLevel &d, int N, int maxN) {
         }
     }
     cudaMemsetAsync(F->flag, 0, sizeof(int), F->st);
-    const dim3 grid(static_cast<unsigned>(std::min<int64_t>(1024, (static_cast<int64_t>(maxN) * maxN + 255) / 256)),
-                    static_cast<unsigned>(F->np));
-    double *X = Adev, *Y = Adev == F->Ainv ? F->AinvT : F->Ainv;
-    for (int c = 0; c < maxN; ++c) {
-        k_gj_pivot<<<(F->np * 32 + 255) / 256, 256, 0, F->st>>>(X, F->moff, F->ustart, F->np, c, F->gj_piv,
-                                                                F->gj_pinv, maxN, F->flag);
-        k_gj_step<<<grid, 256, 0, F->st>>>(X, Y, F->moff, F->ustart, c, F->gj_piv, F->gj_pinv, maxN);
-        std::swap(X, Y);
-    }
-    k_gj_perm<<<(F->np + 127) / 128, 128, 0, F->st>>>(F->gj_piv, F->ustart, F->np, F->gj_src, maxN);
-    k_gj_unpermute<<<grid, 256, 0, F->st>>>(F->AinvT, F->Ainv, F->moff, F->ustart, F->gj_src, maxN);
-    k_gj_transpose<<<grid, 256, 0, F->st>>>(F->Ainv, F->AinvT, F->moff, F->ustart);
+    enqueue_gauss_jordan(F, maxN);
     cudaMemsetAsync(d.u64, 0, d.pool_elems() * sizeof(double), F->st);
 }
 
@@ -866,10 +854,10 @@ mg_status assemble_coarse(mg_forest *F) {
     if (!F->coarse_r) MG_TRY(dalloc(F, &F->coarse_r, d.pool_elems()));
     int maxN = 0;
     for (int p = 0; p < F->np; ++p) maxN = std::max<int>(maxN, static_cast<int>(F->ustart_h[p + 1] - F->ustart_h[p]));
-    if (!F->gj_piv) {
-        MG_TRY(dalloc(F, &F->gj_piv, static_cast<int64_t>(F->np) * maxN));
-        MG_TRY(dalloc(F, &F->gj_src, static_cast<int64_t>(F->np) * maxN));
-        MG_TRY(dalloc(F, &F->gj_pinv, F->np));
+    if (!F->gj_src) {
+        MG_TRY(dalloc(F, &F->gj_panel, static_cast<int64_t>(N) * gj_width(maxN)));
+        MG_TRY(dalloc(F, &F->gj_org, 2 * static_cast<int64_t>(N)));
+        MG_TRY(dalloc(F, &F->gj_src, N));
     }
     // the probe must see the homogeneous operator: no boundary data, no profiling events inside a recorded graph
     double *const gb = F->gb;
