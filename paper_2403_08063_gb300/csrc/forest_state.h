@@ -52,8 +52,10 @@ struct DevLevel {
     float *kap = nullptr;
     int32_t *bprob = nullptr;  // problem of each block
     int32_t *nbr6 = nullptr;   // per block face: same-level neighbour, -1 boundary, -2 refinement interface
-    FaceItem *ifaces = nullptr;  // the C2F faces alone (interface-only exchange)
+    FaceItem *ifaces = nullptr;  // the C2F faces alone: each with the coarse quarter face it covers, an interface item
     int nifaces = 0;
+    FaceItem *sfaces = nullptr;  // the other faces: boundary and same level
+    int nsfaces = 0;
     int8_t *fkind = nullptr;   // per block face (b * 6 + 2 * axis + side): 0 boundary, 1 same, 2 C2F, 3 F2C
     bool all_halve = false;  // every block of the next level is a halved block of this one
     // FP32 smoother launch shape (kind, parameters): {1, ZC, threads, 0, 0} k_smooth32, {2, TY, TZ, D, R}
@@ -80,11 +82,10 @@ struct TailLevel {
     LevelGeom g;
     float *u, *f;
     const float *kap, *h2, *ih2;
-    const FaceItem *faces, *ifaces;
-    const SegItem *segs;
+    const FaceItem *sfaces, *ifaces;
     const XferItem *xfer;  // to the next level
     const int32_t *nbr6, *bprob;
-    int nfaces, nifaces, nsegs;
+    int nsfaces, nifaces;
     int fast;  // the transfers to the next level use the specialised kernels (every block halves, edge 8..128)
     const float *ax, *ay, *az;  // halved face coefficients of a face-averaged coarse level (mode 3)
     int face32;                 // 1: this level's smoothing, ghosts and restriction use them
@@ -92,7 +93,7 @@ struct TailLevel {
 
 // One step of the tail's V-cycle; every step is followed by a grid barrier.
 enum TailOp : int32_t {
-    T_SMOOTH0 = 0, T_SMOOTH1, T_FACES_IFACE, T_FACES_FULL, T_SEGS, T_RESTRICT, T_PROLONG, T_COARSE
+    T_SMOOTH0 = 0, T_SMOOTH1, T_EXCH_IFACE, T_EXCH_FULL, T_RESTRICT, T_PROLONG, T_COARSE
 };
 struct TailPhase {
     int32_t op, level;

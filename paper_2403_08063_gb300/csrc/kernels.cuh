@@ -367,61 +367,6 @@ static __global__ void k_exchange_faces(T *__restrict__ u, const FaceItem *__res
                                    static_cast<int64_t>(gridDim.x) * blockDim.x, c2f, gb);
 }
 
-// Coarse-to-fine ghosts of refinement interfaces only (Sec. 3.3.2), one CTA per fine block face, with the
-// intermediate results shared between neighbouring coarse cells: the normal-direction extrapolation (the 1D step
-// through the current coarse cell and the two inward) of every coarse cell of the segment and of its one-cell
-// tangential border is computed once into shared memory, and each coarse cell's four fine ghosts are the
-// tangential interpolation of 3 x 3 of those values.  Sec. 8 of the paper proposes this reuse of intermediate
-// extrapolation results for neighbouring cells (a ring buffer on CPUs, shared memory on GPUs); it takes 3 loads per
-// intermediate value, about 3.4 per coarse cell, instead of 27 per fine ghost.  Same operations in the same order as
-// exchange_faces_body, so the same bits.  Dynamic shared memory: (n/2 + 2)^2 values of T.
-template <typename T>
-static __global__ void k_exchange_c2f_smem(T *__restrict__ u, const FaceItem *__restrict__ items, LevelGeom g,
-                                           Skip skip, int c2f) {
-    extern __shared__ __align__(16) unsigned char c2f_smem[];
-    T *E = reinterpret_cast<T *>(c2f_smem);
-    const FaceItem F = items[blockIdx.x];
-    if (skip(F.blk)) return;  // uniform over the CTA, before the barrier
-    const int n = g.n, h = n >> 1;
-    // coarse cells [lo1, lo1 + w1) x [lo2, lo2 + w2) of the coarse face: the segment and the neighbours its
-    // stencils reach (remapped bases stay inside the coarse block)
-    const int lo1 = max(0, F.seg1 * h - 1), w1 = min(n - 1, F.seg1 * h + h) - lo1 + 1;
-    const int lo2 = max(0, F.seg2 * h - 1), w2 = min(n - 1, F.seg2 * h + h) - lo2 + 1;
-    for (int q = threadIdx.x; q < w1 * w2; q += blockDim.x) {
-        const int y = lo1 + q % w1, z = lo2 + q / w1;
-        T v = w_normal<T>(c2f, 0) * u[fidx<T>(g, F.nbr, F.axis, 1 - F.side, 1, y, z)];
-        v = fma(w_normal<T>(c2f, 1), u[fidx<T>(g, F.nbr, F.axis, 1 - F.side, 2, y, z)], v);
-        E[q] = fma(w_normal<T>(c2f, 2), u[fidx<T>(g, F.nbr, F.axis, 1 - F.side, 3, y, z)], v);
-    }
-    __syncthreads();
-    for (int q = threadIdx.x; q < h * h; q += blockDim.x) {
-        const int ycl = q % h, zcl = q / h;
-        const int yc = F.seg1 * h + ycl, zc = F.seg2 * h + zcl;
-        const int cy = yc == 0 ? 1 : (yc == n - 1 ? 2 : 0);
-        const int cz = zc == 0 ? 1 : (zc == n - 1 ? 2 : 0);
-        T e[3][3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-#pragma unroll
-            for (int b = 0; b < 3; ++b)
-                e[c][b] = E[(zc + c_base[cz][c] - lo2) * w1 + (yc + c_base[cy][b] - lo1)];
-#pragma unroll
-        for (int a2 = 0; a2 < 2; ++a2)
-#pragma unroll
-            for (int a1 = 0; a1 < 2; ++a1) {
-                T acc = T(0);
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    T accb = T(0);
-#pragma unroll
-                    for (int b = 0; b < 3; ++b) accb = fma(w_tang<T>(c2f, cy, a1, b), e[c][b], accb);
-                    acc = fma(w_tang<T>(c2f, cz, a2, c), accb, acc);
-                }
-                u[fidx<T>(g, F.blk, F.axis, F.side, 0, 2 * ycl + a1, 2 * zcl + a2)] = acc;
-            }
-    }
-}
-
 // ------------------------------------------------------------------------------------------------------------
 // Ghost exchange, part 2: coarse ghost segments next to finer neighbours.
 // FLUX = false: F2C mean of the 2x2x2 fine inner cells overlapping each coarse ghost cell (Sec. 3.3.1).
@@ -481,6 +426,141 @@ static __global__ void k_exchange_segs(T *__restrict__ u, Coef cf, const SegItem
     exchange_segs_body<T, MODE, FLUX>(u, cf, items, nitems, g, skip,
                                       blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x,
                                       static_cast<int64_t>(gridDim.x) * blockDim.x);
+}
+
+// ------------------------------------------------------------------------------------------------------------
+// Both sides of a refinement interface in one pass.  A fine block face next to a coarser block is one FaceItem, and the
+// quarter of the coarse block's face that it covers is filled from that fine block alone, so the work on one coarse cell of
+// the quarter gives its four fine ghosts (C2F, Sec. 3.3.2) and, from these, the coarse ghost across the face (F2C): all it
+// reads is the interior of the two blocks.  `e` holds the normal-direction extrapolations of the 3 x 3 coarse cells of the
+// cell's tangential stencil.  The same operations in the same order as exchange_faces_body and exchange_segs_body.
+// ------------------------------------------------------------------------------------------------------------
+template <typename T, int MODE, bool FLUX, bool CG = false>
+__device__ __forceinline__ void exchange_iface_cell(T *__restrict__ u, const Coef &cf, const FaceItem &F,
+                                                    const LevelGeom &g, int c2f, int ycl, int zcl, const T (&e)[3][3]) {
+    const int n = g.n, h = n >> 1;
+    const int yc = F.seg1 * h + ycl, zc = F.seg2 * h + zcl;
+    const int cy = yc == 0 ? 1 : (yc == n - 1 ? 2 : 0);
+    const int cz = zc == 0 ? 1 : (zc == n - 1 ? 2 : 0);
+    const int64_t gC = fidx<T>(g, F.nbr, F.axis, 1 - F.side, 1, yc, zc);
+    const int64_t g0c = fidx<T>(g, F.nbr, F.axis, 1 - F.side, 0, yc, zc);
+    T flux = T(0);
+#pragma unroll
+    for (int a2 = 0; a2 < 2; ++a2)
+#pragma unroll
+        for (int a1 = 0; a1 < 2; ++a1) {
+            T acc = T(0);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                T accb = T(0);
+#pragma unroll
+                for (int b = 0; b < 3; ++b) accb = fma(w_tang<T>(c2f, cy, a1, b), e[c][b], accb);
+                acc = fma(w_tang<T>(c2f, cz, a2, c), accb, acc);
+            }
+            const int64_t g0 = fidx<T>(g, F.blk, F.axis, F.side, 0, 2 * ycl + a1, 2 * zcl + a2);
+            u[g0] = acc;
+            if constexpr (FLUX) {
+                const int64_t g1 = fidx<T>(g, F.blk, F.axis, F.side, 1, 2 * ycl + a1, 2 * zcl + a2);
+                const T Tj = face_coef<T, MODE>(cf, F.side ? g0 : g1, F.side ? g1 : g0, F.axis);
+                flux = fma(Tj, acc - ldv<CG>(u + g1), flux);
+            }
+        }
+    if constexpr (FLUX) {
+        const T Tc = face_coef<T, MODE>(cf, F.side ? gC : g0c, F.side ? g0c : gC, F.axis);
+        u[g0c] = ldv<CG>(u + gC) - flux / (T(MODE == 1 ? 8 : 2) * Tc);
+    } else {
+        T s = T(0);
+#pragma unroll
+        for (int d = 1; d <= 2; ++d)
+#pragma unroll
+            for (int b = 0; b < 2; ++b)
+#pragma unroll
+                for (int a = 0; a < 2; ++a)
+                    s += ldv<CG>(u + fidx<T>(g, F.blk, F.axis, F.side, d, 2 * ycl + a, 2 * zcl + b));
+        u[g0c] = T(0.125) * s;
+    }
+}
+
+// One interface item by one CTA.  The normal-direction extrapolations of the quarter's coarse cells and of their one-cell
+// tangential border are computed once into shared memory, E[(n/2 + 2)^2] (Sec. 8 of the paper proposes this reuse for
+// neighbouring cells): about 3.4 loads per coarse cell instead of 27.
+template <typename T, int MODE, bool FLUX>
+__device__ __forceinline__ void exchange_iface_cta(T *__restrict__ u, const Coef &cf, const FaceItem &F,
+                                                   const LevelGeom &g, int c2f, T *E) {
+    const int n = g.n, h = n >> 1;
+    // coarse cells [lo1, lo1 + w1) x [lo2, lo2 + w2) of the coarse face: the segment and the neighbours its
+    // stencils reach (remapped bases stay inside the coarse block)
+    const int lo1 = max(0, F.seg1 * h - 1), w1 = min(n - 1, F.seg1 * h + h) - lo1 + 1;
+    const int lo2 = max(0, F.seg2 * h - 1), w2 = min(n - 1, F.seg2 * h + h) - lo2 + 1;
+    for (int q = threadIdx.x; q < w1 * w2; q += blockDim.x) {
+        const int y = lo1 + q % w1, z = lo2 + q / w1;
+        T v = w_normal<T>(c2f, 0) * u[fidx<T>(g, F.nbr, F.axis, 1 - F.side, 1, y, z)];
+        v = fma(w_normal<T>(c2f, 1), u[fidx<T>(g, F.nbr, F.axis, 1 - F.side, 2, y, z)], v);
+        E[q] = fma(w_normal<T>(c2f, 2), u[fidx<T>(g, F.nbr, F.axis, 1 - F.side, 3, y, z)], v);
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < h * h; q += blockDim.x) {
+        const int ycl = q % h, zcl = q / h;
+        const int yc = F.seg1 * h + ycl, zc = F.seg2 * h + zcl;
+        const int cy = yc == 0 ? 1 : (yc == n - 1 ? 2 : 0);
+        const int cz = zc == 0 ? 1 : (zc == n - 1 ? 2 : 0);
+        T e[3][3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int b = 0; b < 3; ++b)
+                e[c][b] = E[(zc + c_base[cz][c] - lo2) * w1 + (yc + c_base[cy][b] - lo1)];
+        exchange_iface_cell<T, MODE, FLUX>(u, cf, F, g, c2f, ycl, zcl, e);
+    }
+}
+
+// The interface items one thread per coarse cell, without shared memory (the persistent tail, whose items are small).
+template <typename T, int MODE, bool FLUX, bool CG>
+__device__ __forceinline__ void exchange_iface_body(T *__restrict__ u, const Coef &cf, const FaceItem *__restrict__ items,
+                                                    int nitems, const LevelGeom &g, Skip skip, int64_t t0, int64_t ts,
+                                                    int c2f = 0) {
+    const int n = g.n, h = n >> 1, lgh = g.lg - 1;
+    const int64_t total = static_cast<int64_t>(nitems) << (2 * lgh);
+    for (int64_t t = t0; t < total; t += ts) {
+        const FaceItem F = items[t >> (2 * lgh)];
+        if (skip(F.blk)) continue;
+        const int r = static_cast<int>(t) & ((1 << (2 * lgh)) - 1), ycl = r & (h - 1), zcl = r >> lgh;
+        const int yc = F.seg1 * h + ycl, zc = F.seg2 * h + zcl;
+        const int cy = yc == 0 ? 1 : (yc == n - 1 ? 2 : 0);
+        const int cz = zc == 0 ? 1 : (zc == n - 1 ? 2 : 0);
+        T e[3][3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                const int y = yc + c_base[cy][b], z = zc + c_base[cz][c];
+                T v = w_normal<T>(c2f, 0) * ldv<CG>(u + fidx<T>(g, F.nbr, F.axis, 1 - F.side, 1, y, z));
+                v = fma(w_normal<T>(c2f, 1), ldv<CG>(u + fidx<T>(g, F.nbr, F.axis, 1 - F.side, 2, y, z)), v);
+                e[c][b] = fma(w_normal<T>(c2f, 2), ldv<CG>(u + fidx<T>(g, F.nbr, F.axis, 1 - F.side, 3, y, z)), v);
+            }
+        exchange_iface_cell<T, MODE, FLUX, CG>(u, cf, F, g, c2f, ycl, zcl, e);
+    }
+}
+
+// Ghost exchange of a level in one launch: CTAs [0, nif) one interface item each, the others the faces filled from one
+// source block (boundary, same level; nsf items, none for the interface-only exchange between half-sweeps), one thread per
+// ghost cell.  Every ghost is computed from block interiors only, so the two parts are independent.  These launches move a
+// few hundred KB and last as long as their latency; two of them (C2F, then F2C from the fine ghosts) took 2 x 3.2 us per
+// half-sweep on 56 + 64 blocks of 32^3, this one 3.5 us.
+template <typename T, int MODE, bool FLUX>
+static __global__ void __launch_bounds__(kThreads) k_exchange(T *__restrict__ u, Coef cf,
+                                                              const FaceItem *__restrict__ ifaces, int nif,
+                                                              const FaceItem *__restrict__ sfaces, int nsf, LevelGeom g,
+                                                              Skip skip, int c2f, const T *__restrict__ gb) {
+    extern __shared__ __align__(16) unsigned char iface_smem[];
+    if (static_cast<int>(blockIdx.x) < nif) {
+        const FaceItem F = ifaces[blockIdx.x];
+        if (skip(F.blk)) return;  // uniform over the CTA, before the barrier
+        exchange_iface_cta<T, MODE, FLUX>(u, cf, F, g, c2f, reinterpret_cast<T *>(iface_smem));
+        return;
+    }
+    exchange_faces_body<T, false>(u, sfaces, nsf, g, skip, (blockIdx.x - nif) * static_cast<int64_t>(blockDim.x) + threadIdx.x,
+                                  static_cast<int64_t>(gridDim.x - nif) * blockDim.x, c2f, gb);
 }
 
 // ------------------------------------------------------------------------------------------------------------

@@ -91,32 +91,34 @@ template <> Coef coef_of<float>(const DevLevel &d) { return d.c32(); }
 Skip skip_of(mg_forest *F, const DevLevel &d) { return Skip{d.bprob, F->pdone}; }
 
 // Ghost exchange of a level: every face (full), or only the refinement-interface faces (C2F and F2C), whose
-// ghosts the smoother's write-through does not maintain.
+// ghosts the smoother's write-through does not maintain.  One launch for block edges up to 128 (the interface items' shared
+// memory, (n/2 + 2)^2 values, then fits 48 KB), two generic ones above.
 template <typename T, int MODE>
 void exchange(mg_forest *F, DevLevel &d, T *u, bool interface_only = false, bool prof = true) {
-    const FaceItem *items = interface_only ? d.ifaces : d.faces;
-    const int nitems = interface_only ? d.nifaces : d.nfaces;
-    if (!nitems && !d.nsegs) return;
-    Prof p(F, prof ? cat_of<T>(P_EXCH64) : -1, (nitems ? 1 : 0) + (d.nsegs ? 1 : 0));
+    const int nif = d.nifaces, nsf = interface_only ? 0 : d.nsfaces, n = d.g.n;
+    if (!nif && !nsf) return;
+    const bool one = n <= 128;
+    Prof p(F, prof ? cat_of<T>(P_EXCH64) : -1, one || !nif ? 1 : 2);
     const T *gb = nullptr;  // inhomogeneous Dirichlet data: FP64 finest level only
     if constexpr (sizeof(T) == 8)
         if (&d == &F->L[0]) gb = F->gb;
-    if (nitems && interface_only) {  // C2F faces only: one CTA per fine face, shared intermediate extrapolations
-        const int w = d.g.n / 2 + 2, threads = d.g.n <= 8 ? 32 : (d.g.n <= 32 ? 128 : 256);
-        k_exchange_c2f_smem<T><<<nitems, threads, static_cast<size_t>(w) * w * sizeof(T), F->st>>>(
-            u, items, d.g, skip_of(F, d), F->cfg.c2f_variant);
+    if (one) {
+        // a CTA per interface item alone takes as many threads as the item has work for; next to the other faces, 256
+        const int threads = nsf ? kThreads : (n <= 8 ? 32 : (n <= 32 ? 128 : 256));
+        const int w = n / 2 + 2, grid = nif + (nsf ? grid_for(static_cast<int64_t>(nsf) * n * n) : 0);
+        auto *fn = F->cfg.interface_flux ? k_exchange<T, MODE, true> : k_exchange<T, MODE, false>;
+        fn<<<grid, threads, nif ? w * w * sizeof(T) : 0, F->st>>>(u, coef_of<T>(d), d.ifaces, nif, d.sfaces, nsf, d.g,
+                                                                  skip_of(F, d), F->cfg.c2f_variant, gb);
+        return;
     }
-    else if (nitems)
-        k_exchange_faces<T, false><<<grid_for(static_cast<int64_t>(nitems) * d.g.n * d.g.n), kThreads, 0, F->st>>>(
-            u, items, nitems, d.g, skip_of(F, d), F->cfg.c2f_variant, gb);
+    const FaceItem *items = interface_only ? d.ifaces : d.faces;
+    const int nitems = interface_only ? d.nifaces : d.nfaces;
+    k_exchange_faces<T, false><<<grid_for(static_cast<int64_t>(nitems) * n * n), kThreads, 0, F->st>>>(
+        u, items, nitems, d.g, skip_of(F, d), F->cfg.c2f_variant, gb);
     if (d.nsegs) {
-        const int64_t tot = static_cast<int64_t>(d.nsegs) * (d.g.n / 2) * (d.g.n / 2);
-        if (F->cfg.interface_flux)
-            k_exchange_segs<T, MODE, true><<<grid_for(tot), kThreads, 0, F->st>>>(u, coef_of<T>(d), d.segs, d.nsegs, d.g,
-                                                                                skip_of(F, d));
-        else
-            k_exchange_segs<T, MODE, false><<<grid_for(tot), kThreads, 0, F->st>>>(u, coef_of<T>(d), d.segs, d.nsegs,
-                                                                                 d.g, skip_of(F, d));
+        const int64_t tot = static_cast<int64_t>(d.nsegs) * (n / 2) * (n / 2);
+        auto *fn = F->cfg.interface_flux ? k_exchange_segs<T, MODE, true> : k_exchange_segs<T, MODE, false>;
+        fn<<<grid_for(tot), kThreads, 0, F->st>>>(u, coef_of<T>(d), d.segs, d.nsegs, d.g, skip_of(F, d));
     }
 }
 
@@ -502,7 +504,7 @@ struct LaunchExec {
         DevLevel &d = F->L[l];
         if (F->cfg.coarse_iters > 0) {  // damped Jacobi sweeps from zero (the paper's coarsest solver)
             const DevLevel &d = F->L[l];
-            Prof p(F, cat_of<T>(P_COARSE64), F->cfg.coarse_iters * (1 + (d.nfaces > 0) + (d.nsegs > 0)));
+            Prof p(F, cat_of<T>(P_COARSE64), F->cfg.coarse_iters * (1 + (d.nfaces > 0)));
             for (int it = 0; it < F->cfg.coarse_iters; ++it) {
                 octmg::exchange<T, MODE>(F, F->L[l], ufield<T>(F->L[l]), false, false);
                 jacobi(l, false);
@@ -551,8 +553,7 @@ struct RecordExec {
     bool tail(int, int) { return false; }
     void exchange(int l, bool iface) {
         const DevLevel &d = F->L[l];
-        if ((iface ? d.nifaces : d.nfaces) > 0) ph.push_back({iface ? T_FACES_IFACE : T_FACES_FULL, l});
-        if (d.nsegs > 0) ph.push_back({T_SEGS, l});
+        if (d.nifaces > 0 || (!iface && d.nsfaces > 0)) ph.push_back({iface ? T_EXCH_IFACE : T_EXCH_FULL, l});
     }
     void smooth(int l, int colour) { ph.push_back({colour ? T_SMOOTH1 : T_SMOOTH0, l}); }
     void jacobi(int) {}  // FP64 only; the tail runs FP32 cycles
@@ -623,8 +624,8 @@ mg_status record_tail(mg_forest *F, int l) {
         std::vector<TailLevel> tl(F->L.size());
         for (size_t m = 0; m < F->L.size(); ++m) {
             const DevLevel &d = F->L[m];
-            tl[m] = TailLevel{d.g, d.u32, d.f32, d.kap, d.h2_32, d.ih2_32, d.faces, d.ifaces, d.segs, d.xfer, d.nbr6,
-                              d.bprob, d.nfaces, d.nifaces, d.nsegs, transfer32_specialised(d) ? 1 : 0,
+            tl[m] = TailLevel{d.g, d.u32, d.f32, d.kap, d.h2_32, d.ih2_32, d.sfaces, d.ifaces, d.xfer, d.nbr6,
+                              d.bprob, d.nsfaces, d.nifaces, transfer32_specialised(d) ? 1 : 0,
                               d.ax32, d.ay32, d.az32, d.face32 ? 1 : 0};
         }
         MG_TRY(upload(F, &F->tail_L, tl));
@@ -1341,16 +1342,18 @@ mg_status create(const mg_config *cfg, mg_forest **out) {
             for (size_t b = 0; b < bp.size(); ++b) bp[b] = h.keys[b].p;
             if ((st = upload(F, &d.bprob, bp)) != MG_OK) return fail(st);
             std::vector<int32_t> nb6(h.keys.size() * 6, -2);
-            std::vector<FaceItem> itf;
+            std::vector<FaceItem> itf, same;
             for (const FaceItem &fi : h.faces) {
                 int32_t &slot = nb6[static_cast<size_t>(fi.blk) * 6 + 2 * fi.axis + fi.side];
                 if (fi.kind == FK_SAME) slot = fi.nbr;
                 else if (fi.kind == FK_BND) slot = -1;
-                else itf.push_back(fi);
+                (fi.kind == FK_C2F ? itf : same).push_back(fi);
             }
             if ((st = upload(F, &d.nbr6, nb6)) != MG_OK) return fail(st);
             d.nifaces = static_cast<int>(itf.size());
             if (!itf.empty() && (st = upload(F, &d.ifaces, itf)) != MG_OK) return fail(st);
+            d.nsfaces = static_cast<int>(same.size());
+            if ((st = upload(F, &d.sfaces, same)) != MG_OK) return fail(st);
         }
         if (!h.to_next.empty() && (st = upload(F, &d.xfer, h.to_next)) != MG_OK) return fail(st);
         if (F->cfg.prolongation == 1) {  // edge and corner ghosts for the trilinear prolongation

@@ -59,8 +59,8 @@ __device__ __forceinline__ void tail_restrict(const TailLevel &d, const TailLeve
                                              t0, ts, d.ax, d.ay, d.az);
 }
 
-// The phases that read the level's coefficients (smoothing, conservative fine-to-coarse ghosts, residual +
-// restriction), in coefficient mode M; the others do not depend on it.
+// The phases that read the level's coefficients (smoothing, exchanges with conservative fine-to-coarse
+// ghosts, residual + restriction), in coefficient mode M; the others do not depend on it.
 template <int M>
 __device__ __forceinline__ void tail_coef_phase(const TailArgs &a, const TailPhase &P, const TailLevel &d, Skip skip,
                                                 int64_t t0, int64_t ts) {
@@ -79,11 +79,14 @@ __device__ __forceinline__ void tail_coef_phase(const TailArgs &a, const TailPha
             }
             break;
         }
-        case T_SEGS:
+        case T_EXCH_FULL:  // the faces filled from one source block, then (independent of them) the interface items
+            exchange_faces_body<float, false, true>(d.u, d.sfaces, d.nsfaces, d.g, skip, t0, ts);
+            [[fallthrough]];
+        case T_EXCH_IFACE:
             if (a.flux)
-                exchange_segs_body<float, M, true, true>(d.u, cf, d.segs, d.nsegs, d.g, skip, t0, ts);
+                exchange_iface_body<float, M, true, true>(d.u, cf, d.ifaces, d.nifaces, d.g, skip, t0, ts);
             else
-                exchange_segs_body<float, M, false, true>(d.u, cf, d.segs, d.nsegs, d.g, skip, t0, ts);
+                exchange_iface_body<float, M, false, true>(d.u, cf, d.ifaces, d.nifaces, d.g, skip, t0, ts);
             break;
         default: {  // T_RESTRICT
             const TailLevel &c = a.L[P.level + 1];
@@ -118,16 +121,11 @@ __device__ __forceinline__ void tail_phase(const TailArgs &a, const TailPhase &P
     switch (P.op) {
         case T_SMOOTH0:
         case T_SMOOTH1:
-        case T_SEGS:
+        case T_EXCH_IFACE:
+        case T_EXCH_FULL:
         case T_RESTRICT:
             if (MODE == 2 && d.face32) tail_coef_phase<3>(a, P, d, skip, t0, ts);
             else tail_coef_phase<MODE>(a, P, d, skip, t0, ts);
-            break;
-        case T_FACES_IFACE:
-            exchange_faces_body<float, false, true>(d.u, d.ifaces, d.nifaces, d.g, skip, t0, ts);
-            break;
-        case T_FACES_FULL:
-            exchange_faces_body<float, false, true>(d.u, d.faces, d.nfaces, d.g, skip, t0, ts);
             break;
         case T_PROLONG: {
             const TailLevel &c = a.L[P.level + 1];
