@@ -1,13 +1,31 @@
-// Adjoint of the octree-block multigrid solve (FP64): the transposed operator, the exact transpose of the forward
-// V-cycle, the adjoint solve by defect correction, and dL/dk.  The paper has no adjoint; every step here is the
-// transpose of a forward step that cites its passage.
+// Adjoint of the octree-block multigrid solve: the transposed operator, the exact transpose of the forward V-cycle, the
+// adjoint solve by defect correction, and dL/dk.  The paper has no adjoint; every step here is the transpose of a forward
+// step that cites its passage.
 //
 // A = S E: E fills ghosts from interiors (reflection, copy, C2F extrapolation of Sec. 3.3.2, F2C mean of Sec. 3.3.1
-// or the conservative flux ghost), S is the 7-point stencil.  A^T = E^T S^T: S^T y is the stencil applied to y with
-// zero ghosts plus, at every ghost next to an interior cell i, the ghost adjoint -T_f y_i / h_i^2; E^T adds every
-// ghost adjoint into the interior cells that ghost was computed from (FP64 atomics), in the reverse order of the
-// forward exchange.  The forward V-cycle is a linear map M of its right-hand side; its transpose M^T runs the cycle's
-// steps backwards, each transposed, so lambda += M^T (g - A^T lambda) converges at the forward cycle's rate.
+// or the conservative flux ghost), S is the 7-point stencil; A^T = E^T S^T.  Between blocks of one level and at the domain
+// boundary E and S transpose into themselves (a copied ghost's adjoint is the neighbour's own coefficient times its value,
+// a reflection's is its own), so away from refinement interfaces A^T y is the forward stencil on y with the forward's
+// ghosts.  At a refinement interface, with a_j the adjoint of fine ghost j, T~ = T / h^2 and y_C the coarse cell behind it:
+//     conservative: the fine ghost reads y_C / 8 and the coarse one y_C (the rows of u_j and u_C in the coarse ghost
+//                   G = u_C - sum_j T_j / (2 T_C) (g_j - u_j)), and a_j = -T~_j (y_j - y_C / 8);
+//     ghost-only:   both read 0, a_j = -T~_j y_j, and each of the eight fine cells of the coarse ghost's mean gets
+//                   -T~_C y_C / 8;
+//     either way (A^T y) gets a_j times the quadratic weights at the coarse cells ghost j was extrapolated from.
+// That last part is the only one that is not a 7-point stencil.  It moves to the right-hand side: with f' = f - (the
+// interface part of A^T y) and the ghosts above, f - A^T y = f' - (stencil of y), so the transposed cycle runs on the
+// forward's kernels, layouts and launch shapes, and one small kernel per exchange (k_adj_iface) keeps ghosts and f' current
+// by adding what changed since the last one.
+//
+// The forward V-cycle is a linear map M of its right-hand side; M^T runs its steps backwards, each transposed.  The
+// transpose of a half-sweep u += Pi_c D^-1 (f - A u) in terms of the accumulated result y is y += Pi_c D^-1 (f - A^T y): the
+// same half-sweep on A^T, with the colours in reverse order.  Prolongation and restriction transpose into the gather
+// k_prolong_T and the injection k_inject.  So lambda += M^T (g - A^T lambda) converges at the forward cycle's rate.
+//
+// What bounds it: HBM, in the half-sweeps (10 B per updated cell) and the FP64 residual's FP64 rate.  The transposed cycle
+// step by step on natural-layout arrays of its own (the correction, its stencil with ghost adjoints, their scatter by
+// atomics over every face, two vector updates per half-sweep: ~70 B per cell and half-sweep) made set-up, forward solve and
+// adjoint on 448 + 512 blocks of 32^3 (31.5M cells) take 174 ms; this form 79.8 ms.
 #include <cmath>
 
 #include "forest_state.h"
@@ -27,323 +45,191 @@ __device__ inline void decode_cell(int64_t t, int lg, int &x, int &y, int &z, in
     for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < (total); \
          t += static_cast<int64_t>(gridDim.x) * blockDim.x)
 
-// The operator's coefficients as the transposed cycle reads them, in its working precision T (natural layout):
-// scaled face coefficients T_f / h^2 (x-, y-, z-faces, stored at the cell with the larger coordinate), their sum
-// (the diagonal) and its inverse.  FP64: the forest's arrays; FP32: rounded copies made by the first adjoint call.
-template <typename T>
-struct ACoef {
-    const T *tx, *ty, *tz, *dg, *dinv;
+// Scaled face coefficient T / h^2 of the face between depth 0 (g0) and depth 1 (g1) of a block face (axis, side).
+template <typename T, int MODE>
+__device__ __forceinline__ T scaled_face(const Coef &cf, const T *ih2, int64_t b, int64_t g0, int64_t g1, int axis,
+                                         int side) {
+    if constexpr (MODE == 0) return ih2[b];
+    const T t = face_coef<T, MODE>(cf, side ? g0 : g1, side ? g1 : g0, axis);
+    return MODE == 1 ? t : t * ih2[b];
+}
+
+// The coarse face quarter of an interface item and the coarse cells its ghosts' stencils reach.
+struct Quarter {
+    int n, h, lo1, w1, lo2, w2;
+    __device__ Quarter(const FaceItem &F, const LevelGeom &g) : n(g.n), h(g.n >> 1) {
+        lo1 = max(0, F.seg1 * h - 1);
+        w1 = min(n - 1, F.seg1 * h + h) - lo1 + 1;
+        lo2 = max(0, F.seg2 * h - 1);
+        w2 = min(n - 1, F.seg2 * h + h) - lo2 + 1;
+    }
 };
 
-// Scaled face coefficient T_f / h^2 between depth 0 and depth 1 of face (axis, side) at those two cells.
-template <int MODE, typename T>
-__device__ inline T face_ts(const ACoef<T> &cf, const T *ih2, int64_t b, int64_t g0, int64_t g1, int axis, int side) {
-    if (MODE == 0) return ih2[b];
-    const T *t = axis == 0 ? cf.tx : (axis == 1 ? cf.ty : cf.tz);
-    return t[side ? g0 : g1];
-}
-
-// Ghost adjoints of the transposed stencil: G[ghost] = -T~ y[adjacent interior], every face of every block.
-template <int MODE, typename T>
-__global__ void k_at_ghosts(const T *__restrict__ y, T *__restrict__ G, ACoef<T> cf, const T *__restrict__ ih2,
-                            LevelGeom g) {
-    const int n = g.n, lg = g.lg, P = g.P;
-    const int64_t total = static_cast<int64_t>(g.nb) * 6 << (2 * lg);
-    GRID_STRIDE(total) {
-        const int cell = static_cast<int>(t & ((1 << (2 * lg)) - 1));
-        const int64_t rest = t >> (2 * lg);
-        const int f = static_cast<int>(rest % 6);
-        const int64_t b = rest / 6;
-        const int axis = f >> 1, side = f & 1;
-        const int i1 = cell & (n - 1), i2 = cell >> lg;
-        const int64_t g0 = b * g.bs + face_off(axis, side, 0, i1, i2, n, P);
-        const int64_t g1 = b * g.bs + face_off(axis, side, 1, i1, i2, n, P);
-        G[g0] = -face_ts<MODE>(cf, ih2, b, g0, g1, axis, side) * y[g1];
+// Adds to E (the quarter's w1 x w2 coarse cells, shared) the tangential transpose of the quadratic C2F rule: the adjoints
+// a[a2][a1] of the four fine ghosts over coarse cell (ycl, zcl) of the quarter.
+template <typename T>
+__device__ __forceinline__ void scatter_tangential(T *E, const Quarter &Q, const FaceItem &F, int ycl, int zcl,
+                                                   const T (&a)[2][2]) {
+    const int yc = F.seg1 * Q.h + ycl, zc = F.seg2 * Q.h + zcl;
+    const int cy = yc == 0 ? 1 : (yc == Q.n - 1 ? 2 : 0);
+    const int cz = zc == 0 ? 1 : (zc == Q.n - 1 ? 2 : 0);
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        const T s0 = fma(w_tang<T>(0, cy, 1, b), a[0][1], w_tang<T>(0, cy, 0, b) * a[0][0]);
+        const T s1 = fma(w_tang<T>(0, cy, 1, b), a[1][1], w_tang<T>(0, cy, 0, b) * a[1][0]);
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            atomicAdd(&E[(zc + c_base[cz][c] - Q.lo2) * Q.w1 + yc + c_base[cy][b] - Q.lo1],
+                      fma(w_tang<T>(0, cz, 1, c), s1, w_tang<T>(0, cz, 0, c) * s0));
     }
 }
 
-// E^T of the conservative coarse ghosts G = u_C - c sum_j (g_j - u_j), c = T_j / (2 T_C) (T~_j / (8 T~_C) scaled).
-template <int MODE, typename T>
-__global__ void k_et_segs_flux(T *__restrict__ G, ACoef<T> cf, const T *__restrict__ ih2,
-                               const SegItem *__restrict__ items, int nitems, LevelGeom g) {
-    const int n = g.n, P = g.P, lgh = g.lg - 1, h = n >> 1;
-    const int64_t total = static_cast<int64_t>(nitems) << (2 * lgh);
-    GRID_STRIDE(total) {
-        const int it = static_cast<int>(t >> (2 * lgh));
-        const int r = static_cast<int>(t) & ((1 << (2 * lgh)) - 1);
-        const int p = r & (h - 1), q = r >> lgh;
-        const SegItem S = items[it];
-        const int64_t cb = S.coarse * g.bs, fb = S.fine * g.bs;
-        const int fs = 1 - S.side;
-        const int yc = S.s1 * h + p, zc = S.s2 * h + q;
-        const int64_t g0c = cb + face_off(S.axis, S.side, 0, yc, zc, n, P);
-        const int64_t gC = cb + face_off(S.axis, S.side, 1, yc, zc, n, P);
-        const T a = G[g0c];
-        atomicAdd(&G[gC], a);
-        const T Tc = face_ts<MODE>(cf, ih2, S.coarse, g0c, gC, S.axis, S.side);
-        const T fac = MODE == 1 ? T(8) : T(2);
-        for (int bb = 0; bb < 2; ++bb)
-            for (int aa = 0; aa < 2; ++aa) {
-                const int64_t g0 = fb + face_off(S.axis, fs, 0, 2 * p + aa, 2 * q + bb, n, P);
-                const int64_t g1 = fb + face_off(S.axis, fs, 1, 2 * p + aa, 2 * q + bb, n, P);
-                const T Tj = MODE == 0 ? T(1) : face_ts<MODE>(cf, ih2, S.fine, g0, g1, S.axis, fs);
-                const T c = (MODE == 0 ? T(1) : Tj) / (fac * (MODE == 0 ? T(1) : Tc)) * a;
-                atomicAdd(&G[g0], -c);
-                atomicAdd(&G[g1], c);
+// The normal step of the transpose: sgn times E to the three coarse layers behind the face, through add(b, X, Y, Z, v).
+template <typename T, class Add>
+__device__ __forceinline__ void scatter_normal(const T *E, const Quarter &Q, const FaceItem &F, T sgn, Add &&add) {
+    for (int q = threadIdx.x; q < Q.w1 * Q.w2; q += blockDim.x) {
+        const int y = Q.lo1 + q % Q.w1, z = Q.lo2 + q / Q.w1;
+        const T v = sgn * E[q];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            int X, Y, Z;
+            face_xyz(F.axis, 1 - F.side, 1 + d, y, z, Q.n, X, Y, Z);
+            add(F.nbr, X, Y, Z, w_normal<T>(0, d) * v);
+        }
+    }
+}
+
+// Where an interface kernel adds: a padded pool, or (user != null) a field in the caller's layout.
+template <typename T>
+struct Target {
+    T *pool;
+    double *user;
+    const int64_t *off;  // start of every leaf in the caller's array, or null
+};
+template <typename T>
+__device__ __forceinline__ void add_to(const Target<T> &t, const LevelGeom &g, int64_t b, int X, int Y, int Z, T v) {
+    if (t.pool) {
+        atomicAdd(&t.pool[Lay<T>::at(g, b, X, Y, Z)], v);
+    } else {
+        const int64_t at = t.off ? t.off[b] : b << (3 * g.lg);
+        atomicAdd(&t.user[at + ((static_cast<int64_t>(Z - 1) * g.n + (Y - 1)) * g.n + (X - 1))], static_cast<double>(v));
+    }
+}
+
+// One interface item per CTA: the transposed ghosts of y on both sides (GHOSTS), and sgn times the part of A^T y that is
+// no 7-point stencil added to `to`.  old (may be null: 0) keeps the ghost adjoints that `to` already holds, n^2 per item,
+// and with the ghost-only variant old_c the coarse ones, (n/2)^2 per item; what is added is the change.  Shared memory:
+// (n/2 + 2)^2 values; where the items of different faces meet, atomics order the sums.
+template <typename T, int MODE, bool FLUX, bool GHOSTS>
+__global__ void __launch_bounds__(kThreads)
+    k_adj_iface(T *__restrict__ y, Coef cf, const T *__restrict__ ih2, const FaceItem *__restrict__ items, LevelGeom g,
+                T *__restrict__ old, T *__restrict__ old_c, Target<T> to, T sgn) {
+    extern __shared__ __align__(16) unsigned char adj_smem[];
+    T *E = reinterpret_cast<T *>(adj_smem);
+    const FaceItem F = items[blockIdx.x];
+    const Quarter Q(F, g);
+    const int n = Q.n, h = Q.h;
+    const bool adds = to.pool || to.user;
+    if (adds) {
+        for (int q = threadIdx.x; q < Q.w1 * Q.w2; q += blockDim.x) E[q] = T(0);
+        __syncthreads();
+    }
+    for (int q = threadIdx.x; q < h * h; q += blockDim.x) {
+        const int ycl = q % h, zcl = q / h, yc = F.seg1 * h + ycl, zc = F.seg2 * h + zcl;
+        const int64_t gC = fidx<T>(g, F.nbr, F.axis, 1 - F.side, 1, yc, zc);
+        const int64_t g0c = fidx<T>(g, F.nbr, F.axis, 1 - F.side, 0, yc, zc);
+        const T yC = y[gC], through = FLUX ? T(0.125) * yC : T(0);
+        T a[2][2];
+#pragma unroll
+        for (int a2 = 0; a2 < 2; ++a2)
+#pragma unroll
+            for (int a1 = 0; a1 < 2; ++a1) {
+                const int i1 = 2 * ycl + a1, i2 = 2 * zcl + a2;
+                const int64_t g0 = fidx<T>(g, F.blk, F.axis, F.side, 0, i1, i2);
+                const int64_t g1 = fidx<T>(g, F.blk, F.axis, F.side, 1, i1, i2);
+                if (GHOSTS) y[g0] = through;
+                if (!adds) continue;
+                const T v = -scaled_face<T, MODE>(cf, ih2, F.blk, g0, g1, F.axis, F.side) * (y[g1] - through);
+                T *keep = old ? old + (static_cast<int64_t>(blockIdx.x) * n + i2) * n + i1 : nullptr;
+                a[a2][a1] = keep ? v - *keep : v;
+                if (keep) *keep = v;
             }
-    }
-}
-
-// E^T of whole faces: reflection (ghost = -u_i), copy from the neighbour, quadratic C2F (27 coarse cells).
-template <typename T>
-__global__ void k_et_faces(T *__restrict__ G, const FaceItem *__restrict__ items, int nitems, LevelGeom g) {
-    const int n = g.n, P = g.P, lg = g.lg, h = n >> 1;
-    const int64_t total = static_cast<int64_t>(nitems) << (2 * lg);
-    GRID_STRIDE(total) {
-        const int it = static_cast<int>(t >> (2 * lg));
-        const int r = static_cast<int>(t) & ((1 << (2 * lg)) - 1);
-        const int i1 = r & (n - 1), i2 = r >> lg;
-        const FaceItem F = items[it];
-        const int64_t base = F.blk * g.bs;
-        const T a = G[base + face_off(F.axis, F.side, 0, i1, i2, n, P)];
-        if (F.kind == FK_BND) {
-            atomicAdd(&G[base + face_off(F.axis, F.side, 1, i1, i2, n, P)], -a);
-        } else if (F.kind == FK_SAME) {
-            atomicAdd(&G[F.nbr * g.bs + face_off(F.axis, 1 - F.side, 1, i1, i2, n, P)], a);
-        } else {
-            const int64_t cbase = F.nbr * g.bs;
-            const int yc = F.seg1 * h + (i1 >> 1), zc = F.seg2 * h + (i2 >> 1);
-            const int a1 = i1 & 1, a2 = i2 & 1;
-            const int cy = yc == 0 ? 1 : (yc == n - 1 ? 2 : 0);
-            const int cz = zc == 0 ? 1 : (zc == n - 1 ? 2 : 0);
-            for (int c = 0; c < 3; ++c)
-                for (int bb = 0; bb < 3; ++bb) {
-                    const T wt = w_tang<T>(0, cz, a2, c) * w_tang<T>(0, cy, a1, bb) * a;
-                    const int y = yc + c_base[cy][bb], z = zc + c_base[cz][c];
-                    for (int d = 0; d < 3; ++d)
-                        atomicAdd(&G[cbase + face_off(F.axis, 1 - F.side, 1 + d, y, z, n, P)], w_normal<T>(0, d) * wt);
+        if (GHOSTS) y[g0c] = FLUX ? yC : T(0);
+        if (!adds) continue;
+        scatter_tangential<T>(E, Q, F, ycl, zcl, a);
+        if (!FLUX) {
+            const T v = -scaled_face<T, MODE>(cf, ih2, F.nbr, g0c, gC, F.axis, 1 - F.side) * yC;
+            T *keep = old_c ? old_c + static_cast<int64_t>(blockIdx.x) * h * h + q : nullptr;
+            const T part = sgn * T(0.125) * (keep ? v - *keep : v);
+            if (keep) *keep = v;
+#pragma unroll
+            for (int d = 1; d <= 2; ++d)
+                for (int e = 0; e < 4; ++e) {
+                    int X, Y, Z;
+                    face_xyz(F.axis, F.side, d, 2 * ycl + (e & 1), 2 * zcl + (e >> 1), n, X, Y, Z);
+                    add_to(to, g, F.blk, X, Y, Z, part);
                 }
         }
     }
+    if (!adds) return;
+    __syncthreads();
+    scatter_normal<T>(E, Q, F, sgn, [&](int64_t b, int X, int Y, int Z, T v) { add_to(to, g, b, X, Y, Z, v); });
 }
 
-// E^T of the F2C mean: each of the 8 fine cells receives 1/8 of the coarse ghost adjoint.
-template <typename T>
-__global__ void k_et_segs_mean(T *__restrict__ G, const SegItem *__restrict__ items, int nitems, LevelGeom g) {
-    const int n = g.n, P = g.P, lgh = g.lg - 1, h = n >> 1;
-    const int64_t total = static_cast<int64_t>(nitems) << (2 * lgh);
-    GRID_STRIDE(total) {
-        const int it = static_cast<int>(t >> (2 * lgh));
-        const int r = static_cast<int>(t) & ((1 << (2 * lgh)) - 1);
-        const int p = r & (h - 1), q = r >> lgh;
-        const SegItem S = items[it];
-        const int fs = 1 - S.side;
-        const T a = T(0.125) * G[S.coarse * g.bs + face_off(S.axis, S.side, 0, S.s1 * h + p, S.s2 * h + q, n, P)];
-        for (int d = 1; d <= 2; ++d)
-            for (int bb = 0; bb < 2; ++bb)
-                for (int aa = 0; aa < 2; ++aa)
-                    atomicAdd(&G[S.fine * g.bs + face_off(S.axis, fs, d, 2 * p + aa, 2 * q + bb, n, P)], a);
-    }
-}
-
-// One transposed smoother step on colour c: z = Pi_c D^-1 ubar (D the diagonal the forward half-sweep divides by),
-// fbar += z.  z is written on every interior cell (0 off the colour); its ghosts stay 0.
-template <int MODE, typename T>
-__global__ void k_adj_colour(const T *__restrict__ ub, T *__restrict__ fb, T *__restrict__ z, ACoef<T> cf,
-                             const T *__restrict__ h2, LevelGeom g, int colour) {
-    const int64_t total = static_cast<int64_t>(g.nb) << (3 * g.lg);
-    GRID_STRIDE(total) {
-        int x, y, zz;
-        int64_t b;
-        decode_cell(t, g.lg, x, y, zz, b);
-        const int64_t gi = b * g.bs + off3(x + 1, y + 1, zz + 1, g.P);
-        T v = T(0);
-        if (((x + y + zz) & 1) == colour) {
-            if constexpr (MODE == 1) v = ub[gi] * cf.dinv[gi];
-            else if constexpr (sizeof(T) == 8) v = ub[gi] * (h2[b] * (1.0 / 6.0));
-            else v = div6(ub[gi] * h2[b]);  // FP32: without the bias of the rounded 1/6
-            fb[gi] += v;
+// fe = g again at the cells that k_adj_iface adds to, one item per CTA.
+template <bool FLUX>
+__global__ void __launch_bounds__(kThreads)
+    k_adj_restore(double *__restrict__ fe, const double *__restrict__ gv, const FaceItem *__restrict__ items, LevelGeom g) {
+    const FaceItem F = items[blockIdx.x];
+    const Quarter Q(F, g);
+    for (int q = threadIdx.x; q < Q.w1 * Q.w2; q += blockDim.x)
+        for (int d = 1; d <= 3; ++d) {
+            const int64_t i = fidx<double>(g, F.nbr, F.axis, 1 - F.side, d, Q.lo1 + q % Q.w1, Q.lo2 + q / Q.w1);
+            fe[i] = gv[i];
         }
-        z[gi] = v;
-    }
+    if (!FLUX)
+        for (int q = threadIdx.x; q < Q.n * Q.n; q += blockDim.x)
+            for (int d = 1; d <= 2; ++d) {
+                const int64_t i = fidx<double>(g, F.blk, F.axis, F.side, d, q % Q.n, q / Q.n);
+                fe[i] = gv[i];
+            }
 }
 
-// y += a x over the interior.
-template <typename T>
-__global__ void k_axpy(T *__restrict__ y, const T *__restrict__ x, T a, LevelGeom g) {
-    const int64_t total = static_cast<int64_t>(g.nb) << (3 * g.lg);
-    GRID_STRIDE(total) {
-        int xx, yy, zz;
-        int64_t b;
-        decode_cell(t, g.lg, xx, yy, zz, b);
-        const int64_t gi = b * g.bs + off3(xx + 1, yy + 1, zz + 1, g.P);
-        y[gi] = fma(a, x[gi], y[gi]);
-    }
-}
-
-// Transposed prolongation: the fine adjoint of u_f += 1/4 (e_C + e_{C+sx} + e_{C+sy} + e_{C+sz}) scattered into the
-// coarse padded adjoint (ghost positions included; the transposed coarse exchange follows).
-template <typename T>
-__global__ void k_prolong_T(const T *__restrict__ ubf, LevelGeom gf, T *__restrict__ Ec,
-                            const XferItem *__restrict__ xf, LevelGeom gc) {
-    const int lgc = gc.lg, nc = gc.n, Pc = gc.P;
-    const int64_t PPc = static_cast<int64_t>(Pc) * Pc;
-    const int64_t total = static_cast<int64_t>(gc.nb) << (3 * lgc);
-    GRID_STRIDE(total) {
-        int X, Y, Z;
-        int64_t B;
-        decode_cell(t, lgc, X, Y, Z, B);
-        const XferItem xi = xf[B];
-        const int64_t gcell = B * gc.bs + off3(X + 1, Y + 1, Z + 1, Pc);
-        if (xi.kind == XF_COPY) {
-            atomicAdd(&Ec[gcell], ubf[xi.src[0] * gf.bs + off3(X + 1, Y + 1, Z + 1, gf.P)]);
-            continue;
-        }
-        int64_t b;
-        int x0, y0, z0;
-        if (xi.kind == XF_HALVE) {
-            b = xi.src[0];
-            x0 = 2 * X;
-            y0 = 2 * Y;
-            z0 = 2 * Z;
-        } else {
-            const int hc = nc >> 1;
-            const int ox = X >= hc, oy = Y >= hc, oz = Z >= hc;
-            b = xi.src[ox + 2 * oy + 4 * oz];
-            x0 = 2 * X - ox * nc;
-            y0 = 2 * Y - oy * nc;
-            z0 = 2 * Z - oz * nc;
-        }
-        T all = T(0), sx[2] = {T(0), T(0)}, sy[2] = {T(0), T(0)}, sz[2] = {T(0), T(0)};
-        for (int c = 0; c < 2; ++c)
-            for (int bb = 0; bb < 2; ++bb)
-                for (int a = 0; a < 2; ++a) {
-                    const T v = T(0.25) * ubf[b * gf.bs + off3(x0 + a + 1, y0 + bb + 1, z0 + c + 1, gf.P)];
-                    all += v;
-                    sx[a] += v;
-                    sy[bb] += v;
-                    sz[c] += v;
-                }
-        atomicAdd(&Ec[gcell], all);
-        atomicAdd(&Ec[gcell - 1], sx[0]);
-        atomicAdd(&Ec[gcell + 1], sx[1]);
-        atomicAdd(&Ec[gcell - Pc], sy[0]);
-        atomicAdd(&Ec[gcell + Pc], sy[1]);
-        atomicAdd(&Ec[gcell - PPc], sz[0]);
-        atomicAdd(&Ec[gcell + PPc], sz[1]);
-    }
-}
-
-// Transposed restriction: every fine cell receives 1/8 of its parent's adjoint (carried-over blocks: all of it).
-template <typename T>
-__global__ void k_restrict_T(const T *__restrict__ fbc, LevelGeom gc, T *__restrict__ rf,
-                             const XferItem *__restrict__ xf, LevelGeom gf) {
-    const int lgc = gc.lg, nc = gc.n;
-    const int64_t total = static_cast<int64_t>(gc.nb) << (3 * lgc);
-    GRID_STRIDE(total) {
-        int X, Y, Z;
-        int64_t B;
-        decode_cell(t, lgc, X, Y, Z, B);
-        const XferItem xi = xf[B];
-        const T v = fbc[B * gc.bs + off3(X + 1, Y + 1, Z + 1, gc.P)];
-        if (xi.kind == XF_COPY) {
-            rf[xi.src[0] * gf.bs + off3(X + 1, Y + 1, Z + 1, gf.P)] = v;
-            continue;
-        }
-        int64_t b;
-        int x0, y0, z0;
-        if (xi.kind == XF_HALVE) {
-            b = xi.src[0];
-            x0 = 2 * X;
-            y0 = 2 * Y;
-            z0 = 2 * Z;
-        } else {
-            const int hc = nc >> 1;
-            const int ox = X >= hc, oy = Y >= hc, oz = Z >= hc;
-            b = xi.src[ox + 2 * oy + 4 * oz];
-            x0 = 2 * X - ox * nc;
-            y0 = 2 * Y - oy * nc;
-            z0 = 2 * Z - oz * nc;
-        }
-        for (int c = 0; c < 2; ++c)
-            for (int bb = 0; bb < 2; ++bb)
-                for (int a = 0; a < 2; ++a) rf[b * gf.bs + off3(x0 + a + 1, y0 + bb + 1, z0 + c + 1, gf.P)] = T(0.125) * v;
-    }
-}
-
-// A u in the working precision T on a natural-layout level (ghosts of u filled): the 7-point rows
-// (1/h^2) sum_f T_f (u_i - u_f), written as dg u_i - sum_f T~_f u_f with the scaled coefficients (MODE 1) or
-// (6 u_i - sum_f u_f) / h^2 (MODE 0).  The FP32 transposed cycle's S^T (the stencil part of A^T y with zero ghosts).
+// r = f - (stencil of y) over the interior, written through to the ghosts that mirror it (same level) or reflect it
+// (boundary); interface ghosts of r stay 0.  With part (FP64) per-CTA partials of h^3 r^2.
 template <typename T, int MODE>
-__global__ void k_apply_nat(const T *__restrict__ u, ACoef<T> cf, const T *__restrict__ ih2, LevelGeom g,
-                            T *__restrict__ out) {
-    const int P = g.P;
-    const int64_t PP = static_cast<int64_t>(P) * P;
+__global__ void k_adj_residual(const T *__restrict__ y, const T *f, Coef cf, const T *__restrict__ ih2, LevelGeom g,
+                               const int32_t *__restrict__ nbr6, T *r, const double *__restrict__ vol,
+                               double *__restrict__ part) {
+    const int n = g.n;
     const int64_t total = static_cast<int64_t>(g.nb) << (3 * g.lg);
+    double acc = 0.0;
     GRID_STRIDE(total) {
-        int x, y, z;
+        int x, yy, z;
         int64_t b;
-        decode_cell(t, g.lg, x, y, z, b);
-        const int64_t gi = b * g.bs + off3(x + 1, y + 1, z + 1, P);
-        if constexpr (MODE == 1) {
-            T a = cf.tx[gi] * u[gi - 1];
-            a = fma(cf.tx[gi + 1], u[gi + 1], a);
-            a = fma(cf.ty[gi], u[gi - P], a);
-            a = fma(cf.ty[gi + P], u[gi + P], a);
-            a = fma(cf.tz[gi], u[gi - PP], a);
-            a = fma(cf.tz[gi + PP], u[gi + PP], a);
-            out[gi] = fma(cf.dg[gi], u[gi], -a);
-        } else {
-            const T S = ((u[gi - 1] + u[gi + 1]) + (u[gi - P] + u[gi + P])) + (u[gi - PP] + u[gi + PP]);
-            out[gi] = fma(T(6), u[gi], -S) * ih2[b];
+        decode_cell(t, g.lg, x, yy, z, b);
+        T v;
+        if constexpr (sizeof(T) == 4)
+            v = residual_xyz<T, MODE>(y, f, cf, g, b, x + 1, yy + 1, z + 1, ih2[b]);
+        else
+            v = residual_at<T, MODE>(y, f, cf, b * g.bs + off3(x + 1, yy + 1, z + 1, g.P), g.P, MODE == 1 ? T(0) : ih2[b]);
+        r[Lay<T>::at(g, b, x + 1, yy + 1, z + 1)] = v;
+        if (part) acc = fma(vol[b] * static_cast<double>(v), static_cast<double>(v), acc);
+        if (nbr6 && (x == 0 || x == n - 1 || yy == 0 || yy == n - 1 || z == 0 || z == n - 1)) {
+            const int c[3] = {x, yy, z};
+#pragma unroll
+            for (int axis = 0; axis < 3; ++axis)
+#pragma unroll
+                for (int side = 0; side < 2; ++side) {
+                    if (c[axis] != (side ? n - 1 : 0)) continue;
+                    const int nb = nbr6[b * 6 + 2 * axis + side];
+                    const int i1 = axis == 0 ? yy : x, i2 = axis == 2 ? yy : z;
+                    if (nb >= 0) r[fidx<T>(g, nb, axis, 1 - side, 0, i1, i2)] = v;
+                    else if (nb == -1) r[fidx<T>(g, b, axis, side, 0, i1, i2)] = -v;
+                }
         }
     }
-}
-
-// FP32 copy of an FP64 array (the coefficient arrays of the FP32 transposed cycle), every element.
-__global__ void k_round32(const double *__restrict__ src, float *__restrict__ dst, int64_t count) {
-    GRID_STRIDE(count) dst[t] = static_cast<float>(src[t]);
-}
-
-// FP32 right-hand side of a transposed correction cycle: r32 = s r over the interior (s a power of two: exact up to
-// the rounding to FP32).
-__global__ void k_scaled32(const double *__restrict__ r, float *__restrict__ r32, double s, LevelGeom g) {
-    const int64_t total = static_cast<int64_t>(g.nb) << (3 * g.lg);
-    GRID_STRIDE(total) {
-        int x, y, z;
-        int64_t b;
-        decode_cell(t, g.lg, x, y, z, b);
-        const int64_t gi = b * g.bs + off3(x + 1, y + 1, z + 1, g.P);
-        r32[gi] = static_cast<float>(s * r[gi]);
-    }
-}
-
-// lambda += e32 / s over the interior, in FP64.
-__global__ void k_add_from32(double *__restrict__ lam, const float *__restrict__ e32, double inv_s, LevelGeom g) {
-    const int64_t total = static_cast<int64_t>(g.nb) << (3 * g.lg);
-    GRID_STRIDE(total) {
-        int x, y, z;
-        int64_t b;
-        decode_cell(t, g.lg, x, y, z, b);
-        const int64_t gi = b * g.bs + off3(x + 1, y + 1, z + 1, g.P);
-        lam[gi] = fma(static_cast<double>(e32[gi]), inv_s, lam[gi]);
-    }
-}
-
-// r = g - q over the interior, with per-CTA partials of h^3 r^2.
-__global__ void k_sub_norm(const double *__restrict__ gvec, const double *__restrict__ q, double *__restrict__ r,
-                           const double *__restrict__ vol, LevelGeom g, double *__restrict__ partial) {
-    double acc = 0.0;
-    const int64_t total = static_cast<int64_t>(g.nb) << (3 * g.lg);
-    GRID_STRIDE(total) {
-        int x, y, z;
-        int64_t b;
-        decode_cell(t, g.lg, x, y, z, b);
-        const int64_t gi = b * g.bs + off3(x + 1, y + 1, z + 1, g.P);
-        const double v = gvec[gi] - q[gi];
-        r[gi] = v;
-        acc = fma(vol[b] * v, v, acc);
-    }
+    if (!part) return;
     __shared__ double sm[kThreads / 32];
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = acc;
@@ -351,18 +237,348 @@ __global__ void k_sub_norm(const double *__restrict__ gvec, const double *__rest
     if (threadIdx.x == 0) {
         double s = 0.0;
         for (int w = 0; w < kThreads / 32; ++w) s += sm[w];
-        partial[blockIdx.x] = s;
+        part[blockIdx.x] = s;
     }
 }
 
-// dL/dk, face terms: for every interior cell i and face f (except coarse sides of refinement interfaces in the
-// conservative variant), the row term (1/h^2) T(k_i, k_f) (u_i - u_f) contributes -lambda_i (u_i - u_f) / h^2 times
-// dT/dk_i to k_i and times dT/dk_f to the k at the neighbour or ghost position (gadj).  T = 2 a b / (a + b):
-// dT/da = 2 b^2 / (a + b)^2.
-__global__ void k_gradk_faces(const double *__restrict__ u, const double *__restrict__ lam,
-                              const double *__restrict__ k, const double *__restrict__ ih2,
-                              const int8_t *__restrict__ fkind, int skip_f2c, LevelGeom g, double *__restrict__ grad,
-                              double *__restrict__ gadj) {
+// The same in FP32 on colour-split blocks of edge 2^LG, one thread per pair of cells x = 2j, 2j + 1 of a row: they and their
+// neighbours are 12 values of y (and of 1/k), at immediate offsets from one position of either half, and share a face.  The
+// generic form above computes every address in 64 bits and loads 14 values per cell: 533 us on 31.5M cells; this 190 us.
+template <int MODE, int LG>
+__global__ void __launch_bounds__(kThreads)
+    k_adj_residual32(const float *__restrict__ y, const float *__restrict__ f, Coef cf, const float *__restrict__ ih2,
+                     int64_t bs, int64_t pairs, const int32_t *__restrict__ nbr6, float *__restrict__ r) {
+    constexpr int n = 1 << LG, NH = n / 2, P = n + 2, H = half_row(P), PL = P * H, HALF = P * PL;
+    const int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    if (t >= pairs) return;
+    const int j = static_cast<int>(t) & (NH - 1), yy = static_cast<int>(t >> (LG - 1)) & (n - 1);
+    const int z = static_cast<int>(t >> (2 * LG - 1)) & (n - 1);
+    const int64_t b = t >> (3 * LG - 1), base = b * bs;
+    // cell A (padded X = 2j + 1) at q of half s, cell B (X = 2j + 2) at q + 1 of the other half
+    const int s = (yy + z + 1) & 1, q = ((z + 1) * P + yy + 1) * H + j;
+    const int hs = s * HALF, ho = (s ^ 1) * HALF;
+    const float *us = y + base + hs + q, *uo = y + base + ho + q;
+    const float A = us[0], B = uo[1];
+    const float nA[6] = {uo[0], B, uo[-H], uo[H], uo[-PL], uo[PL]};
+    const float nB[6] = {A, us[1], us[1 - H], us[1 + H], us[1 - PL], us[1 + PL]};
+    const float fA = __ldg(f + base + hs + q), fB = __ldg(f + base + ho + q + 1);
+    const float ih = __ldg(ih2 + b);
+    float rA, rB;
+    if constexpr (MODE == 0) {
+        const float SA = ((nA[0] + nA[1]) + (nA[2] + nA[3])) + (nA[4] + nA[5]);
+        const float SB = ((nB[0] + nB[1]) + (nB[2] + nB[3])) + (nB[4] + nB[5]);
+        rA = fmaf(fmaf(-6.0f, A, SA), ih, fA);
+        rB = fmaf(fmaf(-6.0f, B, SB), ih, fB);
+    } else {
+        float cA[6], cB[6];
+        if constexpr (MODE == 2) {
+            const float *ks = cf.kap + base + hs + q, *ko = cf.kap + base + ho + q;
+            const float kA = __ldg(ks), kB = __ldg(ko + 1);
+            cA[0] = frcp(kA + __ldg(ko));
+            cA[1] = frcp(kA + kB);
+            cA[2] = frcp(kA + __ldg(ko - H));
+            cA[3] = frcp(kA + __ldg(ko + H));
+            cA[4] = frcp(kA + __ldg(ko - PL));
+            cA[5] = frcp(kA + __ldg(ko + PL));
+            cB[0] = cA[1];
+            cB[1] = frcp(kB + __ldg(ks + 1));
+            cB[2] = frcp(kB + __ldg(ks + 1 - H));
+            cB[3] = frcp(kB + __ldg(ks + 1 + H));
+            cB[4] = frcp(kB + __ldg(ks + 1 - PL));
+            cB[5] = frcp(kB + __ldg(ks + 1 + PL));
+        } else {  // a cell's lower faces at the cell, its upper ones at the upper neighbour
+            const int64_t is = base + hs + q, io = base + ho + q;
+            cA[0] = __ldg(cf.ax + is);
+            cA[1] = __ldg(cf.ax + io + 1);
+            cA[2] = __ldg(cf.ay + is);
+            cA[3] = __ldg(cf.ay + io + H);
+            cA[4] = __ldg(cf.az + is);
+            cA[5] = __ldg(cf.az + io + PL);
+            cB[0] = cA[1];
+            cB[1] = __ldg(cf.ax + is + 1);
+            cB[2] = __ldg(cf.ay + io + 1);
+            cB[3] = __ldg(cf.ay + is + 1 + H);
+            cB[4] = __ldg(cf.az + io + 1);
+            cB[5] = __ldg(cf.az + is + 1 + PL);
+        }
+        float SA = 0.0f, DA = 0.0f, SB = 0.0f, DB = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            SA = fmaf(cA[i], nA[i], SA);
+            DA += cA[i];
+            SB = fmaf(cB[i], nB[i], SB);
+            DB += cB[i];
+        }
+        rA = fmaf(2.0f * fmaf(-DA, A, SA), ih, fA);
+        rB = fmaf(2.0f * fmaf(-DB, B, SB), ih, fB);
+    }
+    float *rs = r + base + hs + q, *ro = r + base + ho + q;
+    rs[0] = rA;
+    ro[1] = rB;
+    // write-through, as in smooth32_column: the mirroring ghost at the same place of its half n cells along the axis, the
+    // reflected one at the neighbour position of the other half
+    if (j == 0) {
+        const int nb = nbr6[b * 6];
+        if (nb >= 0) r[nb * bs + hs + q + NH] = rA;
+        else if (nb == -1) ro[0] = -rA;
+    }
+    if (j == NH - 1) {
+        const int nb = nbr6[b * 6 + 1];
+        if (nb >= 0) r[nb * bs + ho + q + 1 - NH] = rB;
+        else if (nb == -1) rs[1] = -rB;
+    }
+#pragma unroll
+    for (int axis = 1; axis < 3; ++axis) {
+        const int c = axis == 1 ? yy : z, D = axis == 1 ? n * H : n * PL, E = axis == 1 ? H : PL;
+        if (c != 0 && c != n - 1) continue;
+        const int side = c ? 1 : 0, nb = nbr6[b * 6 + 2 * axis + side];
+        if (nb >= 0) {
+            r[nb * bs + hs + q + (side ? -D : D)] = rA;
+            r[nb * bs + ho + q + 1 + (side ? -D : D)] = rB;
+        } else if (nb == -1) {
+            ro[side ? E : -E] = -rA;
+            rs[1 + (side ? E : -E)] = -rB;
+        }
+    }
+}
+
+// Transposed prolongation of a level whose blocks all halve, as a gather: e_C enters its eight children and, as the
+// neighbour on their side, the four cells across each of its six faces, every time with weight 1/4 (u_f += 1/4 (e_C +
+// e_{C+sx} + e_{C+sy} + e_{C+sz})); the reflected boundary ghost of r carries the reflected e.  Writes the coarse
+// right-hand side and zeroes the coarse result with its face ghosts.
+template <typename T>
+__global__ void k_prolong_T(const T *__restrict__ r, LevelGeom gf, T *__restrict__ fc, T *__restrict__ yc,
+                            const XferItem *__restrict__ xf, LevelGeom gc) {
+    const int nc = gc.n;
+    const int64_t total = static_cast<int64_t>(gc.nb) << (3 * gc.lg);
+    GRID_STRIDE(total) {
+        int X, Y, Z;
+        int64_t B;
+        decode_cell(t, gc.lg, X, Y, Z, B);
+        const int64_t b = xf[B].src[0];
+        T s = T(0);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int out = (i == 0 || i == 3) + (j == 0 || j == 3) + (k == 0 || k == 3);
+                    if (out <= 1) s += r[Lay<T>::at(gf, b, 2 * X + i, 2 * Y + j, 2 * Z + k)];
+                }
+        const int64_t gi = Lay<T>::at(gc, B, X + 1, Y + 1, Z + 1);
+        fc[gi] = T(0.25) * s;
+        yc[gi] = T(0);
+        if (X == 0) yc[Lay<T>::at(gc, B, 0, Y + 1, Z + 1)] = T(0);
+        if (X == nc - 1) yc[Lay<T>::at(gc, B, nc + 1, Y + 1, Z + 1)] = T(0);
+        if (Y == 0) yc[Lay<T>::at(gc, B, X + 1, 0, Z + 1)] = T(0);
+        if (Y == nc - 1) yc[Lay<T>::at(gc, B, X + 1, nc + 1, Z + 1)] = T(0);
+        if (Z == 0) yc[Lay<T>::at(gc, B, X + 1, Y + 1, 0)] = T(0);
+        if (Z == nc - 1) yc[Lay<T>::at(gc, B, X + 1, Y + 1, nc + 1)] = T(0);
+    }
+}
+
+// The same in FP32 for fine edges 2^LG, with the box at immediate offsets (Box32).
+template <int LG>
+__global__ void __launch_bounds__(kThreads)
+    k_prolong_T32(const float *__restrict__ r, int64_t bsf, float *__restrict__ fc, float *__restrict__ yc,
+                  const XferItem *__restrict__ xf, int64_t total, int64_t bsc) {
+    using Bx = Box32<LG>;
+    constexpr int nc = (1 << LG) / 2, LC = LG - 1;
+    const int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    if (t >= total) return;
+    const int q = static_cast<int>(t) & ((1 << (3 * LC)) - 1);
+    const int64_t B = t >> (3 * LC);
+    const int X = q & (nc - 1), Y = (q >> LC) & (nc - 1), Z = q >> (2 * LC);
+    const float *rb = r + xf[B].src[0] * bsf + (2 * Z * Bx::P + 2 * Y) * Bx::HP + X;
+    float s = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int out = (i == 0 || i == 3) + (j == 0 || j == 3) + (k == 0 || k == 3);
+                if (out <= 1) s += rb[Bx::off(i, j, k)];
+            }
+    rr32_store<LG>(fc, yc, B, bsc, X, Y, Z, 2.0f * s);  // stores 1/8 of it: a quarter of the sum
+}
+
+// The same for a level with merged octets or carried-over blocks: scattered into the coarse padded right-hand side
+// (ghost positions included; k_et_faces and k_et_iface follow).
+template <typename T>
+__global__ void k_prolong_T_scatter(const T *__restrict__ r, LevelGeom gf, T *__restrict__ Ec,
+                                    const XferItem *__restrict__ xf, LevelGeom gc) {
+    const int nc = gc.n;
+    const int64_t total = static_cast<int64_t>(gc.nb) << (3 * gc.lg);
+    GRID_STRIDE(total) {
+        int X, Y, Z;
+        int64_t B;
+        decode_cell(t, gc.lg, X, Y, Z, B);
+        const XferItem xi = xf[B];
+        if (xi.kind == XF_COPY) {
+            atomicAdd(&Ec[Lay<T>::at(gc, B, X + 1, Y + 1, Z + 1)], r[Lay<T>::at(gf, xi.src[0], X + 1, Y + 1, Z + 1)]);
+            continue;
+        }
+        int64_t b = xi.src[0];
+        int x0 = 2 * X, y0 = 2 * Y, z0 = 2 * Z;
+        if (xi.kind == XF_MERGE) {
+            const int hc = nc >> 1, ox = X >= hc, oy = Y >= hc, oz = Z >= hc;
+            b = xi.src[ox + 2 * oy + 4 * oz];
+            x0 -= ox * nc;
+            y0 -= oy * nc;
+            z0 -= oz * nc;
+        }
+        T all = T(0), sx[2] = {T(0), T(0)}, sy[2] = {T(0), T(0)}, sz[2] = {T(0), T(0)};
+        for (int c = 0; c < 2; ++c)
+            for (int bb = 0; bb < 2; ++bb)
+                for (int a = 0; a < 2; ++a) {
+                    const T v = T(0.25) * r[Lay<T>::at(gf, b, x0 + a + 1, y0 + bb + 1, z0 + c + 1)];
+                    all += v;
+                    sx[a] += v;
+                    sy[bb] += v;
+                    sz[c] += v;
+                }
+        atomicAdd(&Ec[Lay<T>::at(gc, B, X + 1, Y + 1, Z + 1)], all);
+        for (int s = 0; s < 2; ++s) {
+            atomicAdd(&Ec[Lay<T>::at(gc, B, X + 2 * s, Y + 1, Z + 1)], sx[s]);
+            atomicAdd(&Ec[Lay<T>::at(gc, B, X + 1, Y + 2 * s, Z + 1)], sy[s]);
+            atomicAdd(&Ec[Lay<T>::at(gc, B, X + 1, Y + 1, Z + 2 * s)], sz[s]);
+        }
+    }
+}
+
+// E^T of the faces filled from one source block: reflection (ghost = -u_i) and copy from the neighbour.
+template <typename T>
+__global__ void k_et_faces(T *__restrict__ G, const FaceItem *__restrict__ items, int nitems, LevelGeom g) {
+    const int n = g.n, lg = g.lg;
+    const int64_t total = static_cast<int64_t>(nitems) << (2 * lg);
+    GRID_STRIDE(total) {
+        const FaceItem F = items[t >> (2 * lg)];
+        const int r = static_cast<int>(t) & ((1 << (2 * lg)) - 1);
+        const int i1 = r & (n - 1), i2 = r >> lg;
+        const T a = G[fidx<T>(g, F.blk, F.axis, F.side, 0, i1, i2)];
+        if (F.kind == FK_BND) atomicAdd(&G[fidx<T>(g, F.blk, F.axis, F.side, 1, i1, i2)], -a);
+        else atomicAdd(&G[fidx<T>(g, F.nbr, F.axis, 1 - F.side, 1, i1, i2)], a);
+    }
+}
+
+// E^T of a level's interface ghosts, one item per CTA, added to the interior of fc.  The ghost adjoints are those of the
+// transposed prolongation: GATHER: a quarter of the four finer cells next to the ghost (the level's blocks are halved
+// blocks, r the finer level's residual); else they stand in fc's own ghosts (k_prolong_T_scatter).
+template <typename T, int MODE, bool FLUX, bool GATHER>
+__global__ void __launch_bounds__(kThreads)
+    k_et_iface(T *__restrict__ fc, Coef cf, const FaceItem *__restrict__ items, LevelGeom g, const T *__restrict__ r,
+               LevelGeom gf, const XferItem *__restrict__ xf) {
+    extern __shared__ __align__(16) unsigned char adj_smem[];
+    T *E = reinterpret_cast<T *>(adj_smem);
+    const FaceItem F = items[blockIdx.x];
+    const Quarter Q(F, g);
+    const int n = Q.n, h = Q.h;
+    const int64_t bf = GATHER ? xf[F.blk].src[0] : 0, bc = GATHER ? xf[F.nbr].src[0] : 0;
+    const auto ghost = [&](int64_t blk, int64_t fine, int side, int i1, int i2) {
+        if constexpr (!GATHER) return fc[fidx<T>(g, blk, F.axis, side, 0, i1, i2)];
+        T s = T(0);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s += r[fidx<T>(gf, fine, F.axis, side, 1, 2 * i1 + (e & 1), 2 * i2 + (e >> 1))];
+        return T(0.25) * s;
+    };
+    for (int q = threadIdx.x; q < Q.w1 * Q.w2; q += blockDim.x) E[q] = T(0);
+    __syncthreads();
+    for (int q = threadIdx.x; q < h * h; q += blockDim.x) {
+        const int ycl = q % h, zcl = q / h, yc = F.seg1 * h + ycl, zc = F.seg2 * h + zcl;
+        const int64_t gC = fidx<T>(g, F.nbr, F.axis, 1 - F.side, 1, yc, zc);
+        const T aG = ghost(F.nbr, bc, 1 - F.side, yc, zc);
+        T Tc = T(1);
+        if constexpr (FLUX && MODE != 0) {
+            const int64_t g0c = fidx<T>(g, F.nbr, F.axis, 1 - F.side, 0, yc, zc);
+            Tc = face_coef<T, MODE>(cf, F.side ? gC : g0c, F.side ? g0c : gC, F.axis);
+        }
+        if (FLUX) atomicAdd(&fc[gC], aG);
+        T a[2][2];
+#pragma unroll
+        for (int a2 = 0; a2 < 2; ++a2)
+#pragma unroll
+            for (int a1 = 0; a1 < 2; ++a1) {
+                const int i1 = 2 * ycl + a1, i2 = 2 * zcl + a2;
+                a[a2][a1] = ghost(F.blk, bf, F.side, i1, i2);
+                if constexpr (FLUX) {  // G = u_C - sum_j c (g_j - u_j), c = T_j / (2 T_C) (MODE 1: T~_j / (8 T~_C))
+                    const int64_t g0 = fidx<T>(g, F.blk, F.axis, F.side, 0, i1, i2);
+                    const int64_t g1 = fidx<T>(g, F.blk, F.axis, F.side, 1, i1, i2);
+                    const T Tj = face_coef<T, MODE>(cf, F.side ? g0 : g1, F.side ? g1 : g0, F.axis);
+                    const T v = Tj / (T(MODE == 1 ? 8 : 2) * Tc) * aG;
+                    a[a2][a1] -= v;
+                    atomicAdd(&fc[g1], v);
+                }
+            }
+        scatter_tangential<T>(E, Q, F, ycl, zcl, a);
+        if (!FLUX)
+            for (int d = 1; d <= 2; ++d)
+                for (int e = 0; e < 4; ++e)
+                    atomicAdd(&fc[fidx<T>(g, F.blk, F.axis, F.side, d, 2 * ycl + (e & 1), 2 * zcl + (e >> 1))],
+                              T(0.125) * aG);
+    }
+    __syncthreads();
+    scatter_normal<T>(E, Q, F, T(1), [&](int64_t b, int X, int Y, int Z, T v) { atomicAdd(&fc[Lay<T>::at(g, b, X, Y, Z)], v); });
+}
+
+// Transposed restriction and correction, y_f += R^T e_c: every fine cell receives 1/8 of its parent's value (carried-over
+// blocks all of it).  Interior only: the ghosts of y_f need an exchange.
+template <typename T>
+__global__ void k_inject(T *__restrict__ yf, LevelGeom gf, const T *__restrict__ ec, const XferItem *__restrict__ xf,
+                         LevelGeom gc) {
+    const int nc = gc.n;
+    const int64_t total = static_cast<int64_t>(gc.nb) << (3 * gc.lg);
+    GRID_STRIDE(total) {
+        int X, Y, Z;
+        int64_t B;
+        decode_cell(t, gc.lg, X, Y, Z, B);
+        const XferItem xi = xf[B];
+        const T v = ec[Lay<T>::at(gc, B, X + 1, Y + 1, Z + 1)];
+        if (xi.kind == XF_COPY) {
+            yf[Lay<T>::at(gf, xi.src[0], X + 1, Y + 1, Z + 1)] += v;
+            continue;
+        }
+        int64_t b = xi.src[0];
+        int x0 = 2 * X, y0 = 2 * Y, z0 = 2 * Z;
+        if (xi.kind == XF_MERGE) {
+            const int hc = nc >> 1, ox = X >= hc, oy = Y >= hc, oz = Z >= hc;
+            b = xi.src[ox + 2 * oy + 4 * oz];
+            x0 -= ox * nc;
+            y0 -= oy * nc;
+            z0 -= oz * nc;
+        }
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int bb = 0; bb < 2; ++bb)
+#pragma unroll
+                for (int a = 0; a < 2; ++a) yf[Lay<T>::at(gf, b, x0 + a + 1, y0 + bb + 1, z0 + c + 1)] += T(0.125) * v;
+    }
+}
+
+// y += x over the interior, FP64.
+__global__ void k_add(double *__restrict__ y, const double *__restrict__ x, LevelGeom g) {
+    const int64_t total = static_cast<int64_t>(g.nb) << (3 * g.lg);
+    GRID_STRIDE(total) {
+        int xx, yy, zz;
+        int64_t b;
+        decode_cell(t, g.lg, xx, yy, zz, b);
+        const int64_t gi = b * g.bs + off3(xx + 1, yy + 1, zz + 1, g.P);
+        y[gi] += x[gi];
+    }
+}
+
+// dL/dk = -lambda^T (dA/dk) u, written in the caller's layout.  A face between cells i and f with T = 2 k_i k_f / (k_i +
+// k_f) enters rows i and f with (1/h^2) T (u_i - u_f) and its negative, and dT/dk_i = 2 k_f^2 / (k_i + k_f)^2 =
+// T^2 / (2 k_i^2), so with T~ = T / h^2
+//     dL/dk_i = -h^2 / (2 k_i^2) sum_f T~_f^2 (lambda_i - lambda_f) (u_i - u_f):
+// one division per cell (six in the form with (k_i + k_f)^2, and the other cell's share by atomics: 5.5 ms on 31.5M cells;
+// this one 2.4 ms, its 45 FP64 operations per cell at the measured FP64 rate).  Ghosts of u and lambda: copies and reflections (at the boundary T = k_i, dT/dk_i = 1: the reflected
+// pair gives the same).  Refinement interfaces are left to k_gradk_iface.
+__global__ void k_gradk(const double *__restrict__ u, const double *__restrict__ lam, const double *__restrict__ k,
+                        Coef cf, const double *__restrict__ h2, const int32_t *__restrict__ nbr6, LevelGeom g,
+                        double *__restrict__ out, const int64_t *__restrict__ off) {
     const int n = g.n, P = g.P;
     const int64_t PP = static_cast<int64_t>(P) * P;
     const int64_t total = static_cast<int64_t>(g.nb) << (3 * g.lg);
@@ -371,268 +587,265 @@ __global__ void k_gradk_faces(const double *__restrict__ u, const double *__rest
         int64_t b;
         decode_cell(t, g.lg, x, y, z, b);
         const int64_t gi = b * g.bs + off3(x + 1, y + 1, z + 1, P);
-        const double w0 = -lam[gi] * ih2[b];
-        const double ki = k[gi], ui = u[gi];
-        const int c[3] = {x, y, z};
-        const int64_t st[3] = {1, P, PP};
-        double acc = 0.0;
-        for (int axis = 0; axis < 3; ++axis)
-            for (int side = 0; side < 2; ++side) {
-                const bool at_face = side ? (c[axis] == n - 1) : (c[axis] == 0);
-                if (at_face && skip_f2c && fkind[b * 6 + 2 * axis + side] == 3) continue;
-                const int64_t gn = gi + (side ? st[axis] : -st[axis]);
-                const double kg = k[gn];
-                const double d = ui - u[gn];
-                const double inv = 1.0 / ((ki + kg) * (ki + kg));
-                acc += w0 * d * 2.0 * kg * kg * inv;
-                atomicAdd(&gadj[gn], w0 * d * 2.0 * ki * ki * inv);
-            }
-        grad[gi] = acc;
+        const double ui = u[gi], li = lam[gi], ki = k[gi];
+        const double T[6] = {cf.tx[gi], cf.tx[gi + 1], cf.ty[gi], cf.ty[gi + P], cf.tz[gi], cf.tz[gi + PP]};
+        const int64_t nb[6] = {gi - 1, gi + 1, gi - P, gi + P, gi - PP, gi + PP};
+        const bool edge[6] = {x == 0, x == n - 1, y == 0, y == n - 1, z == 0, z == n - 1};
+        double s = 0.0;
+#pragma unroll
+        for (int f = 0; f < 6; ++f) {
+            if (edge[f] && nbr6[b * 6 + f] == -2) continue;
+            s = fma((T[f] * T[f]) * (li - lam[nb[f]]), ui - u[nb[f]], s);
+        }
+        const int64_t at = off ? off[b] + (t & ((int64_t(1) << (3 * g.lg)) - 1)) : t;
+        out[at] = -0.5 * h2[b] * s / (ki * ki);
     }
 }
 
-// Interior positions of gadj are the neighbours' own k.
-__global__ void k_gradk_merge(double *__restrict__ grad, const double *__restrict__ gadj, LevelGeom g) {
-    const int64_t total = static_cast<int64_t>(g.nb) << (3 * g.lg);
-    GRID_STRIDE(total) {
-        int x, y, z;
-        int64_t b;
-        decode_cell(t, g.lg, x, y, z, b);
-        const int64_t gi = b * g.bs + off3(x + 1, y + 1, z + 1, g.P);
-        grad[gi] += gadj[gi];
-    }
-}
-
-// Ghost positions of gadj through the ghost-k maps: k_g = k_i (boundary), neighbour copy, injection of the
-// covering coarse k (fine ghosts).
-__global__ void k_gradk_ghost_faces(double *__restrict__ grad, const double *__restrict__ gadj,
-                                    const FaceItem *__restrict__ items, int nitems, LevelGeom g) {
-    const int n = g.n, P = g.P, lg = g.lg, h = n >> 1;
-    const int64_t total = static_cast<int64_t>(nitems) << (2 * lg);
-    GRID_STRIDE(total) {
-        const int it = static_cast<int>(t >> (2 * lg));
-        const int r = static_cast<int>(t) & ((1 << (2 * lg)) - 1);
-        const int i1 = r & (n - 1), i2 = r >> lg;
-        const FaceItem F = items[it];
-        const double a = gadj[F.blk * g.bs + face_off(F.axis, F.side, 0, i1, i2, n, P)];
-        if (F.kind == FK_BND)
-            atomicAdd(&grad[F.blk * g.bs + face_off(F.axis, F.side, 1, i1, i2, n, P)], a);
-        else if (F.kind == FK_SAME)
-            atomicAdd(&grad[F.nbr * g.bs + face_off(F.axis, 1 - F.side, 1, i1, i2, n, P)], a);
-        else
-            atomicAdd(&grad[F.nbr * g.bs + face_off(F.axis, 1 - F.side, 1, F.seg1 * h + (i1 >> 1), F.seg2 * h + (i2 >> 1),
-                                                     n, P)],
-                      a);
-    }
-}
-
-// Coarse ghost k = mean of the 8 fine k (ghost-only variant): 1/8 of the ghost adjoint to each fine cell.
-__global__ void k_gradk_ghost_segs(double *__restrict__ grad, const double *__restrict__ gadj,
-                                   const SegItem *__restrict__ items, int nitems, LevelGeom g) {
-    const int n = g.n, P = g.P, lgh = g.lg - 1, h = n >> 1;
+// The interface faces' part of dL/dk, one thread per coarse cell of a quarter.  Fine face j (coefficient T_j of k_j and the
+// injected coarse k_C) stands in the fine row with (1/h^2) T_j (u_j - g_j) and, conservative variant, with half of
+// (1/h_C^2) T_j (g_j - u_j) in the coarse row; in the ghost-only variant the coarse row has its own face, of k_C and the mean
+// of the eight fine k.
+template <bool FLUX>
+__global__ void k_gradk_iface(const double *__restrict__ u, const double *__restrict__ lam, const double *__restrict__ k,
+                              Coef cf, const double *__restrict__ h2, const double *__restrict__ ih2,
+                              const FaceItem *__restrict__ items, int nitems, LevelGeom g, Target<double> to) {
+    const int n = g.n, lgh = g.lg - 1, h = n >> 1;
     const int64_t total = static_cast<int64_t>(nitems) << (2 * lgh);
     GRID_STRIDE(total) {
-        const int it = static_cast<int>(t >> (2 * lgh));
-        const int r = static_cast<int>(t) & ((1 << (2 * lgh)) - 1);
-        const int p = r & (h - 1), q = r >> lgh;
-        const SegItem S = items[it];
-        const int fs = 1 - S.side;
-        const double a =
-            0.125 * gadj[S.coarse * g.bs + face_off(S.axis, S.side, 0, S.s1 * h + p, S.s2 * h + q, n, P)];
-        for (int d = 1; d <= 2; ++d)
-            for (int bb = 0; bb < 2; ++bb)
-                for (int aa = 0; aa < 2; ++aa)
-                    atomicAdd(&grad[S.fine * g.bs + face_off(S.axis, fs, d, 2 * p + aa, 2 * q + bb, n, P)], a);
-    }
-}
-
-// Conservative coarse rows: (1/h_C^2) 1/2 sum_j T(k_j, k_C) (g_j - u_j) with weight -lambda_C.
-__global__ void k_gradk_flux_rows(double *__restrict__ grad, const double *__restrict__ u,
-                                  const double *__restrict__ lam, const double *__restrict__ k,
-                                  const double *__restrict__ ih2, const SegItem *__restrict__ items, int nitems,
-                                  LevelGeom g) {
-    const int n = g.n, P = g.P, lgh = g.lg - 1, h = n >> 1;
-    const int64_t total = static_cast<int64_t>(nitems) << (2 * lgh);
-    GRID_STRIDE(total) {
-        const int it = static_cast<int>(t >> (2 * lgh));
-        const int r = static_cast<int>(t) & ((1 << (2 * lgh)) - 1);
-        const int p = r & (h - 1), q = r >> lgh;
-        const SegItem S = items[it];
-        const int fs = 1 - S.side;
-        const int64_t gC = S.coarse * g.bs + face_off(S.axis, S.side, 1, S.s1 * h + p, S.s2 * h + q, n, P);
-        const double lC = lam[gC] * ih2[S.coarse], kC = k[gC];
-        double accC = 0.0;
-        for (int bb = 0; bb < 2; ++bb)
-            for (int aa = 0; aa < 2; ++aa) {
-                const int64_t g0 = S.fine * g.bs + face_off(S.axis, fs, 0, 2 * p + aa, 2 * q + bb, n, P);
-                const int64_t g1 = S.fine * g.bs + face_off(S.axis, fs, 1, 2 * p + aa, 2 * q + bb, n, P);
-                const double kj = k[g1];
-                const double w = -lC * 0.5 * (u[g0] - u[g1]);
-                const double inv = 1.0 / ((kj + kC) * (kj + kC));
-                atomicAdd(&grad[g1], w * 2.0 * kC * kC * inv);
-                accC += w * 2.0 * kj * kj * inv;
-            }
-        atomicAdd(&grad[gC], accC);
+        const FaceItem F = items[t >> (2 * lgh)];
+        const int q = static_cast<int>(t) & ((1 << (2 * lgh)) - 1), ycl = q & (h - 1), zcl = q >> lgh;
+        const int yc = F.seg1 * h + ycl, zc = F.seg2 * h + zcl;
+        int X, Y, Z;
+        face_xyz(F.axis, 1 - F.side, 1, yc, zc, n, X, Y, Z);
+        const int64_t gC = Lay<double>::at(g, F.nbr, X, Y, Z);
+        const int64_t g0c = fidx<double>(g, F.nbr, F.axis, 1 - F.side, 0, yc, zc);
+        const double lC = lam[gC], kC = k[gC], hf = h2[F.blk];
+        const auto add_fine = [&](int d, int e, double v) {
+            int x, y, z;
+            face_xyz(F.axis, F.side, d, 2 * ycl + (e & 1), 2 * zcl + (e >> 1), n, x, y, z);
+            add_to(to, g, F.blk, x, y, z, v);
+        };
+        double toC = 0.0;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int64_t g0 = fidx<double>(g, F.blk, F.axis, F.side, 0, 2 * ycl + (e & 1), 2 * zcl + (e >> 1));
+            const int64_t g1 = fidx<double>(g, F.blk, F.axis, F.side, 1, 2 * ycl + (e & 1), 2 * zcl + (e >> 1));
+            const double T = face_coef<double, 1>(cf, F.side ? g0 : g1, F.side ? g1 : g0, F.axis) * hf;
+            double w = -lam[g1] * ih2[F.blk];
+            if (FLUX) w = fma(0.5 * lC, ih2[F.nbr], w);
+            const double v = 0.5 * T * T * w * (u[g1] - u[g0]), kj = k[g1];
+            add_fine(1, e, v / (kj * kj));
+            toC += v / (kC * kC);
+        }
+        if (!FLUX) {
+            const double T = face_coef<double, 1>(cf, F.side ? gC : g0c, F.side ? g0c : gC, F.axis) * h2[F.nbr];
+            const double v = -0.5 * T * T * lC * ih2[F.nbr] * (u[gC] - u[g0c]), kG = k[g0c];
+            toC += v / (kC * kC);
+            for (int d = 1; d <= 2; ++d)
+                for (int e = 0; e < 4; ++e) add_fine(d, e, 0.125 * v / (kG * kG));
+        }
+        add_to(to, g, F.nbr, X, Y, Z, toC);
     }
 }
 
 // ---------------------------------------------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------------------------------------------
-// The transposed cycle's pools and coefficients in its working precision.
+// The transposed cycle's pools in its working precision: result, right-hand side, residual, interface adjoints.  FP32
+// cycles run on the forward cycle's pools (dead between solves); FP64 ones too, but level 0's right-hand side is the
+// forward solve's and has a pool of its own.
 template <typename T>
 struct APools {
-    T *ub, *fb, *z, *tmp;
+    T *y, *f, *r, *old, *old_c;
 };
-template <typename T> APools<T> apools(DevLevel &d);
-template <> APools<double> apools<double>(DevLevel &d) { return {d.a_ub, d.a_fb, d.a_z, d.a_tmp}; }
-template <> APools<float> apools<float>(DevLevel &d) { return {d.a32_ub, d.a32_fb, d.a32_z, d.a32_tmp}; }
-template <typename T> ACoef<T> acoef(const DevLevel &d);
-template <> ACoef<double> acoef<double>(const DevLevel &d) { return {d.tx, d.ty, d.tz, d.dg, d.dinv}; }
-template <> ACoef<float> acoef<float>(const DevLevel &d) {
-    return {d.a32_tx, d.a32_ty, d.a32_tz, d.a32_dg, d.a32_dinv};
+template <typename T> APools<T> apools(mg_forest *F, int l);
+template <> APools<double> apools<double>(mg_forest *F, int l) {
+    DevLevel &d = F->L[l];
+    return {d.u64, l == 0 ? F->a_fe : d.f64, static_cast<double *>(d.a_r), static_cast<double *>(d.a_old),
+            static_cast<double *>(d.a_old_c)};
+}
+template <> APools<float> apools<float>(mg_forest *F, int l) {
+    DevLevel &d = F->L[l];
+    return {d.u32, d.f32, static_cast<float *>(d.a_r), static_cast<float *>(d.a_old), static_cast<float *>(d.a_old_c)};
 }
 template <typename T> const T *aih2(const DevLevel &d);
 template <> const double *aih2<double>(const DevLevel &d) { return d.ih2_64; }
 template <> const float *aih2<float>(const DevLevel &d) { return d.ih2_32; }
-template <typename T> const T *ah2(const DevLevel &d);
-template <> const double *ah2<double>(const DevLevel &d) { return d.h2_64; }
-template <> const float *ah2<float>(const DevLevel &d) { return d.h2_32; }
+template <typename T> Coef acoef(const DevLevel &d);
+template <> Coef acoef<double>(const DevLevel &d) { return d.c64(); }
+template <> Coef acoef<float>(const DevLevel &d) { return d.c32(); }
 
-template <int MODE, typename T>
-void exchange_T(mg_forest *F, DevLevel &d, T *G) {
-    Prof p(F, P_ADJ, 2);
-    if (d.nsegs && F->cfg.interface_flux)
-        k_et_segs_flux<MODE, T><<<grid_for(static_cast<int64_t>(d.nsegs) << (2 * (d.g.lg - 1))), kThreads, 0, F->st>>>(
-            G, acoef<T>(d), aih2<T>(d), d.segs, d.nsegs, d.g);
-    if (d.nfaces)
-        k_et_faces<T><<<grid_for(static_cast<int64_t>(d.nfaces) << (2 * d.g.lg)), kThreads, 0, F->st>>>(G, d.faces,
-                                                                                                        d.nfaces, d.g);
-    if (d.nsegs && !F->cfg.interface_flux)
-        k_et_segs_mean<T><<<grid_for(static_cast<int64_t>(d.nsegs) << (2 * (d.g.lg - 1))), kThreads, 0, F->st>>>(
-            G, d.segs, d.nsegs, d.g);
+// Calls fn(integral constant) with the coefficient mode of a level in precision T.
+template <typename T, class Fn>
+void with_mode(const mg_forest *F, const DevLevel &d, Fn &&fn) {
+    if (!F->cfg.coeff) fn(std::integral_constant<int, 0>{});
+    else if constexpr (sizeof(T) == 8) fn(std::integral_constant<int, 1>{});
+    else if (d.face32) fn(std::integral_constant<int, 3>{});
+    else fn(std::integral_constant<int, 2>{});
 }
 
-// out = A^T x on level l; x must have zero ghosts; out's ghost positions are left holding ghost adjoints.
-template <int MODE, typename T>
-void apply_T(mg_forest *F, DevLevel &d, const T *x, T *out) {
-    if constexpr (sizeof(T) == 8) {
-        apply64(F, d, x, out);
-    } else {
-        Prof p(F, P_ADJ, 1);
-        k_apply_nat<T, MODE><<<grid_for(d.cells()), kThreads, 0, F->st>>>(x, acoef<T>(d), aih2<T>(d), d.g, out);
-    }
-    {
-        Prof p(F, P_ADJ, 1);
-        k_at_ghosts<MODE, T><<<grid_for(static_cast<int64_t>(d.g.nb) * 6 << (2 * d.g.lg)), kThreads, 0, F->st>>>(
-            x, out, acoef<T>(d), aih2<T>(d), d.g);
-    }
-    exchange_T<MODE, T>(F, d, out);
+template <typename T>
+size_t iface_smem(const DevLevel &d) {
+    const size_t w = d.g.n / 2 + 2;
+    return w * w * sizeof(T);
+}
+int iface_threads(const DevLevel &d) { return d.g.n <= 8 ? 32 : (d.g.n <= 16 ? 64 : 256); }
+
+// Transposed interface ghosts of y (ghosts) and sgn times the interface part of A^T y into `to` (see k_adj_iface).
+template <typename T>
+void adj_iface(mg_forest *F, DevLevel &d, T *y, bool ghosts, T *old, T *old_c, Target<T> to, T sgn) {
+    if (!d.nifaces) return;
+    Prof p(F, P_ADJ, 1);
+    with_mode<T>(F, d, [&](auto m) {
+        constexpr int M = decltype(m)::value;
+        auto *fn = F->cfg.interface_flux ? (ghosts ? k_adj_iface<T, M, true, true> : k_adj_iface<T, M, true, false>)
+                                         : (ghosts ? k_adj_iface<T, M, false, true> : k_adj_iface<T, M, false, false>);
+        if (iface_smem<T>(d) > 48 * 1024)  // block edges above 128
+            cudaFuncSetAttribute(reinterpret_cast<const void *>(fn), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 static_cast<int>(iface_smem<T>(d)));
+        fn<<<d.nifaces, iface_threads(d), iface_smem<T>(d), F->st>>>(y, acoef<T>(d), aih2<T>(d), d.ifaces, d.g, old, old_c,
+                                                                     to, sgn);
+    });
 }
 
-template <int MODE, typename T>
-void smooth_T(mg_forest *F, DevLevel &d, int iters) {
-    const APools<T> a = apools<T>(d);
+// Ghosts of y filled from one source block (same level, boundary).
+template <typename T>
+void exchange_same(mg_forest *F, DevLevel &d, T *y) {
+    if (!d.nsfaces) return;
+    Prof p(F, P_ADJ, 1);
+    k_exchange_faces<T, false><<<grid_for(static_cast<int64_t>(d.nsfaces) << (2 * d.g.lg)), kThreads, 0, F->st>>>(
+        y, d.sfaces, d.nsfaces, d.g);
+}
+
+// Red-black iterations on A^T with the colours in reverse order.  `stale`: y changed since the last interface exchange.
+template <typename T>
+void smooth_T(mg_forest *F, int l, int iters, bool &stale) {
+    DevLevel &d = F->L[l];
+    const APools<T> a = apools<T>(F, l);
     for (int i = 0; i < iters; ++i)
         for (int colour = 1; colour >= 0; --colour) {
-            {
+            if (stale) adj_iface<T>(F, d, a.y, true, a.old, a.old_c, {a.f, nullptr, nullptr}, T(-1));
+            if constexpr (sizeof(T) == 4) {
+                smooth_level32(F, d, colour);
+            } else {
                 Prof p(F, P_ADJ, 1);
-                k_adj_colour<MODE, T><<<grid_for(d.cells()), kThreads, 0, F->st>>>(a.ub, a.fb, a.z, acoef<T>(d),
-                                                                                    ah2<T>(d), d.g, colour);
+                auto *fn = F->cfg.coeff ? k_smooth<double, 1> : k_smooth<double, 0>;
+                fn<<<grid_for(d.cells() / 2), kThreads, 0, F->st>>>(a.y, a.f, d.c64(), d.h2_64, d.g, colour, d.nbr6, Skip{},
+                                                                    nullptr);
             }
-            apply_T<MODE, T>(F, d, a.z, a.tmp);
-            Prof p(F, P_ADJ, 1);
-            k_axpy<T><<<grid_for(d.cells()), kThreads, 0, F->st>>>(a.ub, a.tmp, T(-1), d.g);
+            stale = true;
         }
 }
 
-// fbar = M_l^T ubar (level l's pools ub in, fb out), in precision T; the coarsest level's dense inverse is FP64.
-template <int MODE, typename T>
+// The FP32 residual of a level with block edge 4 .. 128 on its own pools into r.
+void launch_residual32(mg_forest *F, DevLevel &d, float *r) {
+    with_mode<float>(F, d, [&](auto m) {
+        constexpr int M = decltype(m)::value;
+        static constexpr decltype(&k_adj_residual32<M, 2>) fns[6] = {
+            k_adj_residual32<M, 2>, k_adj_residual32<M, 3>, k_adj_residual32<M, 4>,
+            k_adj_residual32<M, 5>, k_adj_residual32<M, 6>, k_adj_residual32<M, 7>};
+        const int64_t pairs = d.cells() / 2;
+        fns[d.g.lg - 2]<<<static_cast<unsigned>((pairs + kThreads - 1) / kThreads), kThreads, 0, F->st>>>(
+            d.u32, d.f32, d.c32(), d.ih2_32, d.g.bs, pairs, d.nbr6, r);
+    });
+}
+
+// y = M_l^T f (level l's pools), in precision T, from y = 0 with zero ghosts; the coarsest level's dense inverse is FP64.
+template <typename T>
 void vcycle_T(mg_forest *F, int l) {
     DevLevel &d = F->L[l];
-    const APools<T> a = apools<T>(d);
+    const APools<T> a = apools<T>(F, l);
     const int last = static_cast<int>(F->L.size()) - 1;
     if (l == last) {
         Prof p(F, P_ADJ, 1);
         k_coarse_solve<T><<<(F->Nc * 32 + kThreads - 1) / kThreads, kThreads, 0, F->st>>>(
-            a.fb, a.ub, F->AinvT, F->cmap, F->uprob, F->ustart, F->moff, F->Nc);
+            a.y, a.f, F->AinvT, sizeof(T) == 4 ? F->cmap32 : F->cmap, F->uprob, F->ustart, F->moff, F->Nc);
         return;
     }
-    cudaMemsetAsync(a.fb, 0, d.pool_elems() * sizeof(T), F->st);
-    smooth_T<MODE, T>(F, d, F->cfg.nu2);
+    const int64_t n2 = static_cast<int64_t>(d.g.n) * d.g.n;
+    if (d.nifaces) {
+        cudaMemsetAsync(a.old, 0, d.nifaces * n2 * sizeof(T), F->st);
+        if (a.old_c) cudaMemsetAsync(a.old_c, 0, d.nifaces * n2 / 4 * sizeof(T), F->st);
+    }
+    const auto iface = [&](bool &stale) {
+        if (stale) adj_iface<T>(F, d, a.y, true, a.old, a.old_c, {a.f, nullptr, nullptr}, T(-1));
+        stale = false;
+    };
+    bool stale = false;
+    smooth_T<T>(F, l, F->cfg.nu2, stale);
+    iface(stale);
     DevLevel &c = F->L[l + 1];
-    const APools<T> ac = apools<T>(c);
-    cudaMemsetAsync(ac.ub, 0, c.pool_elems() * sizeof(T), F->st);
+    const APools<T> ac = apools<T>(F, l + 1);
     {
         Prof p(F, P_ADJ, 1);
-        k_prolong_T<T><<<grid_for(c.cells()), kThreads, 0, F->st>>>(a.ub, d.g, ac.ub, d.xfer, c.g);
+        if (sizeof(T) == 4 && smooth32_specialised(d))
+            launch_residual32(F, d, reinterpret_cast<float *>(a.r));
+        else
+            with_mode<T>(F, d, [&](auto m) {
+                k_adj_residual<T, decltype(m)::value><<<grid_for(d.cells()), kThreads, 0, F->st>>>(
+                    a.y, a.f, acoef<T>(d), aih2<T>(d), d.g, d.nbr6, a.r, nullptr, nullptr);
+            });
     }
-    exchange_T<MODE, T>(F, c, ac.ub);
-    vcycle_T<MODE, T>(F, l + 1);
-    {
+    const bool gather = d.all_halve;
+    if (sizeof(T) == 4 && transfer32_specialised(d)) {
+        Prof p(F, P_ADJ, 1);
+        static constexpr decltype(&k_prolong_T32<3>) fns[5] = {k_prolong_T32<3>, k_prolong_T32<4>, k_prolong_T32<5>,
+                                                               k_prolong_T32<6>, k_prolong_T32<7>};
+        fns[d.g.lg - 3]<<<static_cast<unsigned>((c.cells() + kThreads - 1) / kThreads), kThreads, 0, F->st>>>(
+            reinterpret_cast<float *>(a.r), d.g.bs, c.f32, c.u32, d.xfer, c.cells(), c.g.bs);
+    } else if (gather) {
+        Prof p(F, P_ADJ, 1);
+        k_prolong_T<T><<<grid_for(c.cells()), kThreads, 0, F->st>>>(a.r, d.g, ac.f, ac.y, d.xfer, c.g);
+    } else {
         Prof p(F, P_ADJ, 2);
-        k_restrict_T<T><<<grid_for(c.cells()), kThreads, 0, F->st>>>(ac.fb, c.g, a.z, d.xfer, d.g);
-        k_axpy<T><<<grid_for(d.cells()), kThreads, 0, F->st>>>(a.fb, a.z, T(1), d.g);
+        cudaMemsetAsync(ac.f, 0, c.pool_elems() * sizeof(T), F->st);
+        cudaMemsetAsync(ac.y, 0, c.pool_elems() * sizeof(T), F->st);
+        k_prolong_T_scatter<T><<<grid_for(c.cells()), kThreads, 0, F->st>>>(a.r, d.g, ac.f, d.xfer, c.g);
+        if (c.nsfaces)
+            k_et_faces<T><<<grid_for(static_cast<int64_t>(c.nsfaces) << (2 * c.g.lg)), kThreads, 0, F->st>>>(
+                ac.f, c.sfaces, c.nsfaces, c.g);
     }
-    apply_T<MODE, T>(F, d, a.z, a.tmp);
+    if (c.nifaces) {
+        Prof p(F, P_ADJ, 1);
+        with_mode<T>(F, c, [&](auto m) {
+            constexpr int M = decltype(m)::value;
+            auto *fn = F->cfg.interface_flux ? (gather ? k_et_iface<T, M, true, true> : k_et_iface<T, M, true, false>)
+                                             : (gather ? k_et_iface<T, M, false, true> : k_et_iface<T, M, false, false>);
+            fn<<<c.nifaces, iface_threads(c), iface_smem<T>(c), F->st>>>(ac.f, acoef<T>(c), c.ifaces, c.g, a.r, d.g, d.xfer);
+        });
+    }
+    vcycle_T<T>(F, l + 1);
+    bool through = false;  // the injection wrote same-level and boundary ghosts
     {
         Prof p(F, P_ADJ, 1);
-        k_axpy<T><<<grid_for(d.cells()), kThreads, 0, F->st>>>(a.ub, a.tmp, T(-1), d.g);
+        if constexpr (sizeof(T) == 4) through = inject32(F, d, c);
+        if (!through) k_inject<T><<<grid_for(c.cells()), kThreads, 0, F->st>>>(a.y, d.g, ac.y, d.xfer, c.g);
     }
-    smooth_T<MODE, T>(F, d, F->cfg.nu1);
+    if (!through) exchange_same<T>(F, d, a.y);
+    stale = true;
+    smooth_T<T>(F, l, F->cfg.nu1, stale);
 }
 
 mg_status ensure_adjoint_pools(mg_forest *F) {
-    MG_TRY(ensure_scratch64(F));
     MG_TRY(ensure_fp64_coefficients(F));
     if (F->a_g) return MG_OK;
     const bool fp32 = F->cfg.precision == 1;
-    for (DevLevel &d : F->L) {
-        const int64_t bytes = d.pool_elems() * static_cast<int64_t>(sizeof(double));
-        void *p;
-        MG_TRY(forest_alloc(F, &p, bytes));
-        d.a_ub = static_cast<double *>(p);
-        MG_TRY(forest_alloc(F, &p, bytes));
-        d.a_fb = static_cast<double *>(p);
-        MG_TRY(forest_alloc(F, &p, bytes));
-        d.a_z = static_cast<double *>(p);
-        MG_TRY(forest_alloc(F, &p, bytes));
-        d.a_tmp = static_cast<double *>(p);
-        if (!fp32) continue;
-        // FP32 transposed cycles (forests with FP32 forward cycles): natural-layout FP32 pools and coefficients
-        const int64_t b32 = d.pool_elems() * static_cast<int64_t>(sizeof(float));
-        float **pools[] = {&d.a32_ub, &d.a32_fb, &d.a32_z, &d.a32_tmp};
-        for (float **q : pools) {
-            MG_TRY(forest_alloc(F, &p, b32));
-            *q = static_cast<float *>(p);
-        }
-        if (F->cfg.coeff) {
-            float **coefs[] = {&d.a32_tx, &d.a32_ty, &d.a32_tz, &d.a32_dg, &d.a32_dinv};
-            for (float **q : coefs) {
-                MG_TRY(forest_alloc(F, &p, b32));
-                *q = static_cast<float *>(p);
-            }
-        }
-    }
+    const int64_t tb = fp32 ? sizeof(float) : sizeof(double);
     const int64_t bytes0 = F->L[0].pool_elems() * static_cast<int64_t>(sizeof(double));
     void *p;
+    for (DevLevel &d : F->L) {
+        const int64_t adj = static_cast<int64_t>(d.nifaces) * d.g.n * d.g.n * tb;
+        MG_TRY(forest_alloc(F, &d.a_r, d.pool_elems() * tb));
+        if (adj) MG_TRY(forest_alloc(F, &d.a_old, adj));
+        if (adj && !F->cfg.interface_flux) MG_TRY(forest_alloc(F, &d.a_old_c, adj / 4));
+    }
     MG_TRY(forest_alloc(F, &p, bytes0));
     F->a_lam = static_cast<double *>(p);
     MG_TRY(forest_alloc(F, &p, bytes0));
+    F->a_fe = static_cast<double *>(p);
+    MG_TRY(forest_alloc(F, &p, bytes0));
     F->a_g = static_cast<double *>(p);
-    return MG_OK;
-}
-
-// The FP32 copies of the FP64 coefficients (rebuilt by every adjoint solve: mg_set_rhs may have changed k).
-mg_status round_coefficients32(mg_forest *F) {
-    if (!F->cfg.coeff) return MG_OK;
-    for (DevLevel &d : F->L) {
-        const int64_t cnt = d.pool_elems();
-        const double *src[] = {d.tx, d.ty, d.tz, d.dg, d.dinv};
-        float *dst[] = {d.a32_tx, d.a32_ty, d.a32_tz, d.a32_dg, d.a32_dinv};
-        for (int i = 0; i < 5; ++i) k_round32<<<grid_for(cnt), kThreads, 0, F->st>>>(src[i], dst[i], cnt);
-    }
-    MG_CUDA(cudaGetLastError());
     return MG_OK;
 }
 
@@ -659,6 +872,53 @@ mg_status adjoint_supported(const mg_forest *F) {
     return MG_OK;
 }
 
+// Half a defect-correction step: r = g - A^T lambda (r = g while lambda is 0).  FP32 cycles: r scaled by `mult` into the
+// level-0 FP32 right-hand side, its result zeroed; FP64 cycles: r into the level-0 right-hand side a_fe, u64 zeroed.
+// rr receives the volume-weighted ||r||^2 over all problems.
+template <int MODE>
+mg_status adjoint_residual(mg_forest *F, bool zero, double mult, double *rr) {
+    DevLevel &d = F->L[0];
+    const double *f = F->a_g;
+    if (!zero) {
+        exchange_same<double>(F, d, F->a_lam);
+        if (d.nifaces) {
+            // FP32 cycles leave a_fe alone, so it differs from g only where the last step added to it
+            if (F->cfg.precision == 1) {
+                auto *fn = F->cfg.interface_flux ? k_adj_restore<true> : k_adj_restore<false>;
+                fn<<<d.nifaces, iface_threads(d), 0, F->st>>>(F->a_fe, F->a_g, d.ifaces, d.g);
+            } else {
+                MG_CUDA(cudaMemcpyAsync(F->a_fe, F->a_g, d.pool_elems() * sizeof(double), cudaMemcpyDeviceToDevice, F->st));
+            }
+            adj_iface<double>(F, d, F->a_lam, true, nullptr, nullptr, {F->a_fe, nullptr, nullptr}, -1.0);
+            f = F->a_fe;
+        }
+    }
+    if (F->cfg.precision == 1) {
+        const std::vector<double> m(F->np, mult);
+        set_scales_host(F, m);
+        MG_TRY(enqueue_scales(F));
+        const int cpb = F->bsum_cpb;
+        Prof p(F, P_ADJ, 1);
+        MG_CUDA(cudaMemsetAsync(F->bsum, 0, static_cast<size_t>(d.g.nb) * cpb * sizeof(double), F->st));
+        auto *fn = zero ? k_residual_norm<MODE, true> : k_residual_norm<MODE, false>;
+        fn<<<d.g.nb * cpb, kThreads, 0, F->st>>>(F->a_lam, f, d.c64(), d.ih2_64, d.vol_32, d.g, cpb, d.f32, F->pscale,
+                                                 d.bprob, F->bsum, d.u32, Skip{});
+        MG_TRY(enqueue_problem_sums(F));
+        MG_CUDA(cudaStreamSynchronize(F->st));
+        *rr = 0.0;
+        for (int p2 = 0; p2 < F->np; ++p2) *rr += F->psum_h[p2] / (mult * mult);
+        return MG_OK;
+    }
+    const int grid = grid_for(d.cells());
+    {
+        Prof p(F, P_ADJ, 1);
+        k_adj_residual<double, MODE><<<grid, kThreads, 0, F->st>>>(F->a_lam, f, d.c64(), d.ih2_64, d.g, nullptr, F->a_fe,
+                                                                   d.vol_64, F->partial);
+    }
+    MG_CUDA(cudaMemsetAsync(d.u64, 0, d.pool_elems() * sizeof(double), F->st));
+    return read_sum(F, grid, rr);
+}
+
 template <int MODE>
 mg_status adjoint_solve(mg_forest *F, const double *u_dev, const double *dLdu_dev, double *lambda_dev,
                         double *dLdk_dev, double rtol, int max_cycles) {
@@ -667,60 +927,51 @@ mg_status adjoint_solve(mg_forest *F, const double *u_dev, const double *dLdu_de
     const int grid = grid_for(d.cells());
     MG_CUDA(cudaMemsetAsync(F->a_lam, 0, d.pool_elems() * sizeof(double), F->st));
     k_pack<double><<<grid, kThreads, 0, F->st>>>(F->a_g, dLdu_dev, d.g, F->leaf_off);
+    if (d.nifaces) k_pack<double><<<grid, kThreads, 0, F->st>>>(F->a_fe, dLdu_dev, d.g, F->leaf_off);
     k_norm64<<<grid, kThreads, 0, F->st>>>(F->a_g, d.vol_64, d.g, F->partial);
     double gg = 0.0;
     MG_TRY(read_sum(F, grid, &gg));
     const double gn = std::sqrt(gg);
-    double rel = gn > 0.0 ? 1.0 : 0.0;
+    double rel = gn > 0.0 ? 1.0 : 0.0, mult = pow2_near(1.0 / gn);
     int it = 0;
     // Defect correction lambda += M^T (g - A^T lambda): the residual and the update in FP64; the transposed cycle
     // M^T in FP64, or, on forests with FP32 forward cycles, in FP32 on the residual scaled by a power of two near
-    // 1 / ||r|| (the forward solve's mixed precision, transposed)
-    const bool fp32 = F->cfg.precision == 1;
-    if (fp32) MG_TRY(round_coefficients32(F));
+    // 1 / ||r|| of the step before (the forward solve's mixed precision, transposed)
     for (; gn > 0.0; ++it) {
-        apply_T<MODE, double>(F, d, F->a_lam, d.a_tmp);
-        k_sub_norm<<<grid, kThreads, 0, F->st>>>(F->a_g, d.a_tmp, d.a_ub, d.vol_64, d.g, F->partial);
         double rr = 0.0;
-        MG_TRY(read_sum(F, grid, &rr));
+        MG_TRY(adjoint_residual<MODE>(F, it == 0, mult, &rr));
         rel = std::sqrt(rr) / gn;
         if (!std::isfinite(rel) || rel <= rtol || it >= max_cycles) break;
-        if (fp32) {
-            const double sc = pow2_near(1.0 / std::sqrt(rr));
-            k_scaled32<<<grid, kThreads, 0, F->st>>>(d.a_ub, d.a32_ub, sc, d.g);
-            vcycle_T<MODE, float>(F, 0);
-            k_add_from32<<<grid, kThreads, 0, F->st>>>(F->a_lam, d.a32_fb, 1.0 / sc, d.g);
+        if (F->cfg.precision == 1) {
+            vcycle_T<float>(F, 0);
+            Prof p(F, P_ADJ, 1);
+            k_update_mixed<<<grid, kThreads, 0, F->st>>>(F->a_lam, d.u32, F->pinv, d.bprob, d.g, Skip{});
         } else {
-            vcycle_T<MODE, double>(F, 0);
-            k_axpy<double><<<grid, kThreads, 0, F->st>>>(F->a_lam, d.a_fb, 1.0, d.g);
+            vcycle_T<double>(F, 0);
+            Prof p(F, P_ADJ, 1);
+            k_add<<<grid, kThreads, 0, F->st>>>(F->a_lam, d.u64, d.g);
         }
+        mult = pow2_near(1.0 / std::sqrt(rr));
     }
     k_unpack<double><<<grid, kThreads, 0, F->st>>>(lambda_dev, F->a_lam, d.g, F->leaf_off);
     MG_CUDA(cudaGetLastError());
     if (dLdk_dev && F->cfg.coeff) {
-        // forward ghosts of u, then the face terms, the ghost-k maps and (conservative variant) the coarse rows
-        MG_CUDA(cudaMemsetAsync(F->s64a, 0, d.pool_elems() * sizeof(double), F->st));
+        // forward ghosts of u; lambda's were filled by the last residual (and are 0 while lambda is)
+        MG_TRY(ensure_scratch64(F));
         k_pack<double><<<grid, kThreads, 0, F->st>>>(F->s64a, u_dev, d.g, F->leaf_off);
         exchange_any64(F, d, F->s64a);
-        MG_CUDA(cudaMemsetAsync(F->s64b, 0, d.pool_elems() * sizeof(double), F->st));
-        MG_CUDA(cudaMemsetAsync(d.a_tmp, 0, d.pool_elems() * sizeof(double), F->st));
-        k_gradk_faces<<<grid, kThreads, 0, F->st>>>(F->s64a, F->a_lam, d.k64, d.ih2_64, d.fkind,
-                                                     F->cfg.interface_flux, d.g, F->s64b, d.a_tmp);
-        k_gradk_merge<<<grid, kThreads, 0, F->st>>>(F->s64b, d.a_tmp, d.g);
-        if (d.nfaces)
-            k_gradk_ghost_faces<<<grid_for(static_cast<int64_t>(d.nfaces) << (2 * d.g.lg)), kThreads, 0, F->st>>>(
-                F->s64b, d.a_tmp, d.faces, d.nfaces, d.g);
-        if (d.nsegs) {
-            const int gs = grid_for(static_cast<int64_t>(d.nsegs) << (2 * (d.g.lg - 1)));
-            if (F->cfg.interface_flux)
-                k_gradk_flux_rows<<<gs, kThreads, 0, F->st>>>(F->s64b, F->s64a, F->a_lam, d.k64, d.ih2_64, d.segs,
-                                                              d.nsegs, d.g);
-            else
-                k_gradk_ghost_segs<<<gs, kThreads, 0, F->st>>>(F->s64b, d.a_tmp, d.segs, d.nsegs, d.g);
+        Prof p(F, P_ADJ, 1 + (d.nifaces > 0));
+        k_gradk<<<grid, kThreads, 0, F->st>>>(F->s64a, F->a_lam, d.k64, d.c64(), d.h2_64, d.nbr6, d.g, dLdk_dev,
+                                              F->leaf_off);
+        if (d.nifaces) {
+            auto *fn = F->cfg.interface_flux ? k_gradk_iface<true> : k_gradk_iface<false>;
+            fn<<<grid_for(static_cast<int64_t>(d.nifaces) << (2 * (d.g.lg - 1))), kThreads, 0, F->st>>>(
+                F->s64a, F->a_lam, d.k64, d.c64(), d.h2_64, d.ih2_64, d.ifaces, d.nifaces, d.g,
+                Target<double>{nullptr, dLdk_dev, F->leaf_off});
         }
-        k_unpack<double><<<grid, kThreads, 0, F->st>>>(dLdk_dev, F->s64b, d.g, F->leaf_off);
     }
     MG_CUDA(cudaStreamSynchronize(F->st));
+    if (F->cfg.precision == 1) MG_TRY(check_kernel_waits(F));
     if (!std::isfinite(rel) || rel > rtol) {
         set_error("adjoint: relative residual " + fmt_e(rel) + " above rtol after " + std::to_string(it) +
                   " cycles");
@@ -744,15 +995,16 @@ extern "C" mg_status mg_apply_transpose(mg_forest *F, const double *y_dev, doubl
         return MG_ERR_STATE;
     }
     MG_TRY(adjoint_supported(F));
-    MG_TRY(ensure_adjoint_pools(F));
+    MG_TRY(ensure_fp64_coefficients(F));
+    MG_TRY(ensure_scratch64(F));
     DevLevel &d = F->L[0];
-    MG_CUDA(cudaMemsetAsync(d.a_z, 0, d.pool_elems() * sizeof(double), F->st));
-    k_pack<double><<<grid_for(d.cells()), kThreads, 0, F->st>>>(d.a_z, y_dev, d.g, F->leaf_off);
-    if (F->cfg.coeff)
-        apply_T<1>(F, d, d.a_z, d.a_tmp);
-    else
-        apply_T<0>(F, d, d.a_z, d.a_tmp);
-    k_unpack<double><<<grid_for(d.cells()), kThreads, 0, F->st>>>(ATy_dev, d.a_tmp, d.g, F->leaf_off);
+    // the stencil on y with the transposed ghosts, then the interface part added to the caller's field
+    k_pack<double><<<grid_for(d.cells()), kThreads, 0, F->st>>>(F->s64a, y_dev, d.g, F->leaf_off);
+    exchange_same<double>(F, d, F->s64a);
+    adj_iface<double>(F, d, F->s64a, true, nullptr, nullptr, {nullptr, nullptr, nullptr}, 1.0);
+    apply64(F, d, F->s64a, F->s64b);
+    k_unpack<double><<<grid_for(d.cells()), kThreads, 0, F->st>>>(ATy_dev, F->s64b, d.g, F->leaf_off);
+    adj_iface<double>(F, d, F->s64a, false, nullptr, nullptr, {nullptr, ATy_dev, F->leaf_off}, 1.0);
     MG_CUDA(cudaStreamSynchronize(F->st));
     return MG_OK;
 }

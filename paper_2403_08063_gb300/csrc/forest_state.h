@@ -61,11 +61,9 @@ struct DevLevel {
     // FP32 smoother launch shape (kind, parameters): {1, ZC, threads, 0, 0} k_smooth32, {2, TY, TZ, D, R}
     // k_smooth32t; kind 0 = not chosen yet
     std::array<int32_t, 5> s32{0, 0, 0, 0, 0};
-    // adjoint work pools (allocated by the first adjoint call)
-    double *a_ub = nullptr, *a_fb = nullptr, *a_z = nullptr, *a_tmp = nullptr;
-    // FP32 transposed cycles (forests with FP32 forward cycles): natural-layout pools and rounded coefficients
-    float *a32_ub = nullptr, *a32_fb = nullptr, *a32_z = nullptr, *a32_tmp = nullptr;
-    float *a32_tx = nullptr, *a32_ty = nullptr, *a32_tz = nullptr, *a32_dg = nullptr, *a32_dinv = nullptr;
+    // transposed cycles (allocated by the first adjoint call, in the cycles' precision): residual pool, and per interface
+    // item the ghost adjoints that the right-hand side already holds
+    void *a_r = nullptr, *a_old = nullptr, *a_old_c = nullptr;
     // FP32 cycles on a face-averaged coarse level: its halved face coefficients (colour-split) and mode 3
     float *ax32 = nullptr, *ay32 = nullptr, *az32 = nullptr;
     bool face32 = false;
@@ -174,7 +172,8 @@ struct mg_forest {
     std::vector<double> fnorm_p;                 // ||f|| per problem
     int64_t *leaf_off = nullptr;                 // optional: start of every leaf in the user arrays (elements)
     bool batch_member = false;                   // inputs are checked by the owning batch
-    double *a_g = nullptr, *a_lam = nullptr;  // adjoint right-hand side and solution (level 0)
+    // adjoint right-hand side, solution, and right-hand side with the interface part moved to it (level 0)
+    double *a_g = nullptr, *a_lam = nullptr, *a_fe = nullptr;
     bool rhs_set = false;
     double fnorm = 0.0;
     // per-kernel-family launch counters (always on) and CUDA-event timing (mg_profile)
@@ -278,4 +277,10 @@ mg_status enqueue_problem_sums(mg_forest *F);  // per-problem sums -> pinned psu
 mg_status enqueue_fp32_step(mg_forest *F, int cycles);  // `cycles` FP32 V-cycles and the FP64 update
 
 mg_status ensure_fp64_coefficients(mg_forest *F);
+// solver.cu, for the transposed cycles: one FP32 half-sweep on a level's own pools, and the injection y_f += R^T e_c with
+// its write-through (false: not for this level's transfer)
+bool smooth32_specialised(const DevLevel &d);
+bool transfer32_specialised(const DevLevel &d);
+void smooth_level32(mg_forest *F, DevLevel &d, int colour);
+bool inject32(mg_forest *F, DevLevel &d, DevLevel &c);
 }  // namespace octmg

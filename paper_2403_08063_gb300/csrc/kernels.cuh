@@ -1838,7 +1838,8 @@ __device__ __forceinline__ void prolong32_put(float *__restrict__ uf, int64_t bs
 // FP32 prolongation + correction for a level whose blocks all halve (fine edge 2^LG): one thread per coarse cell
 // adds 1/4 (e_C + e_{C+sx} + e_{C+sy} + e_{C+sz}) to its 8 children, fine offsets as in Box32, and writes them
 // through to the face ghosts (prolong32_put).
-template <int LG, bool CG = false>
+// INJ: the transposed restriction instead, 1/8 e_C to each child.
+template <int LG, bool CG = false, bool INJ = false>
 __device__ __forceinline__ void prolong32_body(float *__restrict__ uf, int64_t bsf, const float *__restrict__ ec,
                                                const XferItem *__restrict__ xf, int32_t nbc, int64_t bsc,
                                                const int32_t *__restrict__ nbr6, Skip skip, int64_t t0, int64_t ts) {
@@ -1856,10 +1857,15 @@ __device__ __forceinline__ void prolong32_body(float *__restrict__ uf, int64_t b
         const float *own = ec + B * bsc + pc * HALFc + row;
         const float *oth = ec + B * bsc + (pc ^ 1) * HALFc + row;
         const float e0 = ldv<CG>(own + (Xc >> 1));
-        const float exm = ldv<CG>(oth + ((Xc - 1) >> 1)), exp_ = ldv<CG>(oth + ((Xc + 1) >> 1));
-        const float eym = ldv<CG>(oth + ((Xc >> 1) - HPc)), eyp = ldv<CG>(oth + ((Xc >> 1) + HPc));
-        const float ezm = ldv<CG>(oth + ((Xc >> 1) - PLc)), ezp = ldv<CG>(oth + ((Xc >> 1) + PLc));
-        const float ex[2] = {exm, exp_}, ey[2] = {eym, eyp}, ez[2] = {ezm, ezp};
+        float ex[2], ey[2], ez[2];
+        if constexpr (!INJ) {
+            ex[0] = ldv<CG>(oth + ((Xc - 1) >> 1));
+            ex[1] = ldv<CG>(oth + ((Xc + 1) >> 1));
+            ey[0] = ldv<CG>(oth + ((Xc >> 1) - HPc));
+            ey[1] = ldv<CG>(oth + ((Xc >> 1) + HPc));
+            ez[0] = ldv<CG>(oth + ((Xc >> 1) - PLc));
+            ez[1] = ldv<CG>(oth + ((Xc >> 1) + PLc));
+        }
         const int64_t b = xf[B].src[0];
         const float *ub = uf + b * bsf + (2 * Z * Bx::P + 2 * Y) * Bx::HP + X;
         float val[2][2][2];
@@ -1870,19 +1876,19 @@ __device__ __forceinline__ void prolong32_body(float *__restrict__ uf, int64_t b
 #pragma unroll
                 for (int a = 0; a < 2; ++a)
                     val[c][bb][a] = ldv<CG>(ub + Bx::off(a + 1, bb + 1, c + 1)) +
-                                    0.25f * ((e0 + ex[a]) + (ey[bb] + ez[c]));
+                                    (INJ ? 0.125f * e0 : 0.25f * ((e0 + ex[a]) + (ey[bb] + ez[c])));
         prolong32_put<LG>(uf, bsf, b, X, Y, Z, val, nbr6);
     }
 }
 
-template <int LG>
+template <int LG, bool INJ = false>
 static __global__ void __launch_bounds__(256) k_prolong32(float *__restrict__ uf, int64_t bsf,
                                                           const float *__restrict__ ec,
                                                           const XferItem *__restrict__ xf, int32_t nbc, int64_t bsc,
                                                           const int32_t *__restrict__ nbr6, Skip skip) {
-    prolong32_body<LG>(uf, bsf, ec, xf, nbc, bsc, nbr6, skip,
-                       blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x,
-                       static_cast<int64_t>(gridDim.x) * blockDim.x);
+    prolong32_body<LG, false, INJ>(uf, bsf, ec, xf, nbc, bsc, nbr6, skip,
+                                   blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x,
+                                   static_cast<int64_t>(gridDim.x) * blockDim.x);
 }
 
 // The same prolongation with one thread per segment of ZC coarse cells of a z-column (X fastest across threads, then
@@ -1890,7 +1896,7 @@ static __global__ void __launch_bounds__(256) k_prolong32(float *__restrict__ uf
 // the four lateral neighbours per cell) and the next cell's 8 children before it stores this cell's: loads touch
 // interior cells only, stores touch other interior cells and ghosts, so the early loads read the values the cell-by-cell
 // order would.  Each child takes the expression of prolong32_body, so the results are bit-identical to it.
-template <int LG, int ZC>
+template <int LG, int ZC, bool INJ = false>
 static __global__ void __launch_bounds__(256) k_prolong32z(float *__restrict__ uf, int64_t bsf,
                                                            const float *__restrict__ ec,
                                                            const XferItem *__restrict__ xf, int32_t nbc, int64_t bsc,
@@ -1914,9 +1920,9 @@ static __global__ void __launch_bounds__(256) k_prolong32z(float *__restrict__ u
     };
     float col[ZC + 2], exm[ZC], exp_[ZC], eym[ZC], eyp[ZC];
 #pragma unroll
-    for (int z = 0; z < ZC + 2; ++z) col[z] = E(Xc, Yc, Z0 + z);  // padded z = Z0 .. Z0 + ZC + 1
+    for (int z = INJ ? 1 : 0; z < ZC + (INJ ? 1 : 2); ++z) col[z] = E(Xc, Yc, Z0 + z);  // padded z = Z0 .. Z0 + ZC + 1
 #pragma unroll
-    for (int z = 0; z < ZC; ++z) {
+    for (int z = 0; z < ZC && !INJ; ++z) {
         const int Zc = Z0 + z + 1;
         exm[z] = E(Xc - 1, Yc, Zc);
         exp_[z] = E(Xc + 1, Yc, Zc);
@@ -1945,14 +1951,19 @@ static __global__ void __launch_bounds__(256) k_prolong32z(float *__restrict__ u
                     for (int a = 0; a < 2; ++a) nxt[c][bb][a] = ub[(z + 1) * ZSTEP + Bx::off(a + 1, bb + 1, c + 1)];
         }
         const float e0 = col[z + 1];
-        const float ex[2] = {exm[z], exp_[z]}, ey[2] = {eym[z], eyp[z]}, ez[2] = {col[z], col[z + 2]};
         float val[2][2][2];
 #pragma unroll
         for (int c = 0; c < 2; ++c)
 #pragma unroll
             for (int bb = 0; bb < 2; ++bb)
 #pragma unroll
-                for (int a = 0; a < 2; ++a) val[c][bb][a] = cur[c][bb][a] + 0.25f * ((e0 + ex[a]) + (ey[bb] + ez[c]));
+                for (int a = 0; a < 2; ++a) {
+                    if constexpr (INJ)
+                        val[c][bb][a] = cur[c][bb][a] + 0.125f * e0;
+                    else
+                        val[c][bb][a] = cur[c][bb][a] + 0.25f * ((e0 + (a ? exp_ : exm)[z]) +
+                                                                 ((bb ? eyp : eym)[z] + col[c ? z + 2 : z]));
+                }
         prolong32_put<LG>(uf, bsf, b, X, Y, Z0 + z, val, nbr6);
         if (z + 1 < ZC) {
 #pragma unroll

@@ -104,7 +104,7 @@ void exchange(mg_forest *F, DevLevel &d, T *u, bool interface_only = false, bool
         if (&d == &F->L[0]) gb = F->gb;
     if (one) {
         // a CTA per interface item alone takes as many threads as the item has work for; next to the other faces, 256
-        const int threads = nsf ? kThreads : (n <= 8 ? 32 : (n <= 32 ? 128 : 256));
+        const int threads = nsf ? kThreads : (n <= 8 ? 32 : (n <= 16 ? 64 : 256));
         const int w = n / 2 + 2, grid = nif + (nsf ? grid_for(static_cast<int64_t>(nsf) * n * n) : 0);
         auto *fn = F->cfg.interface_flux ? k_exchange<T, MODE, true> : k_exchange<T, MODE, false>;
         fn<<<grid, threads, nif ? w * w * sizeof(T) : 0, F->st>>>(u, coef_of<T>(d), d.ifaces, nif, d.sfaces, nsf, d.g,
@@ -325,6 +325,11 @@ const Prolong32Fn kProlong32[5] = {k_prolong32<3>, k_prolong32<4>, k_prolong32<5
 constexpr int kProlongZC = 2;
 const Prolong32Fn kProlong32z[3] = {k_prolong32z<5, kProlongZC>, k_prolong32z<6, kProlongZC>,
                                     k_prolong32z<7, kProlongZC>};
+// the transposed restriction in the same two forms
+const Prolong32Fn kInject32[5] = {k_prolong32<3, true>, k_prolong32<4, true>, k_prolong32<5, true>, k_prolong32<6, true>,
+                                  k_prolong32<7, true>};
+const Prolong32Fn kInject32z[3] = {k_prolong32z<5, kProlongZC, true>, k_prolong32z<6, kProlongZC, true>,
+                                   k_prolong32z<7, kProlongZC, true>};
 
 using Restrict32tFn = void (*)(const float *, const float *, const float *, const float *, int64_t, float *, float *,
                                const XferItem *, int32_t, int64_t, Skip, const float *, const float *, const float *,
@@ -371,15 +376,21 @@ void launch_residual_restrict32(mg_forest *F, DevLevel &d, DevLevel &c) {
         d.az32);
 }
 
-void launch_prolong32(mg_forest *F, DevLevel &d, DevLevel &c) {
+void launch_prolong32(mg_forest *F, DevLevel &d, DevLevel &c, bool inject = false) {
     if (d.g.lg >= 5) {
         const auto grid = static_cast<unsigned>((c.cells() / kProlongZC + kThreads - 1) / kThreads);
-        kProlong32z[d.g.lg - 5]<<<grid, kThreads, 0, F->st>>>(d.u32, d.g.bs, c.u32, d.xfer, c.g.nb, c.g.bs, d.nbr6,
-                                                              skip_of(F, c));
+        const Prolong32Fn fn = (inject ? kInject32z : kProlong32z)[d.g.lg - 5];
+        fn<<<grid, kThreads, 0, F->st>>>(d.u32, d.g.bs, c.u32, d.xfer, c.g.nb, c.g.bs, d.nbr6, skip_of(F, c));
         return;
     }
-    kProlong32[d.g.lg - 3]<<<grid_for(c.cells()), kThreads, 0, F->st>>>(d.u32, d.g.bs, c.u32, d.xfer, c.g.nb, c.g.bs,
-                                                                          d.nbr6, skip_of(F, c));
+    const Prolong32Fn fn = (inject ? kInject32 : kProlong32)[d.g.lg - 3];
+    fn<<<grid_for(c.cells()), kThreads, 0, F->st>>>(d.u32, d.g.bs, c.u32, d.xfer, c.g.nb, c.g.bs, d.nbr6, skip_of(F, c));
+}
+
+bool inject32(mg_forest *F, DevLevel &d, DevLevel &c) {
+    if (!transfer32_specialised(d)) return false;
+    launch_prolong32(F, d, c, true);
+    return true;
 }
 
 template <typename T, int MODE>
@@ -397,6 +408,11 @@ void smooth(mg_forest *F, DevLevel &d, int colour) {
     k_smooth<T, MODE><<<grid_for(d.cells() / 2), kThreads, 0, F->st>>>(ufield<T>(d), ffield<T>(d), coef_of<T>(d),
                                                                        h2_of<T>(d), d.g, colour, d.nbr6, skip_of(F, d),
                                                                        gb);
+}
+
+void smooth_level32(mg_forest *F, DevLevel &d, int colour) {
+    if (F->cfg.coeff) smooth<float, 2>(F, d, colour);
+    else smooth<float, 0>(F, d, colour);
 }
 
 // V(nu1, nu2) on level l.  Exchange schedule: at level entry a full exchange, unless the ghosts are known to be
@@ -1140,24 +1156,20 @@ mg_status ensure_scratch64(mg_forest *F) {
     return MG_OK;
 }
 
-// FP64 coefficient arrays (scaled faces, diagonal, inverse diagonal) on every level, for the FP64 paths a forest
-// with FP32 cycles does not allocate at creation (adjoint cycles, the debug exchange of intermediate levels).
+// FP64 coefficient arrays (scaled faces and diagonal) on every level, for the debug exchange of intermediate levels, which a
+// forest with FP32 cycles does not allocate at creation (the inverse diagonal belongs to FP64 smoothing, which it never
+// does).  The adjoint calls it too, so that mg_exchange_level_noalloc finds the arrays after either.
 mg_status ensure_fp64_coefficients(mg_forest *F) {
     if (!F->cfg.coeff) return MG_OK;
     bool added = false;
     for (DevLevel &d : F->L) {
+        if (d.tx) continue;
         const int64_t pe = d.pool_elems();
-        if (!d.tx) {
-            MG_TRY(dalloc(F, &d.tx, pe));
-            MG_TRY(dalloc(F, &d.ty, pe));
-            MG_TRY(dalloc(F, &d.tz, pe));
-            MG_TRY(dalloc(F, &d.dg, pe));
-            added = true;
-        }
-        if (!d.dinv) {
-            MG_TRY(dalloc(F, &d.dinv, pe));
-            added = true;
-        }
+        MG_TRY(dalloc(F, &d.tx, pe));
+        MG_TRY(dalloc(F, &d.ty, pe));
+        MG_TRY(dalloc(F, &d.tz, pe));
+        MG_TRY(dalloc(F, &d.dg, pe));
+        added = true;
     }
     if (added && F->rhs_set) MG_TRY(build_coefficients(F));
     return MG_OK;
