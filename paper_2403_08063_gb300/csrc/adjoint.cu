@@ -54,46 +54,56 @@ __device__ __forceinline__ T scaled_face(const Coef &cf, const T *ih2, int64_t b
     return MODE == 1 ? t : t * ih2[b];
 }
 
-// The coarse face quarter of an interface item and the coarse cells its ghosts' stencils reach.
-struct Quarter {
-    int n, h, lo1, w1, lo2, w2;
-    __device__ Quarter(const FaceItem &F, const LevelGeom &g) : n(g.n), h(g.n >> 1) {
-        lo1 = max(0, F.seg1 * h - 1);
-        w1 = min(n - 1, F.seg1 * h + h) - lo1 + 1;
-        lo2 = max(0, F.seg2 * h - 1);
-        w2 = min(n - 1, F.seg2 * h + h) - lo2 + 1;
+// Shared memory of the transposed quadratic C2F rule of one strip of an item: the adjoints of its 2 rows x n ghosts, their
+// sums after the first tangential step, 2 rows of the w1 <= n/2 + 2 coarse cells, and the tangential weights [case][a][base].
+__host__ __device__ inline size_t scatter_values(int n) {
+    const size_t lines = n / iface_strips(n);
+    return lines * n + lines * (n / 2 + 2) + 18;
+}
+template <typename T>
+struct ScatterMem {
+    T *D, *S, *W;
+    __device__ ScatterMem(unsigned char *raw, const IfaceStrip &Q)
+        : D(reinterpret_cast<T *>(raw)), S(D + 2 * Q.rows * Q.n), W(S + 2 * Q.rows * (Q.h + 2)) {
+        if (threadIdx.x < 18) W[threadIdx.x] = w_tang<T>(0, threadIdx.x / 6, threadIdx.x / 3 % 2, threadIdx.x % 3);
     }
 };
 
-// Adds to E (the quarter's w1 x w2 coarse cells, shared) the tangential transpose of the quadratic C2F rule: the adjoints
-// a[a2][a1] of the four fine ghosts over coarse cell (ycl, zcl) of the quarter.
+// One tangential step of the transpose: the sum over the fine positions of coarse cells c0 .. c0 + count - 1 (values at
+// v[0], v[stride], ..) of the weight with which the ghost there reads coarse cell y.
 template <typename T>
-__device__ __forceinline__ void scatter_tangential(T *E, const Quarter &Q, const FaceItem &F, int ycl, int zcl,
-                                                   const T (&a)[2][2]) {
-    const int yc = F.seg1 * Q.h + ycl, zc = F.seg2 * Q.h + zcl;
-    const int cy = yc == 0 ? 1 : (yc == Q.n - 1 ? 2 : 0);
-    const int cz = zc == 0 ? 1 : (zc == Q.n - 1 ? 2 : 0);
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-        const T s0 = fma(w_tang<T>(0, cy, 1, b), a[0][1], w_tang<T>(0, cy, 0, b) * a[0][0]);
-        const T s1 = fma(w_tang<T>(0, cy, 1, b), a[1][1], w_tang<T>(0, cy, 0, b) * a[1][0]);
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-            atomicAdd(&E[(zc + c_base[cz][c] - Q.lo2) * Q.w1 + yc + c_base[cy][b] - Q.lo1],
-                      fma(w_tang<T>(0, cz, 1, c), s1, w_tang<T>(0, cz, 0, c) * s0));
+__device__ __forceinline__ T gather_tangential(const T *v, int stride, const T *W, int y, int c0, int count, int n) {
+    T s = T(0);
+    for (int c = max(y - 2, c0); c <= min(y + 2, c0 + count - 1); ++c) {
+        const int cs = tang_case(c, n), k = y - c - tang_first(cs);
+        if (k < 0 || k > 2) continue;
+        const int i = 2 * (c - c0);
+        s = fma(W[cs * 6 + k], v[i * stride], s);
+        s = fma(W[cs * 6 + 3 + k], v[(i + 1) * stride], s);
     }
+    return s;
 }
 
-// The normal step of the transpose: sgn times E to the three coarse layers behind the face, through add(b, X, Y, Z, v).
+// The transposed quadratic C2F rule on a strip of item F: the ghosts' adjoints in m.D[line n + i1] (written by the CTA's
+// threads just before) times sgn to the coarse cells the ghosts were extrapolated from, through add(b, X, Y, Z, v).  One
+// tangential direction after the other, then the three coarse layers behind the face: about 6 + 6 + 3 operations per value,
+// as gathers (sums by floating-point atomics in shared memory, which are compare-and-swap loops, took 34 us on 384 faces of
+// 32 x 32 cells; this 19 us).
 template <typename T, class Add>
-__device__ __forceinline__ void scatter_normal(const T *E, const Quarter &Q, const FaceItem &F, T sgn, Add &&add) {
+__device__ __forceinline__ void scatter_c2f(const ScatterMem<T> &m, const IfaceStrip &Q, const FaceItem &F, T sgn, Add &&add) {
+    __syncthreads();
+    for (int q = threadIdx.x; q < 2 * Q.rows * Q.w1; q += blockDim.x) {
+        const int y = q % Q.w1, line = q / Q.w1;
+        m.S[q] = gather_tangential<T>(m.D + line * Q.n, 1, m.W, Q.lo1 + y, F.seg1 * Q.h, Q.h, Q.n);
+    }
+    __syncthreads();
     for (int q = threadIdx.x; q < Q.w1 * Q.w2; q += blockDim.x) {
-        const int y = Q.lo1 + q % Q.w1, z = Q.lo2 + q / Q.w1;
-        const T v = sgn * E[q];
+        const int y = q % Q.w1, z = Q.lo2 + q / Q.w1;
+        const T v = sgn * gather_tangential<T>(m.S + y, Q.w1, m.W, z, F.seg2 * Q.h + Q.c0, Q.rows, Q.n);
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             int X, Y, Z;
-            face_xyz(F.axis, 1 - F.side, 1 + d, y, z, Q.n, X, Y, Z);
+            face_xyz(F.axis, 1 - F.side, 1 + d, Q.lo1 + y, z, Q.n, X, Y, Z);
             add(F.nbr, X, Y, Z, w_normal<T>(0, d) * v);
         }
     }
@@ -116,81 +126,79 @@ __device__ __forceinline__ void add_to(const Target<T> &t, const LevelGeom &g, i
     }
 }
 
-// One interface item per CTA: the transposed ghosts of y on both sides (GHOSTS), and sgn times the part of A^T y that is
-// no 7-point stencil added to `to`.  old (may be null: 0) keeps the ghost adjoints that `to` already holds, n^2 per item,
-// and with the ghost-only variant old_c the coarse ones, (n/2)^2 per item; what is added is the change.  Shared memory:
-// (n/2 + 2)^2 values; where the items of different faces meet, atomics order the sums.
+// One strip of an interface item per CTA, one lane per fine ghost (a coarse cell's four next to each other): the transposed
+// ghosts of y on both sides (GHOSTS), and sgn times the part of A^T y that is no 7-point stencil added to `to`.  old (may be
+// null: 0) keeps the ghost adjoints that `to` already holds, n^2 per item, and with the ghost-only variant old_c the coarse
+// ones, (n/2)^2 per item; what is added is the change.  Where strips meet, atomics order the sums.
 template <typename T, int MODE, bool FLUX, bool GHOSTS>
 __global__ void __launch_bounds__(kThreads)
     k_adj_iface(T *__restrict__ y, Coef cf, const T *__restrict__ ih2, const FaceItem *__restrict__ items, LevelGeom g,
                 T *__restrict__ old, T *__restrict__ old_c, Target<T> to, T sgn) {
     extern __shared__ __align__(16) unsigned char adj_smem[];
-    T *E = reinterpret_cast<T *>(adj_smem);
-    const FaceItem F = items[blockIdx.x];
-    const Quarter Q(F, g);
+    const int strips = iface_strips(g.n), item = blockIdx.x / strips;
+    const FaceItem F = items[item];
+    const IfaceStrip Q(F, g.n, blockIdx.x % strips);
     const int n = Q.n, h = Q.h;
     const bool adds = to.pool || to.user;
-    if (adds) {
-        for (int q = threadIdx.x; q < Q.w1 * Q.w2; q += blockDim.x) E[q] = T(0);
-        __syncthreads();
-    }
-    for (int q = threadIdx.x; q < h * h; q += blockDim.x) {
-        const int ycl = q % h, zcl = q / h, yc = F.seg1 * h + ycl, zc = F.seg2 * h + zcl;
+    const ScatterMem<T> m(adj_smem, Q);
+    const auto add = [&](int64_t b, int X, int Y, int Z, T v) { add_to(to, g, b, X, Y, Z, v); };
+    for (int q = threadIdx.x; q < 4 * Q.rows * h; q += blockDim.x) {
+        const int a1 = q & 1, a2 = (q >> 1) & 1, ycl = (q >> 2) & (h - 1), zcl = Q.c0 + (q >> (g.lg + 1));
+        const int i1 = 2 * ycl + a1, i2 = 2 * zcl + a2, yc = F.seg1 * h + ycl, zc = F.seg2 * h + zcl;
         const int64_t gC = fidx<T>(g, F.nbr, F.axis, 1 - F.side, 1, yc, zc);
         const int64_t g0c = fidx<T>(g, F.nbr, F.axis, 1 - F.side, 0, yc, zc);
+        const int64_t g0 = fidx<T>(g, F.blk, F.axis, F.side, 0, i1, i2);
+        const int64_t g1 = fidx<T>(g, F.blk, F.axis, F.side, 1, i1, i2);
+        // loads before stores, which the compiler could not move them across
         const T yC = y[gC], through = FLUX ? T(0.125) * yC : T(0);
-        T a[2][2];
-#pragma unroll
-        for (int a2 = 0; a2 < 2; ++a2)
-#pragma unroll
-            for (int a1 = 0; a1 < 2; ++a1) {
-                const int i1 = 2 * ycl + a1, i2 = 2 * zcl + a2;
-                const int64_t g0 = fidx<T>(g, F.blk, F.axis, F.side, 0, i1, i2);
-                const int64_t g1 = fidx<T>(g, F.blk, F.axis, F.side, 1, i1, i2);
-                if (GHOSTS) y[g0] = through;
-                if (!adds) continue;
-                const T v = -scaled_face<T, MODE>(cf, ih2, F.blk, g0, g1, F.axis, F.side) * (y[g1] - through);
-                T *keep = old ? old + (static_cast<int64_t>(blockIdx.x) * n + i2) * n + i1 : nullptr;
-                a[a2][a1] = keep ? v - *keep : v;
-                if (keep) *keep = v;
-            }
-        if (GHOSTS) y[g0c] = FLUX ? yC : T(0);
+        T a = T(0);
+        if (adds) a = -scaled_face<T, MODE>(cf, ih2, F.blk, g0, g1, F.axis, F.side) * (y[g1] - through);
+        if (GHOSTS) {
+            y[g0] = through;
+            if ((q & 3) == 0) y[g0c] = FLUX ? yC : T(0);
+        }
         if (!adds) continue;
-        scatter_tangential<T>(E, Q, F, ycl, zcl, a);
-        if (!FLUX) {
-            const T v = -scaled_face<T, MODE>(cf, ih2, F.nbr, g0c, gC, F.axis, 1 - F.side) * yC;
-            T *keep = old_c ? old_c + static_cast<int64_t>(blockIdx.x) * h * h + q : nullptr;
-            const T part = sgn * T(0.125) * (keep ? v - *keep : v);
-            if (keep) *keep = v;
-#pragma unroll
-            for (int d = 1; d <= 2; ++d)
-                for (int e = 0; e < 4; ++e) {
-                    int X, Y, Z;
-                    face_xyz(F.axis, F.side, d, 2 * ycl + (e & 1), 2 * zcl + (e >> 1), n, X, Y, Z);
-                    add_to(to, g, F.blk, X, Y, Z, part);
-                }
+        if (old) {
+            T *keep = old + (static_cast<int64_t>(item) * n + i2) * n + i1;
+            const T before = *keep;
+            *keep = a;
+            a -= before;
+        }
+        m.D[(i2 - 2 * Q.c0) * n + i1] = a;
+        if (!FLUX && (q & 3) == 0) {
+            T v = -scaled_face<T, MODE>(cf, ih2, F.nbr, g0c, gC, F.axis, 1 - F.side) * yC;
+            if (old_c) {
+                T *keep = old_c + (static_cast<int64_t>(item) * h + zcl) * h + ycl;
+                const T before = *keep;
+                *keep = v;
+                v -= before;
+            }
+            for (int e = 0; e < 8; ++e) {
+                int X, Y, Z;
+                face_xyz(F.axis, F.side, 1 + (e >> 2), 2 * ycl + (e & 1), 2 * zcl + ((e >> 1) & 1), n, X, Y, Z);
+                add(F.blk, X, Y, Z, sgn * T(0.125) * v);
+            }
         }
     }
-    if (!adds) return;
-    __syncthreads();
-    scatter_normal<T>(E, Q, F, sgn, [&](int64_t b, int X, int Y, int Z, T v) { add_to(to, g, b, X, Y, Z, v); });
+    if (adds) scatter_c2f<T>(m, Q, F, sgn, add);
 }
 
-// fe = g again at the cells that k_adj_iface adds to, one item per CTA.
+// fe = g again at the cells that k_adj_iface adds to, one strip of an item per CTA.
 template <bool FLUX>
 __global__ void __launch_bounds__(kThreads)
     k_adj_restore(double *__restrict__ fe, const double *__restrict__ gv, const FaceItem *__restrict__ items, LevelGeom g) {
-    const FaceItem F = items[blockIdx.x];
-    const Quarter Q(F, g);
+    const int strips = iface_strips(g.n);
+    const FaceItem F = items[blockIdx.x / strips];
+    const IfaceStrip Q(F, g.n, blockIdx.x % strips);
     for (int q = threadIdx.x; q < Q.w1 * Q.w2; q += blockDim.x)
         for (int d = 1; d <= 3; ++d) {
             const int64_t i = fidx<double>(g, F.nbr, F.axis, 1 - F.side, d, Q.lo1 + q % Q.w1, Q.lo2 + q / Q.w1);
             fe[i] = gv[i];
         }
     if (!FLUX)
-        for (int q = threadIdx.x; q < Q.n * Q.n; q += blockDim.x)
+        for (int q = threadIdx.x; q < 2 * Q.rows * Q.n; q += blockDim.x)
             for (int d = 1; d <= 2; ++d) {
-                const int64_t i = fidx<double>(g, F.blk, F.axis, F.side, d, q % Q.n, q / Q.n);
+                const int64_t i = fidx<double>(g, F.blk, F.axis, F.side, d, q % Q.n, 2 * Q.c0 + q / Q.n);
                 fe[i] = gv[i];
             }
 }
@@ -463,19 +471,21 @@ __global__ void k_et_faces(T *__restrict__ G, const FaceItem *__restrict__ items
     }
 }
 
-// E^T of a level's interface ghosts, one item per CTA, added to the interior of fc.  The ghost adjoints are those of the
-// transposed prolongation: GATHER: a quarter of the four finer cells next to the ghost (the level's blocks are halved
-// blocks, r the finer level's residual); else they stand in fc's own ghosts (k_prolong_T_scatter).
+// E^T of a level's interface ghosts, one strip of an item per CTA and one lane per fine ghost, added to the interior of fc.
+// The ghost adjoints are those of the transposed prolongation: GATHER: a quarter of the four finer cells next to the ghost (the level's
+// blocks are halved blocks, r the finer level's residual); else they stand in fc's own ghosts (k_prolong_T_scatter).
 template <typename T, int MODE, bool FLUX, bool GATHER>
 __global__ void __launch_bounds__(kThreads)
     k_et_iface(T *__restrict__ fc, Coef cf, const FaceItem *__restrict__ items, LevelGeom g, const T *__restrict__ r,
                LevelGeom gf, const XferItem *__restrict__ xf) {
     extern __shared__ __align__(16) unsigned char adj_smem[];
-    T *E = reinterpret_cast<T *>(adj_smem);
-    const FaceItem F = items[blockIdx.x];
-    const Quarter Q(F, g);
+    const int strips = iface_strips(g.n), item = blockIdx.x / strips;
+    const FaceItem F = items[item];
+    const IfaceStrip Q(F, g.n, blockIdx.x % strips);
     const int n = Q.n, h = Q.h;
+    const ScatterMem<T> m(adj_smem, Q);
     const int64_t bf = GATHER ? xf[F.blk].src[0] : 0, bc = GATHER ? xf[F.nbr].src[0] : 0;
+    const auto add = [&](int64_t b, int X, int Y, int Z, T v) { atomicAdd(&fc[Lay<T>::at(g, b, X, Y, Z)], v); };
     const auto ghost = [&](int64_t blk, int64_t fine, int side, int i1, int i2) {
         if constexpr (!GATHER) return fc[fidx<T>(g, blk, F.axis, side, 0, i1, i2)];
         T s = T(0);
@@ -483,43 +493,32 @@ __global__ void __launch_bounds__(kThreads)
         for (int e = 0; e < 4; ++e) s += r[fidx<T>(gf, fine, F.axis, side, 1, 2 * i1 + (e & 1), 2 * i2 + (e >> 1))];
         return T(0.25) * s;
     };
-    for (int q = threadIdx.x; q < Q.w1 * Q.w2; q += blockDim.x) E[q] = T(0);
-    __syncthreads();
-    for (int q = threadIdx.x; q < h * h; q += blockDim.x) {
-        const int ycl = q % h, zcl = q / h, yc = F.seg1 * h + ycl, zc = F.seg2 * h + zcl;
-        const int64_t gC = fidx<T>(g, F.nbr, F.axis, 1 - F.side, 1, yc, zc);
+    for (int q = threadIdx.x; q < 4 * Q.rows * h; q += blockDim.x) {
+        const int a1 = q & 1, a2 = (q >> 1) & 1, ycl = (q >> 2) & (h - 1), zcl = Q.c0 + (q >> (g.lg + 1));
+        const int i1 = 2 * ycl + a1, i2 = 2 * zcl + a2, yc = F.seg1 * h + ycl, zc = F.seg2 * h + zcl;
+        T a = ghost(F.blk, bf, F.side, i1, i2);
         const T aG = ghost(F.nbr, bc, 1 - F.side, yc, zc);
-        T Tc = T(1);
-        if constexpr (FLUX && MODE != 0) {
+        if constexpr (FLUX) {  // G = u_C - sum_j c (g_j - u_j), c = T_j / (2 T_C) (MODE 1: T~_j / (8 T~_C))
+            const int64_t gC = fidx<T>(g, F.nbr, F.axis, 1 - F.side, 1, yc, zc);
             const int64_t g0c = fidx<T>(g, F.nbr, F.axis, 1 - F.side, 0, yc, zc);
-            Tc = face_coef<T, MODE>(cf, F.side ? gC : g0c, F.side ? g0c : gC, F.axis);
-        }
-        if (FLUX) atomicAdd(&fc[gC], aG);
-        T a[2][2];
-#pragma unroll
-        for (int a2 = 0; a2 < 2; ++a2)
-#pragma unroll
-            for (int a1 = 0; a1 < 2; ++a1) {
-                const int i1 = 2 * ycl + a1, i2 = 2 * zcl + a2;
-                a[a2][a1] = ghost(F.blk, bf, F.side, i1, i2);
-                if constexpr (FLUX) {  // G = u_C - sum_j c (g_j - u_j), c = T_j / (2 T_C) (MODE 1: T~_j / (8 T~_C))
-                    const int64_t g0 = fidx<T>(g, F.blk, F.axis, F.side, 0, i1, i2);
-                    const int64_t g1 = fidx<T>(g, F.blk, F.axis, F.side, 1, i1, i2);
-                    const T Tj = face_coef<T, MODE>(cf, F.side ? g0 : g1, F.side ? g1 : g0, F.axis);
-                    const T v = Tj / (T(MODE == 1 ? 8 : 2) * Tc) * aG;
-                    a[a2][a1] -= v;
-                    atomicAdd(&fc[g1], v);
-                }
+            const int64_t g0 = fidx<T>(g, F.blk, F.axis, F.side, 0, i1, i2);
+            const int64_t g1 = fidx<T>(g, F.blk, F.axis, F.side, 1, i1, i2);
+            const T Tc = face_coef<T, MODE>(cf, F.side ? gC : g0c, F.side ? g0c : gC, F.axis);
+            const T Tj = face_coef<T, MODE>(cf, F.side ? g0 : g1, F.side ? g1 : g0, F.axis);
+            const T v = Tj / (T(MODE == 1 ? 8 : 2) * Tc) * aG;
+            a -= v;
+            atomicAdd(&fc[g1], v);
+            if ((q & 3) == 0) atomicAdd(&fc[gC], aG);
+        } else if ((q & 3) == 0) {
+            for (int e = 0; e < 8; ++e) {
+                int X, Y, Z;
+                face_xyz(F.axis, F.side, 1 + (e >> 2), 2 * ycl + (e & 1), 2 * zcl + ((e >> 1) & 1), n, X, Y, Z);
+                add(F.blk, X, Y, Z, T(0.125) * aG);
             }
-        scatter_tangential<T>(E, Q, F, ycl, zcl, a);
-        if (!FLUX)
-            for (int d = 1; d <= 2; ++d)
-                for (int e = 0; e < 4; ++e)
-                    atomicAdd(&fc[fidx<T>(g, F.blk, F.axis, F.side, d, 2 * ycl + (e & 1), 2 * zcl + (e >> 1))],
-                              T(0.125) * aG);
+        }
+        m.D[(i2 - 2 * Q.c0) * n + i1] = a;
     }
-    __syncthreads();
-    scatter_normal<T>(E, Q, F, T(1), [&](int64_t b, int X, int Y, int Z, T v) { atomicAdd(&fc[Lay<T>::at(g, b, X, Y, Z)], v); });
+    scatter_c2f<T>(m, Q, F, T(1), add);
 }
 
 // Transposed restriction and correction, y_f += R^T e_c: every fine cell receives 1/8 of its parent's value (carried-over
@@ -685,12 +684,12 @@ void with_mode(const mg_forest *F, const DevLevel &d, Fn &&fn) {
     else fn(std::integral_constant<int, 2>{});
 }
 
-template <typename T>
-size_t iface_smem(const DevLevel &d) {
-    const size_t w = d.g.n / 2 + 2;
-    return w * w * sizeof(T);
+// Launch of an interface kernel, one CTA per strip of every item.
+template <typename T, class Fn, class... Args>
+void launch_iface(mg_forest *F, const DevLevel &d, Fn fn, Args... args) {
+    const int n = d.g.n;
+    fn<<<d.nifaces * iface_strips(n), iface_threads(n), scatter_values(n) * sizeof(T), F->st>>>(args...);
 }
-int iface_threads(const DevLevel &d) { return d.g.n <= 8 ? 32 : (d.g.n <= 16 ? 64 : 256); }
 
 // Transposed interface ghosts of y (ghosts) and sgn times the interface part of A^T y into `to` (see k_adj_iface).
 template <typename T>
@@ -701,11 +700,20 @@ void adj_iface(mg_forest *F, DevLevel &d, T *y, bool ghosts, T *old, T *old_c, T
         constexpr int M = decltype(m)::value;
         auto *fn = F->cfg.interface_flux ? (ghosts ? k_adj_iface<T, M, true, true> : k_adj_iface<T, M, true, false>)
                                          : (ghosts ? k_adj_iface<T, M, false, true> : k_adj_iface<T, M, false, false>);
-        if (iface_smem<T>(d) > 48 * 1024)  // block edges above 128
-            cudaFuncSetAttribute(reinterpret_cast<const void *>(fn), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(iface_smem<T>(d)));
-        fn<<<d.nifaces, iface_threads(d), iface_smem<T>(d), F->st>>>(y, acoef<T>(d), aih2<T>(d), d.ifaces, d.g, old, old_c,
-                                                                     to, sgn);
+        launch_iface<T>(F, d, fn, y, acoef<T>(d), aih2<T>(d), d.ifaces, d.g, old, old_c, to, sgn);
+    });
+}
+
+// E^T of level c's interface ghosts, from the finer level d's residual r (gather) or from fc's own ghosts.
+template <typename T>
+void et_iface(mg_forest *F, DevLevel &d, DevLevel &c, T *fc, const T *r, bool gather) {
+    if (!c.nifaces) return;
+    Prof p(F, P_ADJ, 1);
+    with_mode<T>(F, c, [&](auto m) {
+        constexpr int M = decltype(m)::value;
+        auto *fn = F->cfg.interface_flux ? (gather ? k_et_iface<T, M, true, true> : k_et_iface<T, M, true, false>)
+                                         : (gather ? k_et_iface<T, M, false, true> : k_et_iface<T, M, false, false>);
+        launch_iface<T>(F, c, fn, fc, acoef<T>(c), c.ifaces, c.g, r, d.g, d.xfer);
     });
 }
 
@@ -806,15 +814,7 @@ void vcycle_T(mg_forest *F, int l) {
             k_et_faces<T><<<grid_for(static_cast<int64_t>(c.nsfaces) << (2 * c.g.lg)), kThreads, 0, F->st>>>(
                 ac.f, c.sfaces, c.nsfaces, c.g);
     }
-    if (c.nifaces) {
-        Prof p(F, P_ADJ, 1);
-        with_mode<T>(F, c, [&](auto m) {
-            constexpr int M = decltype(m)::value;
-            auto *fn = F->cfg.interface_flux ? (gather ? k_et_iface<T, M, true, true> : k_et_iface<T, M, true, false>)
-                                             : (gather ? k_et_iface<T, M, false, true> : k_et_iface<T, M, false, false>);
-            fn<<<c.nifaces, iface_threads(c), iface_smem<T>(c), F->st>>>(ac.f, acoef<T>(c), c.ifaces, c.g, a.r, d.g, d.xfer);
-        });
-    }
+    et_iface<T>(F, d, c, ac.f, a.r, gather);
     vcycle_T<T>(F, l + 1);
     bool through = false;  // the injection wrote same-level and boundary ghosts
     {
@@ -885,7 +885,7 @@ mg_status adjoint_residual(mg_forest *F, bool zero, double mult, double *rr) {
             // FP32 cycles leave a_fe alone, so it differs from g only where the last step added to it
             if (F->cfg.precision == 1) {
                 auto *fn = F->cfg.interface_flux ? k_adj_restore<true> : k_adj_restore<false>;
-                fn<<<d.nifaces, iface_threads(d), 0, F->st>>>(F->a_fe, F->a_g, d.ifaces, d.g);
+                fn<<<d.nifaces * iface_strips(d.g.n), iface_threads(d.g.n), 0, F->st>>>(F->a_fe, F->a_g, d.ifaces, d.g);
             } else {
                 MG_CUDA(cudaMemcpyAsync(F->a_fe, F->a_g, d.pool_elems() * sizeof(double), cudaMemcpyDeviceToDevice, F->st));
             }

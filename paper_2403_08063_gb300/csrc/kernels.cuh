@@ -13,6 +13,7 @@
 //      the residual is then f + sum_f T~_f u_f - dg u, seven FMAs per cell;
 //   2  variable k in FP32: kap[idx] = 1/k with ghosts; T_f = 2 / (kap_i + kap_nb) evaluated with rcp.approx.
 #pragma once
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 #include <cuda_runtime.h>
@@ -430,137 +431,200 @@ static __global__ void k_exchange_segs(T *__restrict__ u, Coef cf, const SegItem
 
 // ------------------------------------------------------------------------------------------------------------
 // Both sides of a refinement interface in one pass.  A fine block face next to a coarser block is one FaceItem, and the
-// quarter of the coarse block's face that it covers is filled from that fine block alone, so the work on one coarse cell of
-// the quarter gives its four fine ghosts (C2F, Sec. 3.3.2) and, from these, the coarse ghost across the face (F2C): all it
-// reads is the interior of the two blocks.  `e` holds the normal-direction extrapolations of the 3 x 3 coarse cells of the
-// cell's tangential stencil.  The same operations in the same order as exchange_faces_body and exchange_segs_body.
+// quarter of the coarse block's face that it covers is filled from that fine block alone, so the four fine ghosts over a
+// coarse cell (C2F, Sec. 3.3.2) give, with the fine cells next to them, the coarse ghost across the face (F2C): all that is
+// read is the interior of the two blocks.  One lane per fine ghost, the four of a coarse cell next to each other (lane
+// 4 k + 2 a2 + a1), which share the coarse ghost's sum by shuffles.  The same operations in the same order as
+// exchange_faces_body and exchange_segs_body.
 // ------------------------------------------------------------------------------------------------------------
+// Offset inside a block of the cell at `depth` from face (axis, side) with tangential interior coordinates (i1, i2), for
+// blocks of fewer than 2^31 elements.
+template <typename T>
+__device__ __forceinline__ int face_in(const LevelGeom &g, int axis, int side, int depth, int i1, int i2) {
+    int X, Y, Z;
+    face_xyz(axis, side, depth, i1, i2, g.n, X, Y, Z);
+    const int P = g.P;
+    if constexpr (sizeof(T) == 8) return (Z * P + Y) * P + X;
+    const int hp = half_row(P);
+    return ((X + Y + Z) & 1) * (P * P * hp) + (Z * P + Y) * hp + (X >> 1);
+}
+
+// The value of lane k (0 .. 3) of the calling lane's group of four.
+template <typename T>
+__device__ __forceinline__ T quad(T v, int k) {
+    return __shfl_sync(0xfu << (threadIdx.x & 28), v, k, 4);
+}
+
+// Tangential stencil of a coarse coordinate: the case of its weights, and the offset of its first base.
+__device__ __forceinline__ int tang_case(int c, int n) { return c == 0 ? 1 : (c == n - 1 ? 2 : 0); }
+__device__ __forceinline__ int tang_first(int cs) { return cs == 0 ? -1 : (cs == 1 ? 0 : -2); }
+
+// What one fine ghost of an interface needs besides the coarse block's values around it, loaded before anything depends on
+// it: the fine cells next to the ghost and, conservative variant, the coarse cell and the two face coefficients.
 template <typename T, int MODE, bool FLUX, bool CG = false>
-__device__ __forceinline__ void exchange_iface_cell(T *__restrict__ u, const Coef &cf, const FaceItem &F,
-                                                    const LevelGeom &g, int c2f, int ycl, int zcl, const T (&e)[3][3]) {
-    const int n = g.n, h = n >> 1;
-    const int yc = F.seg1 * h + ycl, zc = F.seg2 * h + zcl;
-    const int cy = yc == 0 ? 1 : (yc == n - 1 ? 2 : 0);
-    const int cz = zc == 0 ? 1 : (zc == n - 1 ? 2 : 0);
-    const int64_t gC = fidx<T>(g, F.nbr, F.axis, 1 - F.side, 1, yc, zc);
-    const int64_t g0c = fidx<T>(g, F.nbr, F.axis, 1 - F.side, 0, yc, zc);
-    T flux = T(0);
-#pragma unroll
-    for (int a2 = 0; a2 < 2; ++a2)
-#pragma unroll
-        for (int a1 = 0; a1 < 2; ++a1) {
-            T acc = T(0);
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                T accb = T(0);
-#pragma unroll
-                for (int b = 0; b < 3; ++b) accb = fma(w_tang<T>(c2f, cy, a1, b), e[c][b], accb);
-                acc = fma(w_tang<T>(c2f, cz, a2, c), accb, acc);
-            }
-            const int64_t g0 = fidx<T>(g, F.blk, F.axis, F.side, 0, 2 * ycl + a1, 2 * zcl + a2);
-            u[g0] = acc;
-            if constexpr (FLUX) {
-                const int64_t g1 = fidx<T>(g, F.blk, F.axis, F.side, 1, 2 * ycl + a1, 2 * zcl + a2);
-                const T Tj = face_coef<T, MODE>(cf, F.side ? g0 : g1, F.side ? g1 : g0, F.axis);
-                flux = fma(Tj, acc - ldv<CG>(u + g1), flux);
-            }
+struct IfaceGhost {
+    int64_t g0, g0c;
+    T u1, u2, uC, Tj, Tc;
+    __device__ __forceinline__ IfaceGhost(const T *__restrict__ u, const Coef &cf, const FaceItem &F, const LevelGeom &g,
+                                          int ycl, int zcl, int a1, int a2) {
+        const int h = g.n >> 1, i1 = 2 * ycl + a1, i2 = 2 * zcl + a2, yc = F.seg1 * h + ycl, zc = F.seg2 * h + zcl;
+        const int64_t fb = F.blk * g.bs, cb = F.nbr * g.bs;
+        g0 = fb + face_in<T>(g, F.axis, F.side, 0, i1, i2);
+        g0c = cb + face_in<T>(g, F.axis, 1 - F.side, 0, yc, zc);
+        const int64_t g1 = fb + face_in<T>(g, F.axis, F.side, 1, i1, i2);
+        u1 = ldv<CG>(u + g1);
+        if constexpr (FLUX) {
+            const int64_t gC = cb + face_in<T>(g, F.axis, 1 - F.side, 1, yc, zc);
+            uC = ldv<CG>(u + gC);
+            Tj = face_coef<T, MODE>(cf, F.side ? g0 : g1, F.side ? g1 : g0, F.axis);
+            Tc = face_coef<T, MODE>(cf, F.side ? gC : g0c, F.side ? g0c : gC, F.axis);
+        } else {
+            u2 = ldv<CG>(u + fb + face_in<T>(g, F.axis, F.side, 2, i1, i2));
         }
-    if constexpr (FLUX) {
-        const T Tc = face_coef<T, MODE>(cf, F.side ? gC : g0c, F.side ? g0c : gC, F.axis);
-        u[g0c] = ldv<CG>(u + gC) - flux / (T(MODE == 1 ? 8 : 2) * Tc);
-    } else {
-        T s = T(0);
-#pragma unroll
-        for (int d = 1; d <= 2; ++d)
-#pragma unroll
-            for (int b = 0; b < 2; ++b)
-#pragma unroll
-                for (int a = 0; a < 2; ++a)
-                    s += ldv<CG>(u + fidx<T>(g, F.blk, F.axis, F.side, d, 2 * ycl + a, 2 * zcl + b));
-        u[g0c] = T(0.125) * s;
     }
-}
+    // The ghost from the normal-direction extrapolations e of its coarse cell's 3 x 3 tangential stencil and the tangential
+    // weights wy, wz; then the coarse ghost, by the group's first lane.
+    __device__ __forceinline__ void put(T *__restrict__ u, bool first, const T (&e)[3][3], const T (&wy)[3],
+                                        const T (&wz)[3]) const {
+        T acc = T(0);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            T accb = T(0);
+#pragma unroll
+            for (int b = 0; b < 3; ++b) accb = fma(wy[b], e[c][b], accb);
+            acc = fma(wz[c], accb, acc);
+        }
+        u[g0] = acc;
+        if constexpr (FLUX) {
+            const T diff = acc - u1;
+            T flux = T(0);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) flux = fma(quad(Tj, k), quad(diff, k), flux);
+            if (first) u[g0c] = uC - flux / (T(MODE == 1 ? 8 : 2) * Tc);
+        } else {
+            T s = T(0);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) s += quad(u1, k);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) s += quad(u2, k);
+            if (first) u[g0c] = T(0.125) * s;
+        }
+    }
+};
 
-// One interface item by one CTA.  The normal-direction extrapolations of the quarter's coarse cells and of their one-cell
-// tangential border are computed once into shared memory, E[(n/2 + 2)^2] (Sec. 8 of the paper proposes this reuse for
-// neighbouring cells): about 3.4 loads per coarse cell instead of 27.
+// An interface item's quarter is cut into strips of coarse rows, one CTA each, so that a CTA has one ghost per thread (at
+// most 256 threads; two and more above block edge 128): the work is a chain of dependent loads.
+__host__ __device__ constexpr int iface_strips(int n) {
+    return n * n / kThreads < 1 ? 1 : (n * n / kThreads > n / 2 ? n / 2 : n * n / kThreads);
+}
+inline int iface_threads(int n) { return std::max(32, std::min(kThreads, n * n / iface_strips(n))); }
+
+// Strip `strip` of item F: coarse rows c0 .. c0 + rows - 1 of the quarter, and the coarse cells [lo1, lo1 + w1) x
+// [lo2, lo2 + w2) of the coarse face that the tangential stencils of its ghosts reach (remapped bases stay inside the block).
+struct IfaceStrip {
+    int n, h, rows, c0, lo1, w1, lo2, w2;
+    __device__ __forceinline__ IfaceStrip(const FaceItem &F, int n_, int strip) : n(n_), h(n_ >> 1) {
+        rows = h / iface_strips(n);
+        c0 = strip * rows;
+        const int z0 = F.seg2 * h + c0, z1 = z0 + rows - 1;
+        lo1 = max(0, F.seg1 * h - 1);
+        w1 = min(n - 1, F.seg1 * h + h) - lo1 + 1;
+        lo2 = max(0, z1 == n - 1 ? min(z0 - 1, n - 3) : z0 - 1);
+        w2 = min(n - 1, z0 == 0 ? max(z1 + 1, 2) : z1 + 1) - lo2 + 1;
+    }
+};
+
+// One strip of an interface item by one CTA, one ghost per thread (block edges up to 128).  The normal-direction
+// extrapolations of the strip's coarse cells and of their tangential border are computed once into shared memory, E[w1 w2]
+// (Sec. 8 of the paper proposes this reuse for neighbouring cells); W[18] the tangential weights [case][a][base].  All loads
+// come before the first use of one, and before the done-mask decides (uniformly over the CTA) whether anything is written.
 template <typename T, int MODE, bool FLUX>
-__device__ __forceinline__ void exchange_iface_cta(T *__restrict__ u, const Coef &cf, const FaceItem &F,
-                                                   const LevelGeom &g, int c2f, T *E) {
-    const int n = g.n, h = n >> 1;
-    // coarse cells [lo1, lo1 + w1) x [lo2, lo2 + w2) of the coarse face: the segment and the neighbours its
-    // stencils reach (remapped bases stay inside the coarse block)
-    const int lo1 = max(0, F.seg1 * h - 1), w1 = min(n - 1, F.seg1 * h + h) - lo1 + 1;
-    const int lo2 = max(0, F.seg2 * h - 1), w2 = min(n - 1, F.seg2 * h + h) - lo2 + 1;
-    for (int q = threadIdx.x; q < w1 * w2; q += blockDim.x) {
-        const int y = lo1 + q % w1, z = lo2 + q / w1;
-        T v = w_normal<T>(c2f, 0) * u[fidx<T>(g, F.nbr, F.axis, 1 - F.side, 1, y, z)];
-        v = fma(w_normal<T>(c2f, 1), u[fidx<T>(g, F.nbr, F.axis, 1 - F.side, 2, y, z)], v);
-        E[q] = fma(w_normal<T>(c2f, 2), u[fidx<T>(g, F.nbr, F.axis, 1 - F.side, 3, y, z)], v);
+__device__ __forceinline__ void exchange_iface_cta(T *__restrict__ u, const Coef &cf, const FaceItem &F, int strip,
+                                                   const LevelGeom &g, Skip skip, int c2f, T *E, T *W) {
+    const IfaceStrip Q(F, g.n, strip);
+    const int n = Q.n, h = Q.h, lgh = g.lg - 1, q = threadIdx.x;
+    const int a1 = q & 1, a2 = (q >> 1) & 1, ycl = (q >> 2) & (h - 1), zcl = Q.c0 + (q >> (2 + lgh));
+    const bool mine = q < 4 * Q.rows * h;
+    const IfaceGhost<T, MODE, FLUX> G(u, cf, F, g, ycl, mine ? zcl : Q.c0, a1, a2);
+    const T *uc = u + F.nbr * g.bs;
+    if (q < 18) W[q] = w_tang<T>(c2f, q / 6, q / 3 % 2, q % 3);
+    for (int i = q; i < Q.w1 * Q.w2; i += blockDim.x) {
+        const int y = Q.lo1 + i % Q.w1, z = Q.lo2 + i / Q.w1;
+        T v = w_normal<T>(c2f, 0) * uc[face_in<T>(g, F.axis, 1 - F.side, 1, y, z)];
+        v = fma(w_normal<T>(c2f, 1), uc[face_in<T>(g, F.axis, 1 - F.side, 2, y, z)], v);
+        E[i] = fma(w_normal<T>(c2f, 2), uc[face_in<T>(g, F.axis, 1 - F.side, 3, y, z)], v);
     }
+    if (skip(F.blk)) return;
     __syncthreads();
-    for (int q = threadIdx.x; q < h * h; q += blockDim.x) {
-        const int ycl = q % h, zcl = q / h;
-        const int yc = F.seg1 * h + ycl, zc = F.seg2 * h + zcl;
-        const int cy = yc == 0 ? 1 : (yc == n - 1 ? 2 : 0);
-        const int cz = zc == 0 ? 1 : (zc == n - 1 ? 2 : 0);
-        T e[3][3];
+    if (!mine) return;
+    const int yc = F.seg1 * h + ycl, zc = F.seg2 * h + zcl;
+    const int cy = tang_case(yc, n), cz = tang_case(zc, n);
+    const T *Ec = E + (zc + tang_first(cz) - Q.lo2) * Q.w1 + yc + tang_first(cy) - Q.lo1;
+    T e[3][3], wy[3], wz[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c)
+    for (int c = 0; c < 3; ++c) {
+        wy[c] = W[cy * 6 + a1 * 3 + c];
+        wz[c] = W[cz * 6 + a2 * 3 + c];
 #pragma unroll
-            for (int b = 0; b < 3; ++b)
-                e[c][b] = E[(zc + c_base[cz][c] - lo2) * w1 + (yc + c_base[cy][b] - lo1)];
-        exchange_iface_cell<T, MODE, FLUX>(u, cf, F, g, c2f, ycl, zcl, e);
+        for (int b = 0; b < 3; ++b) e[c][b] = Ec[c * Q.w1 + b];
     }
+    G.put(u, (q & 3) == 0, e, wy, wz);
 }
 
-// The interface items one thread per coarse cell, without shared memory (the persistent tail, whose items are small).
+// The interface items one thread per fine ghost, without shared memory (the persistent tail, whose items are small).
 template <typename T, int MODE, bool FLUX, bool CG>
 __device__ __forceinline__ void exchange_iface_body(T *__restrict__ u, const Coef &cf, const FaceItem *__restrict__ items,
                                                     int nitems, const LevelGeom &g, Skip skip, int64_t t0, int64_t ts,
                                                     int c2f = 0) {
-    const int n = g.n, h = n >> 1, lgh = g.lg - 1;
-    const int64_t total = static_cast<int64_t>(nitems) << (2 * lgh);
+    const int n = g.n, h = n >> 1, lg = g.lg;
+    const int64_t total = static_cast<int64_t>(nitems) << (2 * lg);
     for (int64_t t = t0; t < total; t += ts) {
-        const FaceItem F = items[t >> (2 * lgh)];
+        const FaceItem F = items[t >> (2 * lg)];
         if (skip(F.blk)) continue;
-        const int r = static_cast<int>(t) & ((1 << (2 * lgh)) - 1), ycl = r & (h - 1), zcl = r >> lgh;
+        const int q = static_cast<int>(t) & ((1 << (2 * lg)) - 1);
+        const int a1 = q & 1, a2 = (q >> 1) & 1, ycl = (q >> 2) & (h - 1), zcl = q >> (1 + lg);
         const int yc = F.seg1 * h + ycl, zc = F.seg2 * h + zcl;
-        const int cy = yc == 0 ? 1 : (yc == n - 1 ? 2 : 0);
-        const int cz = zc == 0 ? 1 : (zc == n - 1 ? 2 : 0);
-        T e[3][3];
+        const int cy = tang_case(yc, n), cz = tang_case(zc, n);
+        const int y0 = yc + tang_first(cy), z0 = zc + tang_first(cz);
+        const T *uc = u + F.nbr * g.bs;
+        const IfaceGhost<T, MODE, FLUX, CG> G(u, cf, F, g, ycl, zcl, a1, a2);
+        T e[3][3], wy[3], wz[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c)
+        for (int c = 0; c < 3; ++c) {
+            wy[c] = w_tang<T>(c2f, cy, a1, c);
+            wz[c] = w_tang<T>(c2f, cz, a2, c);
 #pragma unroll
             for (int b = 0; b < 3; ++b) {
-                const int y = yc + c_base[cy][b], z = zc + c_base[cz][c];
-                T v = w_normal<T>(c2f, 0) * ldv<CG>(u + fidx<T>(g, F.nbr, F.axis, 1 - F.side, 1, y, z));
-                v = fma(w_normal<T>(c2f, 1), ldv<CG>(u + fidx<T>(g, F.nbr, F.axis, 1 - F.side, 2, y, z)), v);
-                e[c][b] = fma(w_normal<T>(c2f, 2), ldv<CG>(u + fidx<T>(g, F.nbr, F.axis, 1 - F.side, 3, y, z)), v);
+                T v = w_normal<T>(c2f, 0) * ldv<CG>(uc + face_in<T>(g, F.axis, 1 - F.side, 1, y0 + b, z0 + c));
+                v = fma(w_normal<T>(c2f, 1), ldv<CG>(uc + face_in<T>(g, F.axis, 1 - F.side, 2, y0 + b, z0 + c)), v);
+                e[c][b] = fma(w_normal<T>(c2f, 2), ldv<CG>(uc + face_in<T>(g, F.axis, 1 - F.side, 3, y0 + b, z0 + c)), v);
             }
-        exchange_iface_cell<T, MODE, FLUX, CG>(u, cf, F, g, c2f, ycl, zcl, e);
+        }
+        G.put(u, (q & 3) == 0, e, wy, wz);
     }
 }
 
-// Ghost exchange of a level in one launch: CTAs [0, nif) one interface item each, the others the faces filled from one
-// source block (boundary, same level; nsf items, none for the interface-only exchange between half-sweeps), one thread per
+// Ghost exchange of a level in one launch: CTAs [0, nif strips) one strip of an interface item each, the others the faces
+// filled from one source block (boundary, same level; nsf items, none for the interface-only exchange between half-sweeps), one thread per
 // ghost cell.  Every ghost is computed from block interiors only, so the two parts are independent.  These launches move a
-// few hundred KB and last as long as their latency; two of them (C2F, then F2C from the fine ghosts) took 2 x 3.2 us per
-// half-sweep on 56 + 64 blocks of 32^3, this one 3.5 us.
+// few hundred KB and last as long as their chain of dependent loads and instructions, so an item's work is spread over as
+// many lanes as it has ghosts, with every load ahead of the first use: 12.8 us on 384 faces of 32 x 32 cells and 3.2 us on
+// the coarser levels, where one lane per coarse cell, loading as it went, took 22.7 and 4.7 us.
 template <typename T, int MODE, bool FLUX>
 static __global__ void __launch_bounds__(kThreads) k_exchange(T *__restrict__ u, Coef cf,
                                                               const FaceItem *__restrict__ ifaces, int nif,
                                                               const FaceItem *__restrict__ sfaces, int nsf, LevelGeom g,
                                                               Skip skip, int c2f, const T *__restrict__ gb) {
     extern __shared__ __align__(16) unsigned char iface_smem[];
-    if (static_cast<int>(blockIdx.x) < nif) {
-        const FaceItem F = ifaces[blockIdx.x];
-        if (skip(F.blk)) return;  // uniform over the CTA, before the barrier
-        exchange_iface_cta<T, MODE, FLUX>(u, cf, F, g, c2f, reinterpret_cast<T *>(iface_smem));
+    __shared__ T W[18];
+    const int strips = iface_strips(g.n), nic = nif * strips;
+    if (static_cast<int>(blockIdx.x) < nic) {
+        const FaceItem F = ifaces[blockIdx.x / strips];
+        exchange_iface_cta<T, MODE, FLUX>(u, cf, F, blockIdx.x % strips, g, skip, c2f, reinterpret_cast<T *>(iface_smem), W);
         return;
     }
-    exchange_faces_body<T, false>(u, sfaces, nsf, g, skip, (blockIdx.x - nif) * static_cast<int64_t>(blockDim.x) + threadIdx.x,
-                                  static_cast<int64_t>(gridDim.x - nif) * blockDim.x, c2f, gb);
+    exchange_faces_body<T, false>(u, sfaces, nsf, g, skip, (blockIdx.x - nic) * static_cast<int64_t>(blockDim.x) + threadIdx.x,
+                                  static_cast<int64_t>(gridDim.x - nic) * blockDim.x, c2f, gb);
 }
 
 // ------------------------------------------------------------------------------------------------------------

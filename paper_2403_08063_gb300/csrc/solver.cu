@@ -87,12 +87,13 @@ template <typename T> Coef coef_of(const DevLevel &d);
 template <> Coef coef_of<double>(const DevLevel &d) { return d.c64(); }
 template <> Coef coef_of<float>(const DevLevel &d) { return d.c32(); }
 
-// The done-mask view of a level for its kernels (all problems active outside a solve).
-Skip skip_of(mg_forest *F, const DevLevel &d) { return Skip{d.bprob, F->pdone}; }
+// The done-mask view of a level for its kernels (all problems active outside a solve).  A single problem needs none: its
+// solve ends when it is done, and without a mask a kernel starts two dependent loads earlier (0.5 us of a launch of 3).
+Skip skip_of(mg_forest *F, const DevLevel &d) { return Skip{d.bprob, F->np > 1 ? F->pdone : nullptr}; }
 
 // Ghost exchange of a level: every face (full), or only the refinement-interface faces (C2F and F2C), whose
-// ghosts the smoother's write-through does not maintain.  One launch for block edges up to 128 (the interface items' shared
-// memory, (n/2 + 2)^2 values, then fits 48 KB), two generic ones above.
+// ghosts the smoother's write-through does not maintain.  One launch for block edges up to 128 (its offsets inside a block
+// are 32-bit), two generic ones above.
 template <typename T, int MODE>
 void exchange(mg_forest *F, DevLevel &d, T *u, bool interface_only = false, bool prof = true) {
     const int nif = d.nifaces, nsf = interface_only ? 0 : d.nsfaces, n = d.g.n;
@@ -103,11 +104,11 @@ void exchange(mg_forest *F, DevLevel &d, T *u, bool interface_only = false, bool
     if constexpr (sizeof(T) == 8)
         if (&d == &F->L[0]) gb = F->gb;
     if (one) {
-        // a CTA per interface item alone takes as many threads as the item has work for; next to the other faces, 256
-        const int threads = nsf ? kThreads : (n <= 8 ? 32 : (n <= 16 ? 64 : 256));
-        const int w = n / 2 + 2, grid = nif + (nsf ? grid_for(static_cast<int64_t>(nsf) * n * n) : 0);
+        const int threads = nsf ? kThreads : iface_threads(n), strips = iface_strips(n);
+        const size_t smem = nif ? (n / 2 / strips + 2) * (n / 2 + 2) * sizeof(T) : 0;
+        const int grid = nif * strips + (nsf ? grid_for(static_cast<int64_t>(nsf) * n * n) : 0);
         auto *fn = F->cfg.interface_flux ? k_exchange<T, MODE, true> : k_exchange<T, MODE, false>;
-        fn<<<grid, threads, nif ? w * w * sizeof(T) : 0, F->st>>>(u, coef_of<T>(d), d.ifaces, nif, d.sfaces, nsf, d.g,
+        fn<<<grid, threads, smem, F->st>>>(u, coef_of<T>(d), d.ifaces, nif, d.sfaces, nsf, d.g,
                                                                   skip_of(F, d), F->cfg.c2f_variant, gb);
         return;
     }
