@@ -943,11 +943,11 @@ mg_status adjoint_solve(mg_forest *F, const double *u_dev, const double *dLdu_de
         rel = std::sqrt(rr) / gn;
         if (!std::isfinite(rel) || rel <= rtol || it >= max_cycles) break;
         if (F->cfg.precision == 1) {
-            vcycle_T<float>(F, 0);
+            MG_TRY(replay(F, F->vT_rec, [&] { vcycle_T<float>(F, 0); }));
             Prof p(F, P_ADJ, 1);
             k_update_mixed<<<grid, kThreads, 0, F->st>>>(F->a_lam, d.u32, F->pinv, d.bprob, d.g, Skip{});
         } else {
-            vcycle_T<double>(F, 0);
+            MG_TRY(replay(F, F->vT_rec, [&] { vcycle_T<double>(F, 0); }));
             Prof p(F, P_ADJ, 1);
             k_add<<<grid, kThreads, 0, F->st>>>(F->a_lam, d.u64, d.g);
         }

@@ -121,6 +121,17 @@ struct BatchEntry {
     TailPhase P;
 };
 
+// A launch sequence that depends only on the forest, recorded as a CUDA graph and replayed (see replay below).
+struct Replay {
+    cudaGraphExec_t exec = nullptr;
+    int runs = 0;
+    bool off = false;  // the recording failed or cannot be replayed: launched directly
+    void drop() {
+        if (exec) cudaGraphExecDestroy(exec);
+        exec = nullptr;
+    }
+};
+
 }  // namespace octmg
 
 struct mg_forest {
@@ -146,13 +157,9 @@ struct mg_forest {
     double *AinvT = nullptr;                  // transpose of the coarsest inverses (adjoint cycles)
     double *gj_panel = nullptr;                // device Gauss-Jordan: the eliminated panel, its row exchanges
     int32_t *gj_src = nullptr, *gj_org = nullptr;  // and the composed row origins (two buffers)
-    cudaGraphExec_t coarse_graph = nullptr;    // recorded coarsest-level probe + inversion (assemble_coarse)
-    int coarse_runs = 0;                       // calls of assemble_coarse so far
-    bool coarse_nograph = false;               // its recording failed: launched directly
     cudaStream_t cap_st = nullptr;             // private stream: graph recording, host-input copies
-    cudaGraphExec_t v64_graph = nullptr;       // one recorded FP64 V-cycle (vcycle64_step), replayed per cycle
-    int v64_runs = 0;                          // FP64 V-cycles run so far (recording starts at the second)
-    bool v64_nograph = false;                  // the recording failed or is not replayable: launched directly
+    // recorded sequences: coarsest-level probe + inversion (assemble_coarse), FP64 V-cycle, FP32 V-cycle, transposed V-cycle
+    octmg::Replay coarse_rec, v64_rec, v32_rec, vT_rec;
     double *hst_f = nullptr, *hst_k = nullptr, *hst_u = nullptr;  // mg_solve_host staging buffers (user layout)
     cudaEvent_t hst_ev = nullptr;              // orders the staging copies against the forest's stream
     int8_t *pcol = nullptr;                    // colour probe (interface-free coarsest level): colour per unknown
@@ -233,6 +240,53 @@ inline std::string fmt_e(double v) {
     char b[32];
     std::snprintf(b, sizeof(b), "%.3e", v);
     return b;
+}
+
+// Runs `body` (launches on F->st that depend only on the forest) as a recorded CUDA graph: directly the first time (it loads
+// the kernels, which a capture does not allow), recorded at the second on the private stream (the forest's may be the legacy
+// default stream, which cannot be captured), replayed on the forest's stream from then on.  One launch per step costs the
+// host about 5 us each, more than most of the coarse levels' kernels last.  Directly also while profiling (per-family
+// events), while the caller's stream is being captured, and when the recording fails or `recorded()`, called after it,
+// says that it cannot be replayed.
+template <class Body, class Ok>
+mg_status replay(mg_forest *F, Replay &r, Body &&body, Ok &&recorded) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    MG_CUDA(cudaStreamIsCapturing(F->st, &cap));
+    if (F->prof || r.off || cap != cudaStreamCaptureStatusNone || r.runs++ == 0) {
+        body();
+        MG_CUDA(cudaGetLastError());
+        return MG_OK;
+    }
+    if (!r.exec) {
+        cudaGraph_t graph = nullptr;
+        cudaError_t e = F->cap_st ? cudaSuccess : cudaStreamCreateWithFlags(&F->cap_st, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaStreamBeginCapture(F->cap_st, cudaStreamCaptureModeThreadLocal);
+        bool ok = false;
+        if (e == cudaSuccess) {
+            cudaStream_t own = F->st;
+            F->st = F->cap_st;
+            body();
+            F->st = own;
+            e = cudaStreamEndCapture(F->cap_st, &graph);
+            ok = recorded();
+        }
+        if (e == cudaSuccess && graph && ok) e = cudaGraphInstantiate(&r.exec, graph, 0);
+        if (graph) cudaGraphDestroy(graph);
+        if (e != cudaSuccess || !ok || !r.exec) {
+            r.exec = nullptr;
+            r.off = true;
+            cudaGetLastError();
+            body();
+            MG_CUDA(cudaGetLastError());
+            return MG_OK;
+        }
+    }
+    MG_CUDA(cudaGraphLaunch(r.exec, F->st));
+    return MG_OK;
+}
+template <class Body>
+mg_status replay(mg_forest *F, Replay &r, Body &&body) {
+    return replay(F, r, body, [] { return true; });
 }
 
 // FP64 operator application A u on a level (ghosts of u already exchanged), defined in solver.cu.

@@ -780,8 +780,7 @@ void enqueue_coarse_inverse(mg_forest *F, DevLevel &d, int N, int maxN) {
 }
 
 // Coarsest-level dense operators and their inverses (and transposes), every problem's block at once.  The device
-// part is a few thousand small launches; outside a stream capture it is recorded as a CUDA graph at the second call
-// and replayed by later ones (the pointers it uses never change).
+// part is about a hundred small launches, recorded as a CUDA graph (the pointers it uses never change).
 mg_status assemble_coarse(mg_forest *F) {
     const int l = static_cast<int>(F->L.size()) - 1;
     DevLevel &d = F->L[l];
@@ -882,46 +881,10 @@ mg_status assemble_coarse(mg_forest *F) {
     const bool prof = F->prof;
     F->gb = nullptr;
     F->prof = false;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    cudaError_t ce = cudaStreamIsCapturing(F->st, &cap);
-    // recorded from the second call on (the first one loads every kernel the sequence uses, which a capture does not
-    // allow); a recording that fails is abandoned for good and the sequence launched directly
-    if (ce == cudaSuccess && cap == cudaStreamCaptureStatusNone && F->coarse_runs++ > 0 && !F->coarse_graph &&
-        !F->coarse_nograph) {
-        // recorded on a private stream (the forest's stream may be the legacy default stream, which cannot be
-        // captured); the graph is then launched on the forest's stream
-        cudaGraph_t graph = nullptr;
-        cudaError_t e1 = F->cap_st ? cudaSuccess : cudaStreamCreateWithFlags(&F->cap_st, cudaStreamNonBlocking);
-        if (e1 == cudaSuccess) e1 = cudaStreamBeginCapture(F->cap_st, cudaStreamCaptureModeThreadLocal);
-        if (e1 == cudaSuccess) {
-            cudaStream_t own = F->st;
-            F->st = F->cap_st;
-            enqueue_coarse_inverse(F, d, N, maxN);
-            F->st = own;
-            e1 = cudaStreamEndCapture(F->cap_st, &graph);
-        }
-        if (e1 == cudaSuccess && graph) e1 = cudaGraphInstantiate(&F->coarse_graph, graph, 0);
-        if (graph) cudaGraphDestroy(graph);
-        if (e1 != cudaSuccess || !F->coarse_graph) {
-            F->coarse_graph = nullptr;
-            F->coarse_nograph = true;
-            cudaGetLastError();
-        }
-    }
-    if (ce == cudaSuccess) {
-        if (F->coarse_graph && cap == cudaStreamCaptureStatusNone) {
-            ce = cudaGraphLaunch(F->coarse_graph, F->st);
-        } else {
-            enqueue_coarse_inverse(F, d, N, maxN);
-            ce = cudaGetLastError();
-        }
-    }
+    const mg_status st = replay(F, F->coarse_rec, [&] { enqueue_coarse_inverse(F, d, N, maxN); });
     F->gb = gb;
     F->prof = prof;
-    if (ce != cudaSuccess) {
-        set_error(std::string("coarsest-level inverse: ") + cudaGetErrorString(ce));
-        return MG_ERR_CUDA;
-    }
+    MG_TRY(st);
     int hbad = 0;
     MG_CUDA(cudaMemcpyAsync(&hbad, F->flag, sizeof(int), cudaMemcpyDeviceToHost, F->st));
     MG_CUDA(cudaStreamSynchronize(F->st));
@@ -982,50 +945,21 @@ void vcycle64(mg_forest *F) {
     if (F->cfg.coeff) vcycle<double, 1>(F, 0, ENTRY_FULL);
     else vcycle<double, 0>(F, 0, ENTRY_FULL);
 }
-// One FP64 V-cycle on level 0, replayed from a recorded CUDA graph: the cycle's launch sequence depends only on the
-// forest, so it is recorded once, on the private stream (from the second cycle on: the first one loads the kernels,
-// which a capture does not allow), and each later cycle is one graph launch instead of one launch per step, which
-// is what small, launch-bound forests need.  Launched directly while profiling (per-family events), while the
-// caller's stream is being captured, and when the recorded cycle would not leave the damped-Jacobi ping-pong pools
-// as it found them (an odd number of sweeps per level) or the recording fails.  mg_set_boundary drops the graph.
+// One FP64 V-cycle on level 0, recorded and replayed.  Not replayable when it would not leave the damped-Jacobi ping-pong
+// pools as it found them (an odd number of sweeps per level).  mg_set_boundary drops the graph.
 mg_status vcycle64_step(mg_forest *F) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    MG_CUDA(cudaStreamIsCapturing(F->st, &cap));
-    if (F->prof || F->v64_nograph || cap != cudaStreamCaptureStatusNone || F->v64_runs++ == 0) {
-        vcycle64(F);
-        return MG_OK;
-    }
-    if (!F->v64_graph) {
-        std::vector<std::pair<double *, double *>> before;
+    std::vector<std::pair<double *, double *>> before;
+    if (!F->v64_rec.exec)
         for (const DevLevel &d : F->L) before.emplace_back(d.u64, d.u64b);
-        cudaGraph_t graph = nullptr;
-        cudaError_t e = F->cap_st ? cudaSuccess : cudaStreamCreateWithFlags(&F->cap_st, cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaStreamBeginCapture(F->cap_st, cudaStreamCaptureModeThreadLocal);
-        if (e == cudaSuccess) {
-            cudaStream_t own = F->st;
-            F->st = F->cap_st;
-            vcycle64(F);
-            F->st = own;
-            e = cudaStreamEndCapture(F->cap_st, &graph);
-        }
+    return replay(F, F->v64_rec, [&] { vcycle64(F); }, [&] {
         bool same = true;  // nothing ran during the recording: the iterate is still where it was
         for (size_t i = 0; i < F->L.size(); ++i) {
             same = same && F->L[i].u64 == before[i].first;
             F->L[i].u64 = before[i].first;
             F->L[i].u64b = before[i].second;
         }
-        if (e == cudaSuccess && graph && same) e = cudaGraphInstantiate(&F->v64_graph, graph, 0);
-        if (graph) cudaGraphDestroy(graph);
-        if (e != cudaSuccess || !same || !F->v64_graph) {
-            F->v64_graph = nullptr;
-            F->v64_nograph = true;
-            cudaGetLastError();
-            vcycle64(F);
-            return MG_OK;
-        }
-    }
-    MG_CUDA(cudaGraphLaunch(F->v64_graph, F->st));
-    return MG_OK;
+        return same;
+    });
 }
 
 // The FP32 correction on level 0 either was just zeroed with its face ghosts (k_residual_norm) or ends a previous
@@ -1145,8 +1079,9 @@ mg_status enqueue_update_mixed(mg_forest *F) {
     return MG_OK;
 }
 
+// `cycles` FP32 V-cycles, each the recorded one (mg_set_smoother_shape and mg_set_tail drop it), and the update.
 mg_status finish_mixed_cycle(mg_forest *F, int cycles) {
-    for (int i = 0; i < cycles; ++i) vcycle32(F);
+    for (int i = 0; i < cycles; ++i) MG_TRY(replay(F, F->v32_rec, [&] { vcycle32(F); }));
     return enqueue_update_mixed(F);
 }
 
@@ -1176,7 +1111,11 @@ mg_status ensure_fp64_coefficients(mg_forest *F) {
     return MG_OK;
 }
 
-mg_status enqueue_fp32_step(mg_forest *F, int cycles) { return finish_mixed_cycle(F, cycles); }
+// For a batch, which records the steps of all its forests in one graph.
+mg_status enqueue_fp32_step(mg_forest *F, int cycles) {
+    for (int i = 0; i < cycles; ++i) vcycle32(F);
+    return enqueue_update_mixed(F);
+}
 
 mg_status check_ready(mg_forest *F) {
     if (!F) {
@@ -1639,8 +1578,7 @@ void mg_forest_destroy(mg_forest *F) {
     if (F->pscale_h) cudaFreeHost(F->pscale_h);
     if (F->pinv_h) cudaFreeHost(F->pinv_h);
     if (F->pdone_h) cudaFreeHost(F->pdone_h);
-    if (F->coarse_graph) cudaGraphExecDestroy(F->coarse_graph);
-    if (F->v64_graph) cudaGraphExecDestroy(F->v64_graph);
+    for (Replay *r : {&F->coarse_rec, &F->v64_rec, &F->v32_rec, &F->vT_rec}) r->drop();
     if (F->cap_st) cudaStreamDestroy(F->cap_st);
     if (F->hst_ev) cudaEventDestroy(F->hst_ev);
     delete F;
@@ -1730,6 +1668,15 @@ mg_status mg_exchange_level(mg_forest *F, int32_t level, const double *u_dev, do
     return MG_OK;
 }
 
+// The recorded FP32 cycles hold the launch shapes and the tail they were recorded with.
+static mg_status drop_cycles32(mg_forest *F) {
+    if (!F->v32_rec.exec && !F->vT_rec.exec) return MG_OK;
+    MG_CUDA(cudaStreamSynchronize(F->st));
+    F->v32_rec.drop();
+    F->vT_rec.drop();
+    return MG_OK;
+}
+
 mg_status mg_get_smoother_shape(const mg_forest *F, int32_t level, int32_t *shape) {
     if (!F || level < 0 || level >= static_cast<int32_t>(F->L.size()) || !shape) {
         set_error("null forest or output, or level out of range");
@@ -1757,7 +1704,7 @@ mg_status mg_set_smoother_shape(mg_forest *F, int32_t level, const int32_t *shap
         return MG_ERR_INVALID_ARG;
     }
     d.s32 = sh;
-    return MG_OK;
+    return drop_cycles32(F);
 }
 
 mg_status mg_set_boundary(mg_forest *F, const double *g_dev) {
@@ -1765,10 +1712,9 @@ mg_status mg_set_boundary(mg_forest *F, const double *g_dev) {
         set_error("null forest");
         return MG_ERR_INVALID_ARG;
     }
-    if (F->v64_graph) {  // the recorded FP64 cycle holds the boundary-data pointer it was recorded with
+    if (F->v64_rec.exec) {  // the recorded FP64 cycle holds the boundary-data pointer it was recorded with
         MG_CUDA(cudaStreamSynchronize(F->st));
-        cudaGraphExecDestroy(F->v64_graph);
-        F->v64_graph = nullptr;
+        F->v64_rec.drop();
     }
     DevLevel &d = F->L[0];
     if (!g_dev) {
@@ -1817,6 +1763,7 @@ mg_status mg_set_tail(mg_forest *F, int32_t level) {
         set_error("null forest");
         return MG_ERR_INVALID_ARG;
     }
+    MG_TRY(drop_cycles32(F));
     if (level < 0) {
         F->tail_level = -1;
         F->tail_tuned = true;
