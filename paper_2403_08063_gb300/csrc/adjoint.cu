@@ -134,6 +134,7 @@ template <typename T, int MODE, bool FLUX, bool GHOSTS>
 __global__ void __launch_bounds__(kThreads)
     k_adj_iface(T *__restrict__ y, Coef cf, const T *__restrict__ ih2, const FaceItem *__restrict__ items, LevelGeom g,
                 T *__restrict__ old, T *__restrict__ old_c, Target<T> to, T sgn) {
+    pdl_enter(y, old, old_c, to.pool, to.user);
     extern __shared__ __align__(16) unsigned char adj_smem[];
     const int strips = iface_strips(g.n), item = blockIdx.x / strips;
     const FaceItem F = items[item];
@@ -149,15 +150,13 @@ __global__ void __launch_bounds__(kThreads)
         const int64_t g0c = fidx<T>(g, F.nbr, F.axis, 1 - F.side, 0, yc, zc);
         const int64_t g0 = fidx<T>(g, F.blk, F.axis, F.side, 0, i1, i2);
         const int64_t g1 = fidx<T>(g, F.blk, F.axis, F.side, 1, i1, i2);
-        // loads before stores, which the compiler could not move them across
         const T yC = y[gC], through = FLUX ? T(0.125) * yC : T(0);
-        T a = T(0);
-        if (adds) a = -scaled_face<T, MODE>(cf, ih2, F.blk, g0, g1, F.axis, F.side) * (y[g1] - through);
         if (GHOSTS) {
             y[g0] = through;
             if ((q & 3) == 0) y[g0c] = FLUX ? yC : T(0);
         }
         if (!adds) continue;
+        T a = -scaled_face<T, MODE>(cf, ih2, F.blk, g0, g1, F.axis, F.side) * (y[g1] - through);
         if (old) {
             T *keep = old + (static_cast<int64_t>(item) * n + i2) * n + i1;
             const T before = *keep;
@@ -209,6 +208,7 @@ template <typename T, int MODE>
 __global__ void k_adj_residual(const T *__restrict__ y, const T *f, Coef cf, const T *__restrict__ ih2, LevelGeom g,
                                const int32_t *__restrict__ nbr6, T *r, const double *__restrict__ vol,
                                double *__restrict__ part) {
+    pdl_enter(y, f, r);
     const int n = g.n;
     const int64_t total = static_cast<int64_t>(g.nb) << (3 * g.lg);
     double acc = 0.0;
@@ -256,6 +256,7 @@ template <int MODE, int LG>
 __global__ void __launch_bounds__(kThreads)
     k_adj_residual32(const float *__restrict__ y, const float *__restrict__ f, Coef cf, const float *__restrict__ ih2,
                      int64_t bs, int64_t pairs, const int32_t *__restrict__ nbr6, float *__restrict__ r) {
+    pdl_enter(y, f, r);
     constexpr int n = 1 << LG, NH = n / 2, P = n + 2, H = half_row(P), PL = P * H, HALF = P * PL;
     const int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
     if (t >= pairs) return;
@@ -357,6 +358,7 @@ __global__ void __launch_bounds__(kThreads)
 template <typename T>
 __global__ void k_prolong_T(const T *__restrict__ r, LevelGeom gf, T *__restrict__ fc, T *__restrict__ yc,
                             const XferItem *__restrict__ xf, LevelGeom gc) {
+    pdl_enter(r, fc, yc);
     const int nc = gc.n;
     const int64_t total = static_cast<int64_t>(gc.nb) << (3 * gc.lg);
     GRID_STRIDE(total) {
@@ -391,6 +393,7 @@ template <int LG>
 __global__ void __launch_bounds__(kThreads)
     k_prolong_T32(const float *__restrict__ r, int64_t bsf, float *__restrict__ fc, float *__restrict__ yc,
                   const XferItem *__restrict__ xf, int64_t total, int64_t bsc) {
+    pdl_enter(r, fc, yc);
     using Bx = Box32<LG>;
     constexpr int nc = (1 << LG) / 2, LC = LG - 1;
     const int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
@@ -417,6 +420,7 @@ __global__ void __launch_bounds__(kThreads)
 template <typename T>
 __global__ void k_prolong_T_scatter(const T *__restrict__ r, LevelGeom gf, T *__restrict__ Ec,
                                     const XferItem *__restrict__ xf, LevelGeom gc) {
+    pdl_enter(r, Ec);
     const int nc = gc.n;
     const int64_t total = static_cast<int64_t>(gc.nb) << (3 * gc.lg);
     GRID_STRIDE(total) {
@@ -459,6 +463,7 @@ __global__ void k_prolong_T_scatter(const T *__restrict__ r, LevelGeom gf, T *__
 // E^T of the faces filled from one source block: reflection (ghost = -u_i) and copy from the neighbour.
 template <typename T>
 __global__ void k_et_faces(T *__restrict__ G, const FaceItem *__restrict__ items, int nitems, LevelGeom g) {
+    pdl_enter(G);
     const int n = g.n, lg = g.lg;
     const int64_t total = static_cast<int64_t>(nitems) << (2 * lg);
     GRID_STRIDE(total) {
@@ -478,6 +483,7 @@ template <typename T, int MODE, bool FLUX, bool GATHER>
 __global__ void __launch_bounds__(kThreads)
     k_et_iface(T *__restrict__ fc, Coef cf, const FaceItem *__restrict__ items, LevelGeom g, const T *__restrict__ r,
                LevelGeom gf, const XferItem *__restrict__ xf) {
+    pdl_enter(fc, r);
     extern __shared__ __align__(16) unsigned char adj_smem[];
     const int strips = iface_strips(g.n), item = blockIdx.x / strips;
     const FaceItem F = items[item];
@@ -526,6 +532,7 @@ __global__ void __launch_bounds__(kThreads)
 template <typename T>
 __global__ void k_inject(T *__restrict__ yf, LevelGeom gf, const T *__restrict__ ec, const XferItem *__restrict__ xf,
                          LevelGeom gc) {
+    pdl_enter(yf, ec);
     const int nc = gc.n;
     const int64_t total = static_cast<int64_t>(gc.nb) << (3 * gc.lg);
     GRID_STRIDE(total) {
@@ -688,7 +695,8 @@ void with_mode(const mg_forest *F, const DevLevel &d, Fn &&fn) {
 template <typename T, class Fn, class... Args>
 void launch_iface(mg_forest *F, const DevLevel &d, Fn fn, Args... args) {
     const int n = d.g.n;
-    fn<<<d.nifaces * iface_strips(n), iface_threads(n), scatter_values(n) * sizeof(T), F->st>>>(args...);
+    launch_pdl(F->st, !F->batch_member, fn, d.nifaces * iface_strips(n), iface_threads(n),
+               scatter_values(n) * sizeof(T), args...);
 }
 
 // Transposed interface ghosts of y (ghosts) and sgn times the interface part of A^T y into `to` (see k_adj_iface).
@@ -722,8 +730,9 @@ template <typename T>
 void exchange_same(mg_forest *F, DevLevel &d, T *y) {
     if (!d.nsfaces) return;
     Prof p(F, P_ADJ, 1);
-    k_exchange_faces<T, false><<<grid_for(static_cast<int64_t>(d.nsfaces) << (2 * d.g.lg)), kThreads, 0, F->st>>>(
-        y, d.sfaces, d.nsfaces, d.g);
+    launch_pdl(F->st, !F->batch_member, k_exchange_faces<T, false>,
+               grid_for(static_cast<int64_t>(d.nsfaces) << (2 * d.g.lg)), kThreads, 0, y,
+               d.sfaces, d.nsfaces, d.g, Skip{}, 0, nullptr);
 }
 
 // Red-black iterations on A^T with the colours in reverse order.  `stale`: y changed since the last interface exchange.
@@ -739,7 +748,8 @@ void smooth_T(mg_forest *F, int l, int iters, bool &stale) {
             } else {
                 Prof p(F, P_ADJ, 1);
                 auto *fn = F->cfg.coeff ? k_smooth<double, 1> : k_smooth<double, 0>;
-                fn<<<grid_for(d.cells() / 2), kThreads, 0, F->st>>>(a.y, a.f, d.c64(), d.h2_64, d.g, colour, d.nbr6, Skip{},
+                launch_pdl(F->st, !F->batch_member, fn, grid_for(d.cells() / 2), kThreads, 0, a.y, a.f, d.c64(),
+                           d.h2_64, d.g, colour, d.nbr6, Skip{},
                                                                     nullptr);
             }
             stale = true;
@@ -754,7 +764,8 @@ void launch_residual32(mg_forest *F, DevLevel &d, float *r) {
             k_adj_residual32<M, 2>, k_adj_residual32<M, 3>, k_adj_residual32<M, 4>,
             k_adj_residual32<M, 5>, k_adj_residual32<M, 6>, k_adj_residual32<M, 7>};
         const int64_t pairs = d.cells() / 2;
-        fns[d.g.lg - 2]<<<static_cast<unsigned>((pairs + kThreads - 1) / kThreads), kThreads, 0, F->st>>>(
+        launch_pdl(F->st, !F->batch_member, fns[d.g.lg - 2],
+                   static_cast<unsigned>((pairs + kThreads - 1) / kThreads), kThreads, 0,
             d.u32, d.f32, d.c32(), d.ih2_32, d.g.bs, pairs, d.nbr6, r);
     });
 }
@@ -767,8 +778,9 @@ void vcycle_T(mg_forest *F, int l) {
     const int last = static_cast<int>(F->L.size()) - 1;
     if (l == last) {
         Prof p(F, P_ADJ, 1);
-        k_coarse_solve<T><<<(F->Nc * 32 + kThreads - 1) / kThreads, kThreads, 0, F->st>>>(
-            a.y, a.f, F->AinvT, sizeof(T) == 4 ? F->cmap32 : F->cmap, F->uprob, F->ustart, F->moff, F->Nc);
+        launch_pdl(F->st, !F->batch_member, k_coarse_solve<T>, (F->Nc * 32 + kThreads - 1) / kThreads, kThreads, 0,
+                   a.y, a.f, F->AinvT,
+                   sizeof(T) == 4 ? F->cmap32 : F->cmap, F->uprob, F->ustart, F->moff, F->Nc, nullptr);
         return;
     }
     const int64_t n2 = static_cast<int64_t>(d.g.n) * d.g.n;
@@ -791,7 +803,8 @@ void vcycle_T(mg_forest *F, int l) {
             launch_residual32(F, d, reinterpret_cast<float *>(a.r));
         else
             with_mode<T>(F, d, [&](auto m) {
-                k_adj_residual<T, decltype(m)::value><<<grid_for(d.cells()), kThreads, 0, F->st>>>(
+                launch_pdl(F->st, !F->batch_member, k_adj_residual<T, decltype(m)::value>, grid_for(d.cells()),
+                           kThreads, 0,
                     a.y, a.f, acoef<T>(d), aih2<T>(d), d.g, d.nbr6, a.r, nullptr, nullptr);
             });
     }
@@ -800,18 +813,22 @@ void vcycle_T(mg_forest *F, int l) {
         Prof p(F, P_ADJ, 1);
         static constexpr decltype(&k_prolong_T32<3>) fns[5] = {k_prolong_T32<3>, k_prolong_T32<4>, k_prolong_T32<5>,
                                                                k_prolong_T32<6>, k_prolong_T32<7>};
-        fns[d.g.lg - 3]<<<static_cast<unsigned>((c.cells() + kThreads - 1) / kThreads), kThreads, 0, F->st>>>(
+        launch_pdl(F->st, !F->batch_member, fns[d.g.lg - 3],
+                   static_cast<unsigned>((c.cells() + kThreads - 1) / kThreads), kThreads, 0,
             reinterpret_cast<float *>(a.r), d.g.bs, c.f32, c.u32, d.xfer, c.cells(), c.g.bs);
     } else if (gather) {
         Prof p(F, P_ADJ, 1);
-        k_prolong_T<T><<<grid_for(c.cells()), kThreads, 0, F->st>>>(a.r, d.g, ac.f, ac.y, d.xfer, c.g);
+        launch_pdl(F->st, !F->batch_member, k_prolong_T<T>, grid_for(c.cells()), kThreads, 0, a.r, d.g, ac.f, ac.y,
+                   d.xfer, c.g);
     } else {
         Prof p(F, P_ADJ, 2);
         cudaMemsetAsync(ac.f, 0, c.pool_elems() * sizeof(T), F->st);
         cudaMemsetAsync(ac.y, 0, c.pool_elems() * sizeof(T), F->st);
-        k_prolong_T_scatter<T><<<grid_for(c.cells()), kThreads, 0, F->st>>>(a.r, d.g, ac.f, d.xfer, c.g);
+        launch_pdl(F->st, !F->batch_member, k_prolong_T_scatter<T>, grid_for(c.cells()), kThreads, 0, a.r, d.g, ac.f,
+                   d.xfer, c.g);
         if (c.nsfaces)
-            k_et_faces<T><<<grid_for(static_cast<int64_t>(c.nsfaces) << (2 * c.g.lg)), kThreads, 0, F->st>>>(
+            launch_pdl(F->st, !F->batch_member, k_et_faces<T>,
+                       grid_for(static_cast<int64_t>(c.nsfaces) << (2 * c.g.lg)), kThreads, 0,
                 ac.f, c.sfaces, c.nsfaces, c.g);
     }
     et_iface<T>(F, d, c, ac.f, a.r, gather);
@@ -820,7 +837,8 @@ void vcycle_T(mg_forest *F, int l) {
     {
         Prof p(F, P_ADJ, 1);
         if constexpr (sizeof(T) == 4) through = inject32(F, d, c);
-        if (!through) k_inject<T><<<grid_for(c.cells()), kThreads, 0, F->st>>>(a.y, d.g, ac.y, d.xfer, c.g);
+        if (!through) launch_pdl(F->st, !F->batch_member, k_inject<T>, grid_for(c.cells()), kThreads, 0, a.y, d.g,
+                                 ac.y, d.xfer, c.g);
     }
     if (!through) exchange_same<T>(F, d, a.y);
     stale = true;

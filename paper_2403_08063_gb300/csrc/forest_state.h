@@ -29,6 +29,23 @@ namespace octmg {
         if (s_ != MG_OK) return s_;       \
     } while (0)
 
+// A kernel that begins with pdl_enter, launched so that its start-up overlaps the end of the kernel before it in the stream
+// (programmatic dependent launch; captured as such in the recorded cycles).
+template <class... P, class... A>
+void launch_pdl(cudaStream_t st, bool overlap, void (*fn)(P...), unsigned grid, unsigned threads, size_t smem, A &&...args) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = overlap && grid <= kPdlGrid ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
+}
+
 constexpr int kMaxGrid = 152 * 32;  // grid-stride loops: at most 32 CTAs of 256 threads per SM
 
 inline int grid_for(int64_t total) {
@@ -110,7 +127,7 @@ struct TailArgs {
     const int64_t *ustart, *moff;
     int Nc;
     const uint8_t *done;
-    unsigned *bar;  // [count, generation]
+    unsigned *bar;  // arrivals
     int *err;
 };
 
@@ -195,7 +212,7 @@ struct mg_forest {
     octmg::TailLevel *tail_L = nullptr;  // device copy of the level descriptors
     octmg::TailPhase *tail_ph = nullptr;  // device phase list
     int tail_nph = 0, tail_for = -2;      // phases recorded, and for which tail level
-    unsigned *tail_bar = nullptr;          // grid-barrier counter and generation
+    unsigned *tail_bar = nullptr;          // grid-barrier arrivals
     std::vector<octmg::TailPhase> tail_ph_host;  // host copy of the phase list (merged into a batch's joint tail)
 };
 

@@ -108,14 +108,15 @@ void exchange(mg_forest *F, DevLevel &d, T *u, bool interface_only = false, bool
         const size_t smem = nif ? (n / 2 / strips + 2) * (n / 2 + 2) * sizeof(T) : 0;
         const int grid = nif * strips + (nsf ? grid_for(static_cast<int64_t>(nsf) * n * n) : 0);
         auto *fn = F->cfg.interface_flux ? k_exchange<T, MODE, true> : k_exchange<T, MODE, false>;
-        fn<<<grid, threads, smem, F->st>>>(u, coef_of<T>(d), d.ifaces, nif, d.sfaces, nsf, d.g,
+        launch_pdl(F->st, !F->batch_member, fn, grid, threads, smem, u, coef_of<T>(d), d.ifaces, nif, d.sfaces, nsf,
+                   d.g,
                                                                   skip_of(F, d), F->cfg.c2f_variant, gb);
         return;
     }
     const FaceItem *items = interface_only ? d.ifaces : d.faces;
     const int nitems = interface_only ? d.nifaces : d.nfaces;
-    k_exchange_faces<T, false><<<grid_for(static_cast<int64_t>(nitems) * n * n), kThreads, 0, F->st>>>(
-        u, items, nitems, d.g, skip_of(F, d), F->cfg.c2f_variant, gb);
+    launch_pdl(F->st, !F->batch_member, k_exchange_faces<T, false>, grid_for(static_cast<int64_t>(nitems) * n * n),
+               kThreads, 0, u, items, nitems, d.g, skip_of(F, d), F->cfg.c2f_variant, gb);
     if (d.nsegs) {
         const int64_t tot = static_cast<int64_t>(d.nsegs) * (n / 2) * (n / 2);
         auto *fn = F->cfg.interface_flux ? k_exchange_segs<T, MODE, true> : k_exchange_segs<T, MODE, false>;
@@ -217,7 +218,8 @@ void launch_smooth32(mg_forest *F, DevLevel &d, int colour, const Shape &sh, cud
                                  200 * 1024);
         });
         const int64_t grid = static_cast<int64_t>(d.g.nb) * (n / TY) * (n / TZ);
-        fn<<<static_cast<unsigned>(grid), (n / 2) * TY / R + 32, smem, st>>>(d.u32, d.f32, d.kap, d.h2_32, d.g.bs, colour,
+        launch_pdl(st, !F->batch_member, fn, static_cast<unsigned>(grid), (n / 2) * TY / R + 32, smem, d.u32, d.f32,
+                   d.kap, d.h2_32, d.g.bs, colour,
                                                                          d.nbr6, TY, TZ, D, F->kerr, skip_of(F, d),
                                                                          d.ax32, d.ay32, d.az32);
         return;
@@ -225,8 +227,9 @@ void launch_smooth32(mg_forest *F, DevLevel &d, int colour, const Shape &sh, cud
     const int zc = sh[0] == 1 ? sh[1] : 1, threads = sh[0] == 1 ? sh[2] : kThreads;
     const int64_t work = (d.cells() / 2) >> ridx(zc);  // one thread per column of zc cells
     const int64_t grid = (work + threads - 1) / threads;
-    kSmooth32[mode_index(mode)][d.g.lg - 2][ridx(zc)]<<<static_cast<unsigned>(grid), threads, 0, st>>>(
-        d.u32, d.f32, d.kap, d.h2_32, work, d.g.bs, colour, d.nbr6, skip_of(F, d), d.ax32, d.ay32, d.az32);
+    launch_pdl(st, !F->batch_member, kSmooth32[mode_index(mode)][d.g.lg - 2][ridx(zc)], static_cast<unsigned>(grid),
+               threads, 0, d.u32, d.f32, d.kap, d.h2_32, work, d.g.bs, colour, d.nbr6, skip_of(F, d), d.ax32, d.ay32,
+               d.az32);
 }
 
 // Reads and clears the device error word of bounded waits.
@@ -365,15 +368,16 @@ void launch_residual_restrict32(mg_forest *F, DevLevel &d, DevLevel &c) {
                                  200 * 1024);
         });
         const int64_t grid = static_cast<int64_t>(c.g.nb) * (n / TY) * (n / TZ);
-        fn<<<static_cast<unsigned>(grid), (n / 2) * (TY / 2) + 32, restrict32t_smem(d.g.lg, mode, TY, TZ, D), F->st>>>(
+        launch_pdl(F->st, !F->batch_member, fn, static_cast<unsigned>(grid), (n / 2) * (TY / 2) + 32,
+                   restrict32t_smem(d.g.lg, mode, TY, TZ, D), 
             d.u32, d.f32, d.kap, d.ih2_32, d.g.bs, c.f32, c.u32, d.xfer, c.g.nb, c.g.bs, skip_of(F, c), d.ax32, d.ay32,
             d.az32, TY, TZ, D, F->kerr);
         return;
     }
     // one coarse cell per thread (no grid-stride loop): its load chain xf -> fine block -> 64 loads is latency-bound
     const auto grid = static_cast<unsigned>((c.cells() + kThreads - 1) / kThreads);
-    kRestrict32[mode_index(mode32(F, d))][d.g.lg - 3]<<<grid, kThreads, 0, F->st>>>(
-        d.u32, d.f32, d.kap, d.ih2_32, d.g.bs, c.f32, c.u32, d.xfer, c.g.nb, c.g.bs, skip_of(F, c), d.ax32, d.ay32,
+    launch_pdl(F->st, !F->batch_member, kRestrict32[mode_index(mode32(F, d))][d.g.lg - 3], grid, kThreads, 0, d.u32,
+               d.f32, d.kap, d.ih2_32, d.g.bs, c.f32, c.u32, d.xfer, c.g.nb, c.g.bs, skip_of(F, c), d.ax32, d.ay32,
         d.az32);
 }
 
@@ -381,11 +385,13 @@ void launch_prolong32(mg_forest *F, DevLevel &d, DevLevel &c, bool inject = fals
     if (d.g.lg >= 5) {
         const auto grid = static_cast<unsigned>((c.cells() / kProlongZC + kThreads - 1) / kThreads);
         const Prolong32Fn fn = (inject ? kInject32z : kProlong32z)[d.g.lg - 5];
-        fn<<<grid, kThreads, 0, F->st>>>(d.u32, d.g.bs, c.u32, d.xfer, c.g.nb, c.g.bs, d.nbr6, skip_of(F, c));
+        launch_pdl(F->st, !F->batch_member, fn, grid, kThreads, 0, d.u32, d.g.bs, c.u32, d.xfer, c.g.nb, c.g.bs,
+                   d.nbr6, skip_of(F, c));
         return;
     }
     const Prolong32Fn fn = (inject ? kInject32 : kProlong32)[d.g.lg - 3];
-    fn<<<grid_for(c.cells()), kThreads, 0, F->st>>>(d.u32, d.g.bs, c.u32, d.xfer, c.g.nb, c.g.bs, d.nbr6, skip_of(F, c));
+    launch_pdl(F->st, !F->batch_member, fn, grid_for(c.cells()), kThreads, 0, d.u32, d.g.bs, c.u32, d.xfer, c.g.nb,
+               c.g.bs, d.nbr6, skip_of(F, c));
 }
 
 bool inject32(mg_forest *F, DevLevel &d, DevLevel &c) {
@@ -406,7 +412,8 @@ void smooth(mg_forest *F, DevLevel &d, int colour) {
     const T *gb = nullptr;
     if constexpr (sizeof(T) == 8)
         if (&d == &F->L[0]) gb = F->gb;
-    k_smooth<T, MODE><<<grid_for(d.cells() / 2), kThreads, 0, F->st>>>(ufield<T>(d), ffield<T>(d), coef_of<T>(d),
+    launch_pdl(F->st, !F->batch_member, k_smooth<T, MODE>, grid_for(d.cells() / 2), kThreads, 0, ufield<T>(d),
+               ffield<T>(d), coef_of<T>(d),
                                                                        h2_of<T>(d), d.g, colour, d.nbr6, skip_of(F, d),
                                                                        gb);
 }
@@ -512,7 +519,8 @@ struct LaunchExec {
         if constexpr (sizeof(T) == 8) {
             DevLevel &d = F->L[l];
             Prof p(F, prof ? cat_of<T>(l == 0 ? P_SMOOTH64_L0 : P_SMOOTH64) : -1, 1);
-            k_jacobi64<MODE><<<grid_for(d.cells()), kThreads, 0, F->st>>>(d.u64, d.u64b, d.f64, d.c64(), d.h2_64, d.g,
+            launch_pdl(F->st, !F->batch_member, k_jacobi64<MODE>, grid_for(d.cells()), kThreads, 0, d.u64, d.u64b,
+                       d.f64, d.c64(), d.h2_64, d.g,
                                                                           F->omega, skip_of(F, d));
             std::swap(d.u64, d.u64b);  // the new iterate; its ghosts are refreshed by the next exchange
         }
@@ -520,7 +528,6 @@ struct LaunchExec {
     void coarse(int l) {
         DevLevel &d = F->L[l];
         if (F->cfg.coarse_iters > 0) {  // damped Jacobi sweeps from zero (the paper's coarsest solver)
-            const DevLevel &d = F->L[l];
             Prof p(F, cat_of<T>(P_COARSE64), F->cfg.coarse_iters * (1 + (d.nfaces > 0)));
             for (int it = 0; it < F->cfg.coarse_iters; ++it) {
                 octmg::exchange<T, MODE>(F, F->L[l], ufield<T>(F->L[l]), false, false);
@@ -529,9 +536,10 @@ struct LaunchExec {
             return;
         }
         Prof p(F, cat_of<T>(P_COARSE64), 1);
-        k_coarse_solve<T><<<(F->Nc * 32 + kThreads - 1) / kThreads, kThreads, 0, F->st>>>(
-            ufield<T>(d), ffield<T>(d), F->Ainv, sizeof(T) == 4 ? F->cmap32 : F->cmap, F->uprob, F->ustart, F->moff,
-            F->Nc, F->pdone);
+        launch_pdl(F->st, !F->batch_member, k_coarse_solve<T>, (F->Nc * 32 + kThreads - 1) / kThreads, kThreads, 0,
+                   ufield<T>(d), ffield<T>(d), F->Ainv, sizeof(T) == 4 ? F->cmap32 : F->cmap, F->uprob, F->ustart,
+                   F->moff,
+            F->Nc, F->np > 1 ? F->pdone : nullptr);
     }
     void restrict_to(int l, bool fast) {
         DevLevel &d = F->L[l], &c = F->L[l + 1];
@@ -539,11 +547,12 @@ struct LaunchExec {
         if (fast)
             launch_residual_restrict32(F, d, c);
         else if (sizeof(T) == 4 && d.face32)
-            k_residual_restrict<float, 3><<<grid_for(c.cells()), kThreads, 0, F->st>>>(
-                d.u32, d.f32, d.c32(), d.ih2_32, d.g, c.f32, c.u32, d.xfer, c.g, skip_of(F, c));
+            launch_pdl(F->st, !F->batch_member, k_residual_restrict<float, 3>, grid_for(c.cells()), kThreads, 0,
+                       d.u32, d.f32, d.c32(), d.ih2_32, d.g, c.f32, c.u32, d.xfer, c.g, skip_of(F, c));
         else
-            k_residual_restrict<T, MODE><<<grid_for(c.cells()), kThreads, 0, F->st>>>(
-                ufield<T>(d), ffield<T>(d), coef_of<T>(d), ih2_of<T>(d), d.g, ffield<T>(c), ufield<T>(c), d.xfer, c.g,
+            launch_pdl(F->st, !F->batch_member, k_residual_restrict<T, MODE>, grid_for(c.cells()), kThreads, 0,
+                       ufield<T>(d), ffield<T>(d), coef_of<T>(d), ih2_of<T>(d), d.g, ffield<T>(c), ufield<T>(c),
+                       d.xfer, c.g,
                 skip_of(F, c));
     }
     void prolong_from(int l, bool fast) {
@@ -559,7 +568,8 @@ struct LaunchExec {
         if (fast)
             launch_prolong32(F, d, c);
         else
-            k_prolong<T><<<grid_for(c.cells()), kThreads, 0, F->st>>>(ufield<T>(d), d.g, ufield<T>(c), d.xfer, c.g,
+            launch_pdl(F->st, !F->batch_member, k_prolong<T>, grid_for(c.cells()), kThreads, 0, ufield<T>(d), d.g,
+                       ufield<T>(c), d.xfer, c.g,
                                                                       skip_of(F, c));
     }
 };
@@ -982,8 +992,8 @@ void vcycle32_part(mg_forest *F, int part) {
 }
 
 // Picks the persistent tail's level: every level l whose own and deeper levels have at most 2^20 cells (and
-// specialised smoothers) is a candidate; each candidate and "off" is timed over five FP32 V-cycles (after two
-// untimed ones) on the FP32 pools, which are dead between solves, and the fastest is kept.  Skipped (off) while the
+// specialised smoothers) is a candidate; each candidate and "off" is timed over five recorded FP32 V-cycles (after
+// three untimed ones) on the FP32 pools, which are dead between solves, and the fastest is kept.  Skipped (off) while the
 // stream is being captured.
 mg_status tune_tail(mg_forest *F) {
     if (F->tail_tuned || F->cfg.precision != 1) return MG_OK;
@@ -1008,11 +1018,15 @@ mg_status tune_tail(mg_forest *F) {
     for (int lt : cand) {
         if (lt >= 0) MG_TRY(record_tail(F, lt));
         F->tail_level = lt;
-        for (int w = 0; w < 2; ++w) vcycle32(F);
+        Replay rec;  // as a solve runs it
+        mg_status st = MG_OK;
+        for (int w = 0; w < 3 && st == MG_OK; ++w) st = replay(F, rec, [&] { vcycle32(F); });
         MG_CUDA(cudaEventRecord(e0, F->st));
-        for (int w = 0; w < 5; ++w) vcycle32(F);
+        for (int w = 0; w < 5 && st == MG_OK; ++w) st = replay(F, rec, [&] { vcycle32(F); });
         MG_CUDA(cudaEventRecord(e1, F->st));
         MG_CUDA(cudaEventSynchronize(e1));
+        rec.drop();
+        MG_TRY(st);
         float ms = 0.0f;
         MG_CUDA(cudaEventElapsedTime(&ms, e0, e1));
         if (lt == -1 || ms < best) {
