@@ -321,6 +321,9 @@ octmg::TailArgs tail_args(mg_forest *F);  // tail.cu: the forest's recorded tail
 // groups' tail arguments (device), with a grid of at most `need` CTAs
 mg_status launch_batch_tail32(mg_forest *const *groups, const octmg::TailArgs *args, const octmg::BatchEntry *entries,
                               int ne, unsigned *bar, int64_t need);
+// coarse_jacobi.cu: the coarsest level's Jacobi sweeps in one launch, where it applies
+bool coarse_jacobi_fits(const mg_forest *F, const DevLevel &d);
+void launch_coarse_jacobi(mg_forest *F, DevLevel &d, int iters);
 // gauss_jordan.cu: inverses of the coarsest operators (input buffer, panel width, launches)
 double *gj_input(mg_forest *F, int maxN);
 int gj_width(int maxN);

@@ -528,6 +528,11 @@ struct LaunchExec {
     void coarse(int l) {
         DevLevel &d = F->L[l];
         if (F->cfg.coarse_iters > 0) {  // damped Jacobi sweeps from zero (the paper's coarsest solver)
+            if (coarse_jacobi_fits(F, d)) {
+                Prof p(F, P_COARSE64, 1);
+                launch_coarse_jacobi(F, d, F->cfg.coarse_iters);
+                return;
+            }
             Prof p(F, cat_of<T>(P_COARSE64), F->cfg.coarse_iters * (1 + (d.nfaces > 0)));
             for (int it = 0; it < F->cfg.coarse_iters; ++it) {
                 octmg::exchange<T, MODE>(F, F->L[l], ufield<T>(F->L[l]), false, false);
