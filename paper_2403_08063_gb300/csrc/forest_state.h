@@ -179,8 +179,7 @@ struct mg_forest {
     octmg::Replay coarse_rec, v64_rec, v32_rec, vT_rec;
     double *hst_f = nullptr, *hst_k = nullptr, *hst_u = nullptr;  // mg_solve_host staging buffers (user layout)
     cudaEvent_t hst_ev = nullptr;              // orders the staging copies against the forest's stream
-    int8_t *pcol = nullptr;                    // colour probe (interface-free coarsest level): colour per unknown
-    int32_t *pnbu = nullptr;                   // and the unknowns of its 7-point neighbourhood (-1: outside)
+    int32_t *pnbu = nullptr;                   // interface-free coarsest level: the unknowns of each 7-point row (-1: outside)
     // several independent problems: per-problem reductions, scales, block-diagonal coarsest inverse
     int np = 1;
     int32_t *pstart = nullptr, *pblk = nullptr;  // level-0 blocks of problem p: pblk[pstart[p] .. pstart[p+1])

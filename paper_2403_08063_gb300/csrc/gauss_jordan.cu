@@ -10,11 +10,10 @@
 // with src the row exchanges of the panel.  After all panels the matrix holds (P A)^-1 = A^-1 P^T for the exchanges P,
 // and org[r] the row of A that ended in row r, so A^-1[:, org r] is column r.
 //
-// What bounds it: the chain of N pivot searches (2.2 us each with 512 unknowns, 3.3 us with 1728: one cluster barrier, one
+// What bounds it: the chain of N pivot searches (2.3 us each with 512 unknowns, 2.9 us with 1728: one cluster barrier, one
 // block barrier, a division, and the panel's update on the 2 FP64 FMA per clock of each of the cluster's SMs), then the
-// FP64 rate in the update (N^3 FMA in all: with 1728 unknowns 83.5 us per panel, 0.57 T FMA/s of the 0.63 measured).
-// Elimination of one column per step with two launches per column (every element rewritten each time) took 4.85 ms for
-// 512 unknowns and 58 ms for 1728 (three root blocks per axis); this takes 1.5 ms and 14.8 ms.
+// FP64 rate in the update.  Elimination of one column per step with two launches per column (every element rewritten each
+// time) took 4.85 ms for 512 unknowns and 58 ms for 1728 (three root blocks per axis); this takes 1.5 ms and 10.1 ms.
 #include <cooperative_groups.h>
 
 #include "forest_state.h"
@@ -41,7 +40,7 @@ struct GjRow {
     int32_t id;
 };
 
-// Rows of a problem held by one CTA, and its dynamic shared memory: rows x W doubles (rounded up to whole passes of the
+// Rows of a problem held by one CTA (r % cluster size == rank), and its dynamic shared memory: rows x W doubles (rounded up to whole passes of the
 // CTA) and the rows' origins.
 __host__ __device__ constexpr int gj_rows(int N) { return (N + kGjCluster - 1) / kGjCluster; }
 __host__ __device__ constexpr int64_t gj_panel_elems(int N, int W) {
@@ -49,8 +48,14 @@ __host__ __device__ constexpr int64_t gj_panel_elems(int N, int W) {
 }
 constexpr int64_t gj_smem(int N, int W) { return gj_panel_elems(N, W) * 8 + static_cast<int64_t>(gj_rows(N)) * 4; }
 
-// Eliminates panel columns c0 .. c0 + W - 1 of every problem with more than c0 unknowns, one cluster per problem, rows
-// dealt out in contiguous chunks.  Per column one cluster barrier: before it each CTA sends the others its best pivot
+// The key of a pivot candidate: its magnitude bits + 1, or 0 for NaN.
+__device__ __forceinline__ uint64_t a_key(const double *a, int i) {
+    const uint64_t bits = static_cast<uint64_t>(__double_as_longlong(a[i])) & ~(1ull << 63);
+    return bits <= 0x7ff0000000000000ull ? bits + 1 : 0;
+}
+
+// Eliminates panel columns c0 .. c0 + W - 1 of every problem with more than c0 unknowns, one cluster per problem, row r in
+// CTA r % 8.  Per column one cluster barrier: before it each CTA sends the others its best pivot
 // candidate with the whole panel row and the reciprocal, and the owner of the diagonal row sends that one; after it every
 // CTA picks the same winner (largest magnitude, lowest row on ties) and updates its rows.  Messages alternate between two
 // buffers: a CTA that writes a buffer again has passed a barrier that every reader of it reached afterwards.  A thread
@@ -63,42 +68,50 @@ __global__ void __cluster_dims__(kGjCluster, 1, 1) __launch_bounds__(kGjThreads)
     extern __shared__ __align__(16) unsigned char gj_raw[];
     __shared__ GjCand<W> cand[2][kGjCluster];
     __shared__ GjRow<W> diag[2];
+    __shared__ int act;
     const cg::cluster_group cluster = cg::this_cluster();
     const int p = blockIdx.x / kGjCluster, rank = static_cast<int>(cluster.block_rank());
     const int N = static_cast<int>(ustart[p + 1] - ustart[p]);
     if (c0 >= N) return;  // uniform over the cluster, before any barrier
-    const int wn = min(W, N - c0), per = gj_rows(N), r0 = rank * per, nr = max(0, min(N - r0, per));
+    const int wn = min(W, N - c0), nr = (N - rank + kGjCluster - 1) / kGjCluster;  // row i of this CTA: rank + 8 i
+    const auto row_of = [&](int i) { return rank + i * kGjCluster; };
     double *a = reinterpret_cast<double *>(gj_raw);
     int32_t *id = reinterpret_cast<int32_t *>(a + gj_panel_elems(N, W));
     const int tid = threadIdx.x, lane = tid & 31, col = tid & (W - 1);
     const double *Ap = A + moff[p];
     for (int e = tid; e < gj_panel_elems(N, W); e += kGjThreads) {
         const int row = e / W;
-        a[e] = row < nr && col < wn ? Ap[static_cast<int64_t>(r0 + row) * N + c0 + col] : 0.0;
+        a[e] = row < nr && col < wn ? Ap[static_cast<int64_t>(row_of(row)) * N + c0 + col] : 0.0;
     }
-    for (int i = tid; i < nr; i += kGjThreads) id[i] = r0 + i;
+    for (int i = tid; i < nr; i += kGjThreads) id[i] = row_of(i);
+    // rows of zeros stay as they are (a zero multiplier, never a pivot): the panel ends at the last other row, or at its own
+    // rows, which receive the pivot rows
+    if (tid == 0) act = 0;
+    __syncthreads();
+    int last = (min(c0 + W, N) - 1 - rank + kGjCluster) / kGjCluster;  // local rows up to row c0 + wn - 1
+    for (int e = tid; e < nr * W; e += kGjThreads)
+        if (a[e] != 0.0) last = max(last, e / W + 1);
+    atomicMax(&act, last);
     cluster.sync();
+    const int na = act;
     for (int cc = 0; cc < wn; ++cc) {
         const int c = c0 + cc, buf = cc & 1;
         if (tid < 32) {
             uint64_t best = 0;
             int at = -1;
-            for (int i = max(0, c - r0) + lane; i < nr; i += 32) {
-                const uint64_t bits = static_cast<uint64_t>(__double_as_longlong(a[i * W + cc])) & ~(1ull << 63);
-                if (bits <= 0x7ff0000000000000ull && bits + 1 > best) {
-                    best = bits + 1;
+            for (int i = (max(0, c - rank) + kGjCluster - 1) / kGjCluster + lane; i < na; i += 32) {
+                const uint64_t key = a_key(a, i * W + cc);
+                if (key > best) {
+                    best = key;
                     at = i;
                 }
             }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const uint64_t ob = __shfl_xor_sync(0xffffffffu, best, o);
-                const int oa = __shfl_xor_sync(0xffffffffu, at, o);
-                if (ob > best || (ob == best && oa >= 0 && oa < at)) {
-                    best = ob;
-                    at = oa;
-                }
-            }
+            // the warp's largest, its upper word first, then the lower one, then the lowest row
+            const uint32_t hi = static_cast<uint32_t>(best >> 32), top = __reduce_max_sync(0xffffffffu, hi);
+            const uint32_t lo = __reduce_max_sync(0xffffffffu, hi == top ? static_cast<uint32_t>(best) : 0u);
+            best = static_cast<uint64_t>(top) << 32 | lo;
+            at = static_cast<int>(__reduce_min_sync(
+                0xffffffffu, hi == top && at >= 0 && a_key(a, at * W + cc) == best ? static_cast<uint32_t>(at) : 0x7fffffffu));
             const double rcp = best ? 1.0 / a[at * W + cc] : 0.0;
             for (int to = 0; to < kGjCluster; ++to) {
                 GjCand<W> *m = cluster.map_shared_rank(&cand[buf][rank], to);
@@ -106,22 +119,24 @@ __global__ void __cluster_dims__(kGjCluster, 1, 1) __launch_bounds__(kGjThreads)
                 if (lane == 0) {
                     m->key = best;
                     m->rcp = rcp;
-                    m->r = r0 + at;
+                    m->r = best ? row_of(at) : N;
                     m->id = best ? id[at] : -1;
                 }
             }
-        } else if (tid < 64 && c >= r0 && c < r0 + nr) {
+        } else if (tid < 64 && c % kGjCluster == rank) {
             for (int to = 0; to < kGjCluster; ++to) {
                 GjRow<W> *m = cluster.map_shared_rank(&diag[buf], to);
-                if (lane < W) m->row[lane] = a[(c - r0) * W + lane];
-                if (lane == 0) m->id = id[c - r0];
+                if (lane < W) m->row[lane] = a[c / kGjCluster * W + lane];
+                if (lane == 0) m->id = id[c / kGjCluster];
             }
         }
         cluster.sync();
         int win = 0;
 #pragma unroll
-        for (int i = 1; i < kGjCluster; ++i)
-            if (cand[buf][i].key > cand[buf][win].key) win = i;  // ranks hold ascending rows: the lowest row on ties
+        for (int i = 1; i < kGjCluster; ++i) {
+            const GjCand<W> &x = cand[buf][i], &y = cand[buf][win];
+            if (x.key > y.key || (x.key == y.key && x.r < y.r)) win = i;
+        }
         const GjCand<W> &w = cand[buf][win];
         // usable: found, not zero (key 1) and not infinite
         const bool ok = w.key > 1 && w.key < 0x7ff0000000000001ull;
@@ -131,27 +146,30 @@ __global__ void __cluster_dims__(kGjCluster, 1, 1) __launch_bounds__(kGjThreads)
         const double v = ok ? w.rcp : 1.0 / diag[buf].row[cc];
         const double pv = col == cc ? v : prow[col] * v;  // row c of the eliminated panel
         const double dc = diag[buf].row[col];
-        for (int base = 0; base < nr * W; base += kGjThreads) {
-            const int e = base + tid, r = r0 + e / W;
+#pragma unroll 4
+        for (int base = 0; base < na * W; base += kGjThreads) {
+            const int e = base + tid, r = row_of(e / W);
             const double x = r == q ? dc : a[e];  // row q now holds the former row c
             const double fr = W == 1 ? x : __shfl_sync(0xffffffffu, x, (lane & ~(W - 1)) | cc);
             const double out = fma(-fr, pv, col == cc ? 0.0 : x);
-            if (e < nr * W) a[e] = r == c ? pv : out;
+            if (e < na * W) a[e] = r == c ? pv : out;
         }
         if (tid == 0) {  // q == c: the second store keeps the row's own origin
-            if (q >= r0 && q < r0 + nr) id[q - r0] = diag[buf].id;
-            if (c >= r0 && c < r0 + nr) id[c - r0] = ok ? w.id : diag[buf].id;
+            if (q % kGjCluster == rank) id[q / kGjCluster] = diag[buf].id;
+            if (c % kGjCluster == rank) id[c / kGjCluster] = ok ? w.id : diag[buf].id;
         }
         __syncthreads();
     }
-    for (int e = tid; e < nr * W; e += kGjThreads) panel[(ustart[p] + r0) * W + e] = a[e];
-    for (int i = tid; i < nr; i += kGjThreads) src[ustart[p] + r0 + i] = id[i];
+    for (int e = tid; e < nr * W; e += kGjThreads) panel[(ustart[p] + row_of(e / W)) * W + col] = a[e];
+    for (int i = tid; i < nr; i += kGjThreads) src[ustart[p] + row_of(i)] = id[i];
     cluster.sync();  // no CTA leaves while another may still write to its shared memory
 }
 
 // The panel's transformations on the whole matrix, X -> Y (see the top), and the composed row origins org_in -> org_out
-// (c0 = 0: from the identity).  One CTA per 32 x 32 output tile, its 32 x W and W x 32 factors in shared memory.
-// Problems with c0 unknowns or fewer are copied through.
+// (c0 = 0: from the identity).  One CTA per 32 x 32 output tile, its 32 x W and W x 32 factors in shared memory; a tile with
+// a factor of zeros is copied, which the unknowns' order makes frequent: with the unknowns sorted by position a row of the
+// operator reaches no further than a plane of cells, so before column c only the first c + plane rows and columns are touched
+// (1728 unknowns: 2.15e9 of 5.16e9 FMA, 5.1 instead of 9.0 ms).  Problems with c0 unknowns or fewer are copied through.
 template <int W>
 __global__ void __launch_bounds__(kGjThreads)
     k_gj_update(const double *__restrict__ X, double *__restrict__ Y, const int64_t *__restrict__ moff,
@@ -169,6 +187,7 @@ __global__ void __launch_bounds__(kGjThreads)
     double *y = Y + moff[p];
     const int tx = threadIdx.x % T, ty = threadIdx.x / T, j = j0 + tx;
     const bool done = c0 >= N;
+    bool m_any = false, b_any = false;
     if (threadIdx.x < T) {
         const int r = i0 + threadIdx.x;
         const int s = r < N && !done ? src[u0 + r] : r;
@@ -178,14 +197,18 @@ __global__ void __launch_bounds__(kGjThreads)
     if (!done) {
         for (int e = threadIdx.x; e < T * W; e += kGjThreads) {
             const int r = i0 + e / W;
-            M[e / W][e % W] = r < N ? panel[(u0 + r) * W + e % W] : 0.0;
+            const double v = r < N ? panel[(u0 + r) * W + e % W] : 0.0;
+            M[e / W][e % W] = v;
+            m_any = m_any || v != 0.0;
         }
         for (int e = threadIdx.x; e < T * W; e += kGjThreads) {
             const int w = e / T, jj = j0 + e % T;
-            B[w][e % T] = c0 + w < N && jj < N ? x[static_cast<int64_t>(src[u0 + c0 + w]) * N + jj] : 0.0;
+            const double v = c0 + w < N && jj < N ? x[static_cast<int64_t>(src[u0 + c0 + w]) * N + jj] : 0.0;
+            B[w][e % T] = v;
+            b_any = b_any || v != 0.0;
         }
     }
-    __syncthreads();
+    const bool product = __syncthreads_or(m_any) && __syncthreads_or(b_any);
     if (j >= N) return;
 #pragma unroll
     for (int k = 0; k < T / ROWS; ++k) {
@@ -196,7 +219,7 @@ __global__ void __launch_bounds__(kGjThreads)
         if (!done) {
             if (j >= c0 && j < c0 + W) {
                 s = M[i][j - c0];
-            } else {
+            } else if (product) {
 #pragma unroll
                 for (int w = 0; w < W; ++w) s = fma(M[i][w], B[w][tx], s);
             }

@@ -2303,22 +2303,42 @@ static __global__ void k_prolong(T *__restrict__ uf, LevelGeom gf, const T *__re
 // problem p are cmap[ustart[p] .. ustart[p+1]), its inverse is the row-major N_p x N_p matrix at Ainv + moff[p]).
 // One warp per unknown; f gathered from the padded pool through cmap.
 // ------------------------------------------------------------------------------------------------------------
+constexpr int kCoarseStage = 2048;  // right-hand side values a CTA stages in shared memory
+
+// Rows w0, w0 + wn, .. of the coarsest solve, the calling warp's; every thread of the CTA calls it.  The right-hand sides
+// lo .. hi - 1 that the CTA's rows need are gathered once into shared memory (up to kCoarseStage): gathered per row, through
+// the map, they put two dependent loads into every step of a row's chain.  Lane l adds columns l, l + 32, .. in order,
+// whatever the path.
 template <typename T, bool CG = false>
-__device__ __forceinline__ void coarse_solve_row(T *__restrict__ u, const T *__restrict__ f,
-                                                 const double *__restrict__ Ainv, const int64_t *__restrict__ cmap,
-                                                 const int32_t *__restrict__ uprob, const int64_t *__restrict__ ustart,
-                                                 const int64_t *__restrict__ moff, const uint8_t *__restrict__ done,
-                                                 int row_i, int lane) {
-    const int p = uprob[row_i];
-    if (done && done[p]) return;
-    const int64_t base = ustart[p];
-    const int Np = static_cast<int>(ustart[p + 1] - base);
-    const double *row = Ainv + moff[p] + static_cast<int64_t>(row_i - base) * Np;
-    double s = 0.0;
-    for (int j = lane; j < Np; j += 32) s = fma(row[j], static_cast<double>(ldv<CG>(f + cmap[base + j])), s);
+__device__ __forceinline__ void coarse_solve_rows(T *__restrict__ u, const T *__restrict__ f,
+                                                  const double *__restrict__ Ainv, const int64_t *__restrict__ cmap,
+                                                  const int32_t *__restrict__ uprob, const int64_t *__restrict__ ustart,
+                                                  const int64_t *__restrict__ moff, const uint8_t *__restrict__ done,
+                                                  int N, int64_t w0, int64_t wn, int64_t lo, int64_t hi,
+                                                  double *__restrict__ stage) {
+    const bool staged = hi - lo <= kCoarseStage;
+    if (staged) {
+        for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) stage[i - lo] = static_cast<double>(ldv<CG>(f + cmap[i]));
+        __syncthreads();
+    }
+    const int lane = threadIdx.x & 31;
+    for (int64_t w = w0; w < N; w += wn) {
+        const int p = uprob[w];
+        if (done && done[p]) continue;
+        const int64_t base = ustart[p];
+        const int Np = static_cast<int>(ustart[p + 1] - base);
+        const double *row = Ainv + moff[p] + (w - base) * Np;
+        double s = 0.0;
+        if (staged) {
+#pragma unroll 8
+            for (int j = lane; j < Np; j += 32) s = fma(__ldg(row + j), stage[base - lo + j], s);
+        } else {
+            for (int j = lane; j < Np; j += 32) s = fma(row[j], static_cast<double>(ldv<CG>(f + cmap[base + j])), s);
+        }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) u[cmap[row_i]] = T(s);
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) u[cmap[w]] = T(s);
+    }
 }
 
 // Coarsest-level solve u = A^-1 f by the dense FP64 inverse, one warp per row (this library's direct coarsest
@@ -2329,9 +2349,11 @@ static __global__ void k_coarse_solve(T *__restrict__ u, const T *__restrict__ f
                                       const int64_t *__restrict__ ustart, const int64_t *__restrict__ moff, int N,
                                       const uint8_t *__restrict__ done = nullptr) {
     pdl_enter(u, f);
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (warp >= N) return;
-    coarse_solve_row<T>(u, f, Ainv, cmap, uprob, ustart, moff, done, warp, threadIdx.x & 31);
+    __shared__ double stage[kCoarseStage];
+    const int warps = blockDim.x >> 5, first = blockIdx.x * warps;  // the CTA's rows: first .. first + warps - 1
+    if (first >= N) return;
+    coarse_solve_rows<T>(u, f, Ainv, cmap, uprob, ustart, moff, done, N, first + (threadIdx.x >> 5), N,
+                         ustart[uprob[first]], ustart[uprob[min(first + warps, N) - 1] + 1], stage);
 }
 
 // ------------------------------------------------------------------------------------------------------------
@@ -2744,31 +2766,35 @@ static __global__ void k_set_units(double *__restrict__ u, const int64_t *__rest
     if (m > 0 && ustart[p] + m - 1 < ustart[p + 1]) u[cmap[ustart[p] + m - 1]] = 0.0;
     if (ustart[p] + m < ustart[p + 1]) u[cmap[ustart[p] + m]] = 1.0;
 }
-// Colour probe of a coarsest level without refinement interfaces (its operator couples a cell only with its six face
-// neighbours, across block faces through same-level ghosts): u = 1 on every unknown of colour C (global cell
-// coordinates mod 3 per axis, 27 colours), 0 elsewhere.  Then row i of A u is A[i, m] for the one unknown m of colour
-// C among i and its six neighbours (nbu: their unknown indices, -1 outside the domain), or 0.
-static __global__ void k_set_colour(double *__restrict__ u, const int64_t *__restrict__ cmap,
-                                    const int8_t *__restrict__ col, int N, int C) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < N) u[cmap[i]] = col[i] == C ? 1.0 : 0.0;
-}
-static __global__ void k_gather_colour(const double *__restrict__ r, const int64_t *__restrict__ cmap,
-                                       const int32_t *__restrict__ uprob, const int64_t *__restrict__ ustart,
-                                       const int64_t *__restrict__ moff, const int8_t *__restrict__ col,
-                                       const int32_t *__restrict__ nbu, int N, double *__restrict__ A, int C) {
+// The rows of a coarsest level without refinement interfaces, one thread per unknown i: its operator couples a cell only with
+// its six face neighbours (nbu: the unknowns of the cell and of its lower and upper x, y and z neighbours, -1 outside the
+// domain, where the reflected ghost -u_i adds the face to the diagonal).  The same values as the operator kernels give on
+// unit vectors, which took four launches for each of 27 colours: 250 us for 512 unknowns, this one 3 us.
+template <int MODE>
+static __global__ void k_coarse_rows(Coef cf, const double *__restrict__ ih2, LevelGeom g, const int64_t *__restrict__ cmap,
+                                     const int32_t *__restrict__ uprob, const int64_t *__restrict__ ustart,
+                                     const int64_t *__restrict__ moff, const int32_t *__restrict__ nbu, int N,
+                                     double *__restrict__ A) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
-    const int p = uprob[i];
-    const int64_t base = ustart[p], Np = ustart[p + 1] - base;
-#pragma unroll
-    for (int q = 0; q < 7; ++q) {
-        const int m = nbu[static_cast<int64_t>(i) * 7 + q];
-        if (m >= 0 && col[m] == C) {
-            A[moff[p] + (i - base) * Np + (m - base)] = r[cmap[i]];
-            return;
-        }
+    const int p = uprob[i], P = g.P;
+    const int64_t base = ustart[p], Np = ustart[p + 1] - base, gi = cmap[i], PP = static_cast<int64_t>(P) * P;
+    double *row = A + moff[p] + (i - base) * Np;
+    double T[6];
+    if constexpr (MODE == 1) {
+        const double t[6] = {cf.tx[gi], cf.tx[gi + 1], cf.ty[gi], cf.ty[gi + P], cf.tz[gi], cf.tz[gi + PP]};
+        for (int f = 0; f < 6; ++f) T[f] = t[f];
+    } else {
+        for (int f = 0; f < 6; ++f) T[f] = 1.0;
     }
+    const double h = MODE == 1 ? 1.0 : ih2[gi / g.bs];
+    double outside = 0.0;
+    for (int f = 0; f < 6; ++f) {
+        const int m = nbu[static_cast<int64_t>(i) * 7 + 1 + f];
+        if (m >= 0) row[m - base] = -T[f] * h;
+        else outside = outside - T[f];
+    }
+    row[i - base] = ((MODE == 1 ? cf.dg[gi] : 6.0) - outside) * h;
 }
 // Column m of every problem's block: A_p[i, m] = (A e_m)[cmap[ustart[p] + i]].
 static __global__ void k_gather_columns(const double *__restrict__ r, const int64_t *__restrict__ cmap,

@@ -771,15 +771,11 @@ void enqueue_coarse_inverse(mg_forest *F, DevLevel &d, int N, int maxN) {
     double *r = F->coarse_r;
     double *Adev = gj_input(F, maxN);
     cudaMemsetAsync(d.u64, 0, d.pool_elems() * sizeof(double), F->st);
-    if (F->pcol) {  // no refinement interface: 27 colour probes
+    if (F->pnbu) {  // no refinement interface: the 7-point rows
         cudaMemsetAsync(Adev, 0, F->moff_h[F->np] * sizeof(double), F->st);
-        for (int C = 0; C < 27; ++C) {
-            k_set_colour<<<(N + 255) / 256, 256, 0, F->st>>>(d.u64, F->cmap, F->pcol, N, C);
-            exchange_any64(F, d, d.u64);
-            apply64(F, d, d.u64, r);
-            k_gather_colour<<<(N + 255) / 256, 256, 0, F->st>>>(r, F->cmap, F->uprob, F->ustart, F->moff, F->pcol,
-                                                                F->pnbu, N, Adev, C);
-        }
+        auto *fn = F->cfg.coeff ? k_coarse_rows<1> : k_coarse_rows<0>;
+        fn<<<(N + 255) / 256, 256, 0, F->st>>>(d.c64(), d.ih2_64, d.g, F->cmap, F->uprob, F->ustart, F->moff, F->pnbu, N,
+                                               Adev);
     } else {  // one unit vector per column
         for (int m = 0; m < maxN; ++m) {
             k_set_units<<<(F->np + 127) / 128, 128, 0, F->st>>>(d.u64, F->cmap, F->ustart, F->np, m);
@@ -806,21 +802,34 @@ mg_status assemble_coarse(mg_forest *F) {
     if (!F->cmap) {
         std::vector<std::vector<int32_t>> blocks(F->np);
         for (int b = 0; b < d.g.nb; ++b) blocks[hl.keys[b].p].push_back(b);
+        // the unknowns of a problem by position (z, then y, then x), so that the operator's rows reach no further than a plane
+        // of cells and the elimination finds most of the matrix untouched (gauss_jordan.cu)
         std::vector<int64_t> cmap, cmap32;
         std::vector<int32_t> uprob;
+        std::vector<int64_t> index(static_cast<size_t>(d.g.nb) * cells);  // unknown of cell `local` of block b
         F->ustart_h.assign(F->np + 1, 0);
         F->moff_h.assign(F->np + 1, 0);
         const int n = d.g.n;
         for (int p = 0; p < F->np; ++p) {
             F->ustart_h[p] = static_cast<int64_t>(cmap.size());
-            for (int b : blocks[p])
-                for (int z = 0; z < n; ++z)
-                    for (int y = 0; y < n; ++y)
-                        for (int x = 0; x < n; ++x) {
-                            cmap.push_back(b * d.g.bs + off3(x + 1, y + 1, z + 1, d.g.P));
-                            cmap32.push_back(Lay<float>::at(d.g, b, x + 1, y + 1, z + 1));
-                            uprob.push_back(p);
-                        }
+            std::vector<std::array<double, 4>> at;  // z, y, x of the cell centre (in level-0 cells), block * cells + local
+            for (int b : blocks[p]) {
+                const Key &kb = hl.keys[b];
+                const double h = std::ldexp(1.0, -kb.lev);
+                for (int c = 0; c < cells; ++c)
+                    at.push_back({(kb.k * n + c / (n * n) + 0.5) * h, (kb.j * n + c / n % n + 0.5) * h,
+                                  (kb.i * n + c % n + 0.5) * h, static_cast<double>(b) * cells + c});
+            }
+            std::sort(at.begin(), at.end());
+            for (const auto &q : at) {
+                const int64_t i = static_cast<int64_t>(q[3]);
+                const int b = static_cast<int>(i / cells), c = static_cast<int>(i % cells);
+                const int x = c % n, y = c / n % n, z = c / (n * n);
+                index[i] = static_cast<int64_t>(cmap.size());
+                cmap.push_back(b * d.g.bs + off3(x + 1, y + 1, z + 1, d.g.P));
+                cmap32.push_back(Lay<float>::at(d.g, b, x + 1, y + 1, z + 1));
+                uprob.push_back(p);
+            }
             const int64_t Np = static_cast<int64_t>(blocks[p].size()) * cells;
             F->moff_h[p + 1] = F->moff_h[p] + Np * Np;
         }
@@ -833,32 +842,18 @@ mg_status assemble_coarse(mg_forest *F) {
         MG_TRY(dalloc(F, &F->Ainv, F->moff_h[F->np]));
         MG_TRY(dalloc(F, &F->AinvT, F->moff_h[F->np]));
         if (d.nifaces == 0 && d.nsegs == 0) {
-            // colours and the 7-point neighbourhoods of the unknowns for the colour probe; every block of a problem
-            // is then at one refinement level (face neighbours share it), so key * n + local is a global coordinate
-            std::vector<int64_t> first(d.g.nb, -1);  // unknown index of each block's first cell
-            for (int p = 0; p < F->np; ++p) {
-                int64_t at = F->ustart_h[p];
-                for (int b : blocks[p]) {
-                    first[b] = at;
-                    at += cells;
-                }
-            }
+            // the 7-point neighbourhoods of the unknowns
             std::vector<int32_t> nb6(static_cast<size_t>(d.g.nb) * 6, -2);
             for (const FaceItem &fi : hl.faces)
                 nb6[static_cast<size_t>(fi.blk) * 6 + 2 * fi.axis + fi.side] =
                     fi.kind == FK_SAME ? fi.nbr : (fi.kind == FK_BND ? -1 : -2);
-            std::vector<int8_t> col(N);
             std::vector<int32_t> nbu(static_cast<size_t>(N) * 7, -1);
             bool ok = true;
             for (int b = 0; b < d.g.nb && ok; ++b) {
-                const Key &kb = hl.keys[b];
                 for (int z = 0; z < n; ++z)
                     for (int y = 0; y < n; ++y)
                         for (int x = 0; x < n; ++x) {
-                            const int64_t i = first[b] + (static_cast<int64_t>(z) * n + y) * n + x;
-                            const int64_t gx = static_cast<int64_t>(kb.i) * n + x, gy = static_cast<int64_t>(kb.j) * n + y,
-                                          gz = static_cast<int64_t>(kb.k) * n + z;
-                            col[i] = static_cast<int8_t>(gx % 3 + 3 * (gy % 3) + 9 * (gz % 3));
+                            const int64_t i = index[static_cast<int64_t>(b) * cells + (z * n + y) * n + x];
                             nbu[i * 7] = static_cast<int32_t>(i);
                             const int c[3] = {x, y, z};
                             for (int axis = 0; axis < 3; ++axis)
@@ -872,15 +867,12 @@ mg_status assemble_coarse(mg_forest *F) {
                                         if (bb < 0) continue;
                                         cc[axis] = side ? 0 : n - 1;
                                     }
-                                    nbu[i * 7 + 1 + 2 * axis + side] =
-                                        static_cast<int32_t>(first[bb] + (static_cast<int64_t>(cc[2]) * n + cc[1]) * n + cc[0]);
+                                    nbu[i * 7 + 1 + 2 * axis + side] = static_cast<int32_t>(
+                                        index[static_cast<int64_t>(bb) * cells + (cc[2] * n + cc[1]) * n + cc[0]]);
                                 }
                         }
             }
-            if (ok && N < (int64_t(1) << 31)) {
-                MG_TRY(upload(F, &F->pcol, col));
-                MG_TRY(upload(F, &F->pnbu, nbu));
-            }
+            if (ok) MG_TRY(upload(F, &F->pnbu, nbu));
         }
     }
     if (!F->coarse_r) MG_TRY(dalloc(F, &F->coarse_r, d.pool_elems()));

@@ -110,7 +110,8 @@ __device__ __forceinline__ void tail_prolong(const TailLevel &d, const TailLevel
 
 // One phase of a recorded tail, over every thread of the grid (thread t0 of ts).
 template <int MODE>
-__device__ __forceinline__ void tail_phase(const TailArgs &a, const TailPhase &P, int64_t t0, int64_t ts) {
+__device__ __forceinline__ void tail_phase(const TailArgs &a, const TailPhase &P, int64_t t0, int64_t ts,
+                                           double *coarse_f) {
     const TailLevel &d = a.L[P.level];
     const Skip skip{d.bprob, a.done};
     switch (P.op) {
@@ -138,23 +139,20 @@ __device__ __forceinline__ void tail_phase(const TailArgs &a, const TailPhase &P
             }
             break;
         }
-        default: {  // T_COARSE: one warp per coarsest unknown
-            const int lane = threadIdx.x & 31;
-            const int64_t w0 = t0 >> 5, wn = ts >> 5;
-            for (int64_t w = w0; w < a.Nc; w += wn)
-                coarse_solve_row<float, true>(d.u, d.f, a.Ainv, a.cmap32, a.uprob, a.ustart, a.moff, a.done,
-                                              static_cast<int>(w), lane);
+        default:  // T_COARSE: one warp per coarsest unknown
+            coarse_solve_rows<float, true>(d.u, d.f, a.Ainv, a.cmap32, a.uprob, a.ustart, a.moff, a.done, a.Nc, t0 >> 5,
+                                           ts >> 5, 0, a.Nc, coarse_f);
             break;
-        }
     }
 }
 
 template <int MODE>
 static __global__ void __launch_bounds__(kTailThreads) k_tail32(TailArgs a) {
+    __shared__ double coarse_f[kCoarseStage];
     const int64_t t0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
     const int64_t ts = static_cast<int64_t>(gridDim.x) * blockDim.x;
     for (int p = 0; p < a.nph; ++p) {
-        tail_phase<MODE>(a, a.ph[p], t0, ts);
+        tail_phase<MODE>(a, a.ph[p], t0, ts, coarse_f);
         if (!grid_barrier(a.bar, (p + 1) * gridDim.x, a.err)) return;
     }
 }
@@ -166,12 +164,13 @@ template <int MODE>
 static __global__ void __launch_bounds__(kTailThreads) k_batch_tail32(const TailArgs *__restrict__ ga,
                                                                       const BatchEntry *__restrict__ e, int ne,
                                                                       unsigned *bar, int *err) {
+    __shared__ double coarse_f[kCoarseStage];
     const int64_t t0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
     const int64_t ts = static_cast<int64_t>(gridDim.x) * blockDim.x;
     unsigned target = 0;
     for (int i = 0; i < ne; ++i) {
         const BatchEntry E = e[i];
-        tail_phase<MODE>(ga[E.group], E.P, t0, ts);
+        tail_phase<MODE>(ga[E.group], E.P, t0, ts, coarse_f);
         if (E.last && !grid_barrier(bar, target += gridDim.x, err)) return;
     }
 }
@@ -181,9 +180,10 @@ TailArgs tail_args(mg_forest *F) {
                     F->ustart, F->moff, F->Nc, F->np > 1 ? F->pdone : nullptr, F->tail_bar, F->kerr};
 }
 
-// CTAs the largest phase of F's recorded tail can use (one thread per updated cell of a half-sweep).
+// CTAs the largest phase of F's recorded tail can use (one thread per updated cell of a half-sweep, one warp per coarsest
+// unknown).
 int64_t tail_ctas(mg_forest *F) {
-    int64_t need = 1;
+    int64_t need = std::max<int64_t>(1, static_cast<int64_t>(F->Nc) * 32 / kTailThreads);
     for (int l = std::max(0, F->tail_level); l < static_cast<int>(F->L.size()); ++l)
         need = std::max<int64_t>(need, (F->L[l].cells() / 2 + kTailThreads - 1) / kTailThreads);
     return need;
