@@ -809,7 +809,7 @@ void vcycle_T(mg_forest *F, int l) {
             });
     }
     const bool gather = d.all_halve;
-    if (sizeof(T) == 4 && transfer32_specialised(d)) {
+    if (sizeof(T) == 4 && transfer_specialised(d)) {
         Prof p(F, P_ADJ, 1);
         static constexpr decltype(&k_prolong_T32<3>) fns[5] = {k_prolong_T32<3>, k_prolong_T32<4>, k_prolong_T32<5>,
                                                                k_prolong_T32<6>, k_prolong_T32<7>};

@@ -353,7 +353,7 @@ mg_status ensure_fp64_coefficients(mg_forest *F);
 // solver.cu, for the transposed cycles: one FP32 half-sweep on a level's own pools, and the injection y_f += R^T e_c with
 // its write-through (false: not for this level's transfer)
 bool smooth32_specialised(const DevLevel &d);
-bool transfer32_specialised(const DevLevel &d);
+bool transfer_specialised(const DevLevel &d);
 void smooth_level32(mg_forest *F, DevLevel &d, int colour);
 bool inject32(mg_forest *F, DevLevel &d, DevLevel &c);
 }  // namespace octmg

@@ -458,9 +458,9 @@ static __global__ void k_exchange_segs(T *__restrict__ u, Coef cf, const SegItem
 // Both sides of a refinement interface in one pass.  A fine block face next to a coarser block is one FaceItem, and the
 // quarter of the coarse block's face that it covers is filled from that fine block alone, so the four fine ghosts over a
 // coarse cell (C2F, Sec. 3.3.2) give, with the fine cells next to them, the coarse ghost across the face (F2C): all that is
-// read is the interior of the two blocks.  One lane per fine ghost, the four of a coarse cell next to each other (lane
-// 4 k + 2 a2 + a1), which share the coarse ghost's sum by shuffles.  The same operations in the same order as
-// exchange_faces_body and exchange_segs_body.
+// read is the interior of the two blocks.  Two forms, with the same operations in the same order as exchange_faces_body and
+// exchange_segs_body: a CTA per strip of a face (exchange_iface_cta), and, for the persistent tail, one lane per fine ghost,
+// the four of a coarse cell next to each other (lane 4 k + 2 a2 + a1), which share the coarse ghost's sum by shuffles.
 // ------------------------------------------------------------------------------------------------------------
 // Offset inside a block of the cell at `depth` from face (axis, side) with tangential interior coordinates (i1, i2), for
 // blocks of fewer than 2^31 elements.
@@ -559,19 +559,42 @@ struct IfaceStrip {
     }
 };
 
-// One strip of an interface item by one CTA, one ghost per thread (block edges up to 128).  The normal-direction
-// extrapolations of the strip's coarse cells and of their tangential border are computed once into shared memory, E[w1 w2]
-// (Sec. 8 of the paper proposes this reuse for neighbouring cells); W[18] the tangential weights [case][a][base].  All loads
-// come before the first use of one, and before the done-mask decides (uniformly over the CTA) whether anything is written.
+// One strip of an interface item by one CTA, one ghost per thread (block edges up to 128), in four steps through shared
+// memory, each value computed once (Sec. 8 of the paper proposes this reuse between neighbouring cells):
+//   E[w2][w1]      normal-direction extrapolations of the strip's coarse cells and their tangential border,
+//   S[w2][n]       their first tangential interpolation at the fine positions of every coarse row,
+//   the ghosts     second tangential interpolation; D[lines][n] keeps what the coarse side needs of each (the difference
+//                  ghost - cell and the face coefficient, or the two fine cells of the mean),
+//   coarse ghosts  one thread per coarse cell.
+// All loads come before the first use of one, and before the done-mask decides (uniformly over the CTA) whether anything is
+// written.  The sharing matters in FP64, whose operations bound the kernel: with 12 of them per ghost, and the coarse side's
+// sum and division by one lane in four of every warp, 6.2 us on 96 faces of 32 x 32 cells, this way 5.9 (five damped Jacobi cycles on 22 blocks of 64^3: 7.1 -> 6.7 ms).
 template <typename T, int MODE, bool FLUX>
 __device__ __forceinline__ void exchange_iface_cta(T *__restrict__ u, const Coef &cf, const FaceItem &F, int strip,
-                                                   const LevelGeom &g, Skip skip, int c2f, T *E, T *W) {
+                                                   const LevelGeom &g, Skip skip, int c2f, T *sm) {
     const IfaceStrip Q(F, g.n, strip);
-    const int n = Q.n, h = Q.h, lgh = g.lg - 1, q = threadIdx.x;
-    const int a1 = q & 1, a2 = (q >> 1) & 1, ycl = (q >> 2) & (h - 1), zcl = Q.c0 + (q >> (2 + lgh));
-    const bool mine = q < 4 * Q.rows * h;
-    const IfaceGhost<T, MODE, FLUX> G(u, cf, F, g, ycl, mine ? zcl : Q.c0, a1, a2);
-    const T *uc = u + F.nbr * g.bs;
+    const int n = Q.n, h = Q.h, lg = g.lg, q = threadIdx.x, lines = 2 * Q.rows;
+    T *E = sm, *S = E + Q.w1 * Q.w2, *D = S + Q.w2 * n, *D2 = D + lines * n, *W = D2 + lines * n;  // W[18]: [case][a][base]
+    const bool mine = q < lines * n, coarse = q < Q.rows * h;
+    const int i1 = q & (n - 1), line = mine ? q >> lg : 0, i2 = 2 * Q.c0 + line;
+    const int ycl = q & (h - 1), zcl = Q.c0 + (coarse ? q >> (lg - 1) : 0);  // the thread's coarse cell
+    const int64_t fb = F.blk * g.bs, cb = F.nbr * g.bs;
+    const int64_t g0 = fb + face_in<T>(g, F.axis, F.side, 0, i1, i2);
+    const int64_t g1 = fb + face_in<T>(g, F.axis, F.side, 1, i1, i2);
+    const int64_t g0c = cb + face_in<T>(g, F.axis, 1 - F.side, 0, F.seg1 * h + ycl, F.seg2 * h + zcl);
+    const T u1 = u[g1];
+    T keep = T(0), uC = T(0), Tc = T(0);
+    if constexpr (FLUX) {
+        keep = face_coef<T, MODE>(cf, F.side ? g0 : g1, F.side ? g1 : g0, F.axis);
+        if (coarse) {
+            const int64_t gC = cb + face_in<T>(g, F.axis, 1 - F.side, 1, F.seg1 * h + ycl, F.seg2 * h + zcl);
+            uC = u[gC];
+            Tc = face_coef<T, MODE>(cf, F.side ? gC : g0c, F.side ? g0c : gC, F.axis);
+        }
+    } else {
+        keep = u[fb + face_in<T>(g, F.axis, F.side, 2, i1, i2)];
+    }
+    const T *uc = u + cb;
     if (q < 18) W[q] = w_tang<T>(c2f, q / 6, q / 3 % 2, q % 3);
     for (int i = q; i < Q.w1 * Q.w2; i += blockDim.x) {
         const int y = Q.lo1 + i % Q.w1, z = Q.lo2 + i / Q.w1;
@@ -581,19 +604,46 @@ __device__ __forceinline__ void exchange_iface_cta(T *__restrict__ u, const Coef
     }
     if (skip(F.blk)) return;
     __syncthreads();
-    if (!mine) return;
-    const int yc = F.seg1 * h + ycl, zc = F.seg2 * h + zcl;
-    const int cy = tang_case(yc, n), cz = tang_case(zc, n);
-    const T *Ec = E + (zc + tang_first(cz) - Q.lo2) * Q.w1 + yc + tang_first(cy) - Q.lo1;
-    T e[3][3], wy[3], wz[3];
+    for (int i = q; i < Q.w2 * n; i += blockDim.x) {
+        const int x = i & (n - 1), yc = F.seg1 * h + (x >> 1), cy = tang_case(yc, n);
+        const T *e = E + (i >> lg) * Q.w1 + yc + tang_first(cy) - Q.lo1, *w = W + cy * 6 + (x & 1) * 3;
+        T acc = T(0);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        wy[c] = W[cy * 6 + a1 * 3 + c];
-        wz[c] = W[cz * 6 + a2 * 3 + c];
-#pragma unroll
-        for (int b = 0; b < 3; ++b) e[c][b] = Ec[c * Q.w1 + b];
+        for (int b = 0; b < 3; ++b) acc = fma(w[b], e[b], acc);
+        S[i] = acc;
     }
-    G.put(u, (q & 3) == 0, e, wy, wz);
+    __syncthreads();
+    if (mine) {
+        const int zc = F.seg2 * h + (i2 >> 1), cz = tang_case(zc, n);
+        const T *e = S + (zc + tang_first(cz) - Q.lo2) * n + i1, *w = W + cz * 6 + (i2 & 1) * 3;
+        T acc = T(0);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) acc = fma(w[c], e[c * n], acc);
+        u[g0] = acc;
+        D[q] = FLUX ? acc - u1 : u1;
+        D2[q] = keep;
+    }
+    __syncthreads();
+    if (!coarse) return;
+    const int at = 2 * (zcl - Q.c0) * n + 2 * ycl;  // the four fine faces: at + a2 n + a1
+    if constexpr (FLUX) {
+        T flux = T(0);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) flux = fma(D2[at + (k >> 1) * n + (k & 1)], D[at + (k >> 1) * n + (k & 1)], flux);
+        u[g0c] = uC - flux / (T(MODE == 1 ? 8 : 2) * Tc);
+    } else {
+        T s = T(0);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s += D[at + (k >> 1) * n + (k & 1)];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s += D2[at + (k >> 1) * n + (k & 1)];
+        u[g0c] = T(0.125) * s;
+    }
+}
+// Shared values of one strip.
+__host__ __device__ constexpr int iface_values(int n) {
+    const int rows = n / 2 / iface_strips(n);
+    return (rows + 2) * (n / 2 + 2) + (rows + 2) * n + 2 * 2 * rows * n + 18;
 }
 
 // The interface items one thread per fine ghost, without shared memory (the persistent tail, whose items are small).
@@ -642,11 +692,10 @@ static __global__ void __launch_bounds__(kThreads) k_exchange(T *__restrict__ u,
                                                               Skip skip, int c2f, const T *__restrict__ gb) {
     pdl_enter(u);
     extern __shared__ __align__(16) unsigned char iface_smem[];
-    __shared__ T W[18];
     const int strips = iface_strips(g.n), nic = nif * strips;
     if (static_cast<int>(blockIdx.x) < nic) {
         const FaceItem F = ifaces[blockIdx.x / strips];
-        exchange_iface_cta<T, MODE, FLUX>(u, cf, F, blockIdx.x % strips, g, skip, c2f, reinterpret_cast<T *>(iface_smem), W);
+        exchange_iface_cta<T, MODE, FLUX>(u, cf, F, blockIdx.x % strips, g, skip, c2f, reinterpret_cast<T *>(iface_smem));
         return;
     }
     exchange_faces_body<T, false>(u, sfaces, nsf, g, skip, (blockIdx.x - nic) * static_cast<int64_t>(blockDim.x) + threadIdx.x,
@@ -1871,6 +1920,115 @@ static __global__ void __launch_bounds__(544) k_residual_restrict32t(
         }
     }
     if (bad && (tid & 31) == 0) atomicOr(err, 4);
+}
+
+// ------------------------------------------------------------------------------------------------------------
+// FP64 transfers of a halving level with fine edge 2^LG: k_residual_restrict and k_prolong with the 4^3 box of a coarse cell
+// at immediate offsets, one coarse cell per thread, and with what spares the cycle its full exchanges: the restriction
+// zeroes the coarse correction's face ghosts too, the prolongation writes the corrected block-face cells through.  The same
+// operations in the same order.  On 256^3 cells of 64^3 blocks the finest restriction takes 234 us (its FP64 operations
+// alone 190; 275 with 64-bit index arithmetic and a grid-stride loop), the prolongation 101 us, and four full exchanges per
+// cycle and level are gone: ten cycles on 32^3 cells 833 -> 775 us.
+// ------------------------------------------------------------------------------------------------------------
+// Writes val, just stored at cell (x, y, z) of block b (offset q inside the block), to the ghosts that mirror or reflect it.
+template <int LG>
+__device__ __forceinline__ void write_through64(double *__restrict__ u, int64_t bs, int64_t b, int q, int x, int y, int z,
+                                                double val, const int32_t *__restrict__ nbr6,
+                                                const double *__restrict__ gb) {
+    constexpr int n = 1 << LG, P = n + 2;
+    const int c[3] = {x, y, z}, st[3] = {1, P, P * P};
+#pragma unroll
+    for (int axis = 0; axis < 3; ++axis) {
+        if (c[axis] != 0 && c[axis] != n - 1) continue;
+        const int side = c[axis] ? 1 : 0, nb = nbr6[b * 6 + 2 * axis + side];
+        if (nb >= 0) {
+            u[nb * bs + q + (side ? -n : n) * st[axis]] = val;
+        } else if (nb == -1) {
+            const int i1 = axis == 0 ? y : x, i2 = axis == 2 ? y : z;
+            u[b * bs + q + (side ? st[axis] : -st[axis])] =
+                gb ? gb[(b * 6 + 2 * axis + side) * static_cast<int64_t>(n) * n + i2 * n + i1] - val : -val;
+        }
+    }
+}
+
+template <int MODE, int LG>
+static __global__ void __launch_bounds__(kThreads) k_residual_restrict64(
+        const double *__restrict__ u, const double *__restrict__ f, Coef cf, const double *__restrict__ ih2f, int64_t bsf,
+        double *__restrict__ fc, double *__restrict__ uc, const XferItem *__restrict__ xf, int64_t total, int64_t bsc,
+        Skip skip) {
+    pdl_enter(u, f, fc, uc);
+    constexpr int n = 1 << LG, P = n + 2, PP = P * P, nc = n / 2, LC = LG - 1, Pc = nc + 2;
+    const int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    if (t >= total) return;
+    const int r = static_cast<int>(t) & ((1 << (3 * LC)) - 1);
+    const int64_t B = t >> (3 * LC);
+    if (skip(B)) return;
+    const int X = r & (nc - 1), Y = (r >> LC) & (nc - 1), Z = r >> (2 * LC);
+    const int64_t b = xf[B].src[0];
+    const int64_t corner = b * bsf + ((2 * Z + 1) * P + 2 * Y + 1) * P + 2 * X + 1;  // the first child
+    const double ih2 = MODE == 1 ? 0.0 : ih2f[b];
+    double s = 0.0;
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int bb = 0; bb < 2; ++bb)
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+                s += residual_at<double, MODE>(u, f, cf, corner + (c * PP + bb * P + a), P, ih2);
+    const int64_t gc = B * bsc;
+    const auto at = [&](int x, int y, int z) { return gc + (z * Pc + y) * Pc + x; };
+    fc[at(X + 1, Y + 1, Z + 1)] = 0.125 * s;
+    uc[at(X + 1, Y + 1, Z + 1)] = 0.0;
+    if (X == 0) uc[at(0, Y + 1, Z + 1)] = 0.0;
+    if (X == nc - 1) uc[at(nc + 1, Y + 1, Z + 1)] = 0.0;
+    if (Y == 0) uc[at(X + 1, 0, Z + 1)] = 0.0;
+    if (Y == nc - 1) uc[at(X + 1, nc + 1, Z + 1)] = 0.0;
+    if (Z == 0) uc[at(X + 1, Y + 1, 0)] = 0.0;
+    if (Z == nc - 1) uc[at(X + 1, Y + 1, nc + 1)] = 0.0;
+}
+
+template <int LG>
+static __global__ void __launch_bounds__(kThreads) k_prolong64(double *__restrict__ uf, int64_t bsf,
+                                                               const double *__restrict__ ec,
+                                                               const XferItem *__restrict__ xf, int64_t total, int64_t bsc,
+                                                               const int32_t *__restrict__ nbr6, Skip skip,
+                                                               const double *__restrict__ gb) {
+    pdl_enter(uf, ec);
+    constexpr int n = 1 << LG, P = n + 2, PP = P * P, nc = n / 2, LC = LG - 1, Pc = nc + 2, PPc = Pc * Pc;
+    const int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    if (t >= total) return;
+    const int r = static_cast<int>(t) & ((1 << (3 * LC)) - 1);
+    const int64_t B = t >> (3 * LC);
+    if (skip(B)) return;
+    const int X = r & (nc - 1), Y = (r >> LC) & (nc - 1), Z = r >> (2 * LC);
+    const double *e = ec + B * bsc + ((Z + 1) * Pc + Y + 1) * Pc + X + 1;
+    const double e0 = e[0], ex[2] = {e[-1], e[1]}, ey[2] = {e[-Pc], e[Pc]}, ez[2] = {e[-PPc], e[PPc]};
+    const int64_t b = xf[B].src[0];
+    const int q = ((2 * Z + 1) * P + 2 * Y + 1) * P + 2 * X + 1;
+    double *ub = uf + b * bsf + q;
+    double val[2][2][2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int bb = 0; bb < 2; ++bb)
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+                val[c][bb][a] = ub[c * PP + bb * P + a] + 0.25 * ((e0 + ex[a]) + (ey[bb] + ez[c]));
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int bb = 0; bb < 2; ++bb)
+#pragma unroll
+            for (int a = 0; a < 2; ++a) ub[c * PP + bb * P + a] = val[c][bb][a];
+    if (X != 0 && X != nc - 1 && Y != 0 && Y != nc - 1 && Z != 0 && Z != nc - 1) return;
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int bb = 0; bb < 2; ++bb)
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+                write_through64<LG>(uf, bsf, b, q + c * PP + bb * P + a, 2 * X + a, 2 * Y + bb, 2 * Z + c, val[c][bb][a],
+                                    nbr6, gb);
 }
 
 // The 8 children (2X + a, 2Y + b, 2Z + c), a, b, c in {1, 2}, of coarse cell (X, Y, Z) in fine block b of a halving

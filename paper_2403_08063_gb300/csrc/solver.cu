@@ -105,7 +105,7 @@ void exchange(mg_forest *F, DevLevel &d, T *u, bool interface_only = false, bool
         if (&d == &F->L[0]) gb = F->gb;
     if (one) {
         const int threads = nsf ? kThreads : iface_threads(n), strips = iface_strips(n);
-        const size_t smem = nif ? (n / 2 / strips + 2) * (n / 2 + 2) * sizeof(T) : 0;
+        const size_t smem = nif ? iface_values(n) * sizeof(T) : 0;
         const int grid = nif * strips + (nsf ? grid_for(static_cast<int64_t>(nsf) * n * n) : 0);
         auto *fn = F->cfg.interface_flux ? k_exchange<T, MODE, true> : k_exchange<T, MODE, false>;
         launch_pdl(F->st, !F->batch_member, fn, grid, threads, smem, u, coef_of<T>(d), d.ifaces, nif, d.sfaces, nsf,
@@ -309,8 +309,9 @@ mg_status tune_smooth32(mg_forest *F) {
     return MG_OK;
 }
 
-// FP32 residual + restriction and prolongation specialised for levels whose blocks all halve, fine edges 8..128.
-bool transfer32_specialised(const DevLevel &d) { return d.all_halve && d.g.lg >= 3 && d.g.lg <= 7; }
+// Residual + restriction and prolongation specialised for levels whose blocks all halve, fine edges 8..128 (the FP32 ones
+// with the FP32 cycles' coefficients, the FP64 ones with theirs).
+bool transfer_specialised(const DevLevel &d) { return d.all_halve && d.g.lg >= 3 && d.g.lg <= 7; }
 
 using Restrict32Fn = void (*)(const float *, const float *, const float *, const float *, int64_t, float *, float *,
                               const XferItem *, int32_t, int64_t, Skip, const float *, const float *, const float *);
@@ -395,9 +396,31 @@ void launch_prolong32(mg_forest *F, DevLevel &d, DevLevel &c, bool inject = fals
 }
 
 bool inject32(mg_forest *F, DevLevel &d, DevLevel &c) {
-    if (!transfer32_specialised(d)) return false;
+    if (!transfer_specialised(d)) return false;
     launch_prolong32(F, d, c, true);
     return true;
+}
+
+using Restrict64Fn = decltype(&k_residual_restrict64<0, 3>);
+using Prolong64Fn = decltype(&k_prolong64<3>);
+// [coefficient mode 0, 1][fine block edge 2^3 .. 2^7]
+const Restrict64Fn kRestrict64[2][5] = {
+    {k_residual_restrict64<0, 3>, k_residual_restrict64<0, 4>, k_residual_restrict64<0, 5>, k_residual_restrict64<0, 6>,
+     k_residual_restrict64<0, 7>},
+    {k_residual_restrict64<1, 3>, k_residual_restrict64<1, 4>, k_residual_restrict64<1, 5>, k_residual_restrict64<1, 6>,
+     k_residual_restrict64<1, 7>}};
+const Prolong64Fn kProlong64[5] = {k_prolong64<3>, k_prolong64<4>, k_prolong64<5>, k_prolong64<6>, k_prolong64<7>};
+
+void launch_residual_restrict64(mg_forest *F, DevLevel &d, DevLevel &c) {
+    launch_pdl(F->st, !F->batch_member, kRestrict64[F->cfg.coeff ? 1 : 0][d.g.lg - 3],
+               static_cast<unsigned>((c.cells() + kThreads - 1) / kThreads), kThreads, 0, d.u64, d.f64, d.c64(), d.ih2_64,
+               d.g.bs, c.f64, c.u64, d.xfer, c.cells(), c.g.bs, skip_of(F, c));
+}
+
+void launch_prolong64(mg_forest *F, DevLevel &d, DevLevel &c) {
+    launch_pdl(F->st, !F->batch_member, kProlong64[d.g.lg - 3],
+               static_cast<unsigned>((c.cells() + kThreads - 1) / kThreads), kThreads, 0, d.u64, d.g.bs, c.u64, d.xfer,
+               c.cells(), c.g.bs, d.nbr6, skip_of(F, c), &d == &F->L[0] ? F->gb : nullptr);
 }
 
 template <typename T, int MODE>
@@ -456,7 +479,7 @@ void vcycle_walk(mg_forest *F, int l, int entry, E &ex) {
         ex.smooth(l, 1);
     }
     if (F->cfg.nu1) ex.exchange(l, !jac);
-    const bool fast = sizeof(T) == 4 && MODE != 1 && transfer32_specialised(F->L[l]);
+    const bool fast = transfer_specialised(F->L[l]);
     ex.restrict_to(l, fast);
     vcycle_walk<T, MODE>(F, l + 1, fast ? ENTRY_NONE : ENTRY_FULL, ex);
     if (l + 1 != last) ex.exchange(l + 1, !jac);  // Jacobi sweeps write no ghosts through
@@ -479,7 +502,7 @@ void vcycle_walk(mg_forest *F, int l, int entry, E &ex) {
 // How level l is entered in an FP32 V-cycle (level 0 from vcycle32, deeper levels from the restriction above).
 int entry32(mg_forest *F, int l) {
     if (l == 0) return ENTRY_INTERFACE;
-    return transfer32_specialised(F->L[l - 1]) ? ENTRY_NONE : ENTRY_FULL;
+    return transfer_specialised(F->L[l - 1]) ? ENTRY_NONE : ENTRY_FULL;
 }
 
 // Edge and corner ghosts of a level (trilinear prolongation; the face ghosts are current): edges, then corners.
@@ -549,7 +572,9 @@ struct LaunchExec {
     void restrict_to(int l, bool fast) {
         DevLevel &d = F->L[l], &c = F->L[l + 1];
         Prof p(F, cat_of<T>(P_RESTR64), 1);
-        if (fast)
+        if (fast && sizeof(T) == 8)
+            launch_residual_restrict64(F, d, c);
+        else if (fast)
             launch_residual_restrict32(F, d, c);
         else if (sizeof(T) == 4 && d.face32)
             launch_pdl(F->st, !F->batch_member, k_residual_restrict<float, 3>, grid_for(c.cells()), kThreads, 0,
@@ -570,7 +595,9 @@ struct LaunchExec {
             return;
         }
         Prof p(F, cat_of<T>(P_PROL64), 1);
-        if (fast)
+        if (fast && sizeof(T) == 8)
+            launch_prolong64(F, d, c);
+        else if (fast)
             launch_prolong32(F, d, c);
         else
             launch_pdl(F->st, !F->batch_member, k_prolong<T>, grid_for(c.cells()), kThreads, 0, ufield<T>(d), d.g,
@@ -657,7 +684,7 @@ mg_status record_tail(mg_forest *F, int l) {
         for (size_t m = 0; m < F->L.size(); ++m) {
             const DevLevel &d = F->L[m];
             tl[m] = TailLevel{d.g, d.u32, d.f32, d.kap, d.h2_32, d.ih2_32, d.sfaces, d.ifaces, d.xfer, d.nbr6,
-                              d.bprob, d.nsfaces, d.nifaces, transfer32_specialised(d) ? 1 : 0,
+                              d.bprob, d.nsfaces, d.nifaces, transfer_specialised(d) ? 1 : 0,
                               d.ax32, d.ay32, d.az32, d.face32 ? 1 : 0};
         }
         MG_TRY(upload(F, &F->tail_L, tl));
