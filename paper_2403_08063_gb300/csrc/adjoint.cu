@@ -898,7 +898,7 @@ mg_status adjoint_residual(mg_forest *F, bool zero, double mult, double *rr) {
     DevLevel &d = F->L[0];
     const double *f = F->a_g;
     if (!zero) {
-        exchange_same<double>(F, d, F->a_lam);
+        if (F->cfg.precision == 0) exchange_same<double>(F, d, F->a_lam);  // else k_update_mixed wrote these ghosts
         if (d.nifaces) {
             // FP32 cycles leave a_fe alone, so it differs from g only where the last step added to it
             if (F->cfg.precision == 1) {
@@ -918,9 +918,14 @@ mg_status adjoint_residual(mg_forest *F, bool zero, double mult, double *rr) {
         const int cpb = F->bsum_cpb;
         Prof p(F, P_ADJ, 1);
         MG_CUDA(cudaMemsetAsync(F->bsum, 0, static_cast<size_t>(d.g.nb) * cpb * sizeof(double), F->st));
-        auto *fn = zero ? k_residual_norm<MODE, true> : k_residual_norm<MODE, false>;
-        fn<<<d.g.nb * cpb, kThreads, 0, F->st>>>(F->a_lam, f, d.c64(), d.ih2_64, d.vol_32, d.g, cpb, d.f32, F->pscale,
-                                                 d.bprob, F->bsum, d.u32, Skip{});
+        if (zero) {
+            MG_CUDA(cudaMemsetAsync(d.u32, 0, d.pool_elems() * sizeof(float), F->st));
+            k_scaled_rhs<<<d.g.nb * cpb, kThreads, 0, F->st>>>(f, d.vol_32, d.g, cpb, d.f32, F->pscale, d.bprob, F->bsum,
+                                                               Skip{});
+        } else {
+            k_residual_norm<MODE><<<d.g.nb * cpb, kThreads, 0, F->st>>>(F->a_lam, f, d.c64(), d.ih2_64, d.vol_32, d.g, cpb,
+                                                                        d.f32, F->pscale, d.bprob, F->bsum, d.u32, Skip{});
+        }
         MG_TRY(enqueue_problem_sums(F));
         MG_CUDA(cudaStreamSynchronize(F->st));
         *rr = 0.0;
@@ -963,7 +968,8 @@ mg_status adjoint_solve(mg_forest *F, const double *u_dev, const double *dLdu_de
         if (F->cfg.precision == 1) {
             MG_TRY(replay(F, F->vT_rec, [&] { vcycle_T<float>(F, 0); }));
             Prof p(F, P_ADJ, 1);
-            k_update_mixed<<<grid, kThreads, 0, F->st>>>(F->a_lam, d.u32, F->pinv, d.bprob, d.g, Skip{});
+            k_update_mixed<false><<<update_grid(d), kThreads, 0, F->st>>>(F->a_lam, d.u32, F->pinv, d.bprob, d.g, d.nbr6,
+                                                                        nullptr, Skip{});
         } else {
             MG_TRY(replay(F, F->vT_rec, [&] { vcycle_T<double>(F, 0); }));
             Prof p(F, P_ADJ, 1);
@@ -1020,8 +1026,7 @@ extern "C" mg_status mg_apply_transpose(mg_forest *F, const double *y_dev, doubl
     k_pack<double><<<grid_for(d.cells()), kThreads, 0, F->st>>>(F->s64a, y_dev, d.g, F->leaf_off);
     exchange_same<double>(F, d, F->s64a);
     adj_iface<double>(F, d, F->s64a, true, nullptr, nullptr, {nullptr, nullptr, nullptr}, 1.0);
-    apply64(F, d, F->s64a, F->s64b);
-    k_unpack<double><<<grid_for(d.cells()), kThreads, 0, F->st>>>(ATy_dev, F->s64b, d.g, F->leaf_off);
+    apply64(F, d, F->s64a, ATy_dev, true);
     adj_iface<double>(F, d, F->s64a, false, nullptr, nullptr, {nullptr, ATy_dev, F->leaf_off}, 1.0);
     MG_CUDA(cudaStreamSynchronize(F->st));
     return MG_OK;

@@ -174,7 +174,7 @@ mg_status enqueue_step(mg_batch *B, int m) {
         for (mg_forest *F : B->groups) {
             MG_TRY(enqueue_update_mixed(F));
             MG_TRY(enqueue_scales(F));
-            MG_TRY(enqueue_residual(F));
+            MG_TRY(enqueue_residual(F, false, true));
             MG_TRY(enqueue_problem_sums(F));
         }
         return join(B);
@@ -183,7 +183,7 @@ mg_status enqueue_step(mg_batch *B, int m) {
         MG_TRY(enqueue_done(F));
         MG_TRY(enqueue_fp32_step(F, m));
         MG_TRY(enqueue_scales(F));
-        MG_TRY(enqueue_residual(F));
+        MG_TRY(enqueue_residual(F, false, true));
         MG_TRY(enqueue_problem_sums(F));
     }
     return join(B);
@@ -276,7 +276,7 @@ mg_status batch_solve(mg_batch *B, double *u_dev, double rtol, int max_cycles, i
     for (size_t g = 0; g < G; ++g) {
         mg_forest *F = B->groups[g];
         bool zero_guess = false;
-        MG_TRY(pack_initial_guess(F, u_dev, &zero_guess));
+        MG_TRY(pack_initial_guess(F, u_dev, &zero_guess, true));
         fn[g].resize(F->np);
         mult[g].resize(F->np);
         rel[g].assign(F->np, -1.0);
@@ -288,7 +288,7 @@ mg_status batch_solve(mg_batch *B, double *u_dev, double rtol, int max_cycles, i
         }
         set_scales_host(F, mult[g]);
         MG_TRY(enqueue_scales(F));
-        MG_TRY(enqueue_residual(F, zero_guess));  // a zero guess needs no operator: r = f
+        MG_TRY(enqueue_residual(F, zero_guess, false));  // a zero guess needs no operator: r = f
         MG_TRY(enqueue_problem_sums(F));
     }
     MG_TRY(join(B));

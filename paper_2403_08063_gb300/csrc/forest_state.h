@@ -92,6 +92,11 @@ struct DevLevel {
     int64_t cells() const { return static_cast<int64_t>(g.nb) << (3 * g.lg); }
 };
 
+// CTAs of k_update_mixed: one thread per pair of cells in kUpdatePlanes planes.
+inline unsigned update_grid(const DevLevel &d) {
+    return static_cast<unsigned>((d.cells() / (2 * kUpdatePlanes) + kThreads - 1) / kThreads);
+}
+
 // One FP32 level as the persistent tail kernel sees it.
 struct TailLevel {
     LevelGeom g;
@@ -164,7 +169,7 @@ struct mg_forest {
     double *partial = nullptr;  // 2 * kMaxGrid
     double *sums = nullptr;     // 2 doubles on the device
     double *pinned = nullptr;   // 2 doubles, host pinned
-    double *s64a = nullptr, *s64b = nullptr;  // level-0 FP64 scratch pools
+    double *s64a = nullptr;     // level-0 FP64 scratch pool
     double *coarse_r = nullptr;               // coarsest-level scratch pool (operator assembly)
     int *flag = nullptr;                      // input-check flag
     double *gb = nullptr;                     // 2 g on the finest level's boundary faces (mg_set_boundary), or null
@@ -305,8 +310,9 @@ mg_status replay(mg_forest *F, Replay &r, Body &&body) {
     return replay(F, r, body, [] { return true; });
 }
 
-// FP64 operator application A u on a level (ghosts of u already exchanged), defined in solver.cu.
-void apply64(mg_forest *F, DevLevel &d, const double *u, double *out);
+// FP64 operator application A u on a level (ghosts of u already exchanged) into a padded pool, or into a field in the
+// caller's layout (user, level 0), defined in solver.cu.
+void apply64(mg_forest *F, DevLevel &d, const double *u, double *out, bool user = false);
 
 // FP64 ghost exchange of one level on a pool laid out like the level's pools (defined in solver.cu).
 void exchange_any64(mg_forest *F, DevLevel &d, double *u);
@@ -331,7 +337,8 @@ int64_t tail_ctas(mg_forest *F);  // tail.cu: CTAs the largest phase of F's tail
 // solver.cu: one FP32 V-cycle in two parts around a joint tail: part 1 the steps down to the tail level's entry,
 // part 2 the steps after the tail (0: the whole cycle, its tail launched as usual)
 void vcycle32_part(mg_forest *F, int part);
-mg_status enqueue_update_mixed(mg_forest *F);  // solver.cu: u64 += e32 / scale_p
+// solver.cu: u64 += e32 / scale_p (set: u64 = e32 / scale_p), same-level and boundary ghosts written
+mg_status enqueue_update_mixed(mg_forest *F, bool set = false);
 mg_status record_tail(mg_forest *F, int l);   // solver.cu
 mg_status launch_selftest_wait(mg_forest *F, int which);  // tail.cu (F->tail_bar allocated)
 void reset_done(mg_forest *F);
@@ -343,9 +350,10 @@ mg_status set_rhs(mg_forest *F, const double *f_dev, const double *k_dev);
 double pow2_near(double x);
 void set_scales_host(mg_forest *F, const std::vector<double> &mult);
 mg_status enqueue_scales(mg_forest *F);
-// FP64 residual -> FP32 scaled rhs, zeroed correction, per-block sums (zero_u: u is zero, r = f)
-mg_status enqueue_residual(mg_forest *F, bool zero_u = false);
-mg_status pack_initial_guess(mg_forest *F, const double *u_dev, bool *zero);
+// FP64 residual -> FP32 scaled rhs, zeroed correction, per-block sums (zero_u: u is zero, r = f; current: u's same-level and
+// boundary ghosts are)
+mg_status enqueue_residual(mg_forest *F, bool zero_u, bool current);
+mg_status pack_initial_guess(mg_forest *F, const double *u_dev, bool *zero, bool keep_zero);
 mg_status enqueue_problem_sums(mg_forest *F);  // per-problem sums -> pinned psum_h (no synchronisation)
 mg_status enqueue_fp32_step(mg_forest *F, int cycles);  // `cycles` FP32 V-cycles and the FP64 update
 

@@ -2514,16 +2514,31 @@ static __global__ void k_coarse_solve(T *__restrict__ u, const T *__restrict__ f
                          ustart[uprob[first]], ustart[uprob[min(first + warps, N) - 1] + 1], stage);
 }
 
+// The CTA's partial sum: vol times the sum of its threads' FP32 values, in FP64 by the first warp.
+__device__ __forceinline__ void cta_norm(float acc, float vol, double *__restrict__ bpart) {
+    __shared__ float sm[kThreads];
+    sm[threadIdx.x] = acc;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    double s = 0.0;
+#pragma unroll
+    for (int i = 0; i < kThreads / 32; ++i) s += static_cast<double>(sm[threadIdx.x + 32 * i]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) bpart[blockIdx.x] = s * vol;
+}
+
 // ------------------------------------------------------------------------------------------------------------
 // FP64 residual over the finest level, r = f - A u (Sec. 5, Eq. 1), written as FP32 r * scale_p (scale_p a power of two per
 // problem, so the scaling is exact), with the FP32 correction field zeroed, and per-block sums of h^3 (r scale_p)^2.
 // Grid: nb * cpb CTAs, CTA (b, c) covers the c-th of cpb contiguous chunks of block b and writes its partial sum to
 // bpart[b cpb + c] (cleared before the launch, so 0 for a skipped block), which k_problem_sums adds up in a fixed
-// order, so the norm is the same from run to run.  The squared norm is accumulated in FP32 per thread (it decides convergence and is reported to
-// ~1e-6 relative) and in FP64 across threads.  out / zero_out may be null.  ZU: u is known to be zero (a zero
-// initial guess), so r = f without reading u or the operator.
+// order, so the norm is the same from run to run.  The squared norm is accumulated in FP32 per thread (it decides convergence
+// and is reported to ~1e-6 relative) and in FP64 across threads, by one warp per CTA: a CTA has eight cells per thread, and
+// converting and adding across lanes in every warp took an eighth of the FP64 operations, which bound the kernel
+// (512^3: 2.01 -> 1.86 ms).  out / zero_out may be null.
 // ------------------------------------------------------------------------------------------------------------
-template <int MODE, bool ZU = false>
+template <int MODE>
 static __global__ void __launch_bounds__(kThreads, 5) k_residual_norm(const double *__restrict__ u, const double *__restrict__ f, Coef cf,
                                        const double *__restrict__ ih2, const float *__restrict__ vol, LevelGeom g,
                                        int cpb, float *__restrict__ out, const float *__restrict__ pscale,
@@ -2537,12 +2552,10 @@ static __global__ void __launch_bounds__(kThreads, 5) k_residual_norm(const doub
     const int sexp = static_cast<int>((__float_as_uint(pscale[bprob[b]]) >> 23) & 0xff) - 127;  // scale = 2^sexp
     const double ihb = MODE == 1 ? 0.0 : ih2[b];
     float acc = 0.0f;
-    // the zero-guess form is a stream (f in, r and the zeroed correction out): four cells in flight per thread
-#pragma unroll(ZU ? 4 : 1)
     for (int c = chunk * per + threadIdx.x; c < (chunk + 1) * per; c += blockDim.x) {
         const int x = c & (n - 1), y = (c >> lg) & (n - 1), z = c >> (2 * lg);
         const int64_t gi = b * g.bs + off3(x + 1, y + 1, z + 1, P);
-        const double r = ZU ? f[gi] : residual_at<double, MODE>(u, f, cf, gi, P, ihb);  // ZU: u = 0, r = f
+        const double r = residual_at<double, MODE>(u, f, cf, gi, P, ihb);
         const float rs = f64_to_f32_pow2(r, sexp);
         const int64_t gs = Lay<float>::at(g, b, x + 1, y + 1, z + 1);  // FP32 pools are colour-split
         if (out) out[gs] = rs;
@@ -2558,17 +2571,35 @@ static __global__ void __launch_bounds__(kThreads, 5) k_residual_norm(const doub
         }
         acc = fmaf(rs, rs, acc);
     }
-    __shared__ double sm[kThreads / 32];
-    double a = static_cast<double>(acc) * vol[b];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = a;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < kThreads / 32; ++w) s += sm[w];
-        bpart[blockIdx.x] = s;
+    cta_norm(acc, vol[b], bpart);
+}
+
+// The same for u = 0, r = f (a zero initial guess): a stream, two cells of a row per thread, four of those in flight.  The
+// correction and its ghosts are zeroed by the caller.
+static __global__ void __launch_bounds__(kThreads) k_scaled_rhs(const double *__restrict__ f, const float *__restrict__ vol,
+                                                                LevelGeom g, int cpb, float *__restrict__ out,
+                                                                const float *__restrict__ pscale,
+                                                                const int32_t *__restrict__ bprob,
+                                                                double *__restrict__ bpart, Skip skip) {
+    const int lg = g.lg, n = g.n, P = g.P, hp = half_row(P), half = P * P * hp;
+    const int64_t b = blockIdx.x / cpb;
+    if (skip(b)) return;  // the whole CTA: its partial stays 0
+    const int chunk = blockIdx.x - static_cast<int>(b * cpb), per = (1 << (3 * lg - 1)) / cpb;  // pairs per CTA
+    const int sexp = static_cast<int>((__float_as_uint(pscale[bprob[b]]) >> 23) & 0xff) - 127;  // scale = 2^sexp
+    const double *fb = f + b * g.bs;
+    float *ob = out + b * g.bs;
+    float acc = 0.0f;
+#pragma unroll 4
+    for (int c = chunk * per + threadIdx.x; c < (chunk + 1) * per; c += kThreads) {
+        const int j = c & ((n >> 1) - 1), y = (c >> (lg - 1)) & (n - 1), z = c >> (2 * lg - 1);
+        const int row = (z + 1) * P + y + 1, s = (y + z + 1) & 1;  // cell x = 2j: half s at j; x = 2j + 1: the other at j + 1
+        const double *p = fb + static_cast<int64_t>(row) * P + 2 * j + 1;
+        const float r0 = f64_to_f32_pow2(p[0], sexp), r1 = f64_to_f32_pow2(p[1], sexp);
+        ob[s * half + row * hp + j] = r0;
+        ob[(s ^ 1) * half + row * hp + j + 1] = r1;
+        acc = fmaf(r1, r1, fmaf(r0, r0, acc));
     }
+    cta_norm(acc, vol[b], bpart);
 }
 
 // Per-CTA partial sums of h^3 x^2 over the interior of an FP64 field (same grid shape and partials as
@@ -2634,10 +2665,11 @@ static __global__ void __launch_bounds__(kSumThreads) k_problem_sums(const doubl
     }
 }
 
-// A u over a whole level in FP64 (operator application; ghosts already exchanged).
-template <int MODE>
+// A u over a whole level in FP64 (operator application; ghosts already exchanged) into a padded pool, or (USER) straight into
+// a field in the caller's layout, whose leaf b starts at off[b] (null: b n^3).
+template <int MODE, bool USER>
 static __global__ void k_apply64(const double *__restrict__ u, Coef cf, const double *__restrict__ ih2, LevelGeom g,
-                          double *__restrict__ out) {
+                                 double *__restrict__ out, const int64_t *__restrict__ off) {
     const int lg = g.lg, n = g.n, P = g.P;
     const int64_t total = static_cast<int64_t>(g.nb) << (3 * lg);
     for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < total;
@@ -2647,7 +2679,8 @@ static __global__ void k_apply64(const double *__restrict__ u, Coef cf, const do
         const int z = static_cast<int>((t >> (2 * lg)) & (n - 1));
         const int64_t b = t >> (3 * lg);
         const int64_t gi = b * g.bs + off3(x + 1, y + 1, z + 1, P);
-        out[gi] = apply_at<MODE>(u, cf, gi, P, MODE == 1 ? 0.0 : ih2[b]);
+        const int64_t to = !USER ? gi : (off ? off[b] + (t & ((int64_t(1) << (3 * lg)) - 1)) : t);
+        out[to] = apply_at<MODE>(u, cf, gi, P, MODE == 1 ? 0.0 : ih2[b]);
     }
 }
 
@@ -2736,24 +2769,77 @@ static __global__ void k_unpack(double *__restrict__ user, const T *__restrict__
 }
 
 // u64 += e32 / scale_p over the interior (mixed-precision defect correction update, an extension the paper does not
-// have; pinv = 1 / scale_p per problem)
-static __global__ void k_update_mixed(double *__restrict__ u, const float *__restrict__ e,
-                                      const double *__restrict__ pinv, const int32_t *__restrict__ bprob,
-                                      LevelGeom g, Skip skip = Skip{}) {
-    const int lg = g.lg, n = g.n;
-    const int64_t total = static_cast<int64_t>(g.nb) << (3 * lg);
-#pragma unroll 4  // several cells' loads in flight per thread
-    for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < total;
-         t += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int x = static_cast<int>(t & (n - 1));
-        const int y = static_cast<int>((t >> lg) & (n - 1));
-        const int z = static_cast<int>((t >> (2 * lg)) & (n - 1));
-        const int64_t b = t >> (3 * lg);
-        if (skip(b)) continue;
-        const int64_t gi = b * g.bs + off3(x + 1, y + 1, z + 1, g.P);
-        const int pexp = static_cast<int>((static_cast<uint64_t>(__double_as_longlong(pinv[bprob[b]])) >> 52) & 0x7ff) - 1023;
-        u[gi] += f32_to_f64_pow2(e[Lay<float>::at(g, b, x + 1, y + 1, z + 1)], pexp);  // pinv = 2^pexp: exact
+// have; pinv = 1 / scale_p per problem), or u64 = e32 / scale_p (SET: the first update of a zero guess, which then needs no
+// zeroed pool).  Block-face cells are written through to the ghosts that mirror or reflect them, so the next residual
+// exchanges refinement interfaces only (512^3: a full FP64 exchange of 175 us per step).
+// One thread per pair of cells of a row in kUpdatePlanes planes, all loads first (one pair per thread: 834 instead of 654 us
+// at 512^3, bound by the turnover of CTAs; the branches of the write-through in a loop over single cells: 1174 us).
+constexpr int kUpdatePlanes = 4;
+template <bool SET>
+static __global__ void __launch_bounds__(kThreads) k_update_mixed(double *__restrict__ u, const float *__restrict__ e,
+                                                                  const double *__restrict__ pinv,
+                                                                  const int32_t *__restrict__ bprob, LevelGeom g,
+                                                                  const int32_t *__restrict__ nbr6,
+                                                                  const double *__restrict__ gb, Skip skip) {
+    constexpr int ZC = kUpdatePlanes, LZ = 2;
+    const int lg = g.lg, n = g.n, P = g.P, hp = half_row(P);
+    const int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    const int64_t b = t >> (3 * lg - 1 - LZ);
+    if (b >= g.nb || skip(b)) return;
+    const int j = static_cast<int>(t) & ((n >> 1) - 1), y = static_cast<int>(t >> (lg - 1)) & (n - 1);
+    const int z0 = (static_cast<int>(t >> (2 * lg - 1)) & ((n >> LZ) - 1)) << LZ;
+    const int64_t PP = static_cast<int64_t>(P) * P, half = PP * hp, row0 = (z0 + 1) * static_cast<int64_t>(P) + y + 1;
+    const float *eb = e + b * g.bs + row0 * hp + j;
+    double *ub = u + b * g.bs + row0 * P + 2 * j + 1;
+    const int pexp = static_cast<int>((static_cast<uint64_t>(__double_as_longlong(pinv[bprob[b]])) >> 52) & 0x7ff) - 1023;
+    double v[ZC][2];
+#pragma unroll
+    for (int k = 0; k < ZC; ++k) {  // cell x = 2j: half s; x = 2j + 1: the other half, one further
+        const int s = (y + z0 + k + 1) & 1;
+        const float *p = eb + k * static_cast<int64_t>(P) * hp;
+        v[k][0] = f32_to_f64_pow2(p[s * half], pexp);  // exact
+        v[k][1] = f32_to_f64_pow2(p[(s ^ 1) * half + 1], pexp);
+        if (!SET) {
+            v[k][0] = ub[k * PP] + v[k][0];
+            v[k][1] = ub[k * PP + 1] + v[k][1];
+        }
     }
+#pragma unroll
+    for (int k = 0; k < ZC; ++k) {
+        ub[k * PP] = v[k][0];
+        ub[k * PP + 1] = v[k][1];
+    }
+    const bool xf = j == 0 || j == (n >> 1) - 1, yf = y == 0 || y == n - 1, zf = z0 == 0 || z0 + ZC == n;
+    if (!xf && !yf && !zf) return;
+#pragma unroll
+    for (int k = 0; k < ZC; ++k) {
+        const int z = z0 + k;
+        const auto through = [&](int axis, int side, int a) {  // cell (2j + a, y, z), on that face
+            const int nb = nbr6[b * 6 + 2 * axis + side], x = 2 * j + a;
+            const int64_t st = axis == 0 ? 1 : (axis == 1 ? P : PP), q = row0 * P + k * PP + x + 1;
+            const int i1 = axis == 0 ? y : x, i2 = axis == 2 ? y : z;
+            if (nb >= 0) u[nb * g.bs + q + (side ? -n : n) * st] = v[k][a];
+            else if (nb == -1)
+                u[b * g.bs + q + (side ? st : -st)] =
+                    gb ? gb[(b * 6 + 2 * axis + side) * static_cast<int64_t>(n) * n + i2 * n + i1] - v[k][a] : -v[k][a];
+        };
+        if (j == 0) through(0, 0, 0);
+        if (j == (n >> 1) - 1) through(0, 1, 1);
+        if (yf)
+            for (int a = 0; a < 2; ++a) through(1, y != 0, a);
+        if (z == 0 || z == n - 1)
+            for (int a = 0; a < 2; ++a) through(2, z != 0, a);
+    }
+}
+
+// Whether any entry of x is not zero (NaN counts).
+static __global__ void k_any_nonzero(const double *__restrict__ x, int64_t count, int *__restrict__ flag) {
+    bool any = false;
+#pragma unroll 8
+    for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < count;
+         t += static_cast<int64_t>(gridDim.x) * blockDim.x)
+        any |= !(x[t] == 0.0);
+    if (__ballot_sync(0xffffffffu, any) && (threadIdx.x & 31) == 0) atomicOr(flag, 1);
 }
 
 // Face coefficients of a level from k with ghosts (variable coefficients: future work in Sec. 8; harmonic-mean

@@ -752,23 +752,26 @@ mg_status enqueue_problem_sums(mg_forest *F) {
 // Level-0 FP64 residual r = f - A u (exchange first); optionally written as FP32 r * scale_p with the FP32
 // correction zeroed; returns ||r_p||^2 (volume-weighted, per problem) to rr when rr is not null.  scale_p (set by
 // upload_scales, mult) is a power of two close to 1 / ||r_p|| so the FP32 values stay near unit size.
+// zero_u: u is zero, r = f; current: u's same-level and boundary ghosts are (k_update_mixed wrote them).
 template <int MODE>
 mg_status residual64(mg_forest *F, double *u, const double *f, float *out, float *zero_out,
-                     const std::vector<double> &mult, std::vector<double> *rr, bool zero_u = false) {
+                     const std::vector<double> &mult, std::vector<double> *rr, bool zero_u = false,
+                     bool current = false) {
     DevLevel &d = F->L[0];
-    if (!zero_u) exchange<double, MODE>(F, d, u);
+    if (!zero_u) exchange<double, MODE>(F, d, u, current);
     const int cpb = chunks_per_block(d);
     MG_CUDA(cudaMemsetAsync(F->bsum, 0, static_cast<size_t>(d.g.nb) * cpb * sizeof(double), F->st));
     {
         Prof p(F, P_RESID64, 1);
-        if (zero_u)
-            k_residual_norm<MODE, true><<<d.g.nb * cpb, kThreads, 0, F->st>>>(
-                u, f, d.c64(), d.ih2_64, d.vol_32, d.g, cpb, out, F->pscale, d.bprob, F->bsum, zero_out,
-                skip_of(F, d));
-        else
+        if (zero_u) {
+            MG_CUDA(cudaMemsetAsync(zero_out, 0, d.pool_elems() * sizeof(float), F->st));
+            k_scaled_rhs<<<d.g.nb * cpb, kThreads, 0, F->st>>>(f, d.vol_32, d.g, cpb, out, F->pscale, d.bprob, F->bsum,
+                                                               skip_of(F, d));
+        } else {
             k_residual_norm<MODE><<<d.g.nb * cpb, kThreads, 0, F->st>>>(u, f, d.c64(), d.ih2_64, d.vol_32, d.g, cpb,
                                                                         out, F->pscale, d.bprob, F->bsum, zero_out,
                                                                         skip_of(F, d));
+        }
     }
     if (rr) {
         MG_TRY(read_problem_sums(F));
@@ -785,11 +788,10 @@ mg_status residual64_any(mg_forest *F, double *u, const double *f, const std::ve
     return residual64<0>(F, u, f, nullptr, nullptr, mult, rr);
 }
 
-void apply64(mg_forest *F, DevLevel &d, const double *u, double *out) {
-    if (F->cfg.coeff)
-        k_apply64<1><<<grid_for(d.cells()), kThreads, 0, F->st>>>(u, d.c64(), d.ih2_64, d.g, out);
-    else
-        k_apply64<0><<<grid_for(d.cells()), kThreads, 0, F->st>>>(u, d.c64(), d.ih2_64, d.g, out);
+void apply64(mg_forest *F, DevLevel &d, const double *u, double *out, bool user) {
+    auto *fn = F->cfg.coeff ? (user ? k_apply64<1, true> : k_apply64<1, false>)
+                            : (user ? k_apply64<0, true> : k_apply64<0, false>);
+    fn<<<grid_for(d.cells()), kThreads, 0, F->st>>>(u, d.c64(), d.ih2_64, d.g, out, F->leaf_off);
 }
 
 // The device part of assemble_coarse: the columns A e_m of every problem's coarsest operator (FP64 kernels on unit
@@ -1075,58 +1077,64 @@ double pow2_near(double x) {
 
 // Mixed precision, first half of a defect-correction step: r64 = f - A u (FP64), stored as FP32 r * scale_p
 // with the FP32 correction zeroed; per-problem ||r||^2 to rr.
-mg_status mixed_step(mg_forest *F, const std::vector<double> &mult, std::vector<double> *rr, bool zero_u) {
+mg_status mixed_step(mg_forest *F, const std::vector<double> &mult, std::vector<double> *rr, bool zero_u, bool current) {
     DevLevel &d = F->L[0];
     MG_TRY(upload_scales(F, mult));
     if (F->cfg.coeff)
-        MG_TRY((residual64<1>(F, d.u64, d.f64, d.f32, d.u32, mult, rr, zero_u)));
+        MG_TRY((residual64<1>(F, d.u64, d.f64, d.f32, d.u32, mult, rr, zero_u, current)));
     else
-        MG_TRY((residual64<0>(F, d.u64, d.f64, d.f32, d.u32, mult, rr, zero_u)));
+        MG_TRY((residual64<0>(F, d.u64, d.f64, d.f32, d.u32, mult, rr, zero_u, current)));
     return MG_OK;
 }
 
 // The residual half of a defect-correction step without host synchronisation (graph-capturable).
-mg_status enqueue_residual(mg_forest *F, bool zero_u) {
+mg_status enqueue_residual(mg_forest *F, bool zero_u, bool current) {
     DevLevel &d = F->L[0];
     static const std::vector<double> none;
-    if (F->cfg.coeff) return residual64<1>(F, d.u64, d.f64, d.f32, d.u32, none, nullptr, zero_u);
-    return residual64<0>(F, d.u64, d.f64, d.f32, d.u32, none, nullptr, zero_u);
+    if (F->cfg.coeff) return residual64<1>(F, d.u64, d.f64, d.f32, d.u32, none, nullptr, zero_u, current);
+    return residual64<0>(F, d.u64, d.f64, d.f32, d.u32, none, nullptr, zero_u, current);
 }
 
-// Packs the caller's u into the level-0 FP64 pool and reports whether it is all zero (one read-back).
-mg_status pack_initial_guess(mg_forest *F, const double *u_dev, bool *zero) {
+// Reports whether the caller's u is all zero (one read-back) and packs it into the level-0 FP64 pool; with keep_zero a zero
+// one too.
+mg_status pack_initial_guess(mg_forest *F, const double *u_dev, bool *zero, bool keep_zero) {
     DevLevel &d = F->L[0];
     MG_CUDA(cudaMemsetAsync(F->flag, 0, sizeof(int), F->st));
-    {
+    if (keep_zero) {
         Prof p(F, P_LAYOUT, 1);
         k_pack<double><<<grid_for(d.cells()), kThreads, 0, F->st>>>(d.u64, u_dev, d.g, F->leaf_off, F->flag);
+    } else {
+        Prof p(F, P_LAYOUT, 1);
+        k_any_nonzero<<<grid_for(d.cells()), kThreads, 0, F->st>>>(u_dev, d.cells(), F->flag);
     }
     int h = 1;
     MG_CUDA(cudaMemcpyAsync(&h, F->flag, sizeof(int), cudaMemcpyDeviceToHost, F->st));
     MG_CUDA(cudaStreamSynchronize(F->st));
     *zero = h == 0;
+    if (!keep_zero && h) MG_TRY(pack_user<double>(F, d, d.u64, u_dev));
     return MG_OK;
 }
 
 // Second half: `cycles` FP32 V-cycles on the scaled residual, then u64 += e32 / scale_p (exact).
-mg_status enqueue_update_mixed(mg_forest *F) {
+mg_status enqueue_update_mixed(mg_forest *F, bool set) {
     DevLevel &d = F->L[0];
     Prof p(F, P_UPDATE, 1);
-    k_update_mixed<<<grid_for(d.cells()), kThreads, 0, F->st>>>(d.u64, d.u32, F->pinv, d.bprob, d.g, skip_of(F, d));
+    auto *fn = set ? k_update_mixed<true> : k_update_mixed<false>;
+    fn<<<update_grid(d), kThreads, 0, F->st>>>(d.u64, d.u32, F->pinv, d.bprob, d.g, d.nbr6, F->gb,
+                                             set ? Skip{} : skip_of(F, d));  // set: u = 0 where e is still 0
     MG_CUDA(cudaGetLastError());
     return MG_OK;
 }
 
 // `cycles` FP32 V-cycles, each the recorded one (mg_set_smoother_shape and mg_set_tail drop it), and the update.
-mg_status finish_mixed_cycle(mg_forest *F, int cycles) {
+mg_status finish_mixed_cycle(mg_forest *F, int cycles, bool set) {
     for (int i = 0; i < cycles; ++i) MG_TRY(replay(F, F->v32_rec, [&] { vcycle32(F); }));
-    return enqueue_update_mixed(F);
+    return enqueue_update_mixed(F, set);
 }
 
-// Level-0 FP64 scratch pools (operator application, gradients), allocated on first use.
+// Level-0 FP64 scratch pool (operator application, gradients), allocated on first use.
 mg_status ensure_scratch64(mg_forest *F) {
     if (!F->s64a) MG_TRY(dalloc(F, &F->s64a, F->L[0].pool_elems()));
-    if (!F->s64b) MG_TRY(dalloc(F, &F->s64b, F->L[0].pool_elems()));
     return MG_OK;
 }
 
@@ -1174,8 +1182,11 @@ mg_status run_cycles(mg_forest *F, double *u_dev, double rtol, int max_cycles, i
     MG_TRY(check_ready(F));
     DevLevel &d = F->L[0];
     const int np = F->np;
+    // FP32 cycles from a zero guess (g = 0) need no packed u: r = f, and the first update writes u
+    const bool lazy = F->cfg.precision == 1 && !F->gb && !F->leaf_off;
     bool zero_guess = false;
-    MG_TRY(pack_initial_guess(F, u_dev, &zero_guess));
+    MG_TRY(pack_initial_guess(F, u_dev, &zero_guess, !lazy));
+    bool unset = lazy && zero_guess;  // u64 does not hold u yet
     reset_done(F);
     std::vector<double> fn(np), rel(np, -1.0), mult(np), rr(np, 0.0);
     std::vector<int32_t> met(np, -1);
@@ -1217,20 +1228,21 @@ mg_status run_cycles(mg_forest *F, double *u_dev, double rtol, int max_cycles, i
             }
         }
     } else {
-        MG_TRY(mixed_step(F, mult, &rr, zero_guess && !F->gb));  // a zero guess (g = 0) needs no operator: r = f
+        MG_TRY(mixed_step(F, mult, &rr, unset, false));
         auto st = update_rel(0);
         finite = st.second;
         const int inner = std::max(1, F->cfg.inner_cycles);
         while (finite && done < max_cycles && !st.first) {
             const int m = std::min(inner, max_cycles - done);
-            MG_TRY(finish_mixed_cycle(F, m));
+            MG_TRY(finish_mixed_cycle(F, m, unset));
+            unset = false;
             done += m;
-            MG_TRY(mixed_step(F, mult, &rr, false));
+            MG_TRY(mixed_step(F, mult, &rr, false, true));
             st = update_rel(done);
             finite = st.second;
         }
     }
-    MG_TRY(unpack_user<double>(F, d, u_dev, d.u64));
+    if (!unset) MG_TRY(unpack_user<double>(F, d, u_dev, d.u64));  // else no step ran: the caller's u is the zero it was
     reset_done(F);
     MG_CUDA(cudaStreamSynchronize(F->st));
     if (F->cfg.precision == 1) MG_TRY(check_kernel_waits(F));
@@ -1590,8 +1602,8 @@ mg_status apply_op(mg_forest *F, const double *u_dev, double *Au_dev) {
     MG_TRY(ensure_scratch64(F));
     MG_TRY(pack_user<double>(F, d, F->s64a, u_dev));
     exchange_any64(F, d, F->s64a);
-    apply64(F, d, F->s64a, F->s64b);
-    MG_TRY(unpack_user<double>(F, d, Au_dev, F->s64b));
+    apply64(F, d, F->s64a, Au_dev, true);
+    MG_CUDA(cudaGetLastError());
     return MG_OK;
 }
 
