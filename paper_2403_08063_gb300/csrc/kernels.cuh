@@ -856,7 +856,7 @@ __device__ __forceinline__ void smooth32_column(float *__restrict__ u, const flo
     constexpr int SH = 3 * LG - 1 - LZ;  // log2(columns per block)
     const int r = static_cast<int>(t) & ((1 << SH) - 1);
     const int64_t b = t >> SH;
-    if (skip(b)) return;
+    const bool masked = skip(b);  // decided after the column's loads are on their way: its own two are a chain
     const int j = r & (NH - 1);
     const int y = (r >> (LG - 1)) & (n - 1);
     const int z0 = (r >> (2 * LG - 1)) << LZ;
@@ -915,6 +915,7 @@ __device__ __forceinline__ void smooth32_column(float *__restrict__ u, const flo
         }
     }
     const float hb = __ldg(h2 + b), hh = 0.5f * hb;  // T_f = 2 / (kap_i + kap_f): its 2 cancels against h^2 / 2
+    if (masked) return;
     // ---- updates -----------------------------------------------------------------------------------
     float val[ZC];
 #pragma unroll
@@ -1674,7 +1675,7 @@ __device__ __forceinline__ void residual_restrict32_body(
     for (int64_t t = t0; t < total; t += ts) {
         const int r = static_cast<int>(t) & ((1 << (3 * LC)) - 1);
         const int64_t B = t >> (3 * LC);
-        if (skip(B)) continue;  // the coarse level's problem ids
+        const bool masked = skip(B);  // the coarse level's problem ids; decided after the loads
         const int X = r & (nc - 1), Y = (r >> LC) & (nc - 1), Z = r >> (2 * LC);
         const int64_t b = xf[B].src[0];
         const int64_t corner = b * bsf + (2 * Z * Bx::P + 2 * Y) * Bx::HP + X;
@@ -1709,6 +1710,7 @@ __device__ __forceinline__ void residual_restrict32_body(
         const float sum = rr32_sum<MODE>(U, K, AX, AY, AZ, ih2, [&](int i, int j, int k) {
             return ldr<CG>(f + corner + Bx::off(i, j, k));
         });
+        if (masked) continue;
         rr32_store<LG>(fc, uc, B, bsc, X, Y, Z, sum);
     }
 }
@@ -2104,7 +2106,7 @@ __device__ __forceinline__ void prolong32_body(float *__restrict__ uf, int64_t b
     for (int64_t t = t0; t < total; t += ts) {
         const int r = static_cast<int>(t) & ((1 << (3 * LC)) - 1);
         const int64_t B = t >> (3 * LC);
-        if (skip(B)) continue;
+        const bool masked = skip(B);  // decided after the loads
         const int X = r & (nc - 1), Y = (r >> LC) & (nc - 1), Z = r >> (2 * LC);
         const int Xc = X + 1, Yc = Y + 1, Zc = Z + 1;
         const int pc = (Xc + Yc + Zc) & 1;
@@ -2132,6 +2134,7 @@ __device__ __forceinline__ void prolong32_body(float *__restrict__ uf, int64_t b
                 for (int a = 0; a < 2; ++a)
                     val[c][bb][a] = ldv<CG>(ub + Bx::off(a + 1, bb + 1, c + 1)) +
                                     (INJ ? 0.125f * e0 : 0.25f * ((e0 + ex[a]) + (ey[bb] + ez[c])));
+        if (masked) continue;
         prolong32_put<LG>(uf, bsf, b, X, Y, Z, val, nbr6);
     }
 }
@@ -2163,7 +2166,8 @@ static __global__ void __launch_bounds__(256) k_prolong32z(float *__restrict__ u
     static_assert(nc % ZC == 0 && (ZC & (ZC - 1)) == 0, "ZC: a power of two dividing the coarse edge");
     constexpr int LS = LC - (ZC == 1 ? 0 : ZC == 2 ? 1 : ZC == 4 ? 2 : 3);  // log2 of the segments per column
     static_assert(ZC <= 8, "ZC up to 8");
-    const int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    // backwards, so that the first colour after it finds the blocks it starts with in L2
+    const int64_t t = (gridDim.x - 1 - blockIdx.x) * static_cast<int64_t>(blockDim.x) + threadIdx.x;
     if (t >= (static_cast<int64_t>(nbc) << (2 * LC + LS))) return;
     const int X = static_cast<int>(t) & (nc - 1), Y = static_cast<int>(t >> LC) & (nc - 1);
     const int seg = static_cast<int>(t >> (2 * LC)) & ((1 << LS) - 1);
@@ -2879,9 +2883,10 @@ static __global__ void k_face_coefs(const double *__restrict__ k, const double *
                 rb = 1.0 / sb;
                 rd = 1.0 / sd;
             }
-            if (wx) tx[gi] = 2.0 * ka * kc * ra * s;
-            if (wy) ty[gi] = 2.0 * kb * kc * rb * s;
-            if (wz) tz[gi] = 2.0 * kd * kc * rd * s;
+            const double ks = 2.0 * s * kc;
+            if (wx) tx[gi] = ka * ra * ks;
+            if (wy) ty[gi] = kb * rb * ks;
+            if (wz) tz[gi] = kd * rd * ks;
         }
         const bool face_or_interior = (inX && inY) || (inX && inZ) || (inY && inZ);
         // 1/k for the FP32 cycles: FP32 accuracy suffices (binary32 conversion on exponent bits, FP32 division)

@@ -791,7 +791,9 @@ mg_status residual64_any(mg_forest *F, double *u, const double *f, const std::ve
 void apply64(mg_forest *F, DevLevel &d, const double *u, double *out, bool user) {
     auto *fn = F->cfg.coeff ? (user ? k_apply64<1, true> : k_apply64<1, false>)
                             : (user ? k_apply64<0, true> : k_apply64<0, false>);
-    fn<<<grid_for(d.cells()), kThreads, 0, F->st>>>(u, d.c64(), d.ih2_64, d.g, out, F->leaf_off);
+    // one cell per thread: a grid-stride loop's last round kept a quarter of the SMs busy
+    fn<<<static_cast<unsigned>((d.cells() + kThreads - 1) / kThreads), kThreads, 0, F->st>>>(u, d.c64(), d.ih2_64, d.g, out,
+                                                                                            F->leaf_off);
 }
 
 // The device part of assemble_coarse: the columns A e_m of every problem's coarsest operator (FP64 kernels on unit
