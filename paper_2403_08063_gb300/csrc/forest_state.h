@@ -73,7 +73,6 @@ struct DevLevel {
     int nifaces = 0;
     FaceItem *sfaces = nullptr;  // the other faces: boundary and same level
     int nsfaces = 0;
-    int8_t *fkind = nullptr;   // per block face (b * 6 + 2 * axis + side): 0 boundary, 1 same, 2 C2F, 3 F2C
     bool all_halve = false;  // every block of the next level is a halved block of this one
     // FP32 smoother launch shape (kind, parameters): {1, ZC, threads, 0, 0} k_smooth32, {2, TY, TZ, D, R}
     // k_smooth32t; kind 0 = not chosen yet
@@ -148,6 +147,7 @@ struct Replay {
     cudaGraphExec_t exec = nullptr;
     int runs = 0;
     bool off = false;  // the recording failed or cannot be replayed: launched directly
+    int64_t nlaunch[32] = {};  // its launches per kernel family, counted at every replay
     void drop() {
         if (exec) cudaGraphExecDestroy(exec);
         exec = nullptr;
@@ -284,12 +284,18 @@ mg_status replay(mg_forest *F, Replay &r, Body &&body, Ok &&recorded) {
         if (e == cudaSuccess) e = cudaStreamBeginCapture(F->cap_st, cudaStreamCaptureModeThreadLocal);
         bool ok = false;
         if (e == cudaSuccess) {
+            int64_t before[32];
+            std::copy(F->nlaunch, F->nlaunch + 32, before);
             cudaStream_t own = F->st;
             F->st = F->cap_st;
             body();
             F->st = own;
             e = cudaStreamEndCapture(F->cap_st, &graph);
             ok = recorded();
+            for (int c = 0; c < 32; ++c) {
+                r.nlaunch[c] = F->nlaunch[c] - before[c];
+                F->nlaunch[c] = before[c];
+            }
         }
         if (e == cudaSuccess && graph && ok) e = cudaGraphInstantiate(&r.exec, graph, 0);
         if (graph) cudaGraphDestroy(graph);
@@ -303,6 +309,7 @@ mg_status replay(mg_forest *F, Replay &r, Body &&body, Ok &&recorded) {
         }
     }
     MG_CUDA(cudaGraphLaunch(r.exec, F->st));
+    for (int c = 0; c < 32; ++c) F->nlaunch[c] += r.nlaunch[c];
     return MG_OK;
 }
 template <class Body>

@@ -1334,12 +1334,6 @@ mg_status create(const mg_config *cfg, mg_forest **out) {
         d.nfaces = static_cast<int>(h.faces.size());
         d.nsegs = static_cast<int>(h.segs.size());
         if ((st = upload(F, &d.faces, h.faces)) != MG_OK) return fail(st);
-        {
-            std::vector<int8_t> fk(static_cast<size_t>(h.keys.size()) * 6, 0);
-            for (const FaceItem &fi : h.faces) fk[static_cast<size_t>(fi.blk) * 6 + 2 * fi.axis + fi.side] = fi.kind;
-            for (const SegItem &si : h.segs) fk[static_cast<size_t>(si.coarse) * 6 + 2 * si.axis + si.side] = 3;
-            if ((st = upload(F, &d.fkind, fk)) != MG_OK) return fail(st);
-        }
         if ((st = upload(F, &d.segs, h.segs)) != MG_OK) return fail(st);
         {
             std::vector<int32_t> bp(h.keys.size());
