@@ -337,9 +337,9 @@ mg_status launch_batch_tail32(mg_forest *const *groups, const octmg::TailArgs *a
 bool coarse_jacobi_fits(const mg_forest *F, const DevLevel &d);
 void launch_coarse_jacobi(mg_forest *F, DevLevel &d, int iters);
 // gauss_jordan.cu: inverses of the coarsest operators (input buffer, panel width, launches)
-double *gj_input(mg_forest *F, int maxN);
-int gj_width(int maxN);
-void enqueue_gauss_jordan(mg_forest *F, int maxN);
+double *gj_input(mg_forest *F, int maxN, bool dominant);
+int gj_width(int maxN, bool dominant);
+void enqueue_gauss_jordan(mg_forest *F, int maxN, bool dominant);
 int64_t tail_ctas(mg_forest *F);  // tail.cu: CTAs the largest phase of F's tail can use
 // solver.cu: one FP32 V-cycle in two parts around a joint tail: part 1 the steps down to the tail level's entry,
 // part 2 the steps after the tail (0: the whole cycle, its tail launched as usual)

@@ -798,9 +798,10 @@ void apply64(mg_forest *F, DevLevel &d, const double *u, double *out, bool user)
 
 // The device part of assemble_coarse: the columns A e_m of every problem's coarsest operator (FP64 kernels on unit
 // vectors, all problems probed at once), then Gauss-Jordan on the device into Ainv and AinvT (transposes; gauss_jordan.cu).
-void enqueue_coarse_inverse(mg_forest *F, DevLevel &d, int N, int maxN) {
+// dominant: without row exchanges, for the 7-point rows of a level without interfaces (symmetric, diagonally dominant).
+void enqueue_coarse_inverse(mg_forest *F, DevLevel &d, int N, int maxN, bool dominant) {
     double *r = F->coarse_r;
-    double *Adev = gj_input(F, maxN);
+    double *Adev = gj_input(F, maxN, dominant);
     cudaMemsetAsync(d.u64, 0, d.pool_elems() * sizeof(double), F->st);
     if (F->pnbu) {  // no refinement interface: the 7-point rows
         cudaMemsetAsync(Adev, 0, F->moff_h[F->np] * sizeof(double), F->st);
@@ -817,7 +818,7 @@ void enqueue_coarse_inverse(mg_forest *F, DevLevel &d, int N, int maxN) {
         }
     }
     cudaMemsetAsync(F->flag, 0, sizeof(int), F->st);
-    enqueue_gauss_jordan(F, maxN);
+    enqueue_gauss_jordan(F, maxN, dominant);
     cudaMemsetAsync(d.u64, 0, d.pool_elems() * sizeof(double), F->st);
 }
 
@@ -910,7 +911,7 @@ mg_status assemble_coarse(mg_forest *F) {
     int maxN = 0;
     for (int p = 0; p < F->np; ++p) maxN = std::max<int>(maxN, static_cast<int>(F->ustart_h[p + 1] - F->ustart_h[p]));
     if (!F->gj_src) {
-        MG_TRY(dalloc(F, &F->gj_panel, static_cast<int64_t>(N) * gj_width(maxN)));
+        MG_TRY(dalloc(F, &F->gj_panel, static_cast<int64_t>(N) * gj_width(maxN, F->pnbu != nullptr)));
         MG_TRY(dalloc(F, &F->gj_org, 2 * static_cast<int64_t>(N)));
         MG_TRY(dalloc(F, &F->gj_src, N));
     }
@@ -919,13 +920,22 @@ mg_status assemble_coarse(mg_forest *F) {
     const bool prof = F->prof;
     F->gb = nullptr;
     F->prof = false;
-    const mg_status st = replay(F, F->coarse_rec, [&] { enqueue_coarse_inverse(F, d, N, maxN); });
+    const bool dominant = F->pnbu != nullptr;
+    int hbad = 0;
+    const auto invert = [&](bool diagonal) -> mg_status {
+        if (diagonal || !dominant)
+            MG_TRY(replay(F, F->coarse_rec, [&] { enqueue_coarse_inverse(F, d, N, maxN, diagonal); }));
+        else
+            enqueue_coarse_inverse(F, d, N, maxN, false);
+        MG_CUDA(cudaMemcpyAsync(&hbad, F->flag, sizeof(int), cudaMemcpyDeviceToHost, F->st));
+        MG_CUDA(cudaStreamSynchronize(F->st));
+        return MG_OK;
+    };
+    mg_status st = invert(dominant);
+    if (st == MG_OK && hbad && dominant) st = invert(false);  // a diagonal pivot cancelled: search for pivots
     F->gb = gb;
     F->prof = prof;
     MG_TRY(st);
-    int hbad = 0;
-    MG_CUDA(cudaMemcpyAsync(&hbad, F->flag, sizeof(int), cudaMemcpyDeviceToHost, F->st));
-    MG_CUDA(cudaStreamSynchronize(F->st));
     if (hbad) {
         set_error("a coarsest-level operator is singular");
         return MG_ERR_INVALID_ARG;

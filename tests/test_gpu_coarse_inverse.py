@@ -65,3 +65,67 @@ def test_problems_with_different_unknowns():
         assert torch.equal(v, u[starts[p]:starts[p + 1]])
         G.close()
     F.close()
+
+
+def _dense(F, shape):
+    """The operator's matrix, a column per unit vector."""
+    n = shape[0] * shape[1]
+    A = torch.empty((n, n), dtype=torch.float64, device="cuda")
+    e = torch.zeros(shape, dtype=torch.float64, device="cuda")
+    for m in range(n):
+        e.view(-1)[m] = 1.0
+        A[:, m] = F.apply(e).view(-1)
+        e.view(-1)[m] = 0.0
+    return A
+
+
+@pytest.mark.parametrize("R,sigma", [(1, 1.0), (2, 3.0), (3, 1.0)])
+def test_direct_solve_with_rough_coefficients(R, sigma):
+    """A symmetric, diagonally dominant operator (no interface) is eliminated without row exchanges: the bound above, with
+    the condition number of the assembled matrix."""
+    from paper_2403_08063_gb300 import Forest
+    keys = _uniform(R)
+    N, shape = 64 * len(keys), (len(keys), 64)
+    rng = np.random.default_rng(7)
+    F = Forest(R, 4, keys, coeff=True, max_coarse=N)
+    f = torch.from_numpy(rng.normal(size=shape)).cuda()
+    F.set_rhs(f, torch.from_numpy(np.exp(sigma * rng.normal(size=shape))).cuda())
+    u = torch.zeros_like(f)
+    F.vcycle(u, 1)
+    s = torch.linalg.svdvals(_dense(F, shape).cpu())
+    assert float((F.apply(u) - f).norm() / f.norm()) <= 4 * N * EPS * float(s[0] / s[-1])
+    F.close()
+
+
+def test_coefficients_beyond_binary64_contrast_are_still_accepted():
+    """Two neighbouring cells of k = 2^66 among cells of k = 1: the other faces are lost in their diagonals, the second of the
+    two has no diagonal pivot left, and the elimination exchanges rows as it does for other matrices."""
+    from paper_2403_08063_gb300 import Forest
+    keys = _uniform(1)
+    k = torch.ones((1, 64), dtype=torch.float64, device="cuda")
+    k[0, 21:23] = 2.0 ** 66
+    F = Forest(1, 4, keys, coeff=True)
+    F.set_rhs(torch.ones_like(k), k)
+    u = torch.zeros_like(k)
+    F.vcycle(u, 1)
+    assert bool(torch.isfinite(u).all())
+    k.fill_(1.0)  # and the next coefficients are inverted as usual
+    F.set_rhs(torch.ones_like(k), k)
+    u.zero_()
+    F.vcycle(u, 1)
+    assert float((F.apply(u) - 1.0).norm() / 8.0) <= 4 * 64 * EPS * (8 / math.pi) ** 2
+    F.close()
+
+
+def test_narrow_panels_search_for_pivots():
+    """More unknowns than one cluster's shared memory takes in panels of 16, with interfaces: panels of 4."""
+    from paper_2403_08063_gb300 import Forest
+    keys = one_refined_root(6)
+    N = 64 * len(keys)
+    F = Forest(6, 4, keys, max_coarse=N)
+    f = torch.from_numpy(np.random.default_rng(8).normal(size=(len(keys), 64))).cuda()
+    F.set_rhs(f)
+    u = torch.zeros_like(f)
+    F.vcycle(u, 1)
+    assert float((F.apply(u) - f).norm() / f.norm()) <= 4 * N * EPS * (2 * 48 / math.pi) ** 2
+    F.close()
