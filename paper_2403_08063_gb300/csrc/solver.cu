@@ -798,10 +798,9 @@ void apply64(mg_forest *F, DevLevel &d, const double *u, double *out, bool user)
 
 // The device part of assemble_coarse: the columns A e_m of every problem's coarsest operator (FP64 kernels on unit
 // vectors, all problems probed at once), then Gauss-Jordan on the device into Ainv and AinvT (transposes; gauss_jordan.cu).
-// dominant: without row exchanges, for the 7-point rows of a level without interfaces (symmetric, diagonally dominant).
-void enqueue_coarse_inverse(mg_forest *F, DevLevel &d, int N, int maxN, bool dominant) {
+void enqueue_coarse_inverse(mg_forest *F, DevLevel &d, int N, int maxN, GjPivots pivots) {
     double *r = F->coarse_r;
-    double *Adev = gj_input(F, maxN, dominant);
+    double *Adev = gj_input(F, maxN, pivots);
     cudaMemsetAsync(d.u64, 0, d.pool_elems() * sizeof(double), F->st);
     if (F->pnbu) {  // no refinement interface: the 7-point rows
         cudaMemsetAsync(Adev, 0, F->moff_h[F->np] * sizeof(double), F->st);
@@ -818,7 +817,7 @@ void enqueue_coarse_inverse(mg_forest *F, DevLevel &d, int N, int maxN, bool dom
         }
     }
     cudaMemsetAsync(F->flag, 0, sizeof(int), F->st);
-    enqueue_gauss_jordan(F, maxN, dominant);
+    enqueue_gauss_jordan(F, maxN, pivots);
     cudaMemsetAsync(d.u64, 0, d.pool_elems() * sizeof(double), F->st);
 }
 
@@ -910,8 +909,14 @@ mg_status assemble_coarse(mg_forest *F) {
     if (!F->coarse_r) MG_TRY(dalloc(F, &F->coarse_r, d.pool_elems()));
     int maxN = 0;
     for (int p = 0; p < F->np; ++p) maxN = std::max<int>(maxN, static_cast<int>(F->ustart_h[p + 1] - F->ustart_h[p]));
+    const GjPivots pivots = F->pnbu ? GJ_DIAGONAL : GJ_SEARCH;
     if (!F->gj_src) {
-        MG_TRY(dalloc(F, &F->gj_panel, static_cast<int64_t>(N) * gj_width(maxN, F->pnbu != nullptr)));
+        std::vector<int8_t> sym(static_cast<size_t>(F->np), 1);  // the problems without interfaces
+        for (const FaceItem &fi : hl.faces)
+            if (fi.kind != FK_SAME && fi.kind != FK_BND) sym[hl.keys[fi.blk].p] = 0;
+        for (const SegItem &si : hl.segs) sym[hl.keys[si.coarse].p] = 0;
+        MG_TRY(upload(F, &F->gj_sym, sym));
+        MG_TRY(dalloc(F, &F->gj_panel, static_cast<int64_t>(N) * gj_width(maxN, pivots)));
         MG_TRY(dalloc(F, &F->gj_org, 2 * static_cast<int64_t>(N)));
         MG_TRY(dalloc(F, &F->gj_src, N));
     }
@@ -920,19 +925,18 @@ mg_status assemble_coarse(mg_forest *F) {
     const bool prof = F->prof;
     F->gb = nullptr;
     F->prof = false;
-    const bool dominant = F->pnbu != nullptr;
     int hbad = 0;
-    const auto invert = [&](bool diagonal) -> mg_status {
-        if (diagonal || !dominant)
-            MG_TRY(replay(F, F->coarse_rec, [&] { enqueue_coarse_inverse(F, d, N, maxN, diagonal); }));
+    const auto invert = [&](GjPivots how) -> mg_status {
+        if (how == pivots)
+            MG_TRY(replay(F, F->coarse_rec, [&] { enqueue_coarse_inverse(F, d, N, maxN, how); }));
         else
-            enqueue_coarse_inverse(F, d, N, maxN, false);
+            enqueue_coarse_inverse(F, d, N, maxN, how);
         MG_CUDA(cudaMemcpyAsync(&hbad, F->flag, sizeof(int), cudaMemcpyDeviceToHost, F->st));
         MG_CUDA(cudaStreamSynchronize(F->st));
         return MG_OK;
     };
-    mg_status st = invert(dominant);
-    if (st == MG_OK && hbad && dominant) st = invert(false);  // a diagonal pivot cancelled: search for pivots
+    mg_status st = invert(pivots);
+    if (st == MG_OK && hbad) st = invert(GJ_SEARCH_ALL);
     F->gb = gb;
     F->prof = prof;
     MG_TRY(st);

@@ -117,6 +117,29 @@ def test_coefficients_beyond_binary64_contrast_are_still_accepted():
     F.close()
 
 
+def test_contrast_in_one_problem_leaves_its_neighbour_alone():
+    """The same coefficients in a problem beside one with interfaces, whose pivots are searched for anyway."""
+    from paper_2403_08063_gb300 import Forest
+    refined = [(1, i, j, k) for k in (0, 1) for j in (0, 1) for i in (0, 1) if (i, j, k) != (1, 0, 1)]
+    refined += [(2, 2 + a, b, 2 + c) for c in (0, 1) for b in (0, 1) for a in (0, 1)]
+    rows = [(0, 0, 0, 0, 0)] + [(1, *key) for key in refined]
+    k = torch.ones((len(rows), 64), dtype=torch.float64, device="cuda")
+    k[0, 21:23] = 2.0 ** 66
+    f = torch.from_numpy(np.random.default_rng(9).normal(size=(len(rows), 64))).cuda()
+    F = Forest(1, 4, np.array(rows, np.int32), coeff=True, n_problems=2, max_coarse=2000)
+    F.set_rhs(f, k)
+    u = torch.zeros_like(f)
+    F.vcycle(u, 1)
+    assert bool(torch.isfinite(u).all())
+    G = Forest(1, 4, refined, coeff=True, max_coarse=2000)
+    G.set_rhs(f[1:].contiguous(), k[1:].contiguous())
+    v = torch.zeros_like(f[1:])
+    G.vcycle(v, 1)
+    assert torch.equal(v, u[1:])
+    F.close()
+    G.close()
+
+
 def test_narrow_panels_search_for_pivots():
     """More unknowns than one cluster's shared memory takes in panels of 16, with interfaces: panels of 4."""
     from paper_2403_08063_gb300 import Forest
