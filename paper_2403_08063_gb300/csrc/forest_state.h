@@ -179,7 +179,7 @@ struct mg_forest {
     double *AinvT = nullptr;                  // transpose of the coarsest inverses (adjoint cycles)
     double *gj_panel = nullptr;                // device Gauss-Jordan: the eliminated panel, its row exchanges
     int32_t *gj_src = nullptr, *gj_org = nullptr;  // and the composed row origins (two buffers)
-    int8_t *gj_sym = nullptr;  // per problem: 1 where the coarsest level has no refinement interface
+    int8_t *gj_kind = nullptr;  // per problem: GJ_DOMINANT, GJ_SYMMETRIC (assemble_coarse)
     cudaStream_t cap_st = nullptr;             // private stream: graph recording, host-input copies
     // recorded sequences: coarsest-level probe + inversion (assemble_coarse), FP64 V-cycle, FP32 V-cycle, transposed V-cycle
     octmg::Replay coarse_rec, v64_rec, v32_rec, vT_rec;
@@ -338,9 +338,10 @@ mg_status launch_batch_tail32(mg_forest *const *groups, const octmg::TailArgs *a
 bool coarse_jacobi_fits(const mg_forest *F, const DevLevel &d);
 void launch_coarse_jacobi(mg_forest *F, DevLevel &d, int iters);
 // gauss_jordan.cu: inverses of the coarsest operators (input buffer, panel width, launches)
-// How the coarsest elimination finds its pivots: on the diagonal of every problem; by search, without exchanges in the
-// problems of gj_sym; by search in all (gauss_jordan.cu, enqueue_gauss_jordan).
+// How the coarsest elimination finds its pivots: on the diagonal in all problems; by search, on the diagonal in those of kind
+// GJ_DOMINANT; by search in all (gauss_jordan.cu, enqueue_gauss_jordan).
 enum GjPivots { GJ_DIAGONAL, GJ_SEARCH, GJ_SEARCH_ALL };
+enum GjKind : int8_t { GJ_DOMINANT = 1, GJ_SYMMETRIC = 2 };
 double *gj_input(mg_forest *F, int maxN, GjPivots pivots);
 int gj_width(int maxN, GjPivots pivots);
 void enqueue_gauss_jordan(mg_forest *F, int maxN, GjPivots pivots);

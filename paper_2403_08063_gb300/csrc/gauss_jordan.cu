@@ -62,18 +62,19 @@ __device__ __forceinline__ uint64_t a_key(const double *a, int i) {
 // CTA picks the same winner (largest magnitude, lowest row on ties) and updates its rows.  Messages alternate between two
 // buffers: a CTA that writes a buffer again has passed a barrier that every reader of it reached afterwards.  A thread
 // keeps one column of the panel (W divides the CTA); the W threads of a row share a warp, so the multiplier comes by
-// shuffle.  A zero or non-finite pivot sets *bad and the elimination goes on with the diagonal row; so does a row exchange
-// in a problem whose update relies on there being none (sym).
+// shuffle.  A zero or non-finite pivot sets *bad and the elimination goes on with the diagonal row.  In a problem of kind
+// GJ_DOMINANT the diagonal row is the only candidate.
 template <int W>
 __global__ void __cluster_dims__(kGjCluster, 1, 1) __launch_bounds__(kGjThreads)
     k_gj_panel(const double *__restrict__ A, const int64_t *__restrict__ moff, const int64_t *__restrict__ ustart, int c0,
-               double *__restrict__ panel, int32_t *__restrict__ src, const int8_t *__restrict__ sym, int *__restrict__ bad) {
+               double *__restrict__ panel, int32_t *__restrict__ src, const int8_t *__restrict__ kind, int *__restrict__ bad) {
     extern __shared__ __align__(16) unsigned char gj_raw[];
     __shared__ GjCand<W> cand[2][kGjCluster];
     __shared__ GjRow<W> diag[2];
     __shared__ int act;
     const cg::cluster_group cluster = cg::this_cluster();
     const int p = blockIdx.x / kGjCluster, rank = static_cast<int>(cluster.block_rank());
+    const bool diagonal = kind && kind[p];
     const int N = static_cast<int>(ustart[p + 1] - ustart[p]);
     if (c0 >= N) return;  // uniform over the cluster, before any barrier
     const int wn = min(W, N - c0), nr = (N - rank + kGjCluster - 1) / kGjCluster;  // row i of this CTA: rank + 8 i
@@ -103,7 +104,7 @@ __global__ void __cluster_dims__(kGjCluster, 1, 1) __launch_bounds__(kGjThreads)
             uint64_t best = 0;
             int at = -1;
             for (int i = (max(0, c - rank) + kGjCluster - 1) / kGjCluster + lane; i < na; i += 32) {
-                const uint64_t key = a_key(a, i * W + cc);
+                const uint64_t key = !diagonal || row_of(i) == c ? a_key(a, i * W + cc) : 0;
                 if (key > best) {
                     best = key;
                     at = i;
@@ -143,7 +144,7 @@ __global__ void __cluster_dims__(kGjCluster, 1, 1) __launch_bounds__(kGjThreads)
         const GjCand<W> &w = cand[buf][win];
         // usable: found, not zero (key 1) and not infinite
         const bool ok = w.key > 1 && w.key < 0x7ff0000000000001ull;
-        if (rank == 0 && tid == 0 && (!ok || (w.r != c && sym && sym[p]))) atomicOr(bad, 1);
+        if (!ok && rank == 0 && tid == 0) atomicOr(bad, 1);
         const int q = ok ? w.r : c;
         const double *prow = ok ? w.row : diag[buf].row;
         const double v = ok ? w.rcp : 1.0 / diag[buf].row[cc];
@@ -173,7 +174,7 @@ __global__ void __cluster_dims__(kGjCluster, 1, 1) __launch_bounds__(kGjThreads)
 // a factor of zeros is copied, which the unknowns' order makes frequent: with the unknowns sorted by position a row of the
 // operator reaches no further than a plane of cells, so before column c only the first c + plane rows and columns are touched
 // (1728 unknowns: 2.15e9 of 5.16e9 FMA, 5.1 instead of 9.0 ms).  Problems with c0 unknowns or fewer are copied through.
-// sym (may be null): the problem's matrix is symmetric and eliminated without row exchanges.  It then stays symmetric up to a
+// GJ_SYMMETRIC: the problem's matrix is symmetric and eliminated without row exchanges.  It then stays symmetric up to a
 // sign, Y[j, r] = Y[r, j] where both or neither of r and j are eliminated and -Y[r, j] otherwise, and the tiles above the
 // diagonal are written from those below: with 1728 unknowns 30 us per update instead of 47, and a gradient on 48^3 cells 8.2
 // instead of 9.8 ms.
@@ -182,13 +183,13 @@ __global__ void __launch_bounds__(kGjThreads)
     k_gj_update(const double *__restrict__ X, double *__restrict__ Y, const int64_t *__restrict__ moff,
                 const int64_t *__restrict__ ustart, int c0, const double *__restrict__ panel,
                 const int32_t *__restrict__ src, const int32_t *__restrict__ org_in, int32_t *__restrict__ org_out,
-                const int8_t *__restrict__ sym_of) {
+                const int8_t *__restrict__ kind) {
     constexpr int T = kGjTile, ROWS = kGjThreads / T;  // rows of the tile per pass
     __shared__ double M[T][W], B[W][T];
     __shared__ int32_t from[T];
     __shared__ double low[T][T + 1];
     const int p = blockIdx.z;
-    const bool sym = sym_of && sym_of[p];
+    const bool sym = kind && (kind[p] & GJ_SYMMETRIC);
     if (sym && blockIdx.x > blockIdx.y) return;
     const int64_t u0 = ustart[p];
     const int N = static_cast<int>(ustart[p + 1] - u0);
@@ -277,7 +278,7 @@ __global__ void k_gj_transpose(const double *__restrict__ X, double *__restrict_
 // so each CTA eliminates these and kGjRows others by itself and nothing passes between CTAs.  A thread keeps one entry of
 // the pivot rows and one of its CTA's rows in registers; the W threads of a row share a warp, and the pivot row of a step
 // goes through one of two shared buffers (who writes a buffer again has passed the barrier after its last read).  The
-// operations and their order are those of k_gj_panel when it finds every pivot on the diagonal.  Bound by the chain of a
+// operations and their order are those of k_gj_panel for a problem of kind GJ_DOMINANT.  Bound by the chain of a
 // shuffle, a reciprocal, a barrier and an update per column: about 9 us per panel, where the cluster's search takes 37 us with
 // 512 unknowns and 46 us with 1728 (new coefficients and a solve on 128^3 cells 3.79 -> 2.94 ms, a gradient on 48^3 cells
 // with 1728 coarsest unknowns 13.8 -> 9.8 ms).
@@ -325,7 +326,7 @@ constexpr int64_t kGjMaxSmem = 200 * 1024;
 
 template <int W>
 void invert(mg_forest *F, int maxN, GjPivots pivots) {
-    const int8_t *sym = pivots == GJ_SEARCH_ALL ? nullptr : F->gj_sym;
+    const int8_t *kind = pivots == GJ_SEARCH_ALL ? nullptr : F->gj_kind;
     if (pivots != GJ_DIAGONAL) cudaFuncSetAttribute(k_gj_panel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGjMaxSmem);
     const unsigned tiles = static_cast<unsigned>((maxN + kGjTile - 1) / kGjTile);
     const int steps = (maxN + W - 1) / W;
@@ -337,9 +338,9 @@ void invert(mg_forest *F, int maxN, GjPivots pivots) {
                 X, F->moff, F->ustart, c0, F->gj_panel, F->gj_src, F->flag);
         else
             k_gj_panel<W><<<F->np * kGjCluster, kGjThreads, gj_smem(maxN, W), F->st>>>(
-                X, F->moff, F->ustart, c0, F->gj_panel, F->gj_src, sym, F->flag);
+                X, F->moff, F->ustart, c0, F->gj_panel, F->gj_src, kind, F->flag);
         k_gj_update<W><<<dim3(tiles, tiles, F->np), kGjThreads, 0, F->st>>>(X, Y, F->moff, F->ustart, c0, F->gj_panel,
-                                                                            F->gj_src, in, out, sym);
+                                                                            F->gj_src, in, out, kind);
         std::swap(X, Y);
         std::swap(in, out);
     }
@@ -364,11 +365,11 @@ double *gj_input(mg_forest *F, int maxN, GjPivots pivots) {
 }
 
 // Ainv and AinvT (the transposes) from the operators in gj_input; a singular one sets *F->flag (cleared by the caller).
-// Problems without interfaces (F->gj_sym) have symmetric (to rounding), diagonally dominant operators.  Elimination keeps
-// that of what is left, so the largest entry of a column is on the diagonal (the lowest row on ties), and the search for
-// pivots, left out when all problems are of this kind (GJ_DIAGONAL), would exchange nothing.  Where coefficients differ
-// by more than binary64 resolves, a pivot can cancel all the same: the flag says so, and the caller comes again with
-// GJ_SEARCH_ALL, which relies on nothing.
+// A problem without interfaces on this level (GJ_DOMINANT) has 7-point rows, diagonally dominant by rows.  Elimination on the
+// diagonal keeps that of what is left, so a scaled pivot row's other entries sum to at most 1 and no row's sum of magnitudes
+// grows: nothing is gained by a search for pivots, which is left out when all problems are of this kind (GJ_DIAGONAL).
+// Where coefficients differ by more than binary64 resolves, a pivot can cancel all the same: the flag says so, and the
+// caller comes again with GJ_SEARCH_ALL.
 void enqueue_gauss_jordan(mg_forest *F, int maxN, GjPivots pivots) {
     switch (gj_width(maxN, pivots)) {
         case 16: invert<16>(F, maxN, pivots); break;

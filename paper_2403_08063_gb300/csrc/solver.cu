@@ -911,11 +911,18 @@ mg_status assemble_coarse(mg_forest *F) {
     for (int p = 0; p < F->np; ++p) maxN = std::max<int>(maxN, static_cast<int>(F->ustart_h[p + 1] - F->ustart_h[p]));
     const GjPivots pivots = F->pnbu ? GJ_DIAGONAL : GJ_SEARCH;
     if (!F->gj_src) {
-        std::vector<int8_t> sym(static_cast<size_t>(F->np), 1);  // the problems without interfaces
-        for (const FaceItem &fi : hl.faces)
-            if (fi.kind != FK_SAME && fi.kind != FK_BND) sym[hl.keys[fi.blk].p] = 0;
-        for (const SegItem &si : hl.segs) sym[hl.keys[si.coarse].p] = 0;
-        MG_TRY(upload(F, &F->gj_sym, sym));
+        // Without interfaces on this level a problem's rows are diagonally dominant.  They are also symmetric if the two blocks
+        // at a face agree on its coefficient: faces averaged on either side of a finer level's interface do not.
+        std::vector<int8_t> kind(static_cast<size_t>(F->np), GJ_DOMINANT | GJ_SYMMETRIC);
+        const auto drop = [&](const HostLevel &h, int8_t keep) {
+            for (const FaceItem &fi : h.faces)
+                if (fi.kind != FK_SAME && fi.kind != FK_BND) kind[h.keys[fi.blk].p] &= keep;
+            for (const SegItem &si : h.segs) kind[h.keys[si.coarse].p] &= keep;
+        };
+        drop(hl, 0);
+        if (F->cfg.coeff && F->cfg.coarse_coef == 1)
+            for (const HostLevel &h : F->H.levels) drop(h, GJ_DOMINANT);
+        MG_TRY(upload(F, &F->gj_kind, kind));
         MG_TRY(dalloc(F, &F->gj_panel, static_cast<int64_t>(N) * gj_width(maxN, pivots)));
         MG_TRY(dalloc(F, &F->gj_org, 2 * static_cast<int64_t>(N)));
         MG_TRY(dalloc(F, &F->gj_src, N));

@@ -152,3 +152,27 @@ def test_narrow_panels_search_for_pivots():
     F.vcycle(u, 1)
     assert float((F.apply(u) - f).norm() / f.norm()) <= 4 * N * EPS * (2 * 48 / math.pi) ** 2
     F.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_faces_averaged_beside_a_finer_interface(precision):
+    """A refined root among 4^3: on the merged levels the two sides of its faces average different fine faces, so the
+    coarsest operator has no interface and is not symmetric.  FP64 cycles against the oracle, and the mixed solve's residual."""
+    import synthetic as syn
+    from oracle.octree_mg import OracleMG
+    from paper_2403_08063_gb300 import Forest
+    R, n, keys = 4, 8, one_refined_root(4, (1, 2, 1))
+    k = syn.lognormal_k_rff(R, n, keys, seed=51)
+    f = syn.uniform_rhs(len(keys), n, seed=52)
+    F = Forest(R, n, keys, coeff=True, precision=precision, coarse_coef="faces")
+    F.set_rhs(f.cuda(), k.cuda())
+    u = torch.zeros(f.shape, dtype=torch.float64, device="cuda")
+    ref = OracleMG(R, n, keys, k_user=k.numpy(), coarse_coef="faces")
+    if precision == 0:
+        F.vcycle(u, 3)
+        want, _ = ref.solve(f.numpy(), cycles=3)
+        assert np.linalg.norm(u.cpu().numpy() - want) <= 1e-10 * np.linalg.norm(want)
+    else:
+        F.solve(u, rtol=1e-10)
+        assert ref.rel_residual(u.cpu().numpy(), f.numpy()) <= 1.05e-10
+    F.close()
