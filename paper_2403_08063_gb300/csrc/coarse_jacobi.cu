@@ -91,7 +91,7 @@ void launch_coarse_jacobi(mg_forest *F, DevLevel &d, int iters) {
     auto *fn = F->cfg.coeff ? k_coarse_jacobi<1> : k_coarse_jacobi<0>;
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     launch_pdl(F->st, false, fn, kCjCluster, kCjThreads, smem_bytes(F, d), d.u64, d.f64, d.c64(), d.h2_64, d.nbr6, d.g,
-               F->omega, iters, F->np > 1 ? Skip{d.bprob, F->pdone} : Skip{});
+               F->omega, iters, Skip{d.bprob, done_mask(F)});
 }
 
 }  // namespace octmg

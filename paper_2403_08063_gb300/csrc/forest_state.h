@@ -232,6 +232,11 @@ template <typename T> constexpr int cat_of(int cat64) { return sizeof(T) == 8 ? 
 
 cudaEvent_t next_event(mg_forest *F);
 
+// The done-mask of the forest's problems.  A problem that is solved alone needs none: its solve ends when it is done, and
+// without a mask a kernel starts two dependent loads earlier (0.5 us of a launch of 3).  In a batch it does, also as the
+// only one of its block size: the others go on.
+inline uint8_t *done_mask(const mg_forest *F) { return F->np > 1 || F->batch_member ? F->pdone : nullptr; }
+
 // RAII scope around the launches of one kernel family (a negative family: no accounting).
 struct Prof {
     mg_forest *F;

@@ -87,9 +87,8 @@ template <typename T> Coef coef_of(const DevLevel &d);
 template <> Coef coef_of<double>(const DevLevel &d) { return d.c64(); }
 template <> Coef coef_of<float>(const DevLevel &d) { return d.c32(); }
 
-// The done-mask view of a level for its kernels (all problems active outside a solve).  A single problem needs none: its
-// solve ends when it is done, and without a mask a kernel starts two dependent loads earlier (0.5 us of a launch of 3).
-Skip skip_of(mg_forest *F, const DevLevel &d) { return Skip{d.bprob, F->np > 1 ? F->pdone : nullptr}; }
+// The done-mask view of a level for its kernels (all problems active outside a solve).
+Skip skip_of(mg_forest *F, const DevLevel &d) { return Skip{d.bprob, done_mask(F)}; }
 
 // Ghost exchange of a level: every face (full), or only the refinement-interface faces (C2F and F2C), whose
 // ghosts the smoother's write-through does not maintain.  One launch for block edges up to 128 (its offsets inside a block
@@ -567,7 +566,7 @@ struct LaunchExec {
         launch_pdl(F->st, !F->batch_member, k_coarse_solve<T>, (F->Nc * 32 + kThreads - 1) / kThreads, kThreads, 0,
                    ufield<T>(d), ffield<T>(d), F->Ainv, sizeof(T) == 4 ? F->cmap32 : F->cmap, F->uprob, F->ustart,
                    F->moff,
-            F->Nc, F->np > 1 ? F->pdone : nullptr);
+            F->Nc, done_mask(F));
     }
     void restrict_to(int l, bool fast) {
         DevLevel &d = F->L[l], &c = F->L[l + 1];

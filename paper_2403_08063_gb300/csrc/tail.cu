@@ -177,7 +177,7 @@ static __global__ void __launch_bounds__(kTailThreads) k_batch_tail32(const Tail
 
 TailArgs tail_args(mg_forest *F) {
     return TailArgs{F->tail_L, F->tail_ph, F->tail_nph, F->cfg.interface_flux, F->Ainv, F->cmap32, F->uprob,
-                    F->ustart, F->moff, F->Nc, F->np > 1 ? F->pdone : nullptr, F->tail_bar, F->kerr};
+                    F->ustart, F->moff, F->Nc, done_mask(F), F->tail_bar, F->kerr};
 }
 
 // CTAs the largest phase of F's recorded tail can use (one thread per updated cell of a half-sweep, one warp per coarsest

@@ -183,3 +183,38 @@ def test_converged_problems_stop_where_they_would_stop_alone():
         F.close()
         off += cnt
     B.close()
+
+
+@pytest.mark.parametrize("mode", [0, 1, 2])
+def test_the_only_problem_of_a_block_size_stops_when_it_is_done(mode):
+    """Three block sizes, two of them with one problem each: the iterates and cycle counts of these two are those of a solve
+    of each alone, although the slower problems go on for more steps (problems that share a forest have its levels, also
+    where one alone would have fewer)."""
+    from paper_2403_08063_gb300 import Batch
+    ns = [8, 32, 16, 16]
+    refined = [(1, i, j, k) for k in (0, 1) for j in (0, 1) for i in (0, 1)]
+    keys = [refined, [(0, 0, 0, 0)], refined, [(0, 0, 0, 0)]]
+    sigma = [0.1, 0.5, 1.0, 0.5]
+    rows = [(p, *key) for p in range(4) for key in keys[p]]
+    rng = np.random.default_rng(81)
+    f, k = [], []
+    for p in range(4):
+        f.append(torch.from_numpy(rng.uniform(-1, 1, size=len(keys[p]) * ns[p] ** 3)).to(DEV))
+        k.append(syn.lognormal_k_rff(1, ns[p], keys[p], seed=90 + p, sigma=sigma[p], ell=0.2).reshape(-1).to(DEV))
+    B = Batch(rows, ns, coeff=True, inner_cycles=1)
+    B.set_rhs(torch.cat(f), torch.cat(k))
+    B.set_tail_mode(mode)
+    u = torch.zeros_like(torch.cat(f))
+    cyc, _ = B.solve(u, rtol=1e-8, max_cycles=60)
+    assert len(set(cyc)) > 1
+    off = 0
+    for p in (0, 1):
+        A = Batch([(0, *key) for key in keys[p]], [ns[p]], coeff=True, inner_cycles=1)
+        A.set_rhs(f[p], k[p])
+        A.set_tail_mode(0)
+        v = torch.zeros_like(f[p])
+        alone, _ = A.solve(v, rtol=1e-8, max_cycles=60)
+        assert list(alone) == [cyc[p]] and torch.equal(v, u[off:off + v.numel()]), p
+        off += v.numel()
+        A.close()
+    B.close()
