@@ -25,7 +25,7 @@
 // What bounds it: HBM, in the half-sweeps (10 B per updated cell) and the FP64 residual's FP64 rate.  The transposed cycle
 // step by step on natural-layout arrays of its own (the correction, its stencil with ghost adjoints, their scatter by
 // atomics over every face, two vector updates per half-sweep: ~70 B per cell and half-sweep) made set-up, forward solve and
-// adjoint on 448 + 512 blocks of 32^3 (31.5M cells) take 174 ms; this form, with the later steps' kernels, 63.7 ms.
+// adjoint on 448 + 512 blocks of 32^3 (31.5M cells) take 174 to 183 ms, depending on the inputs; this form, with the later steps' kernels, 63 ms.
 #include <cmath>
 
 #include "forest_state.h"

@@ -14,7 +14,7 @@
 // block barrier, a division, and the panel's update on the 2 FP64 FMA per clock of each of the cluster's SMs), then the
 // FP64 rate in the update.  Elimination of one column per step with two launches per column (every element rewritten each
 // time) took 4.85 ms for 512 unknowns and 58 ms for 1728 (three root blocks per axis); this takes 1.5 ms and 10.1 ms.
-// Symmetric operators whose pivots are known to be on the diagonal need no search (k_gj_panel_diag) and half of the updates:
+// Operators without interfaces take their pivots on the diagonal (k_gj_panel_diag), symmetric ones half of the updates:
 // 0.65 ms and 4.4 ms.
 #include <cooperative_groups.h>
 
