@@ -2470,7 +2470,8 @@ constexpr int kCoarseStage = 2048;  // right-hand side values a CTA stages in sh
 // Rows w0, w0 + wn, .. of the coarsest solve, the calling warp's; every thread of the CTA calls it.  The right-hand sides
 // lo .. hi - 1 that the CTA's rows need are gathered once into shared memory (up to kCoarseStage): gathered per row, through
 // the map, they put two dependent loads into every step of a row's chain.  Lane l adds columns l, l + 32, .. in order,
-// whatever the path.
+// whatever the path.  The persistent tails (CG) call it again with the same stage, a batch's joint tail for one forest after
+// the other without a grid barrier between: the CTA's slower warps have read the last call's values before it is filled.
 template <typename T, bool CG = false>
 __device__ __forceinline__ void coarse_solve_rows(T *__restrict__ u, const T *__restrict__ f,
                                                   const double *__restrict__ Ainv, const int64_t *__restrict__ cmap,
@@ -2480,6 +2481,7 @@ __device__ __forceinline__ void coarse_solve_rows(T *__restrict__ u, const T *__
                                                   double *__restrict__ stage) {
     const bool staged = hi - lo <= kCoarseStage;
     if (staged) {
+        if constexpr (CG) __syncthreads();
         for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) stage[i - lo] = static_cast<double>(ldv<CG>(f + cmap[i]));
         __syncthreads();
     }

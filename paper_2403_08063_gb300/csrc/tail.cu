@@ -158,8 +158,9 @@ static __global__ void __launch_bounds__(kTailThreads) k_tail32(TailArgs a) {
 }
 
 // The joint tail of a batch: the recorded tails of several forests (one per block size) in one launch.  Entries
-// between two barriers are phases of different forests, which share no data, so the grid runs them back to back
-// and synchronises once; each forest's own phases keep their order, each followed by a barrier as in k_tail32.
+// between two barriers are phases of different forests, which share no data in global memory, so the grid runs them
+// back to back and synchronises once; each forest's own phases keep their order, each followed by a barrier as in
+// k_tail32.  Inside a CTA they share coarse_f, which coarse_solve_rows fills only when every warp has read its last use.
 template <int MODE>
 static __global__ void __launch_bounds__(kTailThreads) k_batch_tail32(const TailArgs *__restrict__ ga,
                                                                       const BatchEntry *__restrict__ e, int ne,

@@ -218,3 +218,38 @@ def test_the_only_problem_of_a_block_size_stops_when_it_is_done(mode):
         off += v.numel()
         A.close()
     B.close()
+
+
+def test_coarsest_solves_of_several_groups_between_two_barriers():
+    """The joint tail runs the same phase of every group between two grid barriers.  With uniform problems of block sizes 8,
+    16 and 32 and every tail from the 8^3 level the three groups' coarsest solves (1536 unknowns each, staged in the CTA's
+    one buffer) are such a phase; two problems of the first group are done before the first cycle, so that their rows
+    take no time.  Ten solves, each bit for bit that with every level launched."""
+    import ctypes
+    from paper_2403_08063_gb300 import Batch
+    keys = [(1, i, j, k) for k in (0, 1) for j in (0, 1) for i in (0, 1)]
+    ns = [8, 8, 8, 16, 16, 16, 32, 32, 32]
+    rows = [(p, *key) for p in range(len(ns)) for key in keys]
+    gen = torch.Generator().manual_seed(91)
+    f = [torch.rand(8 * n ** 3, generator=gen, dtype=torch.float64) - 0.5 for n in ns]
+    f[0].zero_()
+    f[1].zero_()
+    k = [syn.lognormal_k_rff(1, n, keys, seed=70 + p, sigma=0.5, ell=0.3).reshape(-1) for p, n in enumerate(ns)]
+    B = Batch(rows, ns, coeff=True, inner_cycles=4, max_coarse=512, coarse_coef="faces")
+    for g, level in enumerate((0, 1, 2)):
+        handle = ctypes.c_void_p(B.lib.mg_batch_group(B.h, g))
+        assert B.lib.mg_set_tail(handle, level) == 0
+    B.set_rhs(torch.cat(f).to(DEV), torch.cat(k).to(DEV))
+    out = {}
+    for mode in (0, 2):
+        B.set_tail_mode(mode)
+        assert B.tail_levels() == ([-1, -1, -1] if mode == 0 else [0, 1, 2])
+        for rep in range(1 if mode == 0 else 10):
+            u = torch.zeros(B.numel, dtype=torch.float64, device=DEV)
+            cyc, rel = B.solve(u, rtol=1e-9, max_cycles=60)
+            assert cyc[0] == cyc[1] == 0
+            if mode == 0:
+                out = {"u": u, "cyc": cyc, "rel": rel}
+            else:
+                assert torch.equal(u, out["u"]) and cyc == out["cyc"] and rel == out["rel"], rep
+    B.close()
