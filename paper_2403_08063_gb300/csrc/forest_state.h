@@ -179,6 +179,7 @@ struct mg_forest {
     double *AinvT = nullptr;                  // transpose of the coarsest inverses (adjoint cycles)
     double *gj_panel = nullptr;                // device Gauss-Jordan: the eliminated panel, its row exchanges
     int32_t *gj_src = nullptr, *gj_org = nullptr;  // and the composed row origins (two buffers)
+    double *gj_diag = nullptr;  // the operators' diagonals before the elimination
     int8_t *gj_kind = nullptr;  // per problem: GJ_DOMINANT, GJ_SYMMETRIC (assemble_coarse)
     cudaStream_t cap_st = nullptr;             // private stream: graph recording, host-input copies
     // recorded sequences: coarsest-level probe + inversion (assemble_coarse), FP64 V-cycle, FP32 V-cycle, transposed V-cycle

@@ -56,6 +56,14 @@ __device__ __forceinline__ uint64_t a_key(const double *a, int i) {
     return bits <= 0x7ff0000000000000ull ? bits + 1 : 0;
 }
 
+// Whether `pivot` can be a diagonal pivot of a problem with N unknowns whose matrix had `before` there.  Elimination of a
+// diagonally dominant matrix leaves a positive pivot; the roundings of up to N updates of this entry, each at most eps / 2 of
+// it, move it by less than N eps times what it was, so a pivot above that has its sign and some digits, and one below may be
+// noise (cells coupled to each other by more than 1 / (N eps) times what couples them to the rest).
+__device__ __forceinline__ bool dominant_pivot(double pivot, double before, int N) {
+    return pivot > N * 2.220446049250313e-16 * before && pivot <= 1.7976931348623157e308;
+}
+
 // Eliminates panel columns c0 .. c0 + W - 1 of every problem with more than c0 unknowns, one cluster per problem, row r in
 // CTA r % 8.  Per column one cluster barrier: before it each CTA sends the others its best pivot
 // candidate with the whole panel row and the reciprocal, and the owner of the diagonal row sends that one; after it every
@@ -63,11 +71,13 @@ __device__ __forceinline__ uint64_t a_key(const double *a, int i) {
 // buffers: a CTA that writes a buffer again has passed a barrier that every reader of it reached afterwards.  A thread
 // keeps one column of the panel (W divides the CTA); the W threads of a row share a warp, so the multiplier comes by
 // shuffle.  A zero or non-finite pivot sets *bad and the elimination goes on with the diagonal row.  In a problem of kind
-// GJ_DOMINANT the diagonal row is the only candidate.
+// GJ_DOMINANT the diagonal row is the only candidate, and one that is no dominant_pivot sets *bad too (dg: the diagonal before
+// the elimination, kept by the first panel).
 template <int W>
 __global__ void __cluster_dims__(kGjCluster, 1, 1) __launch_bounds__(kGjThreads)
     k_gj_panel(const double *__restrict__ A, const int64_t *__restrict__ moff, const int64_t *__restrict__ ustart, int c0,
-               double *__restrict__ panel, int32_t *__restrict__ src, const int8_t *__restrict__ kind, int *__restrict__ bad) {
+               double *__restrict__ panel, int32_t *__restrict__ src, const int8_t *__restrict__ kind,
+               double *__restrict__ dg, int *__restrict__ bad) {
     extern __shared__ __align__(16) unsigned char gj_raw[];
     __shared__ GjCand<W> cand[2][kGjCluster];
     __shared__ GjRow<W> diag[2];
@@ -87,7 +97,10 @@ __global__ void __cluster_dims__(kGjCluster, 1, 1) __launch_bounds__(kGjThreads)
         const int row = e / W;
         a[e] = row < nr && col < wn ? Ap[static_cast<int64_t>(row_of(row)) * N + c0 + col] : 0.0;
     }
-    for (int i = tid; i < nr; i += kGjThreads) id[i] = row_of(i);
+    for (int i = tid; i < nr; i += kGjThreads) {
+        id[i] = row_of(i);
+        if (diagonal && c0 == 0) dg[ustart[p] + row_of(i)] = Ap[static_cast<int64_t>(row_of(i)) * N + row_of(i)];
+    }
     // rows of zeros stay as they are (a zero multiplier, never a pivot): the panel ends at the last other row, or at its own
     // rows, which receive the pivot rows
     if (tid == 0) act = 0;
@@ -100,6 +113,8 @@ __global__ void __cluster_dims__(kGjCluster, 1, 1) __launch_bounds__(kGjThreads)
     const int na = act;
     for (int cc = 0; cc < wn; ++cc) {
         const int c = c0 + cc, buf = cc & 1;
+        const bool checks = diagonal && rank == 0 && tid == 0;
+        const double before = !checks ? 0.0 : (c0 == 0 ? Ap[static_cast<int64_t>(c) * N + c] : dg[ustart[p] + c]);
         if (tid < 32) {
             uint64_t best = 0;
             int at = -1;
@@ -144,7 +159,7 @@ __global__ void __cluster_dims__(kGjCluster, 1, 1) __launch_bounds__(kGjThreads)
         const GjCand<W> &w = cand[buf][win];
         // usable: found, not zero (key 1) and not infinite
         const bool ok = w.key > 1 && w.key < 0x7ff0000000000001ull;
-        if (!ok && rank == 0 && tid == 0) atomicOr(bad, 1);
+        if (rank == 0 && tid == 0 && (!ok || (checks && !dominant_pivot(w.row[cc], before, N)))) atomicOr(bad, 1);
         const int q = ok ? w.r : c;
         const double *prow = ok ? w.row : diag[buf].row;
         const double v = ok ? w.rcp : 1.0 / diag[buf].row[cc];
@@ -285,7 +300,7 @@ __global__ void k_gj_transpose(const double *__restrict__ X, double *__restrict_
 constexpr int kGjRows = 16;
 __global__ void __launch_bounds__(kGjThreads)
     k_gj_panel_diag(const double *__restrict__ A, const int64_t *__restrict__ moff, const int64_t *__restrict__ ustart, int c0,
-                    double *__restrict__ panel, int32_t *__restrict__ src, int *__restrict__ bad) {
+                    double *__restrict__ panel, int32_t *__restrict__ src, double *__restrict__ dg, int *__restrict__ bad) {
     constexpr int W = 16;
     static_assert(kGjRows == W && kGjThreads == W * W, "one entry of each half per thread");
     __shared__ double prow[2][W];
@@ -298,13 +313,22 @@ __global__ void __launch_bounds__(kGjThreads)
     const double *a = A + moff[p];
     double d = i < wn && col < wn ? a[static_cast<int64_t>(c0 + i) * N + c0 + col] : 0.0;
     double x = r < N && col < wn ? a[static_cast<int64_t>(r) * N + c0 + col] : 0.0;
-    bool zero = false;
+    // the diagonal before the elimination, kept by the first panel; the pivot rows' own CTA (c0 is a multiple of W) checks
+    const bool own = r0 == c0;
+    double before = 0.0;
+    if (c0 == 0 && r < N) {
+        before = a[static_cast<int64_t>(r) * N + r];
+        if (col == 0) dg[u0 + r] = before;
+    } else if (own && r < N) {
+        before = dg[u0 + r];
+    }
+    bool lost = false;
     for (int cc = 0; cc < wn; ++cc) {
         const int from = (lane & ~(W - 1)) | cc;
         const double fd = __shfl_sync(0xffffffffu, d, from), fx = __shfl_sync(0xffffffffu, x, from);
         double *row = prow[cc & 1];
         if (i == cc) {
-            zero = zero || !(fabs(fd) > 0.0 && fabs(fd) <= 1.7976931348623157e308);
+            lost = lost || !dominant_pivot(fd, before, N);
             const double v = 1.0 / fd;
             row[col] = col == cc ? v : d * v;
         }
@@ -313,9 +337,9 @@ __global__ void __launch_bounds__(kGjThreads)
         d = i == cc ? pv : fma(-fd, pv, col == cc ? 0.0 : d);
         x = fma(-fx, pv, col == cc ? 0.0 : x);
     }
-    if (r0 == c0) {  // the pivot rows' own CTA (c0 is a multiple of W)
+    if (own) {
         x = d;
-        if (zero) atomicOr(bad, 1);
+        if (lost) atomicOr(bad, 1);
     }
     if (r >= N) return;
     panel[(u0 + r) * W + col] = x;
@@ -335,10 +359,10 @@ void invert(mg_forest *F, int maxN, GjPivots pivots) {
     for (int c0 = 0; c0 < maxN; c0 += W) {
         if (pivots == GJ_DIAGONAL)
             k_gj_panel_diag<<<dim3(static_cast<unsigned>((maxN + kGjRows - 1) / kGjRows), F->np), kGjThreads, 0, F->st>>>(
-                X, F->moff, F->ustart, c0, F->gj_panel, F->gj_src, F->flag);
+                X, F->moff, F->ustart, c0, F->gj_panel, F->gj_src, F->gj_diag, F->flag);
         else
             k_gj_panel<W><<<F->np * kGjCluster, kGjThreads, gj_smem(maxN, W), F->st>>>(
-                X, F->moff, F->ustart, c0, F->gj_panel, F->gj_src, kind, F->flag);
+                X, F->moff, F->ustart, c0, F->gj_panel, F->gj_src, kind, F->gj_diag, F->flag);
         k_gj_update<W><<<dim3(tiles, tiles, F->np), kGjThreads, 0, F->st>>>(X, Y, F->moff, F->ustart, c0, F->gj_panel,
                                                                             F->gj_src, in, out, kind);
         std::swap(X, Y);
@@ -368,8 +392,8 @@ double *gj_input(mg_forest *F, int maxN, GjPivots pivots) {
 // A problem without interfaces on this level (GJ_DOMINANT) has 7-point rows, diagonally dominant by rows.  Elimination on the
 // diagonal keeps that of what is left, so a scaled pivot row's other entries sum to at most 1 and no row's sum of magnitudes
 // grows: nothing is gained by a search for pivots, which is left out when all problems are of this kind (GJ_DIAGONAL).
-// Where coefficients differ by more than binary64 resolves, a pivot can cancel all the same: the flag says so, and the
-// caller comes again with GJ_SEARCH_ALL.
+// Where coefficients differ by more than binary64 resolves, rounding can cancel a pivot all the same or leave noise in its
+// place (dominant_pivot): the flag says so, and the caller comes again with GJ_SEARCH_ALL.
 void enqueue_gauss_jordan(mg_forest *F, int maxN, GjPivots pivots) {
     switch (gj_width(maxN, pivots)) {
         case 16: invert<16>(F, maxN, pivots); break;

@@ -924,6 +924,7 @@ mg_status assemble_coarse(mg_forest *F) {
         MG_TRY(upload(F, &F->gj_kind, kind));
         MG_TRY(dalloc(F, &F->gj_panel, static_cast<int64_t>(N) * gj_width(maxN, pivots)));
         MG_TRY(dalloc(F, &F->gj_org, 2 * static_cast<int64_t>(N)));
+        MG_TRY(dalloc(F, &F->gj_diag, N));
         MG_TRY(dalloc(F, &F->gj_src, N));
     }
     // the probe must see the homogeneous operator: no boundary data, no profiling events inside a recorded graph

@@ -140,6 +140,35 @@ def test_contrast_in_one_problem_leaves_its_neighbour_alone():
     G.close()
 
 
+@pytest.mark.parametrize("cells,exponent", [("pair", 17.0), ("pair", 18.6), ("cube", 17.4), ("cube", 18.2),
+                                            ("cube", 18.9), ("cube", 19.7)])
+def test_pivots_lost_in_rounding_are_searched_for(cells, exponent):
+    """A pair or a cube of cells coupled by about 10^exponent times what couples them to the rest, with coefficients that
+    cancel to rounding noise instead of zero: such an operator is eliminated with row exchanges, bit for bit as beside a
+    problem whose pivots cancel exactly and which therefore has all problems of its forest searched."""
+    from paper_2403_08063_gb300 import Forest
+    rng = np.random.default_rng(int(10 * exponent))
+    k = np.exp(rng.normal(size=(2, 4, 4, 4)))
+    if cells == "pair":
+        k[0, 1, 1, 1:3] = 10.0 ** exponent * rng.uniform(1, 2, size=2)
+    else:
+        k[0, 1:3, 1:3, 1:3] = 10.0 ** exponent * rng.uniform(0.3, 3, size=(2, 2, 2))
+    k[1] = 1.0
+    k[1, 1, 1, 1:3] = 2.0 ** 66
+    k = torch.from_numpy(k.reshape(2, 64)).cuda()
+    f = torch.from_numpy(rng.normal(size=(2, 64))).cuda()
+    got = []
+    for problems in (1, 2):
+        F = Forest(1, 4, [(p, 0, 0, 0, 0) for p in range(problems)], coeff=True, n_problems=problems)
+        F.set_rhs(f[:problems].contiguous(), k[:problems].contiguous())
+        u = torch.zeros_like(f[:problems])
+        F.vcycle(u, 1)
+        assert bool(torch.isfinite(u).all())
+        got.append(u[0])
+        F.close()
+    assert torch.equal(got[0], got[1])
+
+
 def test_narrow_panels_search_for_pivots():
     """More unknowns than one cluster's shared memory takes in panels of 16, with interfaces: panels of 4."""
     from paper_2403_08063_gb300 import Forest
