@@ -892,7 +892,7 @@ mg_status adjoint_supported(const mg_forest *F) {
 
 // Half a defect-correction step: r = g - A^T lambda (r = g while lambda is 0).  FP32 cycles: r scaled by `mult` into the
 // level-0 FP32 right-hand side, its result zeroed; FP64 cycles: r into the level-0 right-hand side a_fe, u64 zeroed.
-// rr receives the volume-weighted ||r||^2 over all problems.
+// rr: the volume-weighted ||g||^2 over all problems on entry, ||r||^2 on exit, in FP64 like the test it is for.
 template <int MODE>
 mg_status adjoint_residual(mg_forest *F, bool zero, double mult, double *rr) {
     DevLevel &d = F->L[0];
@@ -922,14 +922,16 @@ mg_status adjoint_residual(mg_forest *F, bool zero, double mult, double *rr) {
             MG_CUDA(cudaMemsetAsync(d.u32, 0, d.pool_elems() * sizeof(float), F->st));
             k_scaled_rhs<<<d.g.nb * cpb, kThreads, 0, F->st>>>(f, d.vol_32, d.g, cpb, d.f32, F->pscale, d.bprob, F->bsum,
                                                                Skip{});
-        } else {
-            k_residual_norm<MODE><<<d.g.nb * cpb, kThreads, 0, F->st>>>(F->a_lam, f, d.c64(), d.ih2_64, d.vol_32, d.g, cpb,
-                                                                        d.f32, F->pscale, d.bprob, F->bsum, d.u32, Skip{});
+            MG_CUDA(cudaStreamSynchronize(F->st));  // the scales' host copies may change again
+            return MG_OK;
         }
+        k_residual_norm<MODE, true><<<d.g.nb * cpb, kThreads, 0, F->st>>>(F->a_lam, f, d.c64(), d.ih2_64, d.vol_32, d.g,
+                                                                          cpb, d.f32, F->pscale, d.bprob, F->bsum, d.u32,
+                                                                          Skip{}, d.vol_64);
         MG_TRY(enqueue_problem_sums(F));
         MG_CUDA(cudaStreamSynchronize(F->st));
         *rr = 0.0;
-        for (int p2 = 0; p2 < F->np; ++p2) *rr += F->psum_h[p2] / (mult * mult);
+        for (int p2 = 0; p2 < F->np; ++p2) *rr += F->psum_h[p2];
         return MG_OK;
     }
     const int grid = grid_for(d.cells());
@@ -961,7 +963,7 @@ mg_status adjoint_solve(mg_forest *F, const double *u_dev, const double *dLdu_de
     // M^T in FP64, or, on forests with FP32 forward cycles, in FP32 on the residual scaled by a power of two near
     // 1 / ||r|| of the step before (the forward solve's mixed precision, transposed)
     for (; gn > 0.0; ++it) {
-        double rr = 0.0;
+        double rr = gg;
         MG_TRY(adjoint_residual<MODE>(F, it == 0, mult, &rr));
         rel = std::sqrt(rr) / gn;
         if (!std::isfinite(rel) || rel <= rtol || it >= max_cycles) break;

@@ -2520,9 +2520,10 @@ static __global__ void k_coarse_solve(T *__restrict__ u, const T *__restrict__ f
                          ustart[uprob[first]], ustart[uprob[min(first + warps, N) - 1] + 1], stage);
 }
 
-// The CTA's partial sum: vol times the sum of its threads' FP32 values, in FP64 by the first warp.
-__device__ __forceinline__ void cta_norm(float acc, float vol, double *__restrict__ bpart) {
-    __shared__ float sm[kThreads];
+// The CTA's partial sum: vol times the sum of its threads' values, in FP64 by the first warp.
+template <typename T>
+__device__ __forceinline__ void cta_norm(T acc, T vol, double *__restrict__ bpart) {
+    __shared__ T sm[kThreads];
     sm[threadIdx.x] = acc;
     __syncthreads();
     if (threadIdx.x >= 32) return;
@@ -2543,13 +2544,15 @@ __device__ __forceinline__ void cta_norm(float acc, float vol, double *__restric
 // and is reported to ~1e-6 relative) and in FP64 across threads, by one warp per CTA: a CTA has eight cells per thread, and
 // converting and adding across lanes in every warp took an eighth of the FP64 operations, which bound the kernel
 // (512^3: 2.01 -> 1.86 ms).  out / zero_out may be null.
+// EXACT: the sums of h^3 r^2 instead (vol64 = h^3), unscaled and in FP64 throughout: the norm that stops the adjoint solve.
 // ------------------------------------------------------------------------------------------------------------
-template <int MODE>
+template <int MODE, bool EXACT = false>
 static __global__ void __launch_bounds__(kThreads, 5) k_residual_norm(const double *__restrict__ u, const double *__restrict__ f, Coef cf,
                                        const double *__restrict__ ih2, const float *__restrict__ vol, LevelGeom g,
                                        int cpb, float *__restrict__ out, const float *__restrict__ pscale,
                                        const int32_t *__restrict__ bprob, double *__restrict__ bpart,
-                                       float *__restrict__ zero_out, Skip skip = Skip{}) {
+                                       float *__restrict__ zero_out, Skip skip = Skip{},
+                                       const double *__restrict__ vol64 = nullptr) {
     const int lg = g.lg, n = g.n, P = g.P;
     const int64_t b = blockIdx.x / cpb;
     if (skip(b)) return;  // the whole CTA: its partial stays 0
@@ -2557,7 +2560,8 @@ static __global__ void __launch_bounds__(kThreads, 5) k_residual_norm(const doub
     const int per = (1 << (3 * lg)) / cpb;
     const int sexp = static_cast<int>((__float_as_uint(pscale[bprob[b]]) >> 23) & 0xff) - 127;  // scale = 2^sexp
     const double ihb = MODE == 1 ? 0.0 : ih2[b];
-    float acc = 0.0f;
+    using Acc = std::conditional_t<EXACT, double, float>;
+    Acc acc = 0;
     for (int c = chunk * per + threadIdx.x; c < (chunk + 1) * per; c += blockDim.x) {
         const int x = c & (n - 1), y = (c >> lg) & (n - 1), z = c >> (2 * lg);
         const int64_t gi = b * g.bs + off3(x + 1, y + 1, z + 1, P);
@@ -2575,9 +2579,11 @@ static __global__ void __launch_bounds__(kThreads, 5) k_residual_norm(const doub
             if (z == 0) zero_out[Lay<float>::at(g, b, x + 1, y + 1, 0)] = 0.0f;
             if (z == n - 1) zero_out[Lay<float>::at(g, b, x + 1, y + 1, n + 1)] = 0.0f;
         }
-        acc = fmaf(rs, rs, acc);
+        if constexpr (EXACT) acc = fma(r, r, acc);
+        else acc = fmaf(rs, rs, acc);
     }
-    cta_norm(acc, vol[b], bpart);
+    if constexpr (EXACT) cta_norm(acc, vol64[b], bpart);
+    else cta_norm(acc, vol[b], bpart);
 }
 
 // The same for u = 0, r = f (a zero initial guess): a stream, two cells of a row per thread, four of those in flight.  The

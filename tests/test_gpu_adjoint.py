@@ -1,6 +1,8 @@
 """Adjoint path on the GPU: A^T, the adjoint solve, dL/df and dL/dk against the oracle and against finite
 differences.  L = 1/2 sum (u - u_t)^2; lambda solves A^T lambda = u - u_t; dL/df = lambda; dL/dk = -lambda^T dA/dk u.
 """
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -200,3 +202,28 @@ def test_autograd_function_matches_directional_differences():
     an_k = float((kr.grad * dk).sum())
     assert abs(fd_f - an_f) <= 1e-6 * abs(an_f)
     assert abs(fd_k - an_k) <= 1e-5 * abs(an_k)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_the_adjoint_stops_by_its_norm_in_64_bits(precision):
+    """lambda = 0 has the relative residual 1, and lambda after two cycles the one that A^T gives: each is accepted with that
+    tolerance (plus 1e-10 of it, where the two are computed differently) and refused with 1e-10 of it less.  Partial sums in
+    FP32 are off by about 1e-8."""
+    from paper_2403_08063_gb300 import Forest, MGError
+    R, n, keys = syn.workload_forest("uniform_2x16")
+    for seed in range(12):
+        g = syn.uniform_rhs(len(keys), n, seed=seed).to(DEV)
+        F = Forest(R, n, keys, precision=precision)
+        F.set_rhs(g)
+        lam, _ = F.adjoint(g, g, want_k=False, rtol=1.0, max_cycles=0)
+        assert float(lam.abs().max()) == 0.0
+        with pytest.raises(MGError):
+            F.adjoint(g, g, want_k=False, rtol=1.0 - 1e-10, max_cycles=0)
+        lam = torch.empty_like(g)
+        ptr = [ctypes.c_void_p(t.data_ptr()) for t in (g, g, lam)]
+        assert F.lib.mg_adjoint_solve(F.h, *ptr, None, 0.0, 2) == 6  # not converged; lambda after two cycles
+        rel = float((g - F.apply_transpose(lam)).norm() / g.norm())
+        F.adjoint(g, g, want_k=False, rtol=rel * (1 + 1e-10), max_cycles=2)
+        with pytest.raises(MGError):
+            F.adjoint(g, g, want_k=False, rtol=rel * (1 - 1e-10), max_cycles=2)
+        F.close()
