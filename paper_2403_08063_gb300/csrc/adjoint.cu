@@ -3,10 +3,11 @@
 // step that cites its passage.
 //
 // A = S E: E fills ghosts from interiors (reflection, copy, C2F extrapolation of Sec. 3.3.2, F2C mean of Sec. 3.3.1
-// or the conservative flux ghost), S is the 7-point stencil; A^T = E^T S^T.  Between blocks of one level and at the domain
-// boundary E and S transpose into themselves (a copied ghost's adjoint is the neighbour's own coefficient times its value,
-// a reflection's is its own), so away from refinement interfaces A^T y is the forward stencil on y with the forward's
-// ghosts.  At a refinement interface, with a_j the adjoint of fine ghost j, T~ = T / h^2 and y_C the coarse cell behind it:
+// or the conservative flux ghost), S is the 7-point stencil; A^T = E^T S^T.  At the domain boundary, and between blocks of one
+// level that hold the same coefficient of their common face, E and S transpose into themselves, so there A^T y is the
+// forward stencil on y with the forward's ghosts.  (A merged level under face averaging can hold two coefficients of a face,
+// each its own side's mean of finer faces: the neighbour's coefficient then belongs to its value, and the difference times
+// that value goes to the right-hand side, k_adj_uneven.)  At a refinement interface, with a_j the adjoint of fine ghost j, T~ = T / h^2 and y_C the coarse cell behind it:
 //     conservative: the fine ghost reads y_C / 8 and the coarse one y_C (the rows of u_j and u_C in the coarse ghost
 //                   G = u_C - sum_j T_j / (2 T_C) (g_j - u_j)), and a_j = -T~_j (y_j - y_C / 8);
 //     ghost-only:   both read 0, a_j = -T~_j y_j, and each of the eight fine cells of the coarse ghost's mean gets
@@ -180,6 +181,30 @@ __global__ void __launch_bounds__(kThreads)
         }
     }
     if (adds) scatter_c2f<T>(m, Q, F, sgn, add);
+}
+
+// Same-level faces with a coefficient on either side: row i of A^T has the neighbour's one, T_B, where the stencil has the
+// block's own, T_A, so f' takes (T_B - T_A) / h^2 times what changed of the value on the other side (old: what f' holds).
+// One thread per face cell of every item; the cells at a block's edges belong to several.
+template <typename T, int MODE>
+__global__ void __launch_bounds__(kThreads)
+    k_adj_uneven(const T *__restrict__ y, Coef cf, const T *__restrict__ ih2, const FaceItem *__restrict__ items, int nitems,
+                 LevelGeom g, T *__restrict__ old, T *__restrict__ f) {
+    pdl_enter(y, old, f);
+    const int n = g.n, lg = g.lg;
+    const int64_t total = static_cast<int64_t>(nitems) << (2 * lg);
+    GRID_STRIDE(total) {
+        const FaceItem F = items[t >> (2 * lg)];
+        if (F.kind != FK_SAME) continue;
+        const int r = static_cast<int>(t) & ((1 << (2 * lg)) - 1), i1 = r & (n - 1), i2 = r >> lg;
+        const auto at = [&](int64_t b, int side, int depth) { return fidx<T>(g, b, F.axis, side, depth, i1, i2); };
+        const int64_t own = at(F.blk, F.side, 1), other = at(F.nbr, 1 - F.side, 1);
+        const T Ta = scaled_face<T, MODE>(cf, ih2, F.blk, at(F.blk, F.side, 0), own, F.axis, F.side);
+        const T Tb = scaled_face<T, MODE>(cf, ih2, F.nbr, at(F.nbr, 1 - F.side, 0), other, F.axis, 1 - F.side);
+        const T now = y[other], before = old[t];
+        old[t] = now;
+        if (Ta != Tb) atomicAdd(&f[own], (Tb - Ta) * (now - before));
+    }
 }
 
 // fe = g again at the cells that k_adj_iface adds to, one strip of an item per CTA.
@@ -712,6 +737,17 @@ void adj_iface(mg_forest *F, DevLevel &d, T *y, bool ghosts, T *old, T *old_c, T
     });
 }
 
+// What of A^T y on a level is no 7-point stencil with the block's own coefficients, brought up to date in y's ghosts and in f.
+template <typename T>
+void adj_update(mg_forest *F, DevLevel &d, const APools<T> &a) {
+    adj_iface<T>(F, d, a.y, true, a.old, a.old_c, {a.f, nullptr, nullptr}, T(-1));
+    if (!d.a_old_s) return;
+    Prof p(F, P_ADJ, 1);
+    constexpr int M = sizeof(T) == 8 ? 1 : 3;  // face-averaged coarse levels only
+    launch_pdl(F->st, !F->batch_member, k_adj_uneven<T, M>, grid_for(static_cast<int64_t>(d.nsfaces) << (2 * d.g.lg)),
+               kThreads, 0, a.y, acoef<T>(d), aih2<T>(d), d.sfaces, d.nsfaces, d.g, static_cast<T *>(d.a_old_s), a.f);
+}
+
 // E^T of level c's interface ghosts, from the finer level d's residual r (gather) or from fc's own ghosts.
 template <typename T>
 void et_iface(mg_forest *F, DevLevel &d, DevLevel &c, T *fc, const T *r, bool gather) {
@@ -742,7 +778,7 @@ void smooth_T(mg_forest *F, int l, int iters, bool &stale) {
     const APools<T> a = apools<T>(F, l);
     for (int i = 0; i < iters; ++i)
         for (int colour = 1; colour >= 0; --colour) {
-            if (stale) adj_iface<T>(F, d, a.y, true, a.old, a.old_c, {a.f, nullptr, nullptr}, T(-1));
+            if (stale) adj_update<T>(F, d, a);
             if constexpr (sizeof(T) == 4) {
                 smooth_level32(F, d, colour);
             } else {
@@ -788,13 +824,10 @@ void vcycle_T(mg_forest *F, int l) {
         cudaMemsetAsync(a.old, 0, d.nifaces * n2 * sizeof(T), F->st);
         if (a.old_c) cudaMemsetAsync(a.old_c, 0, d.nifaces * n2 / 4 * sizeof(T), F->st);
     }
-    const auto iface = [&](bool &stale) {
-        if (stale) adj_iface<T>(F, d, a.y, true, a.old, a.old_c, {a.f, nullptr, nullptr}, T(-1));
-        stale = false;
-    };
+    if (d.a_old_s) cudaMemsetAsync(d.a_old_s, 0, d.nsfaces * n2 * sizeof(T), F->st);
     bool stale = false;
     smooth_T<T>(F, l, F->cfg.nu2, stale);
-    iface(stale);
+    if (stale) adj_update<T>(F, d, a);
     DevLevel &c = F->L[l + 1];
     const APools<T> ac = apools<T>(F, l + 1);
     {
@@ -852,8 +885,12 @@ mg_status ensure_adjoint_pools(mg_forest *F) {
     const int64_t tb = fp32 ? sizeof(float) : sizeof(double);
     const int64_t bytes0 = F->L[0].pool_elems() * static_cast<int64_t>(sizeof(double));
     void *p;
-    for (DevLevel &d : F->L) {
-        const int64_t adj = static_cast<int64_t>(d.nifaces) * d.g.n * d.g.n * tb;
+    bool uneven = false;  // faces with two coefficients: from where a merge took away an interface, under face averaging
+    for (size_t l = 0; l < F->L.size(); ++l) {
+        DevLevel &d = F->L[l];
+        const int64_t n2 = static_cast<int64_t>(d.g.n) * d.g.n, adj = d.nifaces * n2 * tb;
+        if (l > 0 && F->cfg.coeff && F->cfg.coarse_coef == 1 && !F->L[l - 1].all_halve) uneven |= F->L[l - 1].nifaces > 0;
+        if (uneven && d.nsfaces && l + 1 < F->L.size()) MG_TRY(forest_alloc(F, &d.a_old_s, d.nsfaces * n2 * tb));
         MG_TRY(forest_alloc(F, &d.a_r, d.pool_elems() * tb));
         if (adj) MG_TRY(forest_alloc(F, &d.a_old, adj));
         if (adj && !F->cfg.interface_flux) MG_TRY(forest_alloc(F, &d.a_old_c, adj / 4));

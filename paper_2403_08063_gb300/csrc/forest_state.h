@@ -80,6 +80,9 @@ struct DevLevel {
     // transposed cycles (allocated by the first adjoint call, in the cycles' precision): residual pool, and per interface
     // item the ghost adjoints that the right-hand side already holds
     void *a_r = nullptr, *a_old = nullptr, *a_old_c = nullptr;
+    // same-level faces whose two blocks hold different coefficients (a merged level under face averaging): per face cell the
+    // value on the other side that the right-hand side already holds (null: the level has none)
+    void *a_old_s = nullptr;
     // FP32 cycles on a face-averaged coarse level: its halved face coefficients (colour-split) and mode 3
     float *ax32 = nullptr, *ay32 = nullptr, *az32 = nullptr;
     bool face32 = false;

@@ -227,3 +227,45 @@ def test_the_adjoint_stops_by_its_norm_in_64_bits(precision):
         with pytest.raises(MGError):
             F.adjoint(g, g, want_k=False, rtol=rel * (1 - 1e-10), max_cycles=2)
         F.close()
+
+
+def _one_transposed_cycle(F, g):
+    """lambda after one cycle from 0 (tolerance 0 is not met: status 6, lambda is written)."""
+    lam = torch.empty_like(g)
+    ptr = [ctypes.c_void_p(t.data_ptr()) for t in (g, g, lam)]
+    assert F.lib.mg_adjoint_solve(F.h, *ptr, None, 0.0, 1) == 6
+    return lam
+
+
+@pytest.mark.parametrize("R,n,refined,coeff,coarse_coef,flux", [
+    (2, 16, False, False, "k", True), (2, 64, False, False, "k", True), (1, 128, False, False, "k", True),
+    (2, 16, False, True, "faces", True), (2, 64, False, True, "faces", True), (1, 128, False, True, "faces", True),
+    (2, 64, False, True, "k", True), (2, 8, True, True, "faces", True), (2, 16, True, True, "faces", False),
+    (4, 8, True, True, "faces", True), (2, 16, True, True, "k", False), (2, 32, True, False, "k", True)])
+def test_one_transposed_cycle(R, n, refined, coeff, coarse_coef, flux):
+    """A V-cycle from 0 is a linear map M of its right-hand side and the adjoint's cycle is M^T: <g, M f> = <M^T g, f> up to
+    FP64 rounding.  The FP32 transposed cycle is element by element as close to the FP64 one as the FP32 forward cycle is to
+    the FP64 forward one: the same half-sweeps and transfers in the same arithmetic, so their roundings differ by a small
+    factor (8 in the L2 norm, 16 in the maximum norm), where a wrong index or weight is off by orders of magnitude.  With
+    averaged faces the merged levels of a refined forest hold two coefficients of a face, one per block."""
+    from paper_2403_08063_gb300 import Forest
+    keys = syn.workload_forest(f"sphere_{R}x{n}")[2] if refined else syn.uniform_leaves(R)
+    g, f = (syn.uniform_rhs(len(keys), n, seed=s).to(DEV) for s in (71, 72))
+    k = syn.lognormal_k_rff(R, n, keys, seed=73, device=DEV) if coeff else None
+    Mf, Mg = {}, {}
+    for precision in (0, 1):
+        F = Forest(R, n, keys, coeff=coeff, precision=precision, coarse_coef=coarse_coef, interface_flux=flux)
+        F.set_rhs(f, k)
+        Mf[precision] = torch.zeros_like(f)
+        F.vcycle(Mf[precision], 1)
+        Mg[precision] = _one_transposed_cycle(F, g)
+        F.close()
+    gMf, Mgf = float((g * Mf[0]).sum()), float((Mg[0] * f).sum())
+    assert abs(gMf - Mgf) <= 1e-13 * float(g.norm() * Mf[0].norm())
+    fwd, adj = Mf[1] - Mf[0], Mg[1] - Mg[0]
+    l2 = [float(e.norm() / x.norm()) for e, x in ((fwd, Mf[0]), (adj, Mg[0]))]
+    mx = [float(e.abs().max() / x.abs().max()) for e, x in ((fwd, Mf[0]), (adj, Mg[0]))]
+    print(f"{R} {n} {refined} {coeff} {coarse_coef} {flux}: forward {l2[0]:.2e} ({mx[0]:.2e}), transposed {l2[1]:.2e} "
+          f"({mx[1]:.2e})")
+    assert 1e-9 < l2[0] < 1e-6
+    assert l2[1] <= 8 * l2[0] and mx[1] <= 16 * mx[0]
