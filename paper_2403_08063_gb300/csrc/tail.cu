@@ -3,9 +3,11 @@
 // thousand to a few hundred thousand cells) and their kernels last a few microseconds each, so launching them one
 // by one is latency-bound; here the CTAs stay resident and walk a phase list recorded from the same schedule as the
 // launched V-cycle (smoothing half-sweeps, interface and full exchanges, restriction, prolongation, coarsest
-// solve), separated by grid barriers.  Every phase runs the same device code as the corresponding kernel (loads of
-// data written by earlier phases go through L2), so results are bit-identical to the launched V-cycle.  No
-// counterpart in the paper, whose generated code runs the cycle level by level (Sec. 4).
+// solve), separated by grid barriers.  Every phase but one runs the same device code as the corresponding kernel (loads
+// of data written by earlier phases go through L2).  Refinement interfaces have two forms, the launched one with a strip's
+// values shared by its CTA (exchange_iface_cta), here every lane for itself (exchange_iface_body), with the same
+// operations in the same order.  So results are bit-identical to the launched V-cycle.  No counterpart in the paper, whose
+// generated code runs the cycle level by level (Sec. 4).
 #include "forest_state.h"
 #include "kernels.cuh"
 

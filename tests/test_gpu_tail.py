@@ -59,3 +59,25 @@ def test_tail_arguments_are_checked():
         F.set_tail(len(F.levels()))
     F.set_tail(0)
     assert F.tail_level() == 0
+
+
+@pytest.mark.parametrize("coeff,coarse_coef", [(False, "k"), (True, "k"), (True, "faces")])
+def test_tail_reproduces_ghost_only_interfaces(coeff, coarse_coef):
+    """The launched exchange shares its interface values in shared memory, a CTA per strip of a face, the tail's computes them
+    per ghost in one lane: the same operations in the same order, here for the ghost-only coarse side (the mean of eight
+    cells) in every FP32 coefficient mode, on three levels of interfaces."""
+    from paper_2403_08063_gb300 import Forest
+    R, n, keys = syn.workload_forest("sphere_2x16")
+    dev = torch.device(DEV)
+    f = syn.gaussian_bump_with_noise(R, n, keys, seed=53, device=dev)
+    k = syn.lognormal_k_rff(R, n, keys, seed=54, device=dev) if coeff else None
+    F = Forest(R, n, keys, coeff=coeff, precision=1, inner_cycles=2, coarse_coef=coarse_coef, interface_flux=False)
+    F.set_rhs(f, k)
+    out = []
+    for level in (-1, 0, 1):
+        F.set_tail(level)
+        u = torch.zeros_like(f)
+        out.append((F.vcycle(u, 3), u))
+    for rel, u in out[1:]:
+        assert rel == out[0][0] and torch.equal(u, out[0][1])
+    F.close()
