@@ -151,9 +151,12 @@ struct Replay {
     int runs = 0;
     bool off = false;  // the recording failed or cannot be replayed: launched directly
     int64_t nlaunch[32] = {};  // its launches per kernel family, counted at every replay
+    // What it records has changed: the next run is a first one again, and a recording that failed is tried again.
     void drop() {
         if (exec) cudaGraphExecDestroy(exec);
         exec = nullptr;
+        runs = 0;
+        off = false;
     }
 };
 
@@ -301,6 +304,8 @@ mg_status replay(mg_forest *F, Replay &r, Body &&body, Ok &&recorded) {
             body();
             F->st = own;
             e = cudaStreamEndCapture(F->cap_st, &graph);
+            const cudaError_t launch = cudaGetLastError();  // of one that failed without ending the capture
+            if (e == cudaSuccess) e = launch;
             ok = recorded();
             for (int c = 0; c < 32; ++c) {
                 r.nlaunch[c] = F->nlaunch[c] - before[c];

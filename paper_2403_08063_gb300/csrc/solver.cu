@@ -1737,8 +1737,7 @@ mg_status mg_exchange_level(mg_forest *F, int32_t level, const double *u_dev, do
 
 // The recorded FP32 cycles hold the launch shapes and the tail they were recorded with.
 static mg_status drop_cycles32(mg_forest *F) {
-    if (!F->v32_rec.exec && !F->vT_rec.exec) return MG_OK;
-    MG_CUDA(cudaStreamSynchronize(F->st));
+    if (F->v32_rec.exec || F->vT_rec.exec) MG_CUDA(cudaStreamSynchronize(F->st));
     F->v32_rec.drop();
     F->vT_rec.drop();
     return MG_OK;
