@@ -1040,10 +1040,40 @@ void vcycle32_part(mg_forest *F, int part) {
     }
 }
 
+// The fastest tail level of the candidates (-1: off), each timed over five recorded FP32 V-cycles (after three untimed ones)
+// on the FP32 pools, which are dead between solves; its phases are recorded.
+mg_status time_tails(mg_forest *F, const std::vector<int> &cand, cudaEvent_t e0, cudaEvent_t e1, int *pick) {
+    float best = 0.0f;
+    for (int lt : cand) {
+        if (lt >= 0) MG_TRY(record_tail(F, lt));
+        F->tail_level = lt;
+        Replay rec;  // as a solve runs it
+        float ms = 0.0f;
+        const auto timed = [&]() -> mg_status {
+            for (int w = 0; w < 3; ++w) MG_TRY(replay(F, rec, [&] { vcycle32(F); }));
+            MG_CUDA(cudaEventRecord(e0, F->st));
+            for (int w = 0; w < 5; ++w) MG_TRY(replay(F, rec, [&] { vcycle32(F); }));
+            MG_CUDA(cudaEventRecord(e1, F->st));
+            MG_CUDA(cudaEventSynchronize(e1));
+            MG_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+            return MG_OK;
+        };
+        const mg_status st = timed();
+        rec.drop();
+        MG_TRY(st);
+        if (lt == -1 || ms < best) {
+            best = ms;
+            *pick = lt;
+        }
+    }
+    MG_CUDA(cudaGetLastError());
+    MG_TRY(check_kernel_waits(F));
+    return *pick >= 0 ? record_tail(F, *pick) : MG_OK;
+}
+
 // Picks the persistent tail's level: every level l whose own and deeper levels have at most 2^20 cells (and
-// specialised smoothers) is a candidate; each candidate and "off" is timed over five recorded FP32 V-cycles (after
-// three untimed ones) on the FP32 pools, which are dead between solves, and the fastest is kept.  Skipped (off) while the
-// stream is being captured.
+// specialised smoothers) is a candidate beside "off".  Skipped (off) while the stream is being captured; when it fails the
+// tail is off and still to be tuned.
 mg_status tune_tail(mg_forest *F) {
     if (F->tail_tuned || F->cfg.precision != 1) return MG_OK;
     F->tail_tuned = true;
@@ -1062,33 +1092,12 @@ mg_status tune_tail(mg_forest *F) {
         set_error("cudaEventCreate failed");
         return MG_ERR_CUDA;
     }
-    float best = 0.0f;
     int pick = -1;
-    for (int lt : cand) {
-        if (lt >= 0) MG_TRY(record_tail(F, lt));
-        F->tail_level = lt;
-        Replay rec;  // as a solve runs it
-        mg_status st = MG_OK;
-        for (int w = 0; w < 3 && st == MG_OK; ++w) st = replay(F, rec, [&] { vcycle32(F); });
-        MG_CUDA(cudaEventRecord(e0, F->st));
-        for (int w = 0; w < 5 && st == MG_OK; ++w) st = replay(F, rec, [&] { vcycle32(F); });
-        MG_CUDA(cudaEventRecord(e1, F->st));
-        MG_CUDA(cudaEventSynchronize(e1));
-        rec.drop();
-        MG_TRY(st);
-        float ms = 0.0f;
-        MG_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-        if (lt == -1 || ms < best) {
-            best = ms;
-            pick = lt;
-        }
-    }
+    const mg_status st = time_tails(F, cand, e0, e1, &pick);
     F->ev_used -= 2;
-    MG_CUDA(cudaGetLastError());
-    MG_TRY(check_kernel_waits(F));
-    if (pick >= 0) MG_TRY(record_tail(F, pick));
-    F->tail_level = pick;
-    return MG_OK;
+    F->tail_level = st == MG_OK ? pick : -1;
+    F->tail_tuned = st == MG_OK;
+    return st;
 }
 
 // The power of two nearest to x, kept inside the binary32 normal range (the kernels apply it on exponent bits).

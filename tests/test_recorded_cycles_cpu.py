@@ -116,3 +116,13 @@ g = calls("cudaGraphLaunch")
 fail("launch", n // 2)  # most launches of the call are the cycle's
 assert cycles(h, 1) == 0 and calls("cudaGraphLaunch") == g
 ''')
+
+
+def test_a_failure_while_the_tail_is_tuned_leaves_it_off(scenario):
+    scenario('''
+h = forest()
+fail("cudaGraphLaunch", 9)  # seven per candidate: the first tail's
+assert lib.mg_set_rhs(h, F, None) == 5 and tail_of(h) == -1
+g = calls("cudaGraphLaunch")
+assert lib.mg_set_rhs(h, F, None) == 0 and calls("cudaGraphLaunch") == g + 21  # tuned now: off and two tails
+''')
