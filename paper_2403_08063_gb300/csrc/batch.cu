@@ -193,9 +193,7 @@ mg_status enqueue_step(mg_batch *B, int m) {
 mg_status apply_tail_mode(mg_batch *B, int mode) {
     for (size_t g = 0; g < B->groups.size(); ++g) {
         mg_forest *F = B->groups[g];
-        const int lt = mode == 0 ? -1 : B->tuned_tails[g];
-        if (lt >= 0 && F->tail_for != lt) MG_TRY(record_tail(F, lt));
-        F->tail_level = lt;
+        MG_TRY(set_tail_level(F, mode == 0 ? -1 : B->tuned_tails[g]));
     }
     B->tail_mode = mode;
     if (mode == 2) MG_TRY(build_joint_tail(B));

@@ -365,7 +365,8 @@ int64_t tail_ctas(mg_forest *F);  // tail.cu: CTAs the largest phase of F's tail
 void vcycle32_part(mg_forest *F, int part);
 // solver.cu: u64 += e32 / scale_p (set: u64 = e32 / scale_p), same-level and boundary ghosts written
 mg_status enqueue_update_mixed(mg_forest *F, bool set = false);
-mg_status record_tail(mg_forest *F, int l);   // solver.cu
+mg_status set_tail_level(mg_forest *F, int l);  // solver.cu
+mg_status drop_cycles32(mg_forest *F);          // solver.cu
 mg_status launch_selftest_wait(mg_forest *F, int which);  // tail.cu (F->tail_bar allocated)
 void reset_done(mg_forest *F);
 mg_status enqueue_done(mg_forest *F);

@@ -699,6 +699,23 @@ mg_status record_tail(mg_forest *F, int l) {
     return MG_OK;
 }
 
+// The recorded FP32 cycles hold the launch shapes and the tail they were recorded with.
+mg_status drop_cycles32(mg_forest *F) {
+    if (F->v32_rec.exec || F->vT_rec.exec) MG_CUDA(cudaStreamSynchronize(F->st));
+    F->v32_rec.drop();
+    F->vT_rec.drop();
+    return MG_OK;
+}
+
+// Every change of a forest's tail after its tuning goes through here: the recorded cycles launch the tail's phases, of which
+// there is one list.
+mg_status set_tail_level(mg_forest *F, int l) {
+    MG_TRY(drop_cycles32(F));
+    if (l >= 0 && F->tail_for != l) MG_TRY(record_tail(F, l));
+    F->tail_level = l;
+    return MG_OK;
+}
+
 // CTA chunks per block for the per-block reductions: about 2048 cells per CTA.
 int chunks_per_block(const DevLevel &d) { return std::max(1, static_cast<int>(d.cells() / d.g.nb) / 2048); }
 
@@ -1744,14 +1761,6 @@ mg_status mg_exchange_level(mg_forest *F, int32_t level, const double *u_dev, do
     return MG_OK;
 }
 
-// The recorded FP32 cycles hold the launch shapes and the tail they were recorded with.
-static mg_status drop_cycles32(mg_forest *F) {
-    if (F->v32_rec.exec || F->vT_rec.exec) MG_CUDA(cudaStreamSynchronize(F->st));
-    F->v32_rec.drop();
-    F->vT_rec.drop();
-    return MG_OK;
-}
-
 mg_status mg_get_smoother_shape(const mg_forest *F, int32_t level, int32_t *shape) {
     if (!F || level < 0 || level >= static_cast<int32_t>(F->L.size()) || !shape) {
         set_error("null forest or output, or level out of range");
@@ -1838,19 +1847,12 @@ mg_status mg_set_tail(mg_forest *F, int32_t level) {
         set_error("null forest");
         return MG_ERR_INVALID_ARG;
     }
-    MG_TRY(drop_cycles32(F));
-    if (level < 0) {
-        F->tail_level = -1;
-        F->tail_tuned = true;
-        return MG_OK;
-    }
-    if (!tail_possible(F, level)) {
+    if (level >= 0 && !tail_possible(F, level)) {
         set_error("no persistent tail from level " + std::to_string(level) +
                   " (FP32 cycles and block edges 4..128 on every deeper level required)");
         return MG_ERR_INVALID_ARG;
     }
-    MG_TRY(record_tail(F, level));
-    F->tail_level = level;
+    MG_TRY(set_tail_level(F, std::max(-1, level)));
     F->tail_tuned = true;
     return MG_OK;
 }

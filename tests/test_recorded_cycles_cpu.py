@@ -127,3 +127,18 @@ fake.cudaGetLastError()  # the runtime keeps an error until it is read
 g = calls("cudaGraphLaunch")
 assert lib.mg_set_rhs(h, F, None) == 0 and calls("cudaGraphLaunch") == g + 21  # tuned now: off and two tails
 ''')
+
+
+def test_a_batch_that_changes_a_groups_tail_drops_its_recorded_cycle(scenario):
+    scenario('''
+cfg = config(8, [(0, 0, 0, 0, 0), (1, 0, 0, 0, 0)], 2)
+B = c.c_void_p()
+assert lib.mg_batch_create(c.byref(cfg), (c.c_int32 * 2)(8, 16), c.byref(B)) == 0
+h = c.c_void_p(lib.mg_batch_group(B, 1))
+assert lib.mg_set_tail(h, 0) == 0 and lib.mg_batch_set_rhs(B, F, None) == 0
+assert lib.mg_set_tail(h, 1) == 0 and cycles(h, 3) == 0
+assert lib.mg_batch_set_tail_mode(B, 1) == 0 and tail_of(h) == 0
+b, g = calls("cudaStreamBeginCapture"), calls("cudaGraphLaunch")
+assert cycles(h, 1) == 0 and calls("cudaGraphLaunch") == g  # not the cycle with the tail from level 1
+assert cycles(h, 1) == 0 and calls("cudaStreamBeginCapture") == b + 1
+''')
