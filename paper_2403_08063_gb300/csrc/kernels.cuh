@@ -2844,14 +2844,52 @@ static __global__ void __launch_bounds__(kThreads) k_update_mixed(double *__rest
     }
 }
 
-// Whether any entry of x is not zero (NaN counts).
-static __global__ void k_any_nonzero(const double *__restrict__ x, int64_t count, int *__restrict__ flag) {
+// An initial guess into the padded pool, where it is not zero: CTA (b, c) takes the c-th of cpb chunks of block b (at most
+// kGuessCells cells, all loads first).  With a value that is not 0 (NaN counts) it writes them all and counts itself in
+// *written, else it marks the chunk in zero[].  So a guess of 0 is read once, any other read and written once, as by k_pack; of
+// one that has both kinds of chunks the marked ones are left to k_zero_chunks.
+// 512^3 cells, a solve that ends at its first residual: 2.84 ms (0.80 from a guess of 0); with k_pack alone 3.14 ms, with a
+// pass over u to find out before it 3.21 ms.
+constexpr int kGuessCells = 2048;
+static __global__ void __launch_bounds__(kThreads) k_pack_nonzero(double *__restrict__ pool, const double *__restrict__ user,
+                                                                  LevelGeom g, int cpb, int *__restrict__ written,
+                                                                  uint8_t *__restrict__ zero) {
+    constexpr int K = kGuessCells / kThreads;
+    const int lg = g.lg, n = g.n, per = (1 << (3 * lg)) / cpb;
+    const int64_t b = blockIdx.x / cpb;
+    const int c0 = (blockIdx.x - static_cast<int>(b * cpb)) * per;
+    const double *ub = user + (b << (3 * lg)) + c0;
+    double v[K];
     bool any = false;
-#pragma unroll 8
-    for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < count;
-         t += static_cast<int64_t>(gridDim.x) * blockDim.x)
-        any |= !(x[t] == 0.0);
-    if (__ballot_sync(0xffffffffu, any) && (threadIdx.x & 31) == 0) atomicOr(flag, 1);
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        const int c = threadIdx.x + i * kThreads;
+        v[i] = c < per ? ub[c] : 0.0;
+    }
+#pragma unroll
+    for (int i = 0; i < K; ++i) any |= !(v[i] == 0.0);
+    any = __syncthreads_or(any);
+    if (threadIdx.x == 0) {
+        zero[blockIdx.x] = !any;
+        if (any) atomicAdd(written, 1);
+    }
+    if (!any) return;
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        const int c = c0 + threadIdx.x + i * kThreads;
+        if (c < c0 + per) pool[b * g.bs + off3((c & (n - 1)) + 1, ((c >> lg) & (n - 1)) + 1, (c >> (2 * lg)) + 1, g.P)] = v[i];
+    }
+}
+
+// 0 into the chunks that k_pack_nonzero marked, one warp per chunk.
+static __global__ void k_zero_chunks(double *__restrict__ pool, LevelGeom g, int cpb, const uint8_t *__restrict__ zero) {
+    const int64_t chunk = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
+    if (chunk >= static_cast<int64_t>(g.nb) * cpb || !zero[chunk]) return;
+    const int lg = g.lg, n = g.n, per = (1 << (3 * lg)) / cpb;
+    const int64_t b = chunk / cpb;
+    const int c0 = static_cast<int>(chunk - b * cpb) * per;
+    for (int c = c0 + (threadIdx.x & 31); c < c0 + per; c += 32)
+        pool[b * g.bs + off3((c & (n - 1)) + 1, ((c >> lg) & (n - 1)) + 1, (c >> (2 * lg)) + 1, g.P)] = 0.0;
 }
 
 // Face coefficients of a level from k with ghosts (variable coefficients: future work in Sec. 8; harmonic-mean

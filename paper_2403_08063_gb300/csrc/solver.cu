@@ -716,8 +716,8 @@ mg_status set_tail_level(mg_forest *F, int l) {
     return MG_OK;
 }
 
-// CTA chunks per block for the per-block reductions: about 2048 cells per CTA.
-int chunks_per_block(const DevLevel &d) { return std::max(1, static_cast<int>(d.cells() / d.g.nb) / 2048); }
+// CTA chunks per block for the per-block reductions and the initial guess: at most kGuessCells cells per CTA.
+int chunks_per_block(const DevLevel &d) { return std::max(1, static_cast<int>(d.cells() / d.g.nb) / kGuessCells); }
 
 // Per-problem sums of the per-block sums to the host (pinned psum_h), synchronising the stream.
 mg_status read_problem_sums(mg_forest *F) {
@@ -1145,22 +1145,27 @@ mg_status enqueue_residual(mg_forest *F, bool zero_u, bool current) {
 }
 
 // Reports whether the caller's u is all zero (one read-back) and packs it into the level-0 FP64 pool; with keep_zero a zero
-// one too.
+// one too (without, the pool of a zero one keeps what it held, and the forest has no leaf_off).
 mg_status pack_initial_guess(mg_forest *F, const double *u_dev, bool *zero, bool keep_zero) {
     DevLevel &d = F->L[0];
+    const int cpb = F->bsum_cpb, chunks = d.g.nb * cpb;
     MG_CUDA(cudaMemsetAsync(F->flag, 0, sizeof(int), F->st));
     if (keep_zero) {
         Prof p(F, P_LAYOUT, 1);
         k_pack<double><<<grid_for(d.cells()), kThreads, 0, F->st>>>(d.u64, u_dev, d.g, F->leaf_off, F->flag);
     } else {
         Prof p(F, P_LAYOUT, 1);
-        k_any_nonzero<<<grid_for(d.cells()), kThreads, 0, F->st>>>(u_dev, d.cells(), F->flag);
+        k_pack_nonzero<<<chunks, kThreads, 0, F->st>>>(d.u64, u_dev, d.g, cpb, F->flag, F->guess_zero);
     }
     int h = 1;
     MG_CUDA(cudaMemcpyAsync(&h, F->flag, sizeof(int), cudaMemcpyDeviceToHost, F->st));
     MG_CUDA(cudaStreamSynchronize(F->st));
     *zero = h == 0;
-    if (!keep_zero && h) MG_TRY(pack_user<double>(F, d, d.u64, u_dev));
+    if (!keep_zero && h && h < chunks) {
+        Prof p(F, P_LAYOUT, 1);
+        k_zero_chunks<<<(chunks * 32 + kThreads - 1) / kThreads, kThreads, 0, F->st>>>(d.u64, d.g, cpb, F->guess_zero);
+        MG_CUDA(cudaGetLastError());
+    }
     return MG_OK;
 }
 
@@ -1473,6 +1478,7 @@ mg_status create(const mg_config *cfg, mg_forest **out) {
         if ((st = upload(F, &F->pblk, pblk)) != MG_OK) return fail(st);
         F->bsum_cpb = chunks_per_block(F->L[0]);
         if ((st = dalloc(F, &F->bsum, static_cast<int64_t>(h0.keys.size()) * F->bsum_cpb)) != MG_OK) return fail(st);
+        if ((st = dalloc(F, &F->guess_zero, static_cast<int64_t>(h0.keys.size()) * F->bsum_cpb)) != MG_OK) return fail(st);
         if ((st = dalloc(F, &F->psum, np)) != MG_OK) return fail(st);
         if ((st = dalloc(F, &F->pscale, np)) != MG_OK) return fail(st);
         if ((st = dalloc(F, &F->pinv, np)) != MG_OK) return fail(st);

@@ -78,3 +78,28 @@ def test_recorded_cycles_follow_a_new_launch_shape_and_are_counted(coeff):
     assert counts[0] == counts[1] and counts[0]["smooth_f32_finest"] > 0
     assert np.isfinite(float(runs[0].norm()))
     F.close()
+
+
+@pytest.mark.parametrize("n", [4, 8, 16, 64])
+@pytest.mark.parametrize("what", ["dense", "blocks", "last"])
+def test_a_guess_is_read_and_written_once(n, what):
+    """One layout launch packs a guess without a zero part (and one unpacks the result); parts that are zero are cleared of
+    what an earlier solve left there.  The iterate is that of a forest that has solved nothing."""
+    guess = torch.rand((8, n ** 3), generator=torch.Generator().manual_seed(75), dtype=torch.float64).to(DEV) + 0.5
+    if what == "blocks":
+        guess[::2] = 0.0
+    elif what == "last":
+        guess.view(-1)[:-1] = 0.0
+    out = []
+    for used in (False, True):
+        F, f = _forest(n, inner_cycles=2)
+        if used:
+            F.solve(torch.zeros_like(f), rtol=1e-8)
+        u = guess.clone()
+        F.profile(True)
+        rel = F.vcycle(u, 2)
+        assert F.profile_read()["layout"][1] == (2 if what == "dense" else 3)
+        F.profile(False)
+        out.append((rel, u))
+        F.close()
+    assert out[0][0] == out[1][0] and torch.equal(out[0][1], out[1][1])
