@@ -603,7 +603,8 @@ __global__ void k_add(double *__restrict__ y, const double *__restrict__ x, Leve
 // dL/dk = -lambda^T (dA/dk) u, written in the caller's layout.  A face between cells i and f with T = 2 k_i k_f / (k_i +
 // k_f) enters rows i and f with (1/h^2) T (u_i - u_f) and its negative, and dT/dk_i = 2 k_f^2 / (k_i + k_f)^2 =
 // T^2 / (2 k_i^2), so with T~ = T / h^2
-//     dL/dk_i = -h^2 / (2 k_i^2) sum_f T~_f^2 (lambda_i - lambda_f) (u_i - u_f):
+//     dL/dk_i = -h^2 / 2 sum_f (T~_f / k_i)^2 (lambda_i - lambda_f) (u_i - u_f),
+// where T~_f / k_i <= 2 / h^2 whatever the scale of k (T~_f^2 would overflow from k / h^2 = 2^512 on):
 // one division per cell (six in the form with (k_i + k_f)^2, and the other cell's share by atomics: 5.5 ms on 31.5M cells;
 // this one 2.4 ms, its 45 FP64 operations per cell at the measured FP64 rate).  Ghosts of u and lambda: copies and reflections (at the boundary T = k_i, dT/dk_i = 1: the reflected
 // pair gives the same).  Refinement interfaces are left to k_gradk_iface.
@@ -622,14 +623,16 @@ __global__ void k_gradk(const double *__restrict__ u, const double *__restrict__
         const double T[6] = {cf.tx[gi], cf.tx[gi + 1], cf.ty[gi], cf.ty[gi + P], cf.tz[gi], cf.tz[gi + PP]};
         const int64_t nb[6] = {gi - 1, gi + 1, gi - P, gi + P, gi - PP, gi + PP};
         const bool edge[6] = {x == 0, x == n - 1, y == 0, y == n - 1, z == 0, z == n - 1};
+        const double rk = 1.0 / ki;
         double s = 0.0;
 #pragma unroll
         for (int f = 0; f < 6; ++f) {
             if (edge[f] && nbr6[b * 6 + f] == -2) continue;
-            s = fma((T[f] * T[f]) * (li - lam[nb[f]]), ui - u[nb[f]], s);
+            const double w = T[f] * rk;
+            s = fma((w * w) * (li - lam[nb[f]]), ui - u[nb[f]], s);
         }
         const int64_t at = off ? off[b] + (t & ((int64_t(1) << (3 * g.lg)) - 1)) : t;
-        out[at] = -0.5 * h2[b] * s / (ki * ki);
+        out[at] = -0.5 * h2[b] * s;
     }
 }
 

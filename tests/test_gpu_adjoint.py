@@ -269,3 +269,24 @@ def test_one_transposed_cycle(R, n, refined, coeff, coarse_coef, flux):
           f"({mx[1]:.2e})")
     assert 1e-9 < l2[0] < 1e-6
     assert l2[1] <= 8 * l2[0] and mx[1] <= 16 * mx[0]
+
+
+@pytest.mark.parametrize("name", ["uniform_2x8", "sphere_2x8"])
+def test_gradient_scales_with_the_coefficient(name):
+    """u, lambda and dL/dk of 2^505 k are those of k times 2^-505, 2^-505 and 2^-1010: k is below the square root of the largest
+    number, k / h^2 above.  Solved to 1e-12; 1e-8 leaves the condition number room."""
+    from paper_2403_08063_gb300 import Forest
+    R, n, keys = syn.workload_forest(name)
+    k = syn.lognormal_k_rff(R, n, keys, seed=65, sigma=0.5, ell=0.3).to(DEV)
+    f, g = (2.0 ** 40 * syn.uniform_rhs(len(keys), n, seed=s).to(DEV) for s in (66, 67))
+    out = []
+    for e in (0, 505):
+        F = Forest(R, n, keys, coeff=True)
+        F.set_rhs(f, 2.0 ** e * k)
+        u = torch.zeros_like(f)
+        F.solve(u, rtol=1e-12)
+        lam, gk = F.adjoint(u, g, rtol=1e-12)
+        out.append((2.0 ** e * u, 2.0 ** e * lam, (gk * 2.0 ** e) * 2.0 ** e))
+        F.close()
+    for a, b in zip(*out):
+        assert bool(torch.isfinite(b).all()) and float((a - b).norm()) <= 1e-8 * float(a.norm())
