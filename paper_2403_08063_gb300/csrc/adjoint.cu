@@ -7,7 +7,8 @@
 // level that hold the same coefficient of their common face, E and S transpose into themselves, so there A^T y is the
 // forward stencil on y with the forward's ghosts.  (A merged level under face averaging can hold two coefficients of a face,
 // each its own side's mean of finer faces: the neighbour's coefficient then belongs to its value, and the difference times
-// that value goes to the right-hand side, k_adj_uneven.)  At a refinement interface, with a_j the adjoint of fine ghost j, T~ = T / h^2 and y_C the coarse cell behind it:
+// that value goes to the right-hand side, k_adj_uneven.)  At a refinement interface, with a_j the adjoint of fine ghost j,
+// T~ = T / h^2 and y_C the coarse cell behind it:
 //     conservative: the fine ghost reads y_C / 8 and the coarse one y_C (the rows of u_j and u_C in the coarse ghost
 //                   G = u_C - sum_j T_j / (2 T_C) (g_j - u_j)), and a_j = -T~_j (y_j - y_C / 8);
 //     ghost-only:   both read 0, a_j = -T~_j y_j, and each of the eight fine cells of the coarse ghost's mean gets
@@ -26,7 +27,8 @@
 // What bounds it: HBM, in the half-sweeps (10 B per updated cell) and the FP64 residual's FP64 rate.  The transposed cycle
 // step by step on natural-layout arrays of its own (the correction, its stencil with ghost adjoints, their scatter by
 // atomics over every face, two vector updates per half-sweep: ~70 B per cell and half-sweep) made set-up, forward solve and
-// adjoint on 448 + 512 blocks of 32^3 (31.5M cells) take 174 to 183 ms, depending on the inputs; this form, with the later steps' kernels, 63 ms.
+// adjoint on 448 + 512 blocks of 32^3 (31.5M cells) take 174 to 183 ms, depending on the inputs; this form, with the later
+// steps' kernels, 63 ms.
 #include <cmath>
 
 #include "forest_state.h"
@@ -502,8 +504,9 @@ __global__ void k_et_faces(T *__restrict__ G, const FaceItem *__restrict__ items
 }
 
 // E^T of a level's interface ghosts, one strip of an item per CTA and one lane per fine ghost, added to the interior of fc.
-// The ghost adjoints are those of the transposed prolongation: GATHER: a quarter of the four finer cells next to the ghost (the level's
-// blocks are halved blocks, r the finer level's residual); else they stand in fc's own ghosts (k_prolong_T_scatter).
+// The ghost adjoints are those of the transposed prolongation: GATHER: a quarter of the four finer cells next to the ghost
+// (the level's blocks are halved blocks, r the finer level's residual); else they stand in fc's own ghosts
+// (k_prolong_T_scatter).
 template <typename T, int MODE, bool FLUX, bool GATHER>
 __global__ void __launch_bounds__(kThreads)
     k_et_iface(T *__restrict__ fc, Coef cf, const FaceItem *__restrict__ items, LevelGeom g, const T *__restrict__ r,
@@ -606,8 +609,9 @@ __global__ void k_add(double *__restrict__ y, const double *__restrict__ x, Leve
 //     dL/dk_i = -h^2 / 2 sum_f (T~_f / k_i)^2 (lambda_i - lambda_f) (u_i - u_f),
 // where T~_f / k_i <= 2 / h^2 whatever the scale of k (T~_f^2 would overflow from k / h^2 = 2^512 on):
 // one division per cell (six in the form with (k_i + k_f)^2, and the other cell's share by atomics: 5.5 ms on 31.5M cells;
-// this one 2.4 ms, its 45 FP64 operations per cell at the measured FP64 rate).  Ghosts of u and lambda: copies and reflections (at the boundary T = k_i, dT/dk_i = 1: the reflected
-// pair gives the same).  Refinement interfaces are left to k_gradk_iface.
+// this one 2.4 ms, its 45 FP64 operations per cell at the measured FP64 rate).  Ghosts of u and lambda: copies and
+// reflections (at the boundary T = k_i, dT/dk_i = 1: the reflected pair gives the same).  Refinement interfaces are left to
+// k_gradk_iface.
 __global__ void k_gradk(const double *__restrict__ u, const double *__restrict__ lam, const double *__restrict__ k,
                         Coef cf, const double *__restrict__ h2, const int32_t *__restrict__ nbr6, LevelGeom g,
                         double *__restrict__ out, const int64_t *__restrict__ off) {
@@ -747,8 +751,9 @@ void adj_update(mg_forest *F, DevLevel &d, const APools<T> &a) {
     if (!d.a_old_s) return;
     Prof p(F, P_ADJ, 1);
     constexpr int M = sizeof(T) == 8 ? 1 : 3;  // face-averaged coarse levels only
-    launch_pdl(F->st, !F->batch_member, k_adj_uneven<T, M>, grid_for(static_cast<int64_t>(d.nsfaces) << (2 * d.g.lg)),
-               kThreads, 0, a.y, acoef<T>(d), aih2<T>(d), d.sfaces, d.nsfaces, d.g, static_cast<T *>(d.a_old_s), a.f);
+    launch_pdl(F->st, !F->batch_member, k_adj_uneven<T, M>,
+               grid_for(static_cast<int64_t>(d.nsfaces) << (2 * d.g.lg)), kThreads, 0, a.y, acoef<T>(d), aih2<T>(d),
+               d.sfaces, d.nsfaces, d.g, static_cast<T *>(d.a_old_s), a.f);
 }
 
 // E^T of level c's interface ghosts, from the finer level d's residual r (gather) or from fc's own ghosts.
@@ -770,8 +775,8 @@ void exchange_same(mg_forest *F, DevLevel &d, T *y) {
     if (!d.nsfaces) return;
     Prof p(F, P_ADJ, 1);
     launch_pdl(F->st, !F->batch_member, k_exchange_faces<T, false>,
-               grid_for(static_cast<int64_t>(d.nsfaces) << (2 * d.g.lg)), kThreads, 0, y,
-               d.sfaces, d.nsfaces, d.g, Skip{}, 0, nullptr);
+               grid_for(static_cast<int64_t>(d.nsfaces) << (2 * d.g.lg)), kThreads, 0, y, d.sfaces, d.nsfaces, d.g,
+               Skip{}, 0, nullptr);
 }
 
 // Red-black iterations on A^T with the colours in reverse order.  `stale`: y changed since the last interface exchange.
@@ -788,8 +793,7 @@ void smooth_T(mg_forest *F, int l, int iters, bool &stale) {
                 Prof p(F, P_ADJ, 1);
                 auto *fn = F->cfg.coeff ? k_smooth<double, 1> : k_smooth<double, 0>;
                 launch_pdl(F->st, !F->batch_member, fn, grid_for(d.cells() / 2), kThreads, 0, a.y, a.f, d.c64(),
-                           d.h2_64, d.g, colour, d.nbr6, Skip{},
-                                                                    nullptr);
+                           d.h2_64, d.g, colour, d.nbr6, Skip{}, nullptr);
             }
             stale = true;
         }
@@ -803,9 +807,8 @@ void launch_residual32(mg_forest *F, DevLevel &d, float *r) {
             k_adj_residual32<M, 2>, k_adj_residual32<M, 3>, k_adj_residual32<M, 4>,
             k_adj_residual32<M, 5>, k_adj_residual32<M, 6>, k_adj_residual32<M, 7>};
         const int64_t pairs = d.cells() / 2;
-        launch_pdl(F->st, !F->batch_member, fns[d.g.lg - 2],
-                   static_cast<unsigned>((pairs + kThreads - 1) / kThreads), kThreads, 0,
-            d.u32, d.f32, d.c32(), d.ih2_32, d.g.bs, pairs, d.nbr6, r);
+        launch_pdl(F->st, !F->batch_member, fns[d.g.lg - 2], static_cast<unsigned>((pairs + kThreads - 1) / kThreads),
+                   kThreads, 0, d.u32, d.f32, d.c32(), d.ih2_32, d.g.bs, pairs, d.nbr6, r);
     });
 }
 
@@ -817,9 +820,8 @@ void vcycle_T(mg_forest *F, int l) {
     const int last = static_cast<int>(F->L.size()) - 1;
     if (l == last) {
         Prof p(F, P_ADJ, 1);
-        launch_pdl(F->st, !F->batch_member, k_coarse_solve<T>, (F->Nc * 32 + kThreads - 1) / kThreads, kThreads, 0,
-                   a.y, a.f, F->AinvT,
-                   sizeof(T) == 4 ? F->cmap32 : F->cmap, F->uprob, F->ustart, F->moff, F->Nc, nullptr);
+        launch_pdl(F->st, !F->batch_member, k_coarse_solve<T>, (F->Nc * 32 + kThreads - 1) / kThreads, kThreads, 0, a.y,
+                   a.f, F->AinvT, sizeof(T) == 4 ? F->cmap32 : F->cmap, F->uprob, F->ustart, F->moff, F->Nc, nullptr);
         return;
     }
     const int64_t n2 = static_cast<int64_t>(d.g.n) * d.g.n;
@@ -840,8 +842,7 @@ void vcycle_T(mg_forest *F, int l) {
         else
             with_mode<T>(F, d, [&](auto m) {
                 launch_pdl(F->st, !F->batch_member, k_adj_residual<T, decltype(m)::value>, grid_for(d.cells()),
-                           kThreads, 0,
-                    a.y, a.f, acoef<T>(d), aih2<T>(d), d.g, d.nbr6, a.r, nullptr, nullptr);
+                           kThreads, 0, a.y, a.f, acoef<T>(d), aih2<T>(d), d.g, d.nbr6, a.r, nullptr, nullptr);
             });
     }
     const bool gather = d.all_halve;
@@ -851,7 +852,7 @@ void vcycle_T(mg_forest *F, int l) {
                                                                k_prolong_T32<6>, k_prolong_T32<7>};
         launch_pdl(F->st, !F->batch_member, fns[d.g.lg - 3],
                    static_cast<unsigned>((c.cells() + kThreads - 1) / kThreads), kThreads, 0,
-            reinterpret_cast<float *>(a.r), d.g.bs, c.f32, c.u32, d.xfer, c.cells(), c.g.bs);
+                   reinterpret_cast<float *>(a.r), d.g.bs, c.f32, c.u32, d.xfer, c.cells(), c.g.bs);
     } else if (gather) {
         Prof p(F, P_ADJ, 1);
         launch_pdl(F->st, !F->batch_member, k_prolong_T<T>, grid_for(c.cells()), kThreads, 0, a.r, d.g, ac.f, ac.y,
@@ -864,8 +865,8 @@ void vcycle_T(mg_forest *F, int l) {
                    d.xfer, c.g);
         if (c.nsfaces)
             launch_pdl(F->st, !F->batch_member, k_et_faces<T>,
-                       grid_for(static_cast<int64_t>(c.nsfaces) << (2 * c.g.lg)), kThreads, 0,
-                ac.f, c.sfaces, c.nsfaces, c.g);
+                       grid_for(static_cast<int64_t>(c.nsfaces) << (2 * c.g.lg)), kThreads, 0, ac.f, c.sfaces,
+                       c.nsfaces, c.g);
     }
     et_iface<T>(F, d, c, ac.f, a.r, gather);
     vcycle_T<T>(F, l + 1);
@@ -873,8 +874,9 @@ void vcycle_T(mg_forest *F, int l) {
     {
         Prof p(F, P_ADJ, 1);
         if constexpr (sizeof(T) == 4) through = inject32(F, d, c);
-        if (!through) launch_pdl(F->st, !F->batch_member, k_inject<T>, grid_for(c.cells()), kThreads, 0, a.y, d.g,
-                                 ac.y, d.xfer, c.g);
+        if (!through)
+            launch_pdl(F->st, !F->batch_member, k_inject<T>, grid_for(c.cells()), kThreads, 0, a.y, d.g, ac.y, d.xfer,
+                       c.g);
     }
     if (!through) exchange_same<T>(F, d, a.y);
     stale = true;

@@ -34,7 +34,8 @@ __global__ void __cluster_dims__(kCjCluster, 1, 1) __launch_bounds__(kCjThreads)
             sm[a * stride + i] = src[a][(rank + i / kCjBlock * kCjCluster) * g.bs + i % kCjBlock];
     cluster.sync();
     const double *sf = sm + 2 * stride;
-    const Coef sc{sm + 3 * stride, sm + 4 * stride, sm + 5 * stride, nullptr, sm + 6 * stride, nullptr, nullptr, nullptr, nullptr};
+    const Coef sc{sm + 3 * stride, sm + 4 * stride, sm + 5 * stride, nullptr, sm + 6 * stride,
+                  nullptr,         nullptr,         nullptr,         nullptr};
     for (int it = 0; it < iters; ++it) {
         double *cur = sm + (it & 1) * stride, *nxt = sm + ((it + 1) & 1) * stride;
         for (int i = threadIdx.x; i < mine * 6 * kCjN * kCjN; i += kCjThreads) {

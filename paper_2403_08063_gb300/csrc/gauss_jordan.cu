@@ -42,8 +42,8 @@ struct GjRow {
     int32_t id;
 };
 
-// Rows of a problem held by one CTA (r % cluster size == rank), and its dynamic shared memory: rows x W doubles (rounded up to whole passes of the
-// CTA) and the rows' origins.
+// Rows of a problem held by one CTA (r % cluster size == rank), and its dynamic shared memory: rows x W doubles (rounded up
+// to whole passes of the CTA) and the rows' origins.
 __host__ __device__ constexpr int gj_rows(int N) { return (N + kGjCluster - 1) / kGjCluster; }
 __host__ __device__ constexpr int64_t gj_panel_elems(int N, int W) {
     return (static_cast<int64_t>(gj_rows(N)) * W + kGjThreads - 1) / kGjThreads * kGjThreads;

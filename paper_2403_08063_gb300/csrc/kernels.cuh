@@ -568,7 +568,8 @@ struct IfaceStrip {
 //   coarse ghosts  one thread per coarse cell.
 // All loads come before the first use of one, and before the done-mask decides (uniformly over the CTA) whether anything is
 // written.  The sharing matters in FP64, whose operations bound the kernel: with 12 of them per ghost, and the coarse side's
-// sum and division by one lane in four of every warp, 6.2 us on 96 faces of 32 x 32 cells, this way 5.9 (five damped Jacobi cycles on 22 blocks of 64^3: 7.1 -> 6.7 ms).
+// sum and division by one lane in four of every warp, 6.2 us on 96 faces of 32 x 32 cells, this way 5.9 (five damped Jacobi
+// cycles on 22 blocks of 64^3: 7.1 -> 6.7 ms).
 template <typename T, int MODE, bool FLUX>
 __device__ __forceinline__ void exchange_iface_cta(T *__restrict__ u, const Coef &cf, const FaceItem &F, int strip,
                                                    const LevelGeom &g, Skip skip, int c2f, T *sm) {
@@ -680,11 +681,11 @@ __device__ __forceinline__ void exchange_iface_body(T *__restrict__ u, const Coe
 }
 
 // Ghost exchange of a level in one launch: CTAs [0, nif strips) one strip of an interface item each, the others the faces
-// filled from one source block (boundary, same level; nsf items, none for the interface-only exchange between half-sweeps), one thread per
-// ghost cell.  Every ghost is computed from block interiors only, so the two parts are independent.  These launches move a
-// few hundred KB and last as long as their chain of dependent loads and instructions, so an item's work is spread over as
-// many lanes as it has ghosts, with every load ahead of the first use: 12.8 us on 384 faces of 32 x 32 cells and 3.2 us on
-// the coarser levels, where one lane per coarse cell, loading as it went, took 22.7 and 4.7 us.
+// filled from one source block (boundary, same level; nsf items, none for the interface-only exchange between half-sweeps),
+// one thread per ghost cell.  Every ghost is computed from block interiors only, so the two parts are independent.  These
+// launches move a few hundred KB and last as long as their chain of dependent loads and instructions, so an item's work is
+// spread over as many lanes as it has ghosts, with every load ahead of the first use: 12.8 us on 384 faces of 32 x 32 cells
+// and 3.2 us on the coarser levels, where one lane per coarse cell, loading as it went, took 22.7 and 4.7 us.
 template <typename T, int MODE, bool FLUX>
 static __global__ void __launch_bounds__(kThreads) k_exchange(T *__restrict__ u, Coef cf,
                                                               const FaceItem *__restrict__ ifaces, int nif,
@@ -2547,12 +2548,11 @@ __device__ __forceinline__ void cta_norm(T acc, T vol, double *__restrict__ bpar
 // EXACT: the sums of h^3 r^2 instead (vol64 = h^3), unscaled and in FP64 throughout: the norm that stops the adjoint solve.
 // ------------------------------------------------------------------------------------------------------------
 template <int MODE, bool EXACT = false>
-static __global__ void __launch_bounds__(kThreads, 5) k_residual_norm(const double *__restrict__ u, const double *__restrict__ f, Coef cf,
-                                       const double *__restrict__ ih2, const float *__restrict__ vol, LevelGeom g,
-                                       int cpb, float *__restrict__ out, const float *__restrict__ pscale,
-                                       const int32_t *__restrict__ bprob, double *__restrict__ bpart,
-                                       float *__restrict__ zero_out, Skip skip = Skip{},
-                                       const double *__restrict__ vol64 = nullptr) {
+static __global__ void __launch_bounds__(kThreads, 5)
+    k_residual_norm(const double *__restrict__ u, const double *__restrict__ f, Coef cf, const double *__restrict__ ih2,
+                    const float *__restrict__ vol, LevelGeom g, int cpb, float *__restrict__ out,
+                    const float *__restrict__ pscale, const int32_t *__restrict__ bprob, double *__restrict__ bpart,
+                    float *__restrict__ zero_out, Skip skip = Skip{}, const double *__restrict__ vol64 = nullptr) {
     const int lg = g.lg, n = g.n, P = g.P;
     const int64_t b = blockIdx.x / cpb;
     if (skip(b)) return;  // the whole CTA: its partial stays 0

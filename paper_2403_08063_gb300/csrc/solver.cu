@@ -108,8 +108,7 @@ void exchange(mg_forest *F, DevLevel &d, T *u, bool interface_only = false, bool
         const int grid = nif * strips + (nsf ? grid_for(static_cast<int64_t>(nsf) * n * n) : 0);
         auto *fn = F->cfg.interface_flux ? k_exchange<T, MODE, true> : k_exchange<T, MODE, false>;
         launch_pdl(F->st, !F->batch_member, fn, grid, threads, smem, u, coef_of<T>(d), d.ifaces, nif, d.sfaces, nsf,
-                   d.g,
-                                                                  skip_of(F, d), F->cfg.c2f_variant, gb);
+                   d.g, skip_of(F, d), F->cfg.c2f_variant, gb);
         return;
     }
     const FaceItem *items = interface_only ? d.ifaces : d.faces;
@@ -218,9 +217,7 @@ void launch_smooth32(mg_forest *F, DevLevel &d, int colour, const Shape &sh, cud
         });
         const int64_t grid = static_cast<int64_t>(d.g.nb) * (n / TY) * (n / TZ);
         launch_pdl(st, !F->batch_member, fn, static_cast<unsigned>(grid), (n / 2) * TY / R + 32, smem, d.u32, d.f32,
-                   d.kap, d.h2_32, d.g.bs, colour,
-                                                                         d.nbr6, TY, TZ, D, F->kerr, skip_of(F, d),
-                                                                         d.ax32, d.ay32, d.az32);
+                   d.kap, d.h2_32, d.g.bs, colour, d.nbr6, TY, TZ, D, F->kerr, skip_of(F, d), d.ax32, d.ay32, d.az32);
         return;
     }
     const int zc = sh[0] == 1 ? sh[1] : 1, threads = sh[0] == 1 ? sh[2] : kThreads;
@@ -369,24 +366,23 @@ void launch_residual_restrict32(mg_forest *F, DevLevel &d, DevLevel &c) {
         });
         const int64_t grid = static_cast<int64_t>(c.g.nb) * (n / TY) * (n / TZ);
         launch_pdl(F->st, !F->batch_member, fn, static_cast<unsigned>(grid), (n / 2) * (TY / 2) + 32,
-                   restrict32t_smem(d.g.lg, mode, TY, TZ, D), 
-            d.u32, d.f32, d.kap, d.ih2_32, d.g.bs, c.f32, c.u32, d.xfer, c.g.nb, c.g.bs, skip_of(F, c), d.ax32, d.ay32,
-            d.az32, TY, TZ, D, F->kerr);
+                   restrict32t_smem(d.g.lg, mode, TY, TZ, D), d.u32, d.f32, d.kap, d.ih2_32, d.g.bs, c.f32, c.u32,
+                   d.xfer, c.g.nb, c.g.bs, skip_of(F, c), d.ax32, d.ay32, d.az32, TY, TZ, D, F->kerr);
         return;
     }
     // one coarse cell per thread (no grid-stride loop): its load chain xf -> fine block -> 64 loads is latency-bound
     const auto grid = static_cast<unsigned>((c.cells() + kThreads - 1) / kThreads);
     launch_pdl(F->st, !F->batch_member, kRestrict32[mode_index(mode32(F, d))][d.g.lg - 3], grid, kThreads, 0, d.u32,
                d.f32, d.kap, d.ih2_32, d.g.bs, c.f32, c.u32, d.xfer, c.g.nb, c.g.bs, skip_of(F, c), d.ax32, d.ay32,
-        d.az32);
+               d.az32);
 }
 
 void launch_prolong32(mg_forest *F, DevLevel &d, DevLevel &c, bool inject = false) {
     if (d.g.lg >= 5) {
         const auto grid = static_cast<unsigned>((c.cells() / kProlongZC + kThreads - 1) / kThreads);
         const Prolong32Fn fn = (inject ? kInject32z : kProlong32z)[d.g.lg - 5];
-        launch_pdl(F->st, !F->batch_member, fn, grid, kThreads, 0, d.u32, d.g.bs, c.u32, d.xfer, c.g.nb, c.g.bs,
-                   d.nbr6, skip_of(F, c));
+        launch_pdl(F->st, !F->batch_member, fn, grid, kThreads, 0, d.u32, d.g.bs, c.u32, d.xfer, c.g.nb, c.g.bs, d.nbr6,
+                   skip_of(F, c));
         return;
     }
     const Prolong32Fn fn = (inject ? kInject32 : kProlong32)[d.g.lg - 3];
@@ -412,8 +408,8 @@ const Prolong64Fn kProlong64[5] = {k_prolong64<3>, k_prolong64<4>, k_prolong64<5
 
 void launch_residual_restrict64(mg_forest *F, DevLevel &d, DevLevel &c) {
     launch_pdl(F->st, !F->batch_member, kRestrict64[F->cfg.coeff ? 1 : 0][d.g.lg - 3],
-               static_cast<unsigned>((c.cells() + kThreads - 1) / kThreads), kThreads, 0, d.u64, d.f64, d.c64(), d.ih2_64,
-               d.g.bs, c.f64, c.u64, d.xfer, c.cells(), c.g.bs, skip_of(F, c));
+               static_cast<unsigned>((c.cells() + kThreads - 1) / kThreads), kThreads, 0, d.u64, d.f64, d.c64(),
+               d.ih2_64, d.g.bs, c.f64, c.u64, d.xfer, c.cells(), c.g.bs, skip_of(F, c));
 }
 
 void launch_prolong64(mg_forest *F, DevLevel &d, DevLevel &c) {
@@ -435,9 +431,7 @@ void smooth(mg_forest *F, DevLevel &d, int colour) {
     if constexpr (sizeof(T) == 8)
         if (&d == &F->L[0]) gb = F->gb;
     launch_pdl(F->st, !F->batch_member, k_smooth<T, MODE>, grid_for(d.cells() / 2), kThreads, 0, ufield<T>(d),
-               ffield<T>(d), coef_of<T>(d),
-                                                                       h2_of<T>(d), d.g, colour, d.nbr6, skip_of(F, d),
-                                                                       gb);
+               ffield<T>(d), coef_of<T>(d), h2_of<T>(d), d.g, colour, d.nbr6, skip_of(F, d), gb);
 }
 
 void smooth_level32(mg_forest *F, DevLevel &d, int colour) {
@@ -542,8 +536,7 @@ struct LaunchExec {
             DevLevel &d = F->L[l];
             Prof p(F, prof ? cat_of<T>(l == 0 ? P_SMOOTH64_L0 : P_SMOOTH64) : -1, 1);
             launch_pdl(F->st, !F->batch_member, k_jacobi64<MODE>, grid_for(d.cells()), kThreads, 0, d.u64, d.u64b,
-                       d.f64, d.c64(), d.h2_64, d.g,
-                                                                          F->omega, skip_of(F, d));
+                       d.f64, d.c64(), d.h2_64, d.g, F->omega, skip_of(F, d));
             std::swap(d.u64, d.u64b);  // the new iterate; its ghosts are refreshed by the next exchange
         }
     }
@@ -565,8 +558,7 @@ struct LaunchExec {
         Prof p(F, cat_of<T>(P_COARSE64), 1);
         launch_pdl(F->st, !F->batch_member, k_coarse_solve<T>, (F->Nc * 32 + kThreads - 1) / kThreads, kThreads, 0,
                    ufield<T>(d), ffield<T>(d), F->Ainv, sizeof(T) == 4 ? F->cmap32 : F->cmap, F->uprob, F->ustart,
-                   F->moff,
-            F->Nc, done_mask(F));
+                   F->moff, F->Nc, done_mask(F));
     }
     void restrict_to(int l, bool fast) {
         DevLevel &d = F->L[l], &c = F->L[l + 1];
@@ -576,13 +568,12 @@ struct LaunchExec {
         else if (fast)
             launch_residual_restrict32(F, d, c);
         else if (sizeof(T) == 4 && d.face32)
-            launch_pdl(F->st, !F->batch_member, k_residual_restrict<float, 3>, grid_for(c.cells()), kThreads, 0,
-                       d.u32, d.f32, d.c32(), d.ih2_32, d.g, c.f32, c.u32, d.xfer, c.g, skip_of(F, c));
+            launch_pdl(F->st, !F->batch_member, k_residual_restrict<float, 3>, grid_for(c.cells()), kThreads, 0, d.u32,
+                       d.f32, d.c32(), d.ih2_32, d.g, c.f32, c.u32, d.xfer, c.g, skip_of(F, c));
         else
             launch_pdl(F->st, !F->batch_member, k_residual_restrict<T, MODE>, grid_for(c.cells()), kThreads, 0,
-                       ufield<T>(d), ffield<T>(d), coef_of<T>(d), ih2_of<T>(d), d.g, ffield<T>(c), ufield<T>(c),
-                       d.xfer, c.g,
-                skip_of(F, c));
+                       ufield<T>(d), ffield<T>(d), coef_of<T>(d), ih2_of<T>(d), d.g, ffield<T>(c), ufield<T>(c), d.xfer,
+                       c.g, skip_of(F, c));
     }
     void prolong_from(int l, bool fast) {
         DevLevel &d = F->L[l], &c = F->L[l + 1];
@@ -600,8 +591,7 @@ struct LaunchExec {
             launch_prolong32(F, d, c);
         else
             launch_pdl(F->st, !F->batch_member, k_prolong<T>, grid_for(c.cells()), kThreads, 0, ufield<T>(d), d.g,
-                       ufield<T>(c), d.xfer, c.g,
-                                                                      skip_of(F, c));
+                       ufield<T>(c), d.xfer, c.g, skip_of(F, c));
     }
 };
 
