@@ -28,7 +28,7 @@
 // step by step on natural-layout arrays of its own (the correction, its stencil with ghost adjoints, their scatter by
 // atomics over every face, two vector updates per half-sweep: ~70 B per cell and half-sweep) made set-up, forward solve and
 // adjoint on 448 + 512 blocks of 32^3 (31.5M cells) take 174 to 183 ms, depending on the inputs; this form, with the later
-// steps' kernels, 63 ms.
+// steps' kernels, 65 ms.
 #include <cmath>
 
 #include "forest_state.h"
@@ -187,7 +187,8 @@ __global__ void __launch_bounds__(kThreads)
 
 // Same-level faces with a coefficient on either side: row i of A^T has the neighbour's one, T_B, where the stencil has the
 // block's own, T_A, so f' takes (T_B - T_A) / h^2 times what changed of the value on the other side (old: what f' holds).
-// One thread per face cell of every item; the cells at a block's edges belong to several.
+// One thread per face cell of every item; the cells at a block's edges belong to several.  A launch of 3.7 us like the level's
+// others: 240 of them are 0.9 of 65 ms in a gradient on 448 + 512 blocks of 32^3 (31.5M cells).
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kThreads)
     k_adj_uneven(const T *__restrict__ y, Coef cf, const T *__restrict__ ih2, const FaceItem *__restrict__ items, int nitems,
@@ -609,7 +610,7 @@ __global__ void k_add(double *__restrict__ y, const double *__restrict__ x, Leve
 //     dL/dk_i = -h^2 / 2 sum_f (T~_f / k_i)^2 (lambda_i - lambda_f) (u_i - u_f),
 // where T~_f / k_i <= 2 / h^2 whatever the scale of k (T~_f^2 would overflow from k / h^2 = 2^512 on):
 // one division per cell (six in the form with (k_i + k_f)^2, and the other cell's share by atomics: 5.5 ms on 31.5M cells;
-// this one 2.4 ms, its 45 FP64 operations per cell at the measured FP64 rate).  Ghosts of u and lambda: copies and
+// this one 2.5 ms, its 51 FP64 operations per cell at the measured FP64 rate; ncu: FP64 pipe 86 % active).  Ghosts of u and lambda: copies and
 // reflections (at the boundary T = k_i, dT/dk_i = 1: the reflected pair gives the same).  Refinement interfaces are left to
 // k_gradk_iface.
 __global__ void k_gradk(const double *__restrict__ u, const double *__restrict__ lam, const double *__restrict__ k,

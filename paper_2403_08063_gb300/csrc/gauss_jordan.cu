@@ -294,7 +294,7 @@ __global__ void k_gj_transpose(const double *__restrict__ X, double *__restrict_
 // the pivot rows and one of its CTA's rows in registers; the W threads of a row share a warp, and the pivot row of a step
 // goes through one of two shared buffers (who writes a buffer again has passed the barrier after its last read).  The
 // operations and their order are those of k_gj_panel for a problem of kind GJ_DOMINANT.  Bound by the chain of a
-// shuffle, a reciprocal, a barrier and an update per column: about 9 us per panel, where the cluster's search takes 37 us with
+// shuffle, a reciprocal, a barrier and an update per column: 9.5 us per panel, where the cluster's search takes 37 us with
 // 512 unknowns and 46 us with 1728 (new coefficients and a solve on 128^3 cells 3.79 -> 2.94 ms, a gradient on 48^3 cells
 // with 1728 coarsest unknowns 13.8 -> 9.8 ms).
 constexpr int kGjRows = 16;
